@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -28,6 +29,31 @@ int graphs_enabled() {
     v = e ? (atoi(e) != 0) : 1;
   }
   return v && current_arena() == nullptr;
+}
+
+// Contexts alive; when the last one goes, the pool's kept blocks go back too.
+static std::atomic<int> g_contexts{0};
+
+void configure_pool_once() {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaMemPool_t pool;
+    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+      uint64_t thr = UINT64_MAX;
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+    }
+    cudaGetLastError();
+  });
+}
+
+static void trim_pool() {
+  int dev = 0;
+  cudaMemPool_t pool;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
+    cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
 }
 
 static cudaEvent_t pool_event(bri_ctx* c) {
@@ -165,6 +191,7 @@ int bri_create(bri_ctx** out, const int dims[4], int flags, void* stream) {
     delete c;
     return cuda_fail(e, "bri_create: cudaMallocHost");
   }
+  g_contexts.fetch_add(1);
   *out = c;
   return BRI_OK;
 }
@@ -195,6 +222,7 @@ void bri_destroy(bri_ctx* c) {
   cudaFreeHost(c->host_pinned);
   cudaGetLastError();
   delete c;
+  if (g_contexts.fetch_sub(1) == 1) trim_pool();
 }
 
 int bri_set_stream(bri_ctx* c, void* stream) {
@@ -408,12 +436,6 @@ int overlap_apply_batch(bri_ctx* const* ctxs, int nctx, void* const* ys, const v
   if (!std::isfinite(am) || am >= 2.0 * rho) {
     set_error("overlap_apply_batch: the traditional massive form needs am < 2 rho");
     return BRI_ERR_INVALID;
-  }
-  // autotune every lattice's stencil launches (used by the per-lattice
-  // refinement) first, one lattice at a time
-  for (int i = 0; i < nctx; ++i) {
-    int rc = pretune_stencils(ctxs[i], prec);
-    if (rc) return rc;
   }
   const double k = (1.0 - am / (2.0 * rho)) * rho;
   return batch_sign_apply(ctxs, nctx, ys, xs, nrhs, n, kind, rho, scale, tol, prec, k, k + am, st);

@@ -1,7 +1,9 @@
-// FP64 Brillouin stencil instantiation.
-#include "bri_kernel.cuh"
+// FP64 Brillouin stencil.
+#include "bri_split.cuh"
 
 namespace bri {
-template int launch_bri_t<double, double2>(const Geom&, double*, const double*, const double2*, const double*,
-                                           double, int, int, cudaStream_t, const ShiftDot<double>*, int*);
+int launch_bri_f64(const Geom& g, double* y, const double* x, const double2* W, const double* cl, double diag, int nrhs,
+                   int dagger, cudaStream_t s, const ShiftDot<double>* sd, int* sd_blocks) {
+  return launch_split<double, double2>(g, y, x, W, cl, diag, nrhs, dagger, s, sd, sd_blocks);
+}
 }  // namespace bri

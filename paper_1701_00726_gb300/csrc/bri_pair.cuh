@@ -1,0 +1,497 @@
+// Brillouin stencil on packed FP32 spinors: every 16-byte word holds one
+// complex number of two spinor components, (re_A, re_B, im_A, im_B), so that
+// fma.rn.f32x2 works on two components at a time with the link element
+// broadcast to both halves (a free operand form), a factor i only exchanges the
+// re and im registers (signs go into the scalar weights), and no register pair
+// has to be built or rotated.
+//
+//   two right-hand sides (RP): A, B = the two right-hand sides of a pair,
+//       [group][V/32][12][32] words, row 3 s + c (spin s, colour c);
+//   one right-hand side (SP):  A, B = the two spins of a chirality,
+//       [rhs][V/32][6][32] words, row 3 h + c (chirality h, colour c).
+//
+// A warp of 32 consecutive sites reads whole 512-byte rows without bank
+// conflicts at immediate offsets from one address (the array-of-structs spinor
+// costs a 96-byte stride: 1.7x the L1 wavefronts).
+//
+// D_bri x(n) = sum_{d != 0} W_d(n) M_d x(n+d) + (15/8 + m0) x(n) + C(n) x(n)   (Eq. def_bril, App. C)
+//
+// Per stored offset d the two opposite hops are taken together, in place:
+//   P = W_d(n) x(n+d),  V = W_d(n-d)^dagger x(n-d) - P,
+//   acc += 2 a_k P + a_k V - c_k sum_mu s_mu gamma_mu V
+// (a_k (P + Q) + c_k G (P - Q) with Q = V + P), so one colour-transported
+// spinor is live besides the accumulator.  The next offset's links are loaded
+// into the registers of the present ones as soon as those are dead.
+//
+// Bound: the FP32 pipe (432 paired FMAs per hop pair and pair of right-hand
+// sides; 71 % busy at 16^3 x 32, L1 46 %, DRAM 19 %), for one right-hand side
+// at 24^3 x 48 also the link stream.  GB300, packing pass included, against the
+// kernels before it (array-of-structs spinors, links as five strided streams):
+// 16^3 x 32, 12 rhs 1208 -> 1024 us; 24^3 x 48, 1 rhs 653 -> 578 us; BF16
+// links, 18.15.14.21, 3 rhs 278 -> 237 us.  Two right-hand sides per thread run
+// at 12 warps per SM (168 registers), one at 16 (128); more warps with spills
+// were slower (0.80 against 0.62 ns per site and rhs), as were blocks that
+// stage a 4D tile and its halo in shared memory (0.78: filling the halo takes
+// longer than the gathers it saves), branches around vanishing gamma terms
+// (0.71 against 0.65) and sites numbered by 4D tiles (0.69: rows of 8 sites
+// straddle more lines).
+#pragma once
+
+#include "hops.cuh"
+
+namespace bri {
+
+__device__ __forceinline__ float2 pr_bc(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 pr_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 pr_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 pr_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 pr_swp(float2 a) { return make_float2(a.y, a.x); }
+
+// One complex number of the two components of a word.
+struct CP {
+  float2 re, im;
+};
+__device__ __forceinline__ CP cp_of(const float4& v) { return CP{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+__device__ __forceinline__ float4 cp_word(const CP& v) { return make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
+// o += c v, o += i c v
+__device__ __forceinline__ void cp_add(CP& o, const CP& v, float c) {
+  o.re = pr_fma(v.re, pr_bc(c), o.re);
+  o.im = pr_fma(v.im, pr_bc(c), o.im);
+}
+__device__ __forceinline__ void cp_addi(CP& o, const CP& v, float c) {
+  o.re = pr_fma(v.im, pr_bc(-c), o.re);
+  o.im = pr_fma(v.re, pr_bc(c), o.im);
+}
+
+constexpr int kPackBlock = 32;
+// 16-byte words of one group (rows = 12: a pair of right-hand sides, 6: one)
+__host__ __device__ __forceinline__ int64_t packed_words(int64_t V, int rows) {
+  return (V + kPackBlock - 1) / kPackBlock * kPackBlock * rows;
+}
+template <int ROWS> __device__ __forceinline__ int packed_at(int m) {
+  return (m / kPackBlock) * (ROWS * kPackBlock) + m % kPackBlock;
+}
+
+// Per-offset data of the packed kernels: index of the stored offset,
+// displacement signs, a_k, and the gamma weights for V = -(P - Q), c_mu =
+// -(sign) c_k s_mu.  The offsets come with the most hops (the smallest
+// weights) first, so the accumulator stays small for most of its roundings
+// (relative error against FP64 at 16^3 x 32 and 24^3 x 48: 7.5e-8 sorted, 1.0e-7 in
+// storage order).
+struct PairHops {
+  int j[40];
+  int d[40][4];
+  float a[40];
+  float c[40][4];
+};
+inline const PairHops& pair_hops(int dagger) {
+  static const auto make = [](float sgn) {
+    PairHops t;
+    const HopTable<float>& h = hop_table<float>();
+    int i = 0;
+    for (int k = 4; k >= 1; --k)
+      for (int j = 0; j < 40; ++j) {
+        int hops = 0;
+        for (int mu = 0; mu < 4; ++mu) hops += h.site_d[j][mu] != 0;
+        if (hops != k) continue;
+        t.j[i] = j;
+        t.a[i] = h.a[j];
+        for (int mu = 0; mu < 4; ++mu) {
+          t.d[i][mu] = h.site_d[j][mu];
+          t.c[i][mu] = -sgn * h.cs[j][mu];
+        }
+        ++i;
+      }
+    return t;
+  };
+  static const PairHops t0 = make(1.f), t1 = make(-1.f);
+  return dagger ? t1 : t0;
+}
+
+// P = w x (rows of x: R spinor rows, component q at row 3 q + colour)
+template <int R> __device__ __forceinline__ void pr_fwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    CP v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) v[q] = cp_of(__ldg(x + (q * 3 + b) * kPackBlock));
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        const float2 wr = pr_bc(w[aa][b].re), wi = pr_bc(w[aa][b].im);
+        P[q][aa].re = b == 0 ? pr_mul(v[q].re, wr) : pr_fma(v[q].re, wr, P[q][aa].re);
+        P[q][aa].im = b == 0 ? pr_mul(v[q].re, wi) : pr_fma(v[q].re, wi, P[q][aa].im);
+      }
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        const float2 wr = pr_bc(w[aa][b].re), nw = pr_bc(-w[aa][b].im);
+        P[q][aa].im = pr_fma(v[q].im, wr, P[q][aa].im);
+        P[q][aa].re = pr_fma(v[q].im, nw, P[q][aa].re);
+      }
+    }
+  }
+}
+// P = w^dagger x - P
+template <int R> __device__ __forceinline__ void pr_bwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    CP v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) v[q] = cp_of(__ldg(x + (q * 3 + b) * kPackBlock));
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        const float2 wr = pr_bc(w[b][aa].re), nw = pr_bc(-w[b][aa].im);
+        P[q][aa].re = pr_fma(v[q].re, wr, b == 0 ? pr_neg(P[q][aa].re) : P[q][aa].re);
+        P[q][aa].im = pr_fma(v[q].re, nw, b == 0 ? pr_neg(P[q][aa].im) : P[q][aa].im);
+      }
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        const float2 wr = pr_bc(w[b][aa].re), wi = pr_bc(w[b][aa].im);
+        P[q][aa].im = pr_fma(v[q].im, wr, P[q][aa].im);
+        P[q][aa].re = pr_fma(v[q].im, wi, P[q][aa].re);
+      }
+    }
+  }
+}
+template <int R> __device__ __forceinline__ void pr_axpy(CP (&acc)[R][3], const CP (&v)[R][3], float k) {
+#pragma unroll
+  for (int q = 0; q < R; ++q)
+#pragma unroll
+    for (int aa = 0; aa < 3; ++aa) cp_add(acc[q][aa], v[q][aa], k);
+}
+// acc += sum_mu c_mu gamma_mu V, chiral basis (hops.cuh), on two right-hand sides
+__device__ __forceinline__ void pr_gamma(CP (&acc)[4][3], const CP (&v)[4][3], float c1, float c2, float c3, float c4) {
+#pragma unroll
+  for (int aa = 0; aa < 3; ++aa) {
+    cp_addi(acc[0][aa], v[3][aa], -c1);
+    cp_addi(acc[1][aa], v[2][aa], -c1);
+    cp_addi(acc[2][aa], v[1][aa], c1);
+    cp_addi(acc[3][aa], v[0][aa], c1);
+    cp_add(acc[0][aa], v[3][aa], -c2);
+    cp_add(acc[1][aa], v[2][aa], c2);
+    cp_add(acc[2][aa], v[1][aa], c2);
+    cp_add(acc[3][aa], v[0][aa], -c2);
+    cp_addi(acc[0][aa], v[2][aa], -c3);
+    cp_addi(acc[1][aa], v[3][aa], c3);
+    cp_addi(acc[2][aa], v[0][aa], c3);
+    cp_addi(acc[3][aa], v[1][aa], -c3);
+    cp_add(acc[0][aa], v[2][aa], c4);
+    cp_add(acc[1][aa], v[3][aa], c4);
+    cp_add(acc[2][aa], v[0][aa], c4);
+    cp_add(acc[3][aa], v[1][aa], c4);
+  }
+}
+// the same on two spins per word: gamma_1 and gamma_2 exchange the spins of a
+// chirality, gamma_3 and gamma_4 do not
+__device__ __forceinline__ void pr_gamma(CP (&acc)[2][3], const CP (&v)[2][3], float c1, float c2, float c3, float c4) {
+  const float2 p1 = pr_bc(c1), m1 = pr_bc(-c1), p4 = pr_bc(c4);
+  const float2 k2 = make_float2(-c2, c2), n2 = make_float2(c2, -c2), k3 = make_float2(c3, -c3), n3 = make_float2(-c3, c3);
+#pragma unroll
+  for (int aa = 0; aa < 3; ++aa) {
+    const float2 s0r = pr_swp(v[0][aa].re), s0i = pr_swp(v[0][aa].im);
+    const float2 s1r = pr_swp(v[1][aa].re), s1i = pr_swp(v[1][aa].im);
+    acc[0][aa].re = pr_fma(s1i, p1, acc[0][aa].re);
+    acc[0][aa].im = pr_fma(s1r, m1, acc[0][aa].im);
+    acc[1][aa].re = pr_fma(s0i, m1, acc[1][aa].re);
+    acc[1][aa].im = pr_fma(s0r, p1, acc[1][aa].im);
+    acc[0][aa].re = pr_fma(s1r, k2, acc[0][aa].re);
+    acc[0][aa].im = pr_fma(s1i, k2, acc[0][aa].im);
+    acc[1][aa].re = pr_fma(s0r, n2, acc[1][aa].re);
+    acc[1][aa].im = pr_fma(s0i, n2, acc[1][aa].im);
+    acc[0][aa].re = pr_fma(v[1][aa].im, k3, acc[0][aa].re);
+    acc[0][aa].im = pr_fma(v[1][aa].re, n3, acc[0][aa].im);
+    acc[1][aa].re = pr_fma(v[0][aa].im, n3, acc[1][aa].re);
+    acc[1][aa].im = pr_fma(v[0][aa].re, k3, acc[1][aa].im);
+    acc[0][aa].re = pr_fma(v[1][aa].re, p4, acc[0][aa].re);
+    acc[0][aa].im = pr_fma(v[1][aa].im, p4, acc[0][aa].im);
+    acc[1][aa].re = pr_fma(v[0][aa].re, p4, acc[1][aa].re);
+    acc[1][aa].im = pr_fma(v[0][aa].im, p4, acc[1][aa].im);
+  }
+}
+
+// Sum over the 80 hops at site n into acc; x = packed vector (R = 4: a pair of
+// right-hand sides, R = 2: one).
+template <int R, typename LS>
+__device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, const float4* __restrict__ x,
+                                        const LS* __restrict__ W, const PairHops& H) {
+  const int V = (int)g.V;
+  // index steps to the neighbours in each direction (periodic)
+  int up[4], dn[4];
+  {
+    int r = n;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const int L = g.L[mu], s = (int)g.str[mu];
+      const int c = mu < 3 ? r % L : r;
+      if (mu < 3) r /= L;
+      up[mu] = c == L - 1 ? -(L - 1) * s : s;
+      dn[mu] = c == 0 ? (L - 1) * s : -s;
+    }
+  }
+  auto sites = [&](int j, int& mp, int& mm) {
+    mp = n;
+    mm = n;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const int d = H.d[j][mu];
+      mp += d > 0 ? up[mu] : (d < 0 ? dn[mu] : 0);
+      mm += d > 0 ? dn[mu] : (d < 0 ? up[mu] : 0);
+    }
+  };
+#pragma unroll
+  for (int q = 0; q < R; ++q)
+#pragma unroll
+    for (int aa = 0; aa < 3; ++aa) acc[q][aa] = CP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  C<float> w[3][3], wm[3][3];
+  int mp, mm;
+  sites(0, mp, mm);
+  load_stored_link<float, LS>(w, W, H.j[0], n, V);
+  load_stored_link<float, LS>(wm, W, H.j[0], mm, V);
+#pragma unroll 1
+  for (int j = 0; j < 40; ++j) {
+    const int jn = j < 39 ? j + 1 : 39;
+    const float a = H.a[j];
+    const int op = packed_at<3 * R>(mp), om = packed_at<3 * R>(mm);
+    CP P[R][3];
+    pr_fwd<R>(P, x + op, w);
+    sites(jn, mp, mm);
+    load_stored_link<float, LS>(w, W, H.j[jn], n, V);
+    pr_axpy<R>(acc, P, 2.f * a);
+    pr_bwd<R>(P, x + om, wm);
+    load_stored_link<float, LS>(wm, W, H.j[jn], mm, V);
+    pr_axpy<R>(acc, P, a);
+    pr_gamma(acc, P, H.c[j][0], H.c[j][1], H.c[j][2], H.c[j][3]);
+  }
+}
+
+// Sum of v over the block (FP64, fixed order), valid in thread 0.
+__device__ __forceinline__ double pr_block_total(double v) {
+  __shared__ double sh[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
+  return t;
+}
+
+// Hermitian 6x6 clover block (6 diagonal reals, 15 upper complex, SoA) on a
+// pair of right-hand sides: o = C in.
+__device__ __forceinline__ void pr_clover(CP (&o)[6], const float* __restrict__ cl, int64_t V, int64_t n, const CP (&in)[6]) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const float2 d = pr_bc(__ldg(cl + (int64_t)i * V + n));
+    o[i] = CP{pr_mul(in[i].re, d), pr_mul(in[i].im, d)};
+  }
+  int k = 6;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i + 1; j < 6; ++j) {
+      const float r = __ldg(cl + (int64_t)k * V + n), m = __ldg(cl + (int64_t)(k + 1) * V + n);
+      cp_add(o[i], in[j], r);
+      cp_addi(o[i], in[j], m);
+      cp_add(o[j], in[i], r);
+      cp_addi(o[j], in[i], -m);
+      k += 2;
+    }
+}
+
+// y = D x on packed x.  OUT = 0: y in the spinors' own layout; 1: packed like x.
+// With EPI (OUT = 0): y = D x + sig_s p_s and the site block's partial of
+// Re<p_s, y> in part[s * blocks + block] (p in the spinors' own layout).
+// nrhs: right-hand sides of the whole vector (a pair's second one may not exist:
+// its half of the packed words is a copy, its results are dropped).
+template <int R, typename LS, int OUT, bool EPI>
+__global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
+    bri_pair_kernel(Geom g, float* __restrict__ y, float4* __restrict__ yp, const float4* __restrict__ x,
+                    const LS* __restrict__ W, const float* __restrict__ cl, float diag, int rhs0, int nrhs, int gfirst,
+                    const __grid_constant__ PairHops H, ShiftDot<float> sd) {
+  const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
+  const int n0 = blk * blockDim.x + threadIdx.x;
+  const bool valid = n0 < g.V;
+  if (!EPI && !valid) return;  // with the epilogue every thread takes part in the block's reduction
+  const int n = valid ? n0 : 0;
+  const int64_t rs = g.V * 24;
+  constexpr int NR = R / 2;                // right-hand sides of a word
+  const int s0 = rhs0 + grp * NR;
+  const float4* xg = x + (int64_t)grp * packed_words(g.V, 3 * R);
+  CP acc[R][3];
+  pr_hops<R, LS>(acc, g, n, xg, W, H);
+  const float4* xo = xg + packed_at<3 * R>(n);
+  const bool second = NR == 1 || s0 + 1 < nrhs;
+  double dots[2] = {0.0, 0.0};
+  if constexpr (R == 4) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      CP own[6], out[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        own[i] = cp_of(__ldg(xo + (h * 6 + i) * kPackBlock));
+        out[i] = acc[h * 2 + i / 3][i % 3];
+        cp_add(out[i], own[i], diag);
+      }
+      if (cl) {
+        CP co[6];
+        pr_clover(co, cl + (int64_t)h * 36 * g.V, g.V, n, own);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          out[i].re = make_float2(out[i].re.x + co[i].re.x, out[i].re.y + co[i].re.y);
+          out[i].im = make_float2(out[i].im.x + co[i].im.x, out[i].im.y + co[i].im.y);
+        }
+      }
+      if constexpr (OUT == 1) {
+        float4* yo = yp + (int64_t)grp * packed_words(g.V, 12) + packed_at<12>(n) + h * 6 * kPackBlock;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) yo[i * kPackBlock] = cp_word(out[i]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (r == 1 && !second) break;
+          float o[12];
+#pragma unroll
+          for (int i = 0; i < 6; ++i) {
+            o[2 * i] = r ? out[i].re.y : out[i].re.x;
+            o[2 * i + 1] = r ? out[i].im.y : out[i].im.x;
+          }
+          const int64_t at = (int64_t)(s0 + r) * rs + (int64_t)n * 24 + h * 12;
+          if constexpr (EPI) {
+            const float sg = (float)sd.sig[s0 + r];
+            const float4* pp = reinterpret_cast<const float4*>(sd.p + at);
+            float dt = 0.f;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              const float4 pv = __ldg(pp + i);
+              const float pe[4] = {pv.x, pv.y, pv.z, pv.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                o[4 * i + e] = fmaf(sg, pe[e], o[4 * i + e]);
+                dt = fmaf(pe[e], o[4 * i + e], dt);
+              }
+            }
+            dots[r] += (double)dt;
+          }
+          if (valid) {
+            float4* yo = reinterpret_cast<float4*>(y + at);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) yo[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+          }
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      C<float> in[6], out[6];
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        const CP own = cp_of(__ldg(xo + (h * 3 + aa) * kPackBlock));
+        cp_add(acc[h][aa], own, diag);
+        in[aa] = C<float>{own.re.x, own.im.x};
+        in[3 + aa] = C<float>{own.re.y, own.im.y};
+        out[aa] = C<float>{acc[h][aa].re.x, acc[h][aa].im.x};
+        out[3 + aa] = C<float>{acc[h][aa].re.y, acc[h][aa].im.y};
+      }
+      if (cl) {
+        C<float> co[6];
+        clover_block(co, cl + (int64_t)h * 36 * g.V, g.V, n, in);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) out[i] = out[i] + co[i];
+      }
+      if constexpr (OUT == 1) {
+        float4* yo = yp + (int64_t)grp * packed_words(g.V, 6) + packed_at<6>(n) + h * 3 * kPackBlock;
+#pragma unroll
+        for (int aa = 0; aa < 3; ++aa)
+          yo[aa * kPackBlock] = make_float4(out[aa].re, out[3 + aa].re, out[aa].im, out[3 + aa].im);
+      } else {
+        const int64_t at = (int64_t)s0 * rs + (int64_t)n * 24 + h * 12;
+        if constexpr (EPI) {
+          const float sg = (float)sd.sig[s0];
+          const float4* pp = reinterpret_cast<const float4*>(sd.p + at);
+          float dt = 0.f;
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            const float4 pv = __ldg(pp + i);
+            out[2 * i].re = fmaf(sg, pv.x, out[2 * i].re);
+            out[2 * i].im = fmaf(sg, pv.y, out[2 * i].im);
+            out[2 * i + 1].re = fmaf(sg, pv.z, out[2 * i + 1].re);
+            out[2 * i + 1].im = fmaf(sg, pv.w, out[2 * i + 1].im);
+            dt = fmaf(pv.x, out[2 * i].re, dt);
+            dt = fmaf(pv.y, out[2 * i].im, dt);
+            dt = fmaf(pv.z, out[2 * i + 1].re, dt);
+            dt = fmaf(pv.w, out[2 * i + 1].im, dt);
+          }
+          dots[0] += (double)dt;
+        }
+        if (valid) {
+          float4* yo = reinterpret_cast<float4*>(y + at);
+#pragma unroll
+          for (int i = 0; i < 3; ++i)
+            yo[i] = make_float4(out[2 * i].re, out[2 * i].im, out[2 * i + 1].re, out[2 * i + 1].im);
+        }
+      }
+    }
+  }
+  if constexpr (EPI) {
+    const int nb = gfirst ? gridDim.y : gridDim.x;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const double t = pr_block_total(valid ? dots[r] : 0.0);
+      if (threadIdx.x == 0 && (r == 0 || second)) sd.part[(int64_t)(s0 + r) * nb + blk] = t;
+    }
+  }
+}
+
+// Spinors [nrhs][V][12] complex64 -> packed groups; group g holds the
+// right-hand sides rhs0 + 2g, rhs0 + 2g + 1 (R = 4; the second repeats the
+// first where it does not exist) or rhs0 + g (R = 2).
+template <int R> __global__ void __launch_bounds__(256) k_pack(int64_t V, const float* __restrict__ x, int rhs0, int nrhs, float4* __restrict__ X) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // 16-byte word (R = 4) or spin pair (R = 2) of a site
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
+  if constexpr (R == 4) {
+    const int s = rhs0 + 2 * blockIdx.y;
+    const float* p = x + s * V * 24 + i * 4;
+    const float4 u = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 v = s + 1 < nrhs ? __ldg(reinterpret_cast<const float4*>(p + V * 24)) : u;
+    o[(2 * q) * kPackBlock] = make_float4(u.x, v.x, u.y, v.y);
+    o[(2 * q + 1) * kPackBlock] = make_float4(u.z, v.z, u.w, v.w);
+  } else {
+    const int h = q / 3, b = q - 3 * h;
+    const float2* p = reinterpret_cast<const float2*>(x + (rhs0 + (int64_t)blockIdx.y) * V * 24 + n * 24) + h * 6 + b;
+    const float2 u = __ldg(p), v = __ldg(p + 3);
+    o[q * kPackBlock] = make_float4(u.x, v.x, u.y, v.y);
+  }
+}
+
+template <int R>
+inline void launch_pack(int64_t V, const float* x, int rhs0, int nrhs, int groups, float4* X, cudaStream_t s) {
+  k_pack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, x, rhs0, nrhs, X);
+  note_launch();
+}
+
+// y (or packed yp) = D x for `groups` packed groups starting at right-hand side rhs0.
+template <int R, typename LS>
+inline void launch_pair(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
+                        int dagger, int rhs0, int nrhs, int groups, cudaStream_t s, const ShiftDot<float>* sd) {
+  const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
+  const ShiftDot<float> none{nullptr, nullptr, nullptr};
+  if (sd)
+    bri_pair_kernel<R, LS, 0, true><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), *sd);
+  else if (yp)
+    bri_pair_kernel<R, LS, 1, false><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), none);
+  else
+    bri_pair_kernel<R, LS, 0, false><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), none);
+  note_launch();
+}
+
+}  // namespace bri

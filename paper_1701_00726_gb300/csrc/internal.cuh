@@ -66,10 +66,9 @@ struct bri_ctx {
   double c_sw = 0.0;
   // kernel operator of the overlap solvers: BRI_KERNEL_BRILLOUIN or BRI_KERNEL_WILSON
   int kernel = BRI_KERNEL_BRILLOUIN;
-  // Stored off-axis links, structure-of-arrays: FP64 and BF16 [40][9][V]
-  // complex, element (nu, e, n) at (nu*9 + e)*V + n; FP32 [40][5][V] pairs of
-  // complex (elements 2k, 2k+1 in one 16-byte word, tenth slot padding).  A
-  // warp of consecutive sites reads one contiguous segment per load.
+  // Stored off-axis links, structure-of-arrays: FP64 [40][9][V] complex,
+  // element (nu, e, n) at (nu*9 + e)*V + n; FP32 and BF16 in chunks of 32
+  // sites (load_stored_link).
   double2* W64 = nullptr;
   float2* W32 = nullptr;
   __nv_bfloat162* W16 = nullptr;
@@ -122,7 +121,6 @@ int dirac_bri(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagge
               cudaStream_t s);
 int dirac_wil(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec,
               cudaStream_t s);
-// The solver's fused D^dagger application: y = D^dagger x + sigma_s p_s and the
 // Double-word FP32 Brillouin stencil (bri_dw.cu): y = D x or D^dagger x on
 // double-word vectors ([nrhs][V][12] float4), FP64 in and out through the
 // split/join kernels (tmp: two double-word vectors of nrhs right-hand sides),
@@ -133,6 +131,7 @@ int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int da
 int dirac_bri_dw64(bri_ctx* c, double* y, const double* x, int nrhs, double m0, int dagger, void* tmp,
                    cudaStream_t s);
 int normal_op_dw(bri_ctx* c, double* out, const double* x, int nrhs, double m0, void* t1, void* t2, cudaStream_t s);
+// The solver's fused D^dagger application: y = D^dagger x + sigma_s p_s and the
 // per-site-block partials of Re<p_s, y> (Brillouin kernel only); sd_blocks
 // receives the number of partials per system (part: [nrhs][sd_blocks]).
 int dirac_bri_shiftdot(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int prec, cudaStream_t s,
@@ -141,9 +140,15 @@ int dirac_bri_shiftdot(bri_ctx* c, void* y, const void* x, int nrhs, double m0, 
 // the Brillouin stencil (Eq. def_bril) or the Wilson stencil (Eq. def_wils).
 int dirac_kernel(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec,
                  cudaStream_t s);
-// Makes the stencil autotuner's choices for this lattice (every rhs class and
-// precision a solve of precision prec uses) before concurrent work starts.
-int pretune_stencils(bri_ctx* c, int prec);
+// The FP32 stencil on packed vectors (bri_f32_on_packed): y or yp = D X or
+// D^dagger X for the first na of nrhs right-hand sides; with p the fused
+// epilogue of dirac_bri_shiftdot.
+int dirac_bri_packed(bri_ctx* c, float* y, void* yp, const void* X, int nrhs, int na, double m0, int dagger, int prec,
+                     cudaStream_t s, const float* p = nullptr, const double* sig = nullptr, double* part = nullptr,
+                     int* sd_blocks = nullptr);
+// Keeps freed blocks of the device's stream-ordered pool for the next
+// allocation (set once; the memory goes back when the last context is destroyed).
+void configure_pool_once();
 
 // Device scratch from a caller-provided block (used by the entry point that
 // allocates nothing); when no arena is set the solvers allocate from the

@@ -8,8 +8,7 @@
 //    (nu = 1..40; W_{82-nu}(n) = W_nu(n + d)^dagger) in FP64, FP32 and BF16;
 //  * the clover term -(c_SW/2) sum_{mu<nu} sigma_{mu nu} F_{mu nu} (Eq. def_bril)
 //    in the chiral basis, two Hermitian 6x6 blocks per site.
-#include "internal.cuh"
-#include "cplx.cuh"
+#include "stencil.cuh"
 
 namespace bri {
 namespace {
@@ -148,16 +147,34 @@ __global__ void levelk_kernel(Geom g, const double2* __restrict__ U64, double2* 
   store_soa(T + (int64_t)nu * 9 * g.V, g.V, n, acc);
 }
 
-// FP32 copy in the paired layout [40][5][V] float4 (elements 2k, 2k+1 of one
-// site in one 16-byte word); BF16 copy in the FP64 layout [40][9][V].
-__global__ void narrow_links_kernel(int64_t count, const double2* __restrict__ W64, float2* W32,
-                                    __nv_bfloat162* W16, int64_t V) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  double2 v = W64[i];
-  const int64_t nu9e = i / V, n = i - nu9e * V, nu = nu9e / 9, e = nu9e - nu * 9;
-  W32[((nu * 5 + e / 2) * V + n) * 2 + (e & 1)] = make_float2((float)v.x, (float)v.y);
-  W16[i] = __floats2bfloat162_rn((float)v.x, (float)v.y);
+// FP32 and BF16 copies of one stored link per thread, in the packed layouts
+// that load_stored_link reads.
+__global__ void narrow_links_kernel(int64_t V, const double2* __restrict__ W64, float2* W32, __nv_bfloat162* W16) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= 40 * V) return;
+  const int64_t j = i / V, n = i - j * V;
+  float2 f[9];
+  unsigned h[9];
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    const double2 v = W64[(j * 9 + e) * V + n];
+    f[e] = make_float2((float)v.x, (float)v.y);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(f[e].x, f[e].y);
+    memcpy(&h[e], &b, 4);
+  }
+  const int64_t blk = n / kLinkBlock * 40 + j;
+  const int lane = (int)(n % kLinkBlock);
+  char* q = reinterpret_cast<char*>(W32) + blk * (kLinkBlock * kLinkBytes32);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    reinterpret_cast<float4*>(q)[k * kLinkBlock + lane] =
+        make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y);
+  reinterpret_cast<float2*>(q + 64 * kLinkBlock)[lane] = f[8];
+  char* s = reinterpret_cast<char*>(W16) + blk * (kLinkBlock * kLinkBytes16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    reinterpret_cast<uint4*>(s)[k * kLinkBlock + lane] = make_uint4(h[4 * k], h[4 * k + 1], h[4 * k + 2], h[4 * k + 3]);
+  reinterpret_cast<unsigned*>(s + 32 * kLinkBlock)[lane] = h[8];
 }
 
 // ------------------------------------------------------------------ clover
@@ -290,8 +307,8 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
   };
   int rc;
   if ((rc = alloc((void**)&c->W64, sizeof(double2) * 360 * V))) return rc;
-  if ((rc = alloc((void**)&c->W32, sizeof(float2) * 400 * V))) return rc;
-  if ((rc = alloc((void**)&c->W16, sizeof(__nv_bfloat162) * 360 * V))) return rc;
+  if ((rc = alloc((void**)&c->W32, kLinkBytes32 * kLinkBlock * 40 * link_blocks(V)))) return rc;
+  if ((rc = alloc((void**)&c->W16, kLinkBytes16 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->U64, sizeof(double2) * 36 * V))) return rc;
   if ((rc = alloc((void**)&c->U32, sizeof(float2) * 36 * V))) return rc;
   double2* T = nullptr;
@@ -302,7 +319,7 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
                                                        (c->flags & BRI_ANTIPERIODIC_T) ? 1 : 0); note_launch();
   if ((rc = build_transporters(c, T))) return rc;
   BRI_CUDA(cudaMemcpyAsync(c->W64, T, sizeof(double2) * 360 * V, cudaMemcpyDeviceToDevice, st));
-  narrow_links_kernel<<<blocks_for(360 * V, 256), 256, 0, st>>>(360 * V, c->W64, c->W32, c->W16, V); note_launch();
+  narrow_links_kernel<<<blocks_for(40 * V, 128), 128, 0, st>>>(V, c->W64, c->W32, c->W16); note_launch();
   BRI_LAUNCH_CHECK("narrow_links_kernel");
   c->have_clover = false;
   c->dw_valid = false;

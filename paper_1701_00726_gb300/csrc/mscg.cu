@@ -28,7 +28,8 @@
 // per-system shift, hardest systems first, and converged systems drop out.
 #include "internal.cuh"
 #include "cplx.cuh"
-#include "bri_kernel.cuh"
+#include "bri_pair.cuh"
+#include "bri_site.cuh"
 
 #include <algorithm>
 #include <chrono>
@@ -320,6 +321,52 @@ __global__ void k_update_p0(int64_t n2, const MsState* __restrict__ st, const ty
     pv.x = fma(bt, pv.x, rv.x);
     pv.y = fma(bt, pv.y, rv.y);
     p[s * n2 + i] = pv;
+  }
+}
+
+// The same with the packed copy X of the directions (bri_pair.cuh: pairs of
+// systems, then the odd one) written in the same pass: the next application of
+// D reads X.  One thread per site and 16-byte word (R = 4) or spin pair (R = 2).
+template <int R>
+__global__ void __launch_bounds__(256) k_update_p0_packed(int64_t V, int s0, const MsState* __restrict__ st,
+                                                          const float* __restrict__ r, float* __restrict__ p,
+                                                          float4* __restrict__ X) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
+  if constexpr (R == 4) {
+    const int s = s0 + 2 * blockIdx.y;
+    const bool da = st[s].done, db = st[s + 1].done;
+    if (da && db) return;
+    float4 v[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int64_t at = (s + k) * V * 24 + i * 4;
+      v[k] = *reinterpret_cast<const float4*>(p + at);
+      if (k ? db : da) continue;
+      const float bt = (float)st[s + k].b_s[0];
+      const float4 rv = __ldg(reinterpret_cast<const float4*>(r + at));
+      v[k] = make_float4(fmaf(bt, v[k].x, rv.x), fmaf(bt, v[k].y, rv.y), fmaf(bt, v[k].z, rv.z), fmaf(bt, v[k].w, rv.w));
+      *reinterpret_cast<float4*>(p + at) = v[k];
+    }
+    o[(2 * q) * kPackBlock] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
+    o[(2 * q + 1) * kPackBlock] = make_float4(v[0].z, v[1].z, v[0].w, v[1].w);
+  } else {
+    const int s = s0 + blockIdx.y;
+    if (st[s].done) return;
+    const float bt = (float)st[s].b_s[0];
+    const int64_t at = s * V * 24 + n * 24 + 2 * (q + 3 * (q / 3));  // spins 2h, 2h + 1 of colour q % 3, h = q / 3
+    float2 v[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float2* pp = reinterpret_cast<float2*>(p + at) + 3 * k;
+      const float2 rv = __ldg(reinterpret_cast<const float2*>(r + at) + 3 * k);
+      v[k] = make_float2(fmaf(bt, pp->x, rv.x), fmaf(bt, pp->y, rv.y));
+      *pp = v[k];
+    }
+    o[q * kPackBlock] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
   }
 }
 
@@ -770,20 +817,6 @@ struct DevBuf {
   template <typename T> T* as() const { return (T*)p; }
 };
 
-void configure_pool_once() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-      uint64_t thr = UINT64_MAX;
-      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-    }
-    cudaGetLastError();
-  });
-}
-
 // Operator application for the solver: out = D in (dagger 0) / D^dagger in.
 template <typename R> int op_prec(int prec);
 template <> int op_prec<double>(int) { return BRI_PREC_F64; }
@@ -806,7 +839,9 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   int rc;
   if ((rc = br.alloc(sizeof(T) * n2 * nsys, st))) return rc;
   if ((rc = bp.alloc(sizeof(T) * n2 * nsys * nshift, st))) return rc;
-  if ((rc = bt.alloc(sizeof(T) * n2 * nsys, st))) return rc;
+  // t may hold a packed vector (whole blocks of 32 sites)
+  const size_t t_bytes = sizeof(R) == 4 ? std::max(sizeof(T) * n2 * nsys, bri_f32_packed_bytes(c->g.V, nsys)) : sizeof(T) * n2 * nsys;
+  if ((rc = bt.alloc(t_bytes, st))) return rc;
   if ((rc = bq.alloc(sizeof(T) * n2 * nsys, st))) return rc;
   if ((rc = bst.alloc(sizeof(MsState) * nsys, st))) return rc;
   if ((rc = bpart.alloc(sizeof(double) * nblk * nsys, st))) return rc;
@@ -833,6 +868,11 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   // and the partials of Re<p_0, q> come out of the stencil's epilogue, so
   // k_shift_dot's pass over q and p_0 is not needed.
   const bool fused = op == nullptr && c->kernel == BRI_KERNEL_BRILLOUIN;
+  // FP32 solves large enough for the packed stencil keep p_0 and t = D p_0 in
+  // its layout: D writes t packed, the direction update writes p_0 both ways.
+  const bool packed = sizeof(R) == 4 && fused && bri_f32_packed(c->g.V, nsys);
+  DevBuf bpk;
+  if (packed && (rc = bpk.alloc(bri_f32_packed_bytes(c->g.V, nsys), st))) return rc;
   // Deferred shifted updates (FP32 solve with FP64 solutions): the shifted
   // directions and solutions are advanced every DW iterations from a ring of
   // the residuals of those iterations (same arithmetic, fewer passes).
@@ -849,7 +889,7 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   for (int s = 0; s < nsys; ++s) hsig[s] = hs[s].sig_base;
   if (fused) {
     if ((rc = bsig.alloc(sizeof(double) * nsys, st))) return rc;
-    if ((rc = bpart_sd.alloc(sizeof(double) * nsys * (size_t)blocks_for(c->g.V, 64), st))) return rc;
+    if ((rc = bpart_sd.alloc(sizeof(double) * nsys * (size_t)blocks_for(c->g.V, kMinSiteBlock), st))) return rc;
     BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));
   }
   dim3 vg(nblk, nsys);
@@ -860,6 +900,7 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   note_launch();
   k_scalar_init<<<nsys, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
   BRI_LAUNCH_CHECK("multishift init");
+  if (packed && (rc = bri_f32_pack(c->g.V, (const float*)p, nsys, bpk.p, st))) return rc;
 
   int* hdone = (int*)c->host_pinned;  // pinned scratch, >= 4 KB
   const int check_every = 8;
@@ -880,10 +921,17 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
         if ((q = op->apply((double2*)t, (const double2*)p, na, 0))) return q;
         if ((q = op->apply((double2*)q_vec, (const double2*)t, na, 1))) return q;
       } else if (fused) {
-        if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) return q;
         int nb = 0;
-        if ((q = dirac_bri_shiftdot(c, q_vec, t, na, m0, oprec, st, p, bsig.as<double>(), bpart_sd.as<double>(), &nb)))
+        if (packed) {
+          if ((q = dirac_bri_packed(c, nullptr, t, bpk.p, nsys, na, m0, 0, oprec, st))) return q;
+          if ((q = dirac_bri_packed(c, (float*)q_vec, nullptr, t, nsys, na, m0, 1, oprec, st, (const float*)p,
+                                    bsig.as<double>(), bpart_sd.as<double>(), &nb)))
+            return q;
+        } else if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) {
           return q;
+        } else if ((q = dirac_bri_shiftdot(c, q_vec, t, na, m0, oprec, st, p, bsig.as<double>(), bpart_sd.as<double>(), &nb))) {
+          return q;
+        }
         k_scalar_alpha<<<na, RED_THREADS, 0, st>>>(S, bpart_sd.as<double>(), nb, hist); note_launch();
       } else {
         if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) return q;
@@ -903,7 +951,21 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
         k_update_fused<R><<<vga, RED_THREADS, 0, st>>>(n2, nsys, S, q_vec, r, p, (T*)x, part, it0 + j == 0 ? 1 : 0);
       note_launch();
       k_scalar_beta<<<na, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
-      k_update_p0<R><<<vga, RED_THREADS, 0, st>>>(n2, S, r, p); note_launch();
+      if (packed) {
+        const int pairs = nsys / 2, act = std::min(pairs, (na + 1) / 2);
+        const int vb = blocks_for(c->g.V * 6, 256);
+        if (act) {
+          k_update_p0_packed<4><<<dim3(vb, act), 256, 0, st>>>(c->g.V, 0, S, (const float*)r, (float*)p, bpk.as<float4>());
+          note_launch();
+        }
+        if (nsys % 2 && na == nsys) {
+          k_update_p0_packed<2><<<dim3(vb, 1), 256, 0, st>>>(c->g.V, nsys - 1, S, (const float*)r, (float*)p,
+                                                             bpk.as<float4>() + packed_words(c->g.V, 12) * pairs);
+          note_launch();
+        }
+      } else {
+        k_update_p0<R><<<vga, RED_THREADS, 0, st>>>(n2, S, r, p); note_launch();
+      }
       if (defer && ((j + 1) % DW == 0 || j == count - 1)) {
         k_flush_shifts<<<vga, RED_THREADS, 0, st>>>(n2, nsys, hist, (const float2*)bring.p, (float2*)p,
                                                     (double2*)x64);

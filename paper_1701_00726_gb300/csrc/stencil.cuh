@@ -4,8 +4,6 @@
 #include "internal.cuh"
 #include "cplx.cuh"
 
-#include <mutex>
-
 namespace bri {
 
 template <typename R> struct Spinor {
@@ -68,21 +66,46 @@ __device__ __forceinline__ void load_link(C<R> w[3][3], const LS* __restrict__ p
   }
 }
 
-// Stored link of offset j at site m.  FP64 and BF16 links are [40][9][V]
-// (element e at (j*9 + e)*V + m); FP32 links pair consecutive elements in one
-// 16-byte word, [40][5][V] float4 (elements 2k, 2k+1; the tenth slot is
-// padding), so a link takes five 16-byte loads instead of nine 8-byte ones.
+// Stored link of offset j at site m.  FP64 links are [40][9][V] (element e at
+// (j*9 + e)*V + m).  FP32 and BF16 links come in blocks of 32 sites, one
+// contiguous chunk per offset and block: four (two) rows of 32 16-byte words
+// holding elements 2k, 2k+1 (4k..4k+3), then a row of 32 words with the ninth
+// element.  A link takes five (three) wide loads at immediate offsets from one
+// address, and a warp reads one contiguous 2304-byte (1152-byte) chunk.
+constexpr int kLinkBlock = 32;
+constexpr int kLinkBytes32 = 72, kLinkBytes16 = 36;
+__host__ __device__ __forceinline__ int64_t link_blocks(int64_t V) { return (V + kLinkBlock - 1) / kLinkBlock; }
+
 template <typename R, typename LS>
 __device__ __forceinline__ void load_stored_link(C<R> w[3][3], const LS* __restrict__ W, int j, int m, int V) {
   if constexpr (sizeof(R) == 4 && sizeof(LS) == 8) {
-    const float4* q = reinterpret_cast<const float4*>(W) + (int64_t)j * 5 * V + m;
+    const char* q = reinterpret_cast<const char*>(W) +
+                    ((int64_t)(m / kLinkBlock) * 40 + j) * (kLinkBlock * kLinkBytes32);
+    const int lane = m % kLinkBlock;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const float4 v = __ldg(q + (int64_t)k * V);
+    for (int k = 0; k < 4; ++k) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(q) + k * kLinkBlock + lane);
       const int e0 = 2 * k, e1 = 2 * k + 1;
       w[e0 / 3][e0 % 3] = C<R>{v.x, v.y};
-      if (e1 < 9) w[e1 / 3][e1 % 3] = C<R>{v.z, v.w};
+      w[e1 / 3][e1 % 3] = C<R>{v.z, v.w};
     }
+    const float2 v = __ldg(reinterpret_cast<const float2*>(q + 64 * kLinkBlock) + lane);
+    w[2][2] = C<R>{v.x, v.y};
+  } else if constexpr (sizeof(LS) == 4) {
+    const char* q = reinterpret_cast<const char*>(W) +
+                    ((int64_t)(m / kLinkBlock) * 40 + j) * (kLinkBlock * kLinkBytes16);
+    const int lane = m % kLinkBlock;
+    const unsigned last = __ldg(reinterpret_cast<const unsigned*>(q + 32 * kLinkBlock) + lane);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(q) + k * kLinkBlock + lane);
+      const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)  // BF16 is the upper half of an FP32 word
+        w[(4 * k + i) / 3][(4 * k + i) % 3] =
+            C<R>{(R)__uint_as_float(u[i] << 16), (R)__uint_as_float(u[i] & 0xffff0000u)};
+    }
+    w[2][2] = C<R>{(R)__uint_as_float(last << 16), (R)__uint_as_float(last & 0xffff0000u)};
   } else {
     load_link<R, LS>(w, W + (int64_t)j * 9 * V + m, V);
   }
@@ -126,23 +149,6 @@ __device__ __forceinline__ void add_clover(Spinor<R>& acc, const Spinor<R>& x, c
   }
 }
 
-// Whether FP32 stencils carry two right-hand sides per thread (shared link
-// loads); BRI_PAIR_RHS=0 turns it off.
-int pair_rhs_enabled();
-// Stencil autotuning (BRI_AUTOTUNE=0 disables it) and its process-wide cache.
-int autotune_enabled();
-// Launch configuration of the FP32 stencil: pairs = 0 one right-hand side per
-// thread, 1 two per thread (shared link loads), 2 the paired-FP32 kernel
-// (bri_c2.cuh, one per thread); and the block size.
-struct StencilConfig {
-  int pairs = 1;
-  int threads = 128;
-  int rg = 1;  // right-hand sides on consecutive lanes (shared link loads), instead of pairs
-};
-bool tune_lookup(const char* key, StencilConfig* out);
-void tune_store(const char* key, const StencilConfig& cf);
-std::mutex& tune_mutex();
-
 // Fused solver epilogue of a stencil launch: q = D x + sigma_s p_s at every
 // site, and per block the partial sums of Re<p_s, q> in FP64 (the inner
 // product of the multi-shift CG), written to part[s * blocks + site block] for
@@ -166,10 +172,25 @@ inline StencilGrid stencil_grid(int64_t site_blocks, int groups) {
   return StencilGrid{dim3((unsigned)site_blocks, (unsigned)groups), 0};
 }
 
-// Host-side launchers (one translation unit per precision).
-template <typename R, typename LS>
-int launch_bri_t(const Geom& g, R* y, const R* x, const LS* W, const R* cl, R diag, int nrhs, int dagger,
-                 cudaStream_t s, const ShiftDot<R>* sd = nullptr, int* sd_blocks = nullptr);
+// Host-side launchers (one translation unit per precision).  sd (optional): the
+// fused solver epilogue; sd_blocks receives the number of its partials per
+// system, at most blocks_for(V, kMinSiteBlock).
+constexpr int kMinSiteBlock = 8;
+int launch_bri_f64(const Geom& g, double* y, const double* x, const double2* W, const double* cl, double diag, int nrhs,
+                   int dagger, cudaStream_t s, const ShiftDot<double>* sd = nullptr, int* sd_blocks = nullptr);
+template <typename LS>
+int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const float* cl, float diag, int nrhs,
+                   int dagger, cudaStream_t s, const ShiftDot<float>* sd = nullptr, int* sd_blocks = nullptr);
+// Packed FP32 vectors (bri_pair.cuh) for callers that keep their vectors in that
+// form: whether a launch of nrhs right-hand sides takes the packed kernels, the
+// size of such a vector, packing, and the operator on it (spinors' layout y or
+// packed yp out, first na of nrhs right-hand sides).
+bool bri_f32_packed(int64_t V, int nrhs);
+size_t bri_f32_packed_bytes(int64_t V, int nrhs);
+int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s);
+template <typename LS>
+int bri_f32_on_packed(const Geom& g, float* y, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs,
+                      int na, int dagger, cudaStream_t s, const ShiftDot<float>* sd = nullptr, int* sd_blocks = nullptr);
 template <typename R, typename LS>
 int launch_wil_t(const Geom& g, R* y, const R* x, const LS* U, const R* cl, R diag, int nrhs, int dagger,
                  cudaStream_t s);
