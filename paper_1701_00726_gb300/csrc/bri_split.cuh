@@ -126,18 +126,17 @@ __global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
     o.im = fma(diag, xe.im, o.im);
     if (cl) {  // row of the packed Hermitian 6x6 block (clover_block)
       const int h = e / 6, row = e - 6 * h;
-      const R* c = cl + (int64_t)h * 36 * V + n;
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
         const C<R> xk = xn[6 * h + k];
         if (k == row) {
-          const R d = c[(int64_t)k * V];
+          const R d = clover_real(cl, V, n, h, k);
           o.re = fma(d, xk.re, o.re);
           o.im = fma(d, xk.im, o.im);
         } else {
           const int i0 = min(k, row), j0 = max(k, row);
           const int at = 6 + 2 * (i0 * 5 - i0 * (i0 - 1) / 2 + j0 - i0 - 1);
-          C<R> cij{c[(int64_t)at * V], c[(int64_t)(at + 1) * V]};
+          C<R> cij{clover_real(cl, V, n, h, at), clover_real(cl, V, n, h, at + 1)};
           if (k < row) cij.im = -cij.im;
           cfma(o, cij, xk);
         }

@@ -72,11 +72,12 @@ struct bri_ctx {
   double2* W64 = nullptr;
   float2* W32 = nullptr;
   __nv_bfloat162* W16 = nullptr;
-  // Thin links with the time boundary applied, [4][9][V] (Wilson kernel).
+  // Thin links with the time boundary applied (Wilson kernel): FP64 [4][9][V],
+  // FP32 in chunks of 32 sites like the off-axis links.
   double2* U64 = nullptr;
   float2* U32 = nullptr;
-  // Clover: two Hermitian 6x6 chiral blocks per site, packed as 72 reals:
-  // [block][36][V]: 6 diagonal reals, then 15 upper off-diagonal complex.
+  // Clover: two Hermitian 6x6 chiral blocks per site, packed as 72 reals (6
+  // diagonal, then 15 upper off-diagonal complex per block; load_clover).
   double* C64 = nullptr;
   float* C32 = nullptr;
   // Double-word FP32 copies (h, l) of W64 and C64 for the FP64-class stencil

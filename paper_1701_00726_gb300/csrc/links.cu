@@ -55,21 +55,33 @@ __device__ __forceinline__ void store_soa(double2* base, int64_t V, int64_t n, c
   for (int e = 0; e < 9; ++e) base[(int64_t)e * V + n] = make_double2(m.m[e / 3][e % 3].re, m.m[e / 3][e % 3].im);
 }
 
-// AoS caller layout [V][4][3][3] complex128 -> SoA [4][9][V] FP64 and FP32,
-// with the antiperiodic sign on U_t of the last time slice.
+// One FP32 link into row-of-32 chunk c at lane (load_link_chunk's layout).
+__device__ __forceinline__ void store_link_chunk(float2* W, int64_t c, int lane, const float2 (&f)[9]) {
+  char* q = reinterpret_cast<char*>(W) + c * (kLinkBlock * kLinkBytes32);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    reinterpret_cast<float4*>(q)[k * kLinkBlock + lane] = make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y);
+  reinterpret_cast<float2*>(q + 64 * kLinkBlock)[lane] = f[8];
+}
+
+// AoS caller layout [V][4][3][3] complex128 -> SoA [4][9][V] FP64 and chunked
+// FP32, with the antiperiodic sign on U_t of the last time slice.
 __global__ void thin_links_kernel(Geom g, const double2* __restrict__ U, double2* U64, float2* U32, int anti) {
   int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= g.V) return;
   int t = (int)(n / g.str[3]);
   for (int mu = 0; mu < 4; ++mu) {
     double sgn = (anti && mu == 3 && t == g.L[3] - 1) ? -1.0 : 1.0;
+    float2 f[9];
+#pragma unroll
     for (int e = 0; e < 9; ++e) {
       double2 v = U[(n * 4 + mu) * 9 + e];
       v.x *= sgn;
       v.y *= sgn;
       U64[((int64_t)mu * 9 + e) * g.V + n] = v;
-      U32[((int64_t)mu * 9 + e) * g.V + n] = make_float2((float)v.x, (float)v.y);
+      f[e] = make_float2((float)v.x, (float)v.y);
     }
+    store_link_chunk(U32, n / kLinkBlock * 4 + mu, (int)(n % kLinkBlock), f);
   }
 }
 
@@ -164,12 +176,7 @@ __global__ void narrow_links_kernel(int64_t V, const double2* __restrict__ W64, 
   }
   const int64_t blk = n / kLinkBlock * 40 + j;
   const int lane = (int)(n % kLinkBlock);
-  char* q = reinterpret_cast<char*>(W32) + blk * (kLinkBlock * kLinkBytes32);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    reinterpret_cast<float4*>(q)[k * kLinkBlock + lane] =
-        make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y);
-  reinterpret_cast<float2*>(q + 64 * kLinkBlock)[lane] = f[8];
+  store_link_chunk(W32, blk, lane, f);
   char* s = reinterpret_cast<char*>(W16) + blk * (kLinkBlock * kLinkBytes16);
 #pragma unroll
   for (int k = 0; k < 2; ++k)
@@ -252,15 +259,15 @@ __global__ void clover_kernel(Geom g, const double2* __restrict__ U64, double c_
     int64_t base = (int64_t)blk * 36;
     for (int i = 0; i < 6; ++i) {
       C64[(base + i) * g.V + n] = full[i][i].re;
-      C32[(base + i) * g.V + n] = (float)full[i][i].re;
+      C32[clover_at32(n, blk, i)] = (float)full[i][i].re;
     }
     int k = 6;
     for (int i = 0; i < 6; ++i)
       for (int j = i + 1; j < 6; ++j) {
         C64[(base + k) * g.V + n] = full[i][j].re;
         C64[(base + k + 1) * g.V + n] = full[i][j].im;
-        C32[(base + k) * g.V + n] = (float)full[i][j].re;
-        C32[(base + k + 1) * g.V + n] = (float)full[i][j].im;
+        C32[clover_at32(n, blk, k)] = (float)full[i][j].re;
+        C32[clover_at32(n, blk, k + 1)] = (float)full[i][j].im;
         k += 2;
       }
   }
@@ -310,7 +317,7 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
   if ((rc = alloc((void**)&c->W32, kLinkBytes32 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->W16, kLinkBytes16 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->U64, sizeof(double2) * 36 * V))) return rc;
-  if ((rc = alloc((void**)&c->U32, sizeof(float2) * 36 * V))) return rc;
+  if ((rc = alloc((void**)&c->U32, kLinkBytes32 * kLinkBlock * 4 * link_blocks(V)))) return rc;
   double2* T = nullptr;
   if ((rc = alloc((void**)&T, sizeof(double2) * 81 * 9 * V))) return rc;
 
@@ -326,7 +333,7 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
   c->c_sw = c_sw;
   if (c_sw != 0.0) {
     if ((rc = alloc((void**)&c->C64, sizeof(double) * 72 * V))) return rc;
-    if ((rc = alloc((void**)&c->C32, sizeof(float) * 72 * V))) return rc;
+    if ((rc = alloc((void**)&c->C32, sizeof(float4) * clover_words32(V)))) return rc;
     clover_kernel<<<blocks_for(V, 64), 64, 0, st>>>(g, c->U64, c_sw, c->C64, c->C32); note_launch();
     BRI_LAUNCH_CHECK("clover_kernel");
     c->have_clover = true;

@@ -76,21 +76,25 @@ constexpr int kLinkBlock = 32;
 constexpr int kLinkBytes32 = 72, kLinkBytes16 = 36;
 __host__ __device__ __forceinline__ int64_t link_blocks(int64_t V) { return (V + kLinkBlock - 1) / kLinkBlock; }
 
+// FP32 link j of the n a block of sites holds (40 stored off-axis links, 4 thin links).
+template <int N> __device__ __forceinline__ void load_link_chunk(C<float> w[3][3], const float2* __restrict__ W, int j, int m) {
+  const char* q = reinterpret_cast<const char*>(W) + ((int64_t)(m / kLinkBlock) * N + j) * (kLinkBlock * kLinkBytes32);
+  const int lane = m % kLinkBlock;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(q) + k * kLinkBlock + lane);
+    const int e0 = 2 * k, e1 = 2 * k + 1;
+    w[e0 / 3][e0 % 3] = C<float>{v.x, v.y};
+    w[e1 / 3][e1 % 3] = C<float>{v.z, v.w};
+  }
+  const float2 v = __ldg(reinterpret_cast<const float2*>(q + 64 * kLinkBlock) + lane);
+  w[2][2] = C<float>{v.x, v.y};
+}
+
 template <typename R, typename LS>
 __device__ __forceinline__ void load_stored_link(C<R> w[3][3], const LS* __restrict__ W, int j, int m, int V) {
   if constexpr (sizeof(R) == 4 && sizeof(LS) == 8) {
-    const char* q = reinterpret_cast<const char*>(W) +
-                    ((int64_t)(m / kLinkBlock) * 40 + j) * (kLinkBlock * kLinkBytes32);
-    const int lane = m % kLinkBlock;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(q) + k * kLinkBlock + lane);
-      const int e0 = 2 * k, e1 = 2 * k + 1;
-      w[e0 / 3][e0 % 3] = C<R>{v.x, v.y};
-      w[e1 / 3][e1 % 3] = C<R>{v.z, v.w};
-    }
-    const float2 v = __ldg(reinterpret_cast<const float2*>(q + 64 * kLinkBlock) + lane);
-    w[2][2] = C<R>{v.x, v.y};
+    load_link_chunk<40>(w, W, j, m);
   } else if constexpr (sizeof(LS) == 4) {
     const char* q = reinterpret_cast<const char*>(W) +
                     ((int64_t)(m / kLinkBlock) * 40 + j) * (kLinkBlock * kLinkBytes16);
@@ -113,21 +117,47 @@ __device__ __forceinline__ void load_stored_link(C<R> w[3][3], const LS* __restr
 
 __device__ __forceinline__ int wrap(int c, int L) { return c < 0 ? c + L : (c >= L ? c - L : c); }
 
-// Packed Hermitian 6x6 times a 6-vector: diag reals [0..5], then upper complex.
-template <typename R>
-__device__ __forceinline__ void clover_block(C<R> out[6], const R* __restrict__ cl, int64_t V, int64_t n,
-                                             const C<R> in[6]) {
+// Clover storage: per chirality 36 reals (6 diagonal, then 15 upper
+// off-diagonal complex, row by row).  FP64 [2][36][V]; FP32 in chunks of 32
+// sites, [V/32][2][9][32] words of 16 bytes (reals 4r..4r+3 of a block).
+constexpr int kCloverBlock = 32;
+__host__ __device__ __forceinline__ int64_t clover_words32(int64_t V) { return (V + kCloverBlock - 1) / kCloverBlock * kCloverBlock * 18; }
+__device__ __forceinline__ int64_t clover_at32(int64_t n, int h, int k) {
+  return (((n / kCloverBlock * 18 + 9 * h + k / 4) * kCloverBlock) + n % kCloverBlock) * 4 + k % 4;
+}
+__device__ __forceinline__ double clover_real(const double* __restrict__ cl, int64_t V, int64_t n, int h, int k) {
+  return __ldg(cl + ((int64_t)h * 36 + k) * V + n);
+}
+__device__ __forceinline__ float clover_real(const float* __restrict__ cl, int64_t, int64_t n, int h, int k) {
+  return __ldg(cl + clover_at32(n, h, k));
+}
+// The 36 reals of block h at site n.
+__device__ __forceinline__ void load_clover(double (&c)[36], const double* __restrict__ cl, int64_t V, int64_t n, int h) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    R d = __ldg(cl + (int64_t)i * V + n);
-    out[i] = C<R>{d * in[i].re, d * in[i].im};
+  for (int k = 0; k < 36; ++k) c[k] = clover_real(cl, V, n, h, k);
+}
+__device__ __forceinline__ void load_clover(float (&c)[36], const float* __restrict__ cl, int64_t V, int64_t n, int h) {
+  const float4* q = reinterpret_cast<const float4*>(cl + clover_at32(n, h, 0));
+#pragma unroll
+  for (int r = 0; r < 9; ++r) {
+    const float4 v = __ldg(q + r * kCloverBlock);
+    c[4 * r] = v.x;
+    c[4 * r + 1] = v.y;
+    c[4 * r + 2] = v.z;
+    c[4 * r + 3] = v.w;
   }
+}
+// out = C in for one chirality block.
+template <typename R>
+__device__ __forceinline__ void clover_block(C<R> out[6], const R (&c)[36], const C<R> in[6]) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) out[i] = C<R>{c[i] * in[i].re, c[i] * in[i].im};
   int k = 6;
 #pragma unroll
   for (int i = 0; i < 6; ++i)
 #pragma unroll
     for (int j = i + 1; j < 6; ++j) {
-      C<R> cij{__ldg(cl + (int64_t)k * V + n), __ldg(cl + (int64_t)(k + 1) * V + n)};
+      const C<R> cij{c[k], c[k + 1]};
       cfma(out[i], cij, in[j]);
       cfma_cj(out[j], cij, in[i]);
       k += 2;
@@ -141,9 +171,11 @@ __device__ __forceinline__ void add_clover(Spinor<R>& acc, const Spinor<R>& x, c
 #pragma unroll
   for (int blk = 0; blk < 2; ++blk) {
     C<R> in[6], out[6];
+    R c[36];
+    load_clover(c, cl, V, n, blk);
 #pragma unroll
     for (int i = 0; i < 6; ++i) in[i] = x.v[2 * blk + i / 3][i % 3];
-    clover_block(out, cl + (int64_t)blk * 36 * V, V, n, in);
+    clover_block(out, c, in);
 #pragma unroll
     for (int i = 0; i < 6; ++i) acc.v[2 * blk + i / 3][i % 3] = acc.v[2 * blk + i / 3][i % 3] + out[i];
   }

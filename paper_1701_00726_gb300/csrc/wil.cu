@@ -1,6 +1,14 @@
 // Wilson stencil (Eq. def_wils) with spin projection (App. C, Wilson operator
 // flop count): for each of the 8 hops the 4-spinor is projected to 2 spin
 // components with (1 -+ gamma_mu), transported, and rebuilt.
+//
+// The FP32 kernel is bound by HBM (thin links 288, clover 288 and two spinors of
+// 96 bytes per site): links and clover come in 16-byte words of 32-site chunks
+// and serve NR right-hand sides per thread.  GB300, 24^3 x 48, 2 rhs, clover:
+// 302 us with element-wise link and clover streams read once per right-hand
+// side, 168 us now (3.8 TB/s of the bytes it cannot do without); one rhs per
+// thread 176 us at 5 blocks per SM, 206 us unbounded; two 176 us unbounded,
+// 197 us at 5 blocks.
 #include "stencil.cuh"
 
 namespace bri {
@@ -81,25 +89,29 @@ __device__ __forceinline__ void reconstruct(Spinor<R>& acc, const C<R> uh[2][3])
   }
 }
 
-template <int MU, typename R, typename LS, bool DAG>
-__device__ __forceinline__ void wil_dir(Spinor<R>& acc, const R* __restrict__ xin, const LS* __restrict__ U,
+__device__ __forceinline__ void load_thin(C<double> u[3][3], const double2* __restrict__ U, int mu, int64_t m, int64_t V) {
+#pragma unroll
+  for (int e = 0; e < 9; ++e) u[e / 3][e % 3] = ld2(U + ((int64_t)mu * 9 + e) * V + m);
+}
+__device__ __forceinline__ void load_thin(C<float> u[3][3], const float2* __restrict__ U, int mu, int64_t m, int64_t) {
+  load_link_chunk<4>(u, U, mu, (int)m);
+}
+
+// forward: -1/2 (1 - gamma_mu) U_mu(n) x(n+mu); backward: -1/2 (1 + gamma_mu) U_mu(n-mu)^+ x(n-mu)
+// (dagger swaps the two projectors).
+template <int MU, int NR, typename R, typename LS, bool DAG>
+__device__ __forceinline__ void wil_dir(Spinor<R> (&acc)[NR], const R* __restrict__ xin, int64_t rs, const LS* __restrict__ U,
                                         int64_t V, int64_t n, const Nb<R>& nb) {
-  // forward: -1/2 (1 - gamma_mu) U_mu(n) x(n+mu); backward: -1/2 (1 + gamma_mu) U_mu(n-mu)^+ x(n-mu)
-  // (dagger swaps the two projectors).
-  int64_t mf = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][2];
-  int64_t mb = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][0];
-  {
+  const int64_t mf = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][2];
+  const int64_t mb = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][0];
+  C<R> u[3][3];
+  load_thin(u, U, MU, n, V);
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
     Spinor<R> xs;
-    load_spinor(xs, xin + mf * 24);
+    load_spinor(xs, xin + r * rs + mf * 24);
     C<R> h[2][3], uh[2][3];
     project<MU, DAG>(xs, h);
-    C<R> u[3][3];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      C<float> f;
-      if constexpr (sizeof(R) == 8) u[e / 3][e % 3] = ld2(reinterpret_cast<const double2*>(U) + ((int64_t)MU * 9 + e) * V + n);
-      else { f = ld2(U + ((int64_t)MU * 9 + e) * V + n); u[e / 3][e % 3] = C<R>{(R)f.re, (R)f.im}; }
-    }
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -108,20 +120,15 @@ __device__ __forceinline__ void wil_dir(Spinor<R>& acc, const R* __restrict__ xi
 #pragma unroll
         for (int b = 0; b < 3; ++b) cfma(uh[s][a], u[a][b], h[s][b]);
       }
-    reconstruct<MU, DAG>(acc, uh);
+    reconstruct<MU, DAG>(acc[r], uh);
   }
-  {
+  load_thin(u, U, MU, mb, V);
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
     Spinor<R> xs;
-    load_spinor(xs, xin + mb * 24);
+    load_spinor(xs, xin + r * rs + mb * 24);
     C<R> h[2][3], uh[2][3];
     project<MU, !DAG>(xs, h);
-    C<R> u[3][3];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      C<float> f;
-      if constexpr (sizeof(R) == 8) u[e / 3][e % 3] = ld2(reinterpret_cast<const double2*>(U) + ((int64_t)MU * 9 + e) * V + mb);
-      else { f = ld2(U + ((int64_t)MU * 9 + e) * V + mb); u[e / 3][e % 3] = C<R>{(R)f.re, (R)f.im}; }
-    }
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
@@ -130,31 +137,67 @@ __device__ __forceinline__ void wil_dir(Spinor<R>& acc, const R* __restrict__ xi
 #pragma unroll
         for (int b = 0; b < 3; ++b) cfma_cj(uh[s][a], u[b][a], h[s][b]);
       }
-    reconstruct<MU, !DAG>(acc, uh);
+    reconstruct<MU, !DAG>(acc[r], uh);
   }
 }
 
-template <typename R, typename LS, bool DAG, bool CLOV>
-__global__ void __launch_bounds__(128) wil_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x,
+template <typename R, typename LS, int NR, bool DAG, bool CLOV>
+__global__ void __launch_bounds__(128, sizeof(R) == 8 ? 1 : (NR == 2 ? 4 : 5)) wil_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, int rhs0,
                                                   const LS* __restrict__ U, const R* __restrict__ cl, R diag) {
   const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= g.V) return;
-  const int64_t rhs_off = (int64_t)blockIdx.y * g.V * 24;
+  const int64_t rs = g.V * 24, rhs_off = (rhs0 + (int64_t)blockIdx.y * NR) * rs;
   const R* xin = x + rhs_off;
   Nb<R> nb;
   neighbours(g, n, nb);
-  Spinor<R> acc, xc;
-  load_spinor(xc, xin + n * 24);
+  Spinor<R> acc[NR];
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+  for (int r = 0; r < NR; ++r) {
+    Spinor<R> xc;
+    load_spinor(xc, xin + r * rs + n * 24);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) acc.v[s][a] = diag * xc.v[s][a];
-  wil_dir<0, R, LS, DAG>(acc, xin, U, g.V, n, nb);
-  wil_dir<1, R, LS, DAG>(acc, xin, U, g.V, n, nb);
-  wil_dir<2, R, LS, DAG>(acc, xin, U, g.V, n, nb);
-  wil_dir<3, R, LS, DAG>(acc, xin, U, g.V, n, nb);
-  if constexpr (CLOV) add_clover(acc, xc, cl, g.V, n);
-  store_spinor(y + rhs_off + n * 24, acc);
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) acc[r].v[s][a] = diag * xc.v[s][a];
+  }
+  wil_dir<0, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
+  wil_dir<1, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
+  wil_dir<2, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
+  wil_dir<3, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
+  if constexpr (CLOV) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      R c[36];
+      load_clover(c, cl, g.V, n, h);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const C<R>* xn = reinterpret_cast<const C<R>*>(xin + r * rs + n * 24) + 6 * h;
+        C<R> in[6], out[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) in[i] = xn[i];
+        clover_block(out, c, in);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) acc[r].v[2 * h + i / 3][i % 3] = acc[r].v[2 * h + i / 3][i % 3] + out[i];
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < NR; ++r) store_spinor(y + rhs_off + r * rs + n * 24, acc[r]);
+}
+
+template <typename R, typename LS, int NR>
+void launch_wil_nr(const Geom& g, R* y, const R* x, int rhs0, int groups, const LS* U, const R* cl, R diag, int dagger,
+                   cudaStream_t s) {
+  const int th = 128;
+  const dim3 grid(blocks_for(g.V, th), groups);
+  if (dagger) {
+    if (cl) wil_kernel<R, LS, NR, true, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    else wil_kernel<R, LS, NR, true, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+  } else {
+    if (cl) wil_kernel<R, LS, NR, false, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    else wil_kernel<R, LS, NR, false, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+  }
+  note_launch();
 }
 
 }  // namespace
@@ -162,16 +205,10 @@ __global__ void __launch_bounds__(128) wil_kernel(Geom g, R* __restrict__ y, con
 template <typename R, typename LS>
 int launch_wil_t(const Geom& g, R* y, const R* x, const LS* U, const R* cl, R diag, int nrhs, int dagger,
                  cudaStream_t s) {
-  const int th = 128;
-  dim3 grid(blocks_for(g.V, th), nrhs);
-  if (dagger) {
-    if (cl) wil_kernel<R, LS, true, true><<<grid, th, 0, s>>>(g, y, x, U, cl, diag);
-    else wil_kernel<R, LS, true, false><<<grid, th, 0, s>>>(g, y, x, U, cl, diag);
-  } else {
-    if (cl) wil_kernel<R, LS, false, true><<<grid, th, 0, s>>>(g, y, x, U, cl, diag);
-    else wil_kernel<R, LS, false, false><<<grid, th, 0, s>>>(g, y, x, U, cl, diag);
-  }
-  note_launch();
+  constexpr int NR = sizeof(R) == 4 ? 2 : 1;
+  const int groups = nrhs / NR;
+  if (groups) launch_wil_nr<R, LS, NR>(g, y, x, 0, groups, U, cl, diag, dagger, s);
+  if (nrhs > groups * NR) launch_wil_nr<R, LS, 1>(g, y, x, groups * NR, nrhs - groups * NR, U, cl, diag, dagger, s);
   BRI_LAUNCH_CHECK("wil_kernel");
   return BRI_OK;
 }
