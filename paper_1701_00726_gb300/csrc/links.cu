@@ -1,13 +1,22 @@
 // Link preparation (once per gauge configuration):
 //  * thin links with the time boundary applied, structure-of-arrays;
-//  * the 80 path-averaged off-axis transporters W_d(n) (App. C: average over
-//    the k! shortest paths, no SU(3) back-projection), built level by level
+//  * the 40 stored path-averaged off-axis transporters W_d(n) (App. C: average
+//    over the k! shortest paths, no SU(3) back-projection), built level by level
 //    with the last-step recursion
 //        W_d(n) = (1/k) sum_{mu: d_mu != 0} W_{d - s_mu e_mu}(n) U_step(n + d - s_mu e_mu, mu, s_mu)
-//    which groups the k! paths by their final hop; 40 of them are kept
-//    (nu = 1..40; W_{82-nu}(n) = W_nu(n + d)^dagger) in FP64, FP32 and BF16;
+//    which groups the k! paths by their final hop; a lower transporter that is
+//    not stored is the mirrored one, W_{82-nu}(n) = W_nu(n + d)^dagger.  FP64, and
+//    FP32 and BF16 copies from the same registers;
 //  * the clover term -(c_SW/2) sum_{mu<nu} sigma_{mu nu} F_{mu nu} (Eq. def_bril)
-//    in the chiral basis, two Hermitian 6x6 blocks per site.
+//    in the chiral basis, two Hermitian 6x6 blocks per site, its leaves products
+//    of the two-hop paths of the link construction.
+//
+// The construction is bound by FP64 arithmetic (104 products of 3x3 complex
+// matrices per site for the links, 24 for the clover leaves: 2.9 ms at 16^3 x 32
+// at the measured FP64 rate).  GB300, 16^3 x 32 with clover, construction and
+// export of the stored links: 10.6 ms with all 80 transporters in a scratch array
+// (allocated and freed on each call), twelve products per clover plane and a
+// strided export, 4.4 ms now.
 #include "stencil.cuh"
 
 namespace bri {
@@ -118,9 +127,19 @@ LevelList level_list(int k) {
   return lst;
 }
 
+// The stored ones among them (nu <= 40).
+static LevelList stored_level(int k) {
+  LevelList all = level_list(k), lst;
+  lst.count = 0;
+  for (int i = 0; i < all.count; ++i)
+    if (all.nu[i] < 40) lst.nu[lst.count++] = all.nu[i];
+  return lst;
+}
+
 namespace {
 
-// k-hop transporters from (k-1)-hop ones at the same site (last-step recursion).
+// k-hop transporters from (k-1)-hop ones at the same site (last-step recursion),
+// all 80 offsets (the adjoint's recursion needs them).
 __global__ void levelk_kernel(Geom g, const double2* __restrict__ U64, double2* T, LevelList lst, int k) {
   int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int which = blockIdx.y;
@@ -159,18 +178,17 @@ __global__ void levelk_kernel(Geom g, const double2* __restrict__ U64, double2* 
   store_soa(T + (int64_t)nu * 9 * g.V, g.V, n, acc);
 }
 
-// FP32 and BF16 copies of one stored link per thread, in the packed layouts
-// that load_stored_link reads.
-__global__ void narrow_links_kernel(int64_t V, const double2* __restrict__ W64, float2* W32, __nv_bfloat162* W16) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= 40 * V) return;
-  const int64_t j = i / V, n = i - j * V;
+// One stored link: FP64 structure-of-arrays element planes and the FP32 and BF16
+// chunks that load_stored_link reads.
+__device__ __forceinline__ void store_link(double2* W64, float2* W32, __nv_bfloat162* W16, int64_t V, int64_t n, int j,
+                                           const M3<double>& m) {
   float2 f[9];
   unsigned h[9];
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
-    const double2 v = W64[(j * 9 + e) * V + n];
-    f[e] = make_float2((float)v.x, (float)v.y);
+    const C<double> v = m.m[e / 3][e % 3];
+    W64[((int64_t)j * 9 + e) * V + n] = make_double2(v.re, v.im);
+    f[e] = make_float2((float)v.re, (float)v.im);
     const __nv_bfloat162 b = __floats2bfloat162_rn(f[e].x, f[e].y);
     memcpy(&h[e], &b, 4);
   }
@@ -184,44 +202,123 @@ __global__ void narrow_links_kernel(int64_t V, const double2* __restrict__ W64, 
   reinterpret_cast<unsigned*>(s + 32 * kLinkBlock)[lane] = h[8];
 }
 
-// ------------------------------------------------------------------ clover
-__device__ __forceinline__ M3<double> linkU(const Geom& g, const double2* U64, const SiteCoord& s, int mu,
-                                            int dx, int dy, int dz, int dt) {
-  int64_t m = displaced(g, s, dx, dy, dz, dt);
-  return load_soa(U64 + (int64_t)mu * 9 * g.V, g.V, m);
+// acc += a b, and acc += a b^dagger
+__device__ __forceinline__ void mmac(M3<double>& acc, const M3<double>& a, const M3<double>& b) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cfma(acc.m[i][j], a.m[i][k], b.m[k][j]);
+}
+__device__ __forceinline__ void mzero(M3<double>& a) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) a.m[i][j] = C<double>{0.0, 0.0};
 }
 
-// F_{mu nu}(n): traceless part of (Q - Q^dagger)/(8i), Q the sum of the four
-// counter-clockwise plaquette leaves around n in the (mu, nu) plane.
-__device__ M3<double> field_strength(const Geom& g, const double2* U64, const SiteCoord& s, int mu, int nu) {
-  int em[4] = {0, 0, 0, 0}, en[4] = {0, 0, 0, 0};
-  em[mu] = 1;
-  en[nu] = 1;
-#define SH(a, b) (a * em[0] + b * en[0]), (a * em[1] + b * en[1]), (a * em[2] + b * en[2]), (a * em[3] + b * en[3])
+// One step of a path from the site n + at: U_mu(n + at) or U_mu(n + at - mu)^dagger.
+__device__ __forceinline__ M3<double> path_step(const Geom& g, const double2* __restrict__ U64, const SiteCoord& s,
+                                                const int at[4], int mu, int sg) {
+  int q[4] = {at[0], at[1], at[2], at[3]};
+  if (sg < 0) q[mu] -= 1;
+  const M3<double> u = load_soa(U64 + (int64_t)mu * 9 * g.V, g.V, displaced(g, s, q[0], q[1], q[2], q[3]));
+  return sg > 0 ? u : adj(u);
+}
+
+// The stored one-hop links W_{-mu}(n) = U_mu(n - mu)^dagger (offset lists hold
+// the stored offsets of one level).
+__global__ void stored1_kernel(Geom g, const double2* __restrict__ U64, double2* W64, float2* W32, __nv_bfloat162* W16) {
+  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (n >= g.V) return;
+  const SiteCoord s = coords(g, n);
+  const int mu = blockIdx.y;
+  const int zero[4] = {0, 0, 0, 0};
+  int e[4] = {0, 0, 0, 0};
+  e[mu] = -1;
+  store_link(W64, W32, W16, g.V, n, nu_of(e[0], e[1], e[2], e[3]), path_step(g, U64, s, zero, mu, -1));
+}
+
+// Stored k-hop links from the (k-1)-hop ones, one thread per site and offset.
+// With AB (two-hop level, clover wanted) the two paths of the offset d =
+// s1 e_mu + s2 e_nu, mu < nu, go to AB[2 * entry][9][V] (mu first) and
+// AB[2 * entry + 1] (nu first).
+__global__ void __launch_bounds__(128) storedk_kernel(Geom g, const double2* __restrict__ U64, double2* W64, float2* W32,
+                                                      __nv_bfloat162* W16, LevelList lst, int k, double2* AB) {
+  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (n >= g.V) return;
+  const int which = blockIdx.y, nu = lst.nu[which];
+  const int d[4] = {nu % 3 - 1, (nu / 3) % 3 - 1, (nu / 9) % 3 - 1, (nu / 27) % 3 - 1};
+  const SiteCoord s = coords(g, n);
+  M3<double> acc;
+  mzero(acc);
+  int path = 0;
+#pragma unroll 1
+  for (int mu = 3; mu >= 0; --mu) {  // last hop; two hops: last hop nu (mu first) comes first
+    if (d[mu] == 0) continue;
+    int dp[4] = {d[0], d[1], d[2], d[3]};
+    dp[mu] = 0;
+    const int at = nu_of(dp[0], dp[1], dp[2], dp[3]);
+    const int64_t m = at < 40 ? n : displaced(g, s, dp[0], dp[1], dp[2], dp[3]);
+    M3<double> w = load_soa(W64 + (int64_t)(at < 40 ? at : 80 - at) * 9 * g.V, g.V, m);
+    if (at > 40) w = adj(w);
+    const M3<double> u = path_step(g, U64, s, dp, mu, d[mu]);
+    if (AB) {
+      M3<double> p;
+      mzero(p);
+      mmac(p, w, u);
+      store_soa(AB + (int64_t)(2 * which + path) * 9 * g.V, g.V, n, p);
+      madd(acc, p);
+      ++path;
+    } else {
+      mmac(acc, w, u);
+    }
+  }
+  const double inv = 1.0 / k;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) acc.m[i][j] = inv * acc.m[i][j];
+  store_link(W64, W32, W16, g.V, n, nu, acc);
+}
+
+// ------------------------------------------------------------------ clover
+// F_{mu nu}(n), mu < nu: traceless part of (Q - Q^dagger)/(8i), Q the sum of the
+// four counter-clockwise plaquette leaves around n in the (mu, nu) plane.  With
+// A_d, B_d the two paths of a stored offset (mu first, nu first):
+//   Q = A_-(n) B_-(n)^+ + B_-(m)^+ A_-(m) + B_+(n) A_+(n)^+ + A_+(p)^+ B_+(p),
+// d_- = (-mu, -nu), m = n + mu + nu, d_+ = (+mu, -nu), p = n + nu - mu.
+__device__ __forceinline__ M3<double> field_strength(const Geom& g, const double2* __restrict__ AB, const LevelList& two,
+                                                     const SiteCoord& s, int64_t n, int mu, int nu) {
+  int em[4] = {0, 0, 0, 0}, ep[4] = {0, 0, 0, 0}, tm[4] = {0, 0, 0, 0}, tp[4] = {0, 0, 0, 0};
+  em[mu] = -1; em[nu] = -1; ep[mu] = 1; ep[nu] = -1;
+  tm[mu] = 1; tm[nu] = 1; tp[mu] = -1; tp[nu] = 1;
+  const int im = nu_of(em[0], em[1], em[2], em[3]), ip = nu_of(ep[0], ep[1], ep[2], ep[3]);
+  int km = 0, kp = 0;
+  for (int i = 0; i < two.count; ++i) {
+    if (two.nu[i] == im) km = i;
+    if (two.nu[i] == ip) kp = i;
+  }
+  auto ld = [&](int entry, int path, int64_t m) { return load_soa(AB + (int64_t)(2 * entry + path) * 9 * g.V, g.V, m); };
   M3<double> q;
-  // l1 = U_mu(n) U_nu(n+mu) U_mu(n+nu)^+ U_nu(n)^+
-  q = mmul(mmul(linkU(g, U64, s, mu, SH(0, 0)), linkU(g, U64, s, nu, SH(1, 0))),
-           mmul(adj(linkU(g, U64, s, mu, SH(0, 1))), adj(linkU(g, U64, s, nu, SH(0, 0)))));
-  // l2 = U_nu(n) U_mu(n+nu-mu)^+ U_nu(n-mu)^+ U_mu(n-mu)
-  madd(q, mmul(mmul(linkU(g, U64, s, nu, SH(0, 0)), adj(linkU(g, U64, s, mu, SH(-1, 1)))),
-               mmul(adj(linkU(g, U64, s, nu, SH(-1, 0))), linkU(g, U64, s, mu, SH(-1, 0)))));
-  // l3 = U_mu(n-mu)^+ U_nu(n-mu-nu)^+ U_mu(n-mu-nu) U_nu(n-nu)
-  madd(q, mmul(mmul(adj(linkU(g, U64, s, mu, SH(-1, 0))), adj(linkU(g, U64, s, nu, SH(-1, -1)))),
-               mmul(linkU(g, U64, s, mu, SH(-1, -1)), linkU(g, U64, s, nu, SH(0, -1)))));
-  // l4 = U_nu(n-nu)^+ U_mu(n-nu) U_nu(n-nu+mu) U_mu(n)^+
-  madd(q, mmul(mmul(adj(linkU(g, U64, s, nu, SH(0, -1))), linkU(g, U64, s, mu, SH(0, -1))),
-               mmul(linkU(g, U64, s, nu, SH(1, -1)), adj(linkU(g, U64, s, mu, SH(0, 0))))));
-#undef SH
+  mzero(q);
+  mmac(q, ld(km, 0, n), adj(ld(km, 1, n)));
+  const int64_t m = displaced(g, s, tm[0], tm[1], tm[2], tm[3]);
+  mmac(q, adj(ld(km, 1, m)), ld(km, 0, m));
+  mmac(q, ld(kp, 1, n), adj(ld(kp, 0, n)));
+  const int64_t p = displaced(g, s, tp[0], tp[1], tp[2], tp[3]);
+  mmac(q, adj(ld(kp, 0, p)), ld(kp, 1, p));
   M3<double> f;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       // (Q - Q^+)_{ij} / (8i) = -i (Q_ij - conj(Q_ji)) / 8
-      C<double> a = q.m[i][j] - conj(q.m[j][i]);
+      const C<double> a = q.m[i][j] - conj(q.m[j][i]);
       f.m[i][j] = C<double>{a.im / 8.0, -a.re / 8.0};
     }
-  C<double> tr = f.m[0][0] + f.m[1][1] + f.m[2][2];
+  const C<double> tr = f.m[0][0] + f.m[1][1] + f.m[2][2];
 #pragma unroll
   for (int i = 0; i < 3; ++i) f.m[i][i] = f.m[i][i] - (1.0 / 3.0) * tr;
   return f;
@@ -230,54 +327,86 @@ __device__ M3<double> field_strength(const Geom& g, const double2* U64, const Si
 // Chiral basis: sigma_{jk} = -eps_{jkl} diag(s_l, s_l), sigma_{j4} = diag(s_j, -s_j)
 // (s = Pauli, sigma_{mu nu} = (i/2)[gamma_mu, gamma_nu]).  Hence the upper
 // (lower) 6x6 block of sum_{mu<nu} sigma_{mu nu} F_{mu nu} is sum_l s_l (x) X_l with
-//   X_1 = -F_23 +- F_14,  X_2 = F_13 +- F_24,  X_3 = -F_12 +- F_34.
-__global__ void clover_kernel(Geom g, const double2* __restrict__ U64, double c_sw, double* C64, float* C32) {
-  int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+//   X_1 = -F_23 +- F_14,  X_2 = F_13 +- F_24,  X_3 = -F_12 +- F_34:
+// [[X_3, X_1 - i X_2], [h.c., -X_3]].  blockIdx.y = 0: the X_3 entries of both
+// blocks, 1: the spin-off-diagonal ones.
+__global__ void __launch_bounds__(64) clover_kernel(Geom g, const double2* __restrict__ AB, LevelList two, double c_sw,
+                                                    double* C64, float* C32) {
+  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (n >= g.V) return;
-  SiteCoord s = coords(g, n);
-  M3<double> F12 = field_strength(g, U64, s, 0, 1), F13 = field_strength(g, U64, s, 0, 2);
-  M3<double> F14 = field_strength(g, U64, s, 0, 3), F23 = field_strength(g, U64, s, 1, 2);
-  M3<double> F24 = field_strength(g, U64, s, 1, 3), F34 = field_strength(g, U64, s, 2, 3);
+  const SiteCoord s = coords(g, n);
   const double pre = -0.5 * c_sw;
-  for (int blk = 0; blk < 2; ++blk) {
-    const double sg = blk == 0 ? 1.0 : -1.0;
-    C<double> full[6][6];
+  auto put = [&](int blk, int k, double v) {
+    C64[((int64_t)blk * 36 + k) * g.V + n] = v;
+    C32[clover_at32(n, blk, k)] = (float)v;
+  };
+  auto at = [](int i, int j) { return 6 + 2 * (i * 5 - i * (i - 1) / 2 + j - i - 1); };  // entry (i, j), i < j
+  // S and D: the two blocks' values are S + D and S - D
+  M3<double> S, D;
+  if (blockIdx.y == 0) {
+    S = field_strength(g, AB, two, s, n, 0, 1);  // X_3 = -F_12 +- F_34
+    D = field_strength(g, AB, two, s, n, 2, 3);
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = a; b < 3; ++b) {
+          const double sg = blk == 0 ? 1.0 : -1.0;
+          const double re = pre * (sg * D.m[a][b].re - S.m[a][b].re), im = pre * (sg * D.m[a][b].im - S.m[a][b].im);
+          if (a == b) {
+            put(blk, a, re);
+            put(blk, 3 + a, -re);
+          } else {
+            put(blk, at(a, b), re);
+            put(blk, at(a, b) + 1, im);
+            put(blk, at(3 + a, 3 + b), -re);
+            put(blk, at(3 + a, 3 + b) + 1, -im);
+          }
+        }
+  } else {
+    // X_1 - i X_2 = (-F_23 - i F_13) +- (F_14 - i F_24)
+    S = field_strength(g, AB, two, s, n, 1, 2);
+    M3<double> f = field_strength(g, AB, two, s, n, 0, 2);
+#pragma unroll
     for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) {
-        C<double> x1, x2, x3;
-        x1 = C<double>{-F23.m[a][b].re + sg * F14.m[a][b].re, -F23.m[a][b].im + sg * F14.m[a][b].im};
-        x2 = C<double>{F13.m[a][b].re + sg * F24.m[a][b].re, F13.m[a][b].im + sg * F24.m[a][b].im};
-        x3 = C<double>{-F12.m[a][b].re + sg * F34.m[a][b].re, -F12.m[a][b].im + sg * F34.m[a][b].im};
-        // s_1 X_1 + s_2 X_2 + s_3 X_3 = [[X3, X1 - i X2], [X1 + i X2, -X3]]
-        C<double> m01 = C<double>{x1.re + x2.im, x1.im - x2.re};
-        C<double> m10 = C<double>{x1.re - x2.im, x1.im + x2.re};
-        full[0 * 3 + a][0 * 3 + b] = pre * x3;
-        full[1 * 3 + a][1 * 3 + b] = (-pre) * x3;
-        full[0 * 3 + a][1 * 3 + b] = pre * m01;
-        full[1 * 3 + a][0 * 3 + b] = pre * m10;
-      }
-    int64_t base = (int64_t)blk * 36;
-    for (int i = 0; i < 6; ++i) {
-      C64[(base + i) * g.V + n] = full[i][i].re;
-      C32[clover_at32(n, blk, i)] = (float)full[i][i].re;
-    }
-    int k = 6;
-    for (int i = 0; i < 6; ++i)
-      for (int j = i + 1; j < 6; ++j) {
-        C64[(base + k) * g.V + n] = full[i][j].re;
-        C64[(base + k + 1) * g.V + n] = full[i][j].im;
-        C32[clover_at32(n, blk, k)] = (float)full[i][j].re;
-        C32[clover_at32(n, blk, k + 1)] = (float)full[i][j].im;
-        k += 2;
-      }
+#pragma unroll
+      for (int b = 0; b < 3; ++b) S.m[a][b] = C<double>{-S.m[a][b].re + f.m[a][b].im, -S.m[a][b].im - f.m[a][b].re};
+    D = field_strength(g, AB, two, s, n, 0, 3);
+    f = field_strength(g, AB, two, s, n, 1, 3);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) D.m[a][b] = C<double>{D.m[a][b].re + f.m[a][b].im, D.m[a][b].im - f.m[a][b].re};
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const double sg = blk == 0 ? 1.0 : -1.0;
+          put(blk, at(a, 3 + b), pre * (S.m[a][b].re + sg * D.m[a][b].re));
+          put(blk, at(a, 3 + b) + 1, pre * (S.m[a][b].im + sg * D.m[a][b].im));
+        }
   }
 }
 
-__global__ void export_links_kernel(Geom g, const double2* __restrict__ W64, double2* out) {
-  int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
-  for (int nu = 0; nu < 40; ++nu)
-    for (int e = 0; e < 9; ++e) out[(n * 40 + nu) * 9 + e] = W64[((int64_t)nu * 9 + e) * g.V + n];
+// Caller layout [V][40][3][3] from the element planes, 32 sites x 40 elements at
+// a time through shared memory so that both sides are contiguous.
+__global__ void __launch_bounds__(256) export_links_kernel(Geom g, const double2* __restrict__ W64, double2* out) {
+  __shared__ double2 t[40][33];
+  const int64_t n0 = blockIdx.x * (int64_t)32;
+  const int k0 = blockIdx.y * 40;
+  const int m = (int)min((int64_t)32, g.V - n0);
+  for (int i = threadIdx.x; i < 40 * 32; i += 256) {
+    const int k = i / 32, l = i % 32;
+    if (l < m) t[k][l] = W64[(int64_t)(k0 + k) * g.V + n0 + l];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 40 * m; i += 256) {
+    const int l = i / 40, k = i - 40 * l;
+    out[(n0 + l) * 360 + k0 + k] = t[k][l];
+  }
 }
 
 }  // namespace
@@ -318,34 +447,43 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
   if ((rc = alloc((void**)&c->W16, kLinkBytes16 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->U64, sizeof(double2) * 36 * V))) return rc;
   if ((rc = alloc((void**)&c->U32, kLinkBytes32 * kLinkBlock * 4 * link_blocks(V)))) return rc;
-  double2* T = nullptr;
-  if ((rc = alloc((void**)&T, sizeof(double2) * 81 * 9 * V))) return rc;
-
   const int th = 128;
   thin_links_kernel<<<blocks_for(V, th), th, 0, st>>>(g, (const double2*)U, c->U64, c->U32,
                                                        (c->flags & BRI_ANTIPERIODIC_T) ? 1 : 0); note_launch();
-  if ((rc = build_transporters(c, T))) return rc;
-  BRI_CUDA(cudaMemcpyAsync(c->W64, T, sizeof(double2) * 360 * V, cudaMemcpyDeviceToDevice, st));
-  narrow_links_kernel<<<blocks_for(40 * V, 128), 128, 0, st>>>(V, c->W64, c->W32, c->W16); note_launch();
-  BRI_LAUNCH_CHECK("narrow_links_kernel");
   c->have_clover = false;
   c->dw_valid = false;
   c->c_sw = c_sw;
+  // the two paths of every stored two-hop offset, kept for the clover leaves
+  LevelList two = stored_level(2);
+  double2* AB = nullptr;
   if (c_sw != 0.0) {
     if ((rc = alloc((void**)&c->C64, sizeof(double) * 72 * V))) return rc;
     if ((rc = alloc((void**)&c->C32, sizeof(float4) * clover_words32(V)))) return rc;
-    clover_kernel<<<blocks_for(V, 64), 64, 0, st>>>(g, c->U64, c_sw, c->C64, c->C32); note_launch();
-    BRI_LAUNCH_CHECK("clover_kernel");
+    configure_pool_once();
+    const cudaError_t e = cudaMallocAsync(&AB, sizeof(double2) * 9 * 2 * two.count * V, st);
+    if (e != cudaSuccess) return cuda_fail(e, "bri_build_links: cudaMallocAsync");
+    note_device_alloc();
+  }
+  stored1_kernel<<<dim3(blocks_for(V, th), 4), th, 0, st>>>(g, c->U64, c->W64, c->W32, c->W16); note_launch();
+  for (int k = 2; k <= 4; ++k) {
+    const LevelList lst = stored_level(k);
+    storedk_kernel<<<dim3(blocks_for(V, th), lst.count), th, 0, st>>>(g, c->U64, c->W64, c->W32, c->W16, lst, k,
+                                                                     k == 2 ? AB : nullptr);
+    note_launch();
+  }
+  if (AB) {
+    clover_kernel<<<dim3(blocks_for(V, 64), 2), 64, 0, st>>>(g, AB, two, c_sw, c->C64, c->C32); note_launch();
+    cudaFreeAsync(AB, st);
     c->have_clover = true;
   }
+  BRI_LAUNCH_CHECK("link construction kernels");
   BRI_CUDA(cudaStreamSynchronize(st));
-  BRI_CUDA(cudaFree(T));
   c->have_links = true;
   return BRI_OK;
 }
 
 int launch_export_links(bri_ctx* c, double* W) {
-  export_links_kernel<<<blocks_for(c->g.V, 128), 128, 0, c->stream>>>(c->g, c->W64, (double2*)W); note_launch();
+  export_links_kernel<<<dim3(blocks_for(c->g.V, 32), 9), 256, 0, c->stream>>>(c->g, c->W64, (double2*)W); note_launch();
   BRI_LAUNCH_CHECK("export_links_kernel");
   return BRI_OK;
 }
