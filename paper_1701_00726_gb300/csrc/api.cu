@@ -305,7 +305,8 @@ int bri_apply(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagge
   if (rc) return rc;
   if (prec != BRI_PREC_DW) return dirac_bri(c, y, x, nrhs, m0, dagger ? 1 : 0, prec, c->stream);
   void* tmp = nullptr;
-  const size_t bytes = sizeof(float4) * 2 * (size_t)c->g.V * 12 * nrhs;
+  const size_t bytes = 2 * dw_vector_bytes(c->g.V) * nrhs;
+  configure_pool_once();
   cudaError_t e = cudaMallocAsync(&tmp, bytes, c->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();

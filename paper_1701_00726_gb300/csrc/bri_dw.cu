@@ -18,19 +18,32 @@
 // The products and sums of the transformations are written with the _rn
 // intrinsics, which the compiler never contracts into fused operations.
 //
-// The stencil is that of the FP32/FP64 kernels (Eq. def_bril, App. C), but the
-// spin matrix of each hop is applied before the colour transport:
-//   W_d(n) M_d x(n+d) = W_d(n) (M_d x(n+d)),   M_{+-d} = a_k 1 +- c_k S_d,
-//   S_d = sum_mu d_mu gamma_mu,
-// so that every colour product accumulates straight into the site's
-// double-word accumulators.  a_k = -2^{-k-3} is a power of two (exact
-// scaling); c_k = 4^{2-k}/27 is carried as a double-word constant.
+// The transformations run on fma/add/mul.rn.f32x2: a word holds the two spins of
+// a chirality (A, B), the link elements are broadcast to both, so half of the
+// instructions do the same arithmetic and no component is moved between
+// registers (bri_pair.cuh has the FP32 form of the same scheme).
 //
-// Storage: spinors as [rhs][V][12] float4 (re_h, re_l, im_h, im_l), links
-// [40][9][V] float4 and clover [2][36][V] float2 (h, l): the byte layout of the
-// FP64 arrays, so an FP64 vector and its double-word copy have the same size.
+// The stencil (Eq. def_bril, App. C) takes the two hops of a stored offset
+// together, colour transport first:
+//   P = W_d(n) x(n+d),  V = W_d(n-d)^dagger x(n-d) - P,
+//   acc += 2 a_k P + a_k V - c_k S_d V,   S_d = sum_mu d_mu gamma_mu.
+// a_k = -2^{-k-3} is a power of two (exact scaling); c_k = 4^{2-k}/27 is carried
+// as a double-word constant.
+//
+// Storage: spinors as [rhs][V/32][12][32] 16-byte words (re_A, re_B, im_A, im_B),
+// rows 0..5 the leading words of (chirality, colour), rows 6..11 the second
+// ones; links [V/32][40][9][32] words (re_h, re_l, im_h, im_l); clover
+// [V/32][2][36][32] pairs (h, l).
+//
+// Bound: the FP32 pipe, about 4600 operations per hop pair, site and right-hand
+// side (12 per real multiply-add; 2.4 ms for 4 right-hand sides at 16^3 x 32).
+// GB300, 16^3 x 32, 4 rhs, with the split and join passes: 4.46 ms with scalar
+// arithmetic, spin combination before each of the two transports and strided
+// links, 3.28 ms now; error against FP64 1.4e-14 -> 0.96e-14.  12 warps per SM with
+// the colour loop unrolled; rolled 3.37 ms, both hops unrolled 3.51 ms
+// (instruction fetch), 16 warps 3.42 ms (spills).
 #include "stencil.cuh"
-#include "hops.cuh"
+#include "bri_pair.cuh"
 
 #include <string>
 
@@ -41,302 +54,357 @@ namespace {
 struct DW {
   float h, l;
 };
-// accumulator: h + l, l not normalised against h between renormalisations
-struct Acc {
-  float h, l;
+// two double-word values (A, B): leading and second words
+struct DP {
+  float2 h, l;
+};
+struct CDP {
+  DP re, im;
 };
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  e = __fsub_rn(b, __fsub_rn(s, a));
-}
+__device__ __forceinline__ float2 d_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 d_sub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+__device__ __forceinline__ float2 d_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 d_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 d_neg(float2 a) { return make_float2(-a.x, -a.y); }
 
 // acc += u v (one Dot2 step with double-word operands)
-__device__ __forceinline__ void mac(Acc& acc, float uh, float ul, float vh, float vl) {
-  const float p = __fmul_rn(uh, vh);
-  const float pe = __fmaf_rn(uh, vh, -p);
-  float s, e;
-  two_sum(acc.h, p, s, e);
+__device__ __forceinline__ void mac(DP& acc, float2 uh, float2 ul, float2 vh, float2 vl) {
+  const float2 p = d_mul(uh, vh);
+  const float2 pe = d_fma(uh, vh, d_neg(p));
+  const float2 s = d_add(acc.h, p);
+  const float2 bb = d_sub(s, acc.h);
+  float2 t = d_add(d_sub(acc.h, d_sub(s, bb)), d_sub(p, bb));
   acc.h = s;
-  float t = __fadd_rn(e, pe);
-  t = __fmaf_rn(uh, vl, t);
-  t = __fmaf_rn(ul, vh, t);
-  acc.l = __fadd_rn(acc.l, t);
+  t = d_add(t, pe);
+  t = d_fma(uh, vl, t);
+  t = d_fma(ul, vh, t);
+  acc.l = d_add(acc.l, t);
 }
-__device__ __forceinline__ void mac(Acc& acc, DW u, DW v) { mac(acc, u.h, u.l, v.h, v.l); }
-// acc += t (double-word addend)
-__device__ __forceinline__ void add(Acc& acc, float th, float tl) {
-  float s, e;
-  two_sum(acc.h, th, s, e);
+// acc += k t for a factor k of powers of two (the products are exact)
+__device__ __forceinline__ void add(DP& acc, const DP& t, float2 k) {
+  const float2 s = d_fma(t.h, k, acc.h);
+  const float2 bb = d_sub(s, acc.h);
+  const float2 e = d_add(d_sub(acc.h, d_sub(s, bb)), d_fma(t.h, k, d_neg(bb)));
   acc.h = s;
-  acc.l = __fadd_rn(acc.l, __fadd_rn(e, tl));
+  acc.l = d_add(d_fma(t.l, k, acc.l), e);
 }
-__device__ __forceinline__ DW renorm(const Acc& a) {
-  DW r;
-  fast_two_sum(a.h, a.l, r.h, r.l);
-  return r;
+// Fast2Sum
+__device__ __forceinline__ void renorm(DP& a) {
+  const float2 s = d_add(a.h, a.l);
+  a.l = d_sub(a.l, d_sub(s, a.h));
+  a.h = s;
 }
-__device__ __forceinline__ DW finish(const Acc& a) {
-  DW r;
-  two_sum(a.h, a.l, r.h, r.l);
-  return r;
+// TwoSum
+__device__ __forceinline__ void finish(DP& a) {
+  const float2 s = d_add(a.h, a.l);
+  const float2 bb = d_sub(s, a.h);
+  a.l = d_add(d_sub(a.h, d_sub(s, bb)), d_sub(a.l, bb));
+  a.h = s;
+}
+__device__ __forceinline__ DP swapped(const DP& a) { return DP{pr_swp(a.h), pr_swp(a.l)}; }
+__device__ __forceinline__ DP zero_dp() { return DP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+
+// word rows r (leading) and r + 6 (second) of a packed spinor
+__device__ __forceinline__ CDP ld_cdp(const float4* __restrict__ x, int r) {
+  const float4 h = __ldg(x + r * kPackBlock), l = __ldg(x + (r + 6) * kPackBlock);
+  return CDP{DP{make_float2(h.x, h.y), make_float2(l.x, l.y)}, DP{make_float2(h.z, h.w), make_float2(l.z, l.w)}};
+}
+// acc += w v, w = (re_h, re_l, im_h, im_l)
+__device__ __forceinline__ void cmac(CDP& acc, const float4& w, const CDP& v) {
+  const float2 rh = pr_bc(w.x), rl = pr_bc(w.y), ih = pr_bc(w.z), il = pr_bc(w.w);
+  mac(acc.re, rh, rl, v.re.h, v.re.l);
+  mac(acc.im, rh, rl, v.im.h, v.im.l);
+  mac(acc.re, d_neg(ih), d_neg(il), v.im.h, v.im.l);
+  mac(acc.im, ih, il, v.re.h, v.re.l);
 }
 
-struct CDW {
-  DW re, im;
-};
-struct CAcc {
-  Acc re, im;
-};
-
-// acc += w v and acc += conj(w) v (complex, double-word)
-__device__ __forceinline__ void cmac(CAcc& acc, const float4& w, const CDW& v) {
-  mac(acc.re, w.x, w.y, v.re.h, v.re.l);
-  mac(acc.re, -w.z, -w.w, v.im.h, v.im.l);
-  mac(acc.im, w.x, w.y, v.im.h, v.im.l);
-  mac(acc.im, w.z, w.w, v.re.h, v.re.l);
-}
-__device__ __forceinline__ void cmac_cj(CAcc& acc, const float4& w, const CDW& v) {
-  mac(acc.re, w.x, w.y, v.re.h, v.re.l);
-  mac(acc.re, w.z, w.w, v.im.h, v.im.l);
-  mac(acc.im, w.x, w.y, v.im.h, v.im.l);
-  mac(acc.im, -w.z, -w.w, v.re.h, v.re.l);
-}
-
-// Per-offset constants: a_k (exact in FP32), c_k as a double-word pair.
+// Per-offset constants: signs, a_k (exact in FP32), c_k as a double-word pair.
 struct HopTableDW {
-  int site_d[40][4];
+  int d[40][4];
   float a[40];
   float ch[40], cl[40];
 };
 
-HopTableDW make_hop_table_dw() {
-  const HopTable<double>& h = hop_table<double>();
-  HopTableDW t;
-  for (int j = 0; j < 40; ++j) {
-    double c = 0.0;
-    for (int mu = 0; mu < 4; ++mu) {
-      t.site_d[j][mu] = h.site_d[j][mu];
-      if (h.cs[j][mu] != 0.0) c = h.cs[j][mu] > 0 ? h.cs[j][mu] : -h.cs[j][mu];
-    }
-    t.a[j] = (float)h.a[j];
-    t.ch[j] = (float)c;
-    t.cl[j] = (float)(c - (double)t.ch[j]);
-  }
-  return t;
-}
-
 const HopTableDW& hop_table_dw() {
-  static const HopTableDW t = make_hop_table_dw();
+  static const HopTableDW t = [] {
+    const HopTable<double>& h = hop_table<double>();
+    HopTableDW t;
+    for (int j = 0; j < 40; ++j) {
+      double c = 0.0;
+      for (int mu = 0; mu < 4; ++mu) {
+        t.d[j][mu] = h.site_d[j][mu];
+        if (h.cs[j][mu] != 0.0) c = h.cs[j][mu] > 0 ? h.cs[j][mu] : -h.cs[j][mu];
+      }
+      t.a[j] = (float)h.a[j];
+      t.ch[j] = (float)c;
+      t.cl[j] = (float)(c - (double)t.ch[j]);
+    }
+    return t;
+  }();
   return t;
 }
 
-__device__ __forceinline__ CDW ld_cdw(const float4* p) {
-  const float4 v = __ldg(p);
-  return CDW{DW{v.x, v.y}, DW{v.z, v.w}};
-}
-
-// phase * z for phase = 1, i, -1, -i (q = 0..3), times sign sg = +-1
-__device__ __forceinline__ void phased(const CDW& z, int q, float sg, float& rh, float& rl, float& ih, float& il) {
-  // i z = (-z_im, z_re)
-  float ar = z.re.h, arl = z.re.l, ai = z.im.h, ail = z.im.l;
-  if (q == 1) {
-    ar = -z.im.h; arl = -z.im.l; ai = z.re.h; ail = z.re.l;
-  } else if (q == 2) {
-    ar = -ar; arl = -arl; ai = -ai; ail = -ail;
-  } else if (q == 3) {
-    ar = z.im.h; arl = z.im.l; ai = -z.re.h; ail = -z.re.l;
-  }
-  rh = sg * ar; rl = sg * arl; ih = sg * ai; il = sg * ail;
-}
-
-// y = a x + c S_d x over one colour (four spins), S_d = sum_mu d_mu gamma_mu in
-// the chiral basis (the spin structure of gamma_term):
-//   gamma_1 x = (-i x3, -i x2, i x1, i x0), gamma_2 x = (-x3, x2, x1, -x0),
-//   gamma_3 x = (-i x2, i x3, i x0, -i x1), gamma_4 x = (x2, x3, x0, x1).
-__device__ __forceinline__ void spin_apply(CDW y[4], const CDW x[4], float a, DW c, const int d[4]) {
-  // source spin and phase (1, i, -1, -i as 0..3) of gamma_mu x at spin s
-  constexpr int src[4][4] = {{3, 2, 1, 0}, {3, 2, 1, 0}, {2, 3, 0, 1}, {2, 3, 0, 1}};
-  constexpr int ph[4][4] = {{3, 3, 1, 1}, {2, 0, 0, 2}, {3, 1, 1, 3}, {0, 0, 0, 0}};
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    CAcc S{{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      if (d[mu] == 0) continue;
-      float rh, rl, ih, il;
-      phased(x[src[mu][s]], ph[mu][s], (float)d[mu], rh, rl, ih, il);
-      add(S.re, rh, rl);
-      add(S.im, ih, il);
-    }
-    // y_s = a x_s + c S (a x_s exact: a is a power of two)
-    CAcc Y{{0.f, 0.f}, {0.f, 0.f}};
-    Y.re.h = a * x[s].re.h;
-    Y.re.l = a * x[s].re.l;
-    Y.im.h = a * x[s].im.h;
-    Y.im.l = a * x[s].im.l;
-    mac(Y.re, c.h, c.l, S.re.h, S.re.l);
-    mac(Y.im, c.h, c.l, S.im.h, S.im.l);
-    y[s].re = renorm(Y.re);
-    y[s].im = renorm(Y.im);
-  }
-}
+constexpr int kDwLinkWords = 9 * kLinkBlock;  // one offset of one block of sites
 
 // One thread per site and right-hand side (grid groups = right-hand sides, in
-// the order of stencil_grid).  One source colour at a time keeps 128
-// registers (16 warps per SM) without spills.
-__global__ void __launch_bounds__(128, 4)
+// the order of stencil_grid).  The hop loop is rolled so that the body fits the
+// instruction cache.
+__global__ void __launch_bounds__(128, 3)
     bri_kernel_dw(Geom g, float4* __restrict__ y, const float4* __restrict__ x, const float4* __restrict__ W,
                   const float2* __restrict__ cl, DW diag, float sgn, int gfirst, const __grid_constant__ HopTableDW H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   const int n = blk * blockDim.x + threadIdx.x;
   if (n >= g.V) return;
-  const int64_t V = g.V;
-  const int64_t roff = (int64_t)grp * V * 12;
+  const int64_t roff = (int64_t)grp * packed_words(g.V, 12);
   const float4* xin = x + roff;
-  int co[4], L[4], str[4];
+  int up[4], dn[4];
   {
     int r = n;
 #pragma unroll
-    for (int mu = 0; mu < 3; ++mu) {
-      co[mu] = r % g.L[mu];
-      r /= g.L[mu];
+    for (int mu = 0; mu < 4; ++mu) {
+      const int L = g.L[mu], s = (int)g.str[mu];
+      const int c = mu < 3 ? r % L : r;
+      if (mu < 3) r /= L;
+      up[mu] = c == L - 1 ? -(L - 1) * s : s;
+      dn[mu] = c == 0 ? (L - 1) * s : -s;
     }
-    co[3] = r;
   }
+  CDP acc[2][3];
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    L[mu] = g.L[mu];
-    str[mu] = (int)g.str[mu];
-  }
-  CAcc acc[4][3];
+  for (int q = 0; q < 2; ++q)
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
-#pragma unroll
-    for (int aa = 0; aa < 3; ++aa) acc[s][aa] = CAcc{{0.f, 0.f}, {0.f, 0.f}};
+    for (int aa = 0; aa < 3; ++aa) acc[q][aa] = CDP{zero_dp(), zero_dp()};
 
 #pragma unroll 1
   for (int j = 0; j < 40; ++j) {
-    int d[4], mp = 0, mm = 0;
+    int mp = n, mm = n;
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-      d[mu] = H.site_d[j][mu];
-      mp += wrap(co[mu] + d[mu], L[mu]) * str[mu];
-      mm += wrap(co[mu] - d[mu], L[mu]) * str[mu];
+      const int d = H.d[j][mu];
+      mp += d > 0 ? up[mu] : (d < 0 ? dn[mu] : 0);
+      mm += d > 0 ? dn[mu] : (d < 0 ? up[mu] : 0);
     }
     const float a = H.a[j];
-    const DW c{sgn * H.ch[j], sgn * H.cl[j]};
-    const DW cm{-c.h, -c.l};
-    // The two hops of the pair, one source colour b at a time (the spin matrix
-    // mixes spins only), as rolled loops so that the body fits the instruction
-    // cache:
-    //   forward  (h = 0): acc[.][aa] += W_d(n)[aa][b] (M_d x(n+d))[.][b]
-    //   backward (h = 1): acc[.][aa] += conj(W_d(n-d)[b][aa]) (M_{-d} x(n-d))[.][b]
+    CDP P[2][3];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) P[q][aa] = CDP{zero_dp(), zero_dp()};
+    // hop 0: P = W_d(n) x(n+d); hop 1: V = W_d(n-d)^dagger x(n-d) - P (conj(w) = (w_re, -w_im))
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
-      const int m = h ? mm : mp;
-      const float4* wp = W + (int64_t)j * 9 * V + (h ? mm : n);
-      const DW ch = h ? cm : c;
-      const float cs = h ? -1.f : 1.f;  // conj(w) = (w_re, -w_im)
-#pragma unroll 1
-      for (int b = 0; b < 3; ++b) {
-        CDW xs[4], ys[4];
+      const int m = h ? mm : n;
+      const float4* wp = W + ((int64_t)(m / kLinkBlock) * 40 + j) * kDwLinkWords + m % kLinkBlock;
+      const float4* xs = xin + packed_at<12>(h ? mm : mp);
+      const float cs = h ? -1.f : 1.f;
+      const int wb = (h ? 3 : 1) * kLinkBlock, wa = (h ? 1 : 3) * kLinkBlock;
 #pragma unroll
-        for (int s = 0; s < 4; ++s) xs[s] = ld_cdw(xin + (int64_t)m * 12 + s * 3 + b);
-        spin_apply(ys, xs, a, ch, d);
+      for (int b = 0; b < 3; ++b) {
+        const CDP x0 = ld_cdp(xs, b), x1 = ld_cdp(xs, 3 + b);
 #pragma unroll
         for (int aa = 0; aa < 3; ++aa) {
-          float4 w = __ldg(wp + (int64_t)(h ? b * 3 + aa : aa * 3 + b) * V);
+          float4 w = __ldg(wp + b * wb + aa * wa);
           w.z *= cs;
           w.w *= cs;
-#pragma unroll
-          for (int s = 0; s < 4; ++s) cmac(acc[s][aa], w, ys[s]);
+          cmac(P[0][aa], w, x0);
+          cmac(P[1][aa], w, x1);
         }
       }
-    }
+      // acc += 2 a P and P -> -P (hop 0), acc += a V (hop 1)
+      const float2 k = pr_bc(h ? a : 2.f * a), f = pr_bc(-cs);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int aa = 0; aa < 3; ++aa) {
+          add(acc[q][aa].re, P[q][aa].re, k);
+          add(acc[q][aa].im, P[q][aa].im, k);
+          P[q][aa].re = DP{d_mul(P[q][aa].re.h, f), d_mul(P[q][aa].re.l, f)};
+          P[q][aa].im = DP{d_mul(P[q][aa].im.h, f), d_mul(P[q][aa].im.l, f)};
+        }
+    }
+    // V times c_k, then the signed spin permutations of -S_d (bri_pair.cuh)
+    const float2 ch = pr_bc(H.ch[j]), clo = pr_bc(H.cl[j]);
+    auto scale = [&](DP& v) {
+      const float2 h = d_mul(v.h, ch);
+      float2 e = d_fma(v.h, ch, d_neg(h));
+      e = d_fma(v.l, ch, e);
+      v.l = d_fma(v.h, clo, e);
+      v.h = h;
+    };
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
 #pragma unroll
       for (int aa = 0; aa < 3; ++aa) {
-        const DW r = renorm(acc[s][aa].re), i = renorm(acc[s][aa].im);
-        acc[s][aa] = CAcc{{r.h, r.l}, {i.h, i.l}};
+        scale(P[q][aa].re);
+        scale(P[q][aa].im);
+      }
+    const float s1 = -sgn * (float)H.d[j][0], s2 = -sgn * (float)H.d[j][1], s3 = -sgn * (float)H.d[j][2], s4 = -sgn * (float)H.d[j][3];
+    if (s1 != 0.f) {
+      const float2 p = pr_bc(s1), m = pr_bc(-s1);
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        add(acc[0][aa].re, swapped(P[1][aa].im), p);
+        add(acc[0][aa].im, swapped(P[1][aa].re), m);
+        add(acc[1][aa].re, swapped(P[0][aa].im), m);
+        add(acc[1][aa].im, swapped(P[0][aa].re), p);
+      }
+    }
+    if (s2 != 0.f) {
+      const float2 k = make_float2(-s2, s2), m = make_float2(s2, -s2);
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        add(acc[0][aa].re, swapped(P[1][aa].re), k);
+        add(acc[0][aa].im, swapped(P[1][aa].im), k);
+        add(acc[1][aa].re, swapped(P[0][aa].re), m);
+        add(acc[1][aa].im, swapped(P[0][aa].im), m);
+      }
+    }
+    if (s3 != 0.f) {
+      const float2 k = make_float2(s3, -s3), m = make_float2(-s3, s3);
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        add(acc[0][aa].re, P[1][aa].im, k);
+        add(acc[0][aa].im, P[1][aa].re, m);
+        add(acc[1][aa].re, P[0][aa].im, m);
+        add(acc[1][aa].im, P[0][aa].re, k);
+      }
+    }
+    if (s4 != 0.f) {
+      const float2 k = pr_bc(s4);
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        add(acc[0][aa].re, P[1][aa].re, k);
+        add(acc[0][aa].im, P[1][aa].im, k);
+        add(acc[1][aa].re, P[0][aa].re, k);
+        add(acc[1][aa].im, P[0][aa].im, k);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) {
+        renorm(acc[q][aa].re);
+        renorm(acc[q][aa].im);
       }
   }
-  // diagonal and clover terms at the site itself
-  CDW xc[4][3];
+  // diagonal and clover terms at the site itself.  A chirality's clover block is
+  // [[X, M], [M^dagger, -X]] on its two spins: X (3 reals, 3 complex above the
+  // diagonal) acts with the signs (+, -), M and M^dagger on the exchanged spins.
+  const float4* xo = xin + packed_at<12>(n);
+  float4* yo = y + roff + packed_at<12>(n);
+  const float2 dh = pr_bc(diag.h), dl = pr_bc(diag.l);
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+  for (int q = 0; q < 2; ++q) {
+    CDP in[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      xc[s][b] = ld_cdw(xin + (int64_t)n * 12 + s * 3 + b);
-      mac(acc[s][b].re, diag, xc[s][b].re);
-      mac(acc[s][b].im, diag, xc[s][b].im);
+      in[b] = ld_cdp(xo, 3 * q + b);
+      mac(acc[q][b].re, dh, dl, in[b].re.h, in[b].re.l);
+      mac(acc[q][b].im, dh, dl, in[b].im.h, in[b].im.l);
     }
-  if (cl) {
-    // two Hermitian 6x6 chiral blocks: 6 diagonal reals, then the 15 upper
-    // off-diagonal complex entries row by row (the FP64 packing)
+    if (cl) {
+      const float2* cb = cl + ((int64_t)(n / kCloverBlock * 2 + q) * 36) * kCloverBlock + n % kCloverBlock;
+      auto real = [&](int k) { return __ldg(cb + k * kCloverBlock); };
+      auto at = [](int i, int j) { return 6 + 2 * (i * 5 - i * (i - 1) / 2 + j - i - 1); };
+      const float2 pm = make_float2(1.f, -1.f);
+      // (+-) X: entry (a, b) as a complex double-word number, conjugated below the diagonal
 #pragma unroll
-    for (int blk6 = 0; blk6 < 2; ++blk6) {
-      const float2* cb = cl + (int64_t)blk6 * 36 * V + n;
+      for (int b = 0; b < 3; ++b) {
+        CDP v = in[b];  // signs (+, -) on the two spins
+        v.re = DP{d_mul(v.re.h, pm), d_mul(v.re.l, pm)};
+        v.im = DP{d_mul(v.im.h, pm), d_mul(v.im.l, pm)};
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
-        const float2 dd = __ldg(cb + (int64_t)i * V);
-        const CDW& in = xc[2 * blk6 + i / 3][i % 3];
-        CAcc& o = acc[2 * blk6 + i / 3][i % 3];
-        mac(o.re, dd.x, dd.y, in.re.h, in.re.l);
-        mac(o.im, dd.x, dd.y, in.im.h, in.im.l);
-      }
-      int k = 6;
-#pragma unroll
-      for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int jj = i + 1; jj < 6; ++jj) {
-          const float2 cr = __ldg(cb + (int64_t)k * V), ci = __ldg(cb + (int64_t)(k + 1) * V);
-          const float4 cij = make_float4(cr.x, cr.y, ci.x, ci.y);
-          cmac(acc[2 * blk6 + i / 3][i % 3], cij, xc[2 * blk6 + jj / 3][jj % 3]);
-          cmac_cj(acc[2 * blk6 + jj / 3][jj % 3], cij, xc[2 * blk6 + i / 3][i % 3]);
-          k += 2;
+        for (int aa = 0; aa < 3; ++aa) {
+          if (aa == b) {
+            const float2 d = real(aa);
+            mac(acc[q][aa].re, pr_bc(d.x), pr_bc(d.y), v.re.h, v.re.l);
+            mac(acc[q][aa].im, pr_bc(d.x), pr_bc(d.y), v.im.h, v.im.l);
+          } else {
+            const int k = aa < b ? at(aa, b) : at(b, aa);
+            const float2 r = real(k), i = real(k + 1);
+            const float sg = aa < b ? 1.f : -1.f;
+            cmac(acc[q][aa], make_float4(r.x, r.y, sg * i.x, sg * i.y), v);
+          }
         }
-    }
-  }
-  float4* yo = y + roff + (int64_t)n * 12;
+      }
+      // out_A += M in_B, out_B += M^dagger in_A: pair operands (M[aa][b], conj M[b][aa])
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+      for (int b = 0; b < 3; ++b) {
+        const DP vr = swapped(in[b].re), vi = swapped(in[b].im);
+#pragma unroll
+        for (int aa = 0; aa < 3; ++aa) {
+          const float2 ra = real(at(aa, 3 + b)), ia = real(at(aa, 3 + b) + 1);
+          const float2 rb = real(at(b, 3 + aa)), ib = real(at(b, 3 + aa) + 1);
+          const float2 rh = make_float2(ra.x, rb.x), rl = make_float2(ra.y, rb.y);
+          const float2 ih = make_float2(ia.x, -ib.x), il = make_float2(ia.y, -ib.y);
+          mac(acc[q][aa].re, rh, rl, vr.h, vr.l);
+          mac(acc[q][aa].im, rh, rl, vi.h, vi.l);
+          mac(acc[q][aa].re, d_neg(ih), d_neg(il), vi.h, vi.l);
+          mac(acc[q][aa].im, ih, il, vr.h, vr.l);
+        }
+      }
+    }
 #pragma unroll
     for (int aa = 0; aa < 3; ++aa) {
-      const DW r = finish(acc[s][aa].re), i = finish(acc[s][aa].im);
-      yo[s * 3 + aa] = make_float4(r.h, r.l, i.h, i.l);
+      CDP o = acc[q][aa];
+      finish(o.re);
+      finish(o.im);
+      yo[(3 * q + aa) * kPackBlock] = make_float4(o.re.h.x, o.re.h.y, o.im.h.x, o.im.h.y);
+      yo[(3 * q + aa + 6) * kPackBlock] = make_float4(o.re.l.x, o.re.l.y, o.im.l.x, o.im.l.y);
     }
+  }
 }
 
-// FP64 (re, im) -> double-word (re_h, re_l, im_h, im_l), element by element
-__global__ void k_split_dw(int64_t n, const double2* __restrict__ in, float4* out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = in[i];
-    const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-    out[i] = make_float4(rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih));
-  }
+__device__ __forceinline__ float2 split_dw(double v) {
+  const float h = __double2float_rn(v);
+  return make_float2(h, __double2float_rn(v - (double)h));
 }
-__global__ void k_split_dw_real(int64_t n, const double* __restrict__ in, float2* out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = in[i];
-    const float h = __double2float_rn(v);
-    out[i] = make_float2(h, __double2float_rn(v - (double)h));
-  }
+
+// FP64 spinors [rhs][V][12] -> packed double-word spinors and back; one thread
+// per site, chirality and colour, blockIdx.y = right-hand side.
+__global__ void __launch_bounds__(256) k_split_dw(int64_t V, const double2* __restrict__ in, float4* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  const double2* p = in + (blockIdx.y * V + n) * 12 + q + 3 * (q / 3);
+  const double2 u = __ldg(p), v = __ldg(p + 3);
+  const float2 ur = split_dw(u.x), ui = split_dw(u.y), vr = split_dw(v.x), vi = split_dw(v.y);
+  float4* o = out + (int64_t)blockIdx.y * packed_words(V, 12) + packed_at<12>((int)n) + q * kPackBlock;
+  o[0] = make_float4(ur.x, vr.x, ui.x, vi.x);
+  o[6 * kPackBlock] = make_float4(ur.y, vr.y, ui.y, vi.y);
 }
-__global__ void k_join_dw(int64_t n, const float4* __restrict__ in, double2* out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 v = in[i];
-    out[i] = make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
-  }
+__global__ void __launch_bounds__(256) k_join_dw(int64_t V, const float4* __restrict__ in, double2* __restrict__ out) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  const float4* o = in + (int64_t)blockIdx.y * packed_words(V, 12) + packed_at<12>((int)n) + q * kPackBlock;
+  const float4 h = __ldg(o), l = __ldg(o + 6 * kPackBlock);
+  double2* p = out + (blockIdx.y * V + n) * 12 + q + 3 * (q / 3);
+  p[0] = make_double2((double)h.x + (double)l.x, (double)h.z + (double)l.z);
+  p[3] = make_double2((double)h.y + (double)l.y, (double)h.w + (double)l.w);
+}
+// FP64 links [40][9][V] and clover [2][36][V] into the chunked double-word
+// layouts, one thread per element and site.
+__global__ void __launch_bounds__(256) k_links_dw(int64_t V, const double2* __restrict__ in, float4* __restrict__ out) {
+  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (n >= V) return;
+  const int je = blockIdx.y;
+  const double2 v = in[(int64_t)je * V + n];
+  const float2 r = split_dw(v.x), m = split_dw(v.y);
+  out[(n / kLinkBlock * 360 + je) * kLinkBlock + n % kLinkBlock] = make_float4(r.x, r.y, m.x, m.y);
+}
+__global__ void __launch_bounds__(256) k_clover_dw(int64_t V, const double* __restrict__ in, float2* __restrict__ out) {
+  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (n >= V) return;
+  out[(n / kCloverBlock * 72 + blockIdx.y) * kCloverBlock + n % kCloverBlock] = split_dw(in[(int64_t)blockIdx.y * V + n]);
 }
 
 }  // namespace
+
+size_t dw_vector_bytes(int64_t V) { return sizeof(float4) * (size_t)packed_words(V, 12); }
 
 // Double-word copies of the FP64 links and clover, made on first use after
 // each bri_build_links.
@@ -356,11 +424,12 @@ int ensure_dw_links(bri_ctx* c) {
     return BRI_OK;
   };
   int rc;
-  if ((rc = alloc(&c->Wdw, sizeof(float4) * 360 * V))) return rc;
-  k_split_dw<<<1024, 256, 0, st>>>(360 * V, c->W64, (float4*)c->Wdw); note_launch();
+  const int64_t Vp = link_blocks(V) * kLinkBlock;
+  if ((rc = alloc(&c->Wdw, sizeof(float4) * 360 * Vp))) return rc;
+  k_links_dw<<<dim3(blocks_for(V, 256), 360), 256, 0, st>>>(V, c->W64, (float4*)c->Wdw); note_launch();
   if (c->have_clover) {
-    if ((rc = alloc(&c->Cdw, sizeof(float2) * 72 * V))) return rc;
-    k_split_dw_real<<<1024, 256, 0, st>>>(72 * V, c->C64, (float2*)c->Cdw); note_launch();
+    if ((rc = alloc(&c->Cdw, sizeof(float2) * 72 * Vp))) return rc;
+    k_clover_dw<<<dim3(blocks_for(V, 256), 72), 256, 0, st>>>(V, c->C64, (float2*)c->Cdw); note_launch();
   }
   BRI_LAUNCH_CHECK("double-word links");
   c->dw_valid = true;
@@ -386,16 +455,17 @@ int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int da
 }
 
 // FP64 in, FP64 out: split, stencil, join (tmp: two double-word vectors of
-// nrhs right-hand sides, 16 bytes per complex element each).
+// nrhs right-hand sides).
 int dirac_bri_dw64(bri_ctx* c, double* y, const double* x, int nrhs, double m0, int dagger, void* tmp,
                    cudaStream_t s) {
-  const int64_t ne = c->g.V * 12 * nrhs;
+  const int64_t V = c->g.V;
+  const dim3 eg(blocks_for(V * 6, 256), nrhs);
   float4* xa = (float4*)tmp;
-  float4* ya = xa + ne;
-  k_split_dw<<<1024, 256, 0, s>>>(ne, (const double2*)x, xa); note_launch();
+  float4* ya = xa + packed_words(V, 12) * nrhs;
+  k_split_dw<<<eg, 256, 0, s>>>(V, (const double2*)x, xa); note_launch();
   int rc = dirac_bri_dw(c, ya, xa, nrhs, m0, dagger, s);
   if (rc) return rc;
-  k_join_dw<<<1024, 256, 0, s>>>(ne, ya, (double2*)y); note_launch();
+  k_join_dw<<<eg, 256, 0, s>>>(V, ya, (double2*)y); note_launch();
   BRI_LAUNCH_CHECK("double-word apply");
   return BRI_OK;
 }
@@ -403,13 +473,14 @@ int dirac_bri_dw64(bri_ctx* c, double* y, const double* x, int nrhs, double m0, 
 // A x = D^dagger D x on FP64 vectors through double-word stencils; out = A x
 // (FP64).  t1, t2: double-word scratch of nrhs vectors each.
 int normal_op_dw(bri_ctx* c, double* out, const double* x, int nrhs, double m0, void* t1, void* t2, cudaStream_t s) {
-  const int64_t ne = c->g.V * 12 * nrhs;
-  k_split_dw<<<1024, 256, 0, s>>>(ne, (const double2*)x, (float4*)t1); note_launch();
+  const int64_t V = c->g.V;
+  const dim3 eg(blocks_for(V * 6, 256), nrhs);
+  k_split_dw<<<eg, 256, 0, s>>>(V, (const double2*)x, (float4*)t1); note_launch();
   int rc = dirac_bri_dw(c, t2, t1, nrhs, m0, 0, s);
   if (rc) return rc;
   rc = dirac_bri_dw(c, t1, t2, nrhs, m0, 1, s);
   if (rc) return rc;
-  k_join_dw<<<1024, 256, 0, s>>>(ne, (const float4*)t1, (double2*)out); note_launch();
+  k_join_dw<<<eg, 256, 0, s>>>(V, (const float4*)t1, (double2*)out); note_launch();
   BRI_LAUNCH_CHECK("double-word normal operator");
   return BRI_OK;
 }

@@ -81,8 +81,8 @@ struct bri_ctx {
   double* C64 = nullptr;
   float* C32 = nullptr;
   // Double-word FP32 copies (h, l) of W64 and C64 for the FP64-class stencil
-  // on the FP32 pipe: [40][9][V] float4 and [2][36][V] float2, made on first
-  // use after each bri_build_links (dw_valid).
+  // on the FP32 pipe, in chunks of 32 sites (bri_dw.cu), made on first use after
+  // each bri_build_links (dw_valid).
   void* Wdw = nullptr;
   void* Cdw = nullptr;
   bool dw_valid = false;
@@ -123,10 +123,11 @@ int dirac_bri(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagge
 int dirac_wil(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec,
               cudaStream_t s);
 // Double-word FP32 Brillouin stencil (bri_dw.cu): y = D x or D^dagger x on
-// double-word vectors ([nrhs][V][12] float4), FP64 in and out through the
+// packed double-word vectors (dw_vector_bytes each), FP64 in and out through the
 // split/join kernels (tmp: two double-word vectors of nrhs right-hand sides),
 // and the normal operator D^dagger D on FP64 vectors (t1, t2 double-word
 // scratch; t2 may be out).
+size_t dw_vector_bytes(int64_t V);
 int ensure_dw_links(bri_ctx* c);
 int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, cudaStream_t s);
 int dirac_bri_dw64(bri_ctx* c, double* y, const double* x, int nrhs, double m0, int dagger, void* tmp,

@@ -1131,8 +1131,9 @@ int refine_mixed(bri_ctx* c, const double* b, int nrhs, int n, const double* sig
   int& refinements = info.refinements;
   // phase 2: one FP64 residual per (shift, rhs), r_i = b - (A + sigma_i) X_i
   DevBuf btmp1, btmp2, bpart, bdsum, bres;
-  if ((rc = btmp1.alloc(sizeof(double) * nreal * nrhs, st))) return rc;
-  if ((rc = btmp2.alloc(sizeof(double) * nreal * nrhs, st))) return rc;
+  const size_t tmp_bytes = std::max(sizeof(double) * nreal, dw_vector_bytes(c->g.V));  // one FP64 or double-word vector
+  if ((rc = btmp1.alloc(tmp_bytes * nrhs, st))) return rc;
+  if ((rc = btmp2.alloc(tmp_bytes * nrhs, st))) return rc;
   // The partials buffer serves three grids: the nrhs-wide residuals below,
   // the correction update (up to 32 systems) and the single-system FP64
   // verification residuals; grid_for caps every one of them at kMaxPartials.
@@ -1278,8 +1279,8 @@ int refine_mixed(bri_ctx* c, const double* b, int nrhs, int n, const double* sig
       if (rlog) fprintf(stderr, "bri refine: round %d: %zu verification residuals\n", round, verify.size());
       if (!verify.empty()) {
         DevBuf v1, v2;
-        if ((rc = v1.alloc(sizeof(double) * nreal, st))) return rc;
-        if ((rc = v2.alloc(sizeof(double) * nreal, st))) return rc;
+        if ((rc = v1.alloc(tmp_bytes, st))) return rc;
+        if ((rc = v2.alloc(tmp_bytes, st))) return rc;
         for (int slot : verify) {
           const int k = slot / nrhs, sidx = slot % nrhs;
           // the solution has changed by a correction of ~1e-7 of its norm, so
