@@ -22,33 +22,46 @@ size_t bri_f32_packed_bytes(int64_t V, int nrhs) {
 int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s) {
   const int pairs = nrhs / 2;
   float4* X4 = (float4*)X;
-  if (pairs) launch_pack<4>(V, x, 0, nrhs, pairs, X4, s);
-  if (nrhs % 2) launch_pack<2>(V, x, nrhs - 1, nrhs, 1, X4 + packed_words(V, 12) * pairs, s);
+  if (pairs) launch_pack<4>(V, x, 0, pairs, X4, s);
+  if (nrhs % 2) launch_pack<2>(V, x, nrhs - 1, 1, X4 + packed_words(V, 12) * pairs, s);
   BRI_LAUNCH_CHECK("k_pack");
+  return BRI_OK;
+}
+
+int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s) {
+  const int pairs = nrhs / 2;
+  const float4* X4 = (const float4*)X;
+  if (pairs) launch_unpack<4>(V, X4, 0, pairs, x, s);
+  if (nrhs % 2) launch_unpack<2>(V, X4 + packed_words(V, 12) * pairs, nrhs - 1, 1, x, s);
+  BRI_LAUNCH_CHECK("k_unpack");
   return BRI_OK;
 }
 
 // y (spinors' layout) or yp (packed) = D x for the first na of nrhs right-hand
 // sides of the packed vector X (a pair whose second member is not asked for is
-// still computed whole; y holds nrhs right-hand sides).
+// still computed whole).  With p (packed; yp only) the fused epilogue of
+// ShiftDot, sd_blocks partials per system.
 template <typename LS>
 int bri_f32_on_packed(const Geom& g, float* y, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs,
-                      int na, int dagger, cudaStream_t s, const ShiftDot<float>* sd, int* sd_blocks) {
+                      int na, int dagger, cudaStream_t s, const void* p, const double* sig, double* part, int* sd_blocks) {
   const int pairs = nrhs / 2, act = std::min(pairs, (na + 1) / 2);
   const int64_t o = packed_words(g.V, 12) * pairs;
-  const float4* X4 = (const float4*)X;
+  const float4 *X4 = (const float4*)X, *P4 = (const float4*)p;
   float4* Y4 = (float4*)yp;
   if (sd_blocks) *sd_blocks = blocks_for(g.V, 128);
-  if (act) launch_pair<4, LS>(g, y, Y4, X4, W, cl, diag, dagger, 0, nrhs, act, s, sd);
-  if (nrhs % 2 && na == nrhs)
-    launch_pair<2, LS>(g, y, Y4 ? Y4 + o : nullptr, X4 + o, W, cl, diag, dagger, nrhs - 1, nrhs, 1, s, sd);
+  PackedDot sd{P4, sig, part};
+  if (act) launch_pair<4, LS>(g, y, Y4, X4, W, cl, diag, dagger, 0, act, s, p ? &sd : nullptr);
+  if (nrhs % 2 && na == nrhs) {
+    sd.p = P4 + (p ? o : 0);
+    launch_pair<2, LS>(g, y, Y4 ? Y4 + o : nullptr, X4 + o, W, cl, diag, dagger, nrhs - 1, 1, s, p ? &sd : nullptr);
+  }
   BRI_LAUNCH_CHECK("bri_pair_kernel");
   return BRI_OK;
 }
 template int bri_f32_on_packed<float2>(const Geom&, float*, void*, const void*, const float2*, const float*, float, int, int,
-                                       int, cudaStream_t, const ShiftDot<float>*, int*);
+                                       int, cudaStream_t, const void*, const double*, double*, int*);
 template int bri_f32_on_packed<__nv_bfloat162>(const Geom&, float*, void*, const void*, const __nv_bfloat162*, const float*,
-                                               float, int, int, int, cudaStream_t, const ShiftDot<float>*, int*);
+                                               float, int, int, int, cudaStream_t, const void*, const double*, double*, int*);
 
 // Spinors in their own layout in and out.  The packed copy of x lives in a
 // stream-ordered allocation of at most kChunk right-hand sides; where there is
@@ -67,7 +80,7 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
         const int nr = std::min(kChunk, nrhs - r0);
         const int64_t at = r0 * g.V * 24;
         rc = bri_f32_pack(g.V, x + at, nr, X, s);
-        if (rc == BRI_OK) rc = bri_f32_on_packed<LS>(g, y + at, nullptr, X, W, cl, diag, nr, nr, dagger, s, nullptr, nullptr);
+        if (rc == BRI_OK) rc = bri_f32_on_packed<LS>(g, y + at, nullptr, X, W, cl, diag, nr, nr, dagger, s);
       }
       cudaFreeAsync(X, s);
       return rc;

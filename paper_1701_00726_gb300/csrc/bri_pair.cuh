@@ -311,33 +311,44 @@ __device__ __forceinline__ void pr_clover(CP (&o)[6], const float* __restrict__ 
     }
 }
 
-// y = D x on packed x.  OUT = 0: y in the spinors' own layout; 1: packed like x.
-// With EPI (OUT = 0): y = D x + sig_s p_s and the site block's partial of
-// Re<p_s, y> in part[s * blocks + block] (p in the spinors' own layout).
-// nrhs: right-hand sides of the whole vector (a pair's second one may not exist:
-// its half of the packed words is a copy, its results are dropped).
+// The solver's epilogue on packed vectors: y = D x + sig_s p_s and the site
+// block's partial of Re<p_s, y> in part[s * blocks + block].
+struct PackedDot {
+  const float4* p;    // packed base directions
+  const double* sig;  // per system
+  double* part;       // [nsys][blocks]
+};
+
+// D x (EPI: + sig p, dA and dB this site's Re<p, y> of the two components'
+// systems) at site n of one packed group: x, yo, p are the group's packed
+// vectors, y0 its first right-hand side in the spinors' own layout (rs reals
+// apart).  OUT = 0 writes y0, OUT = 1 writes yo.
 template <int R, typename LS, int OUT, bool EPI>
-__global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
-    bri_pair_kernel(Geom g, float* __restrict__ y, float4* __restrict__ yp, const float4* __restrict__ x,
-                    const LS* __restrict__ W, const float* __restrict__ cl, float diag, int rhs0, int nrhs, int gfirst,
-                    const __grid_constant__ PairHops H, ShiftDot<float> sd) {
-  const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  const int n0 = blk * blockDim.x + threadIdx.x;
-  const bool valid = n0 < g.V;
-  if (!EPI && !valid) return;  // with the epilogue every thread takes part in the block's reduction
-  const int n = valid ? n0 : 0;
-  const int64_t rs = g.V * 24;
-  constexpr int NR = R / 2;                // right-hand sides of a word
-  const int s0 = rhs0 + grp * NR;
-  const float4* xg = x + (int64_t)grp * packed_words(g.V, 3 * R);
+__device__ __forceinline__ void pr_site(const Geom& g, int n, bool valid, float* __restrict__ y0, int64_t rs,
+                                        float4* __restrict__ yo, const float4* __restrict__ x, const LS* __restrict__ W,
+                                        const float* __restrict__ cl, float diag, const PairHops& H,
+                                        const float4* __restrict__ p, float sA, float sB, float& dA, float& dB) {
   CP acc[R][3];
-  pr_hops<R, LS>(acc, g, n, xg, W, H);
-  const float4* xo = xg + packed_at<3 * R>(n);
-  const bool second = NR == 1 || s0 + 1 < nrhs;
-  double dots[2] = {0.0, 0.0};
-  if constexpr (R == 4) {
+  pr_hops<R, LS>(acc, g, n, x, W, H);
+  const float4* xo = x + packed_at<3 * R>(n);
+  const float2 sig = make_float2(sA, sB);
+  // one word: epilogue and packed store
+  auto put = [&](int row, CP v) {
+    const int64_t at = packed_at<3 * R>(n) + row * kPackBlock;
+    if constexpr (EPI) {
+      const CP pv = cp_of(__ldg(p + at));
+      v.re = pr_fma(pv.re, sig, v.re);
+      v.im = pr_fma(pv.im, sig, v.im);
+      dA = fmaf(pv.re.x, v.re.x, dA);
+      dB = fmaf(pv.re.y, v.re.y, dB);
+      dA = fmaf(pv.im.x, v.im.x, dA);
+      dB = fmaf(pv.im.y, v.im.y, dB);
+    }
+    if (valid) yo[at] = cp_word(v);
+  };
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < 2; ++h) {
+    if constexpr (R == 4) {
       CP own[6], out[6];
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
@@ -355,47 +366,18 @@ __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
         }
       }
       if constexpr (OUT == 1) {
-        float4* yo = yp + (int64_t)grp * packed_words(g.V, 12) + packed_at<12>(n) + h * 6 * kPackBlock;
 #pragma unroll
-        for (int i = 0; i < 6; ++i) yo[i * kPackBlock] = cp_word(out[i]);
-      } else {
+        for (int i = 0; i < 6; ++i) put(h * 6 + i, out[i]);
+      } else if (valid) {
+        float4* ya = reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
+        float4* yb = reinterpret_cast<float4*>(y0 + rs + (int64_t)n * 24 + h * 12);
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          if (r == 1 && !second) break;
-          float o[12];
-#pragma unroll
-          for (int i = 0; i < 6; ++i) {
-            o[2 * i] = r ? out[i].re.y : out[i].re.x;
-            o[2 * i + 1] = r ? out[i].im.y : out[i].im.x;
-          }
-          const int64_t at = (int64_t)(s0 + r) * rs + (int64_t)n * 24 + h * 12;
-          if constexpr (EPI) {
-            const float sg = (float)sd.sig[s0 + r];
-            const float4* pp = reinterpret_cast<const float4*>(sd.p + at);
-            float dt = 0.f;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-              const float4 pv = __ldg(pp + i);
-              const float pe[4] = {pv.x, pv.y, pv.z, pv.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                o[4 * i + e] = fmaf(sg, pe[e], o[4 * i + e]);
-                dt = fmaf(pe[e], o[4 * i + e], dt);
-              }
-            }
-            dots[r] += (double)dt;
-          }
-          if (valid) {
-            float4* yo = reinterpret_cast<float4*>(y + at);
-#pragma unroll
-            for (int i = 0; i < 3; ++i) yo[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-          }
+        for (int i = 0; i < 3; ++i) {
+          ya[i] = make_float4(out[2 * i].re.x, out[2 * i].im.x, out[2 * i + 1].re.x, out[2 * i + 1].im.x);
+          yb[i] = make_float4(out[2 * i].re.y, out[2 * i].im.y, out[2 * i + 1].re.y, out[2 * i + 1].im.y);
         }
       }
-    }
-  } else {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    } else {
       C<float> in[6], out[6];
 #pragma unroll
       for (int aa = 0; aa < 3; ++aa) {
@@ -415,63 +397,67 @@ __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
         for (int i = 0; i < 6; ++i) out[i] = out[i] + co[i];
       }
       if constexpr (OUT == 1) {
-        float4* yo = yp + (int64_t)grp * packed_words(g.V, 6) + packed_at<6>(n) + h * 3 * kPackBlock;
 #pragma unroll
         for (int aa = 0; aa < 3; ++aa)
-          yo[aa * kPackBlock] = make_float4(out[aa].re, out[3 + aa].re, out[aa].im, out[3 + aa].im);
-      } else {
-        const int64_t at = (int64_t)s0 * rs + (int64_t)n * 24 + h * 12;
-        if constexpr (EPI) {
-          const float sg = (float)sd.sig[s0];
-          const float4* pp = reinterpret_cast<const float4*>(sd.p + at);
-          float dt = 0.f;
+          put(h * 3 + aa, CP{make_float2(out[aa].re, out[3 + aa].re), make_float2(out[aa].im, out[3 + aa].im)});
+      } else if (valid) {
+        float4* ya = reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
 #pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            const float4 pv = __ldg(pp + i);
-            out[2 * i].re = fmaf(sg, pv.x, out[2 * i].re);
-            out[2 * i].im = fmaf(sg, pv.y, out[2 * i].im);
-            out[2 * i + 1].re = fmaf(sg, pv.z, out[2 * i + 1].re);
-            out[2 * i + 1].im = fmaf(sg, pv.w, out[2 * i + 1].im);
-            dt = fmaf(pv.x, out[2 * i].re, dt);
-            dt = fmaf(pv.y, out[2 * i].im, dt);
-            dt = fmaf(pv.z, out[2 * i + 1].re, dt);
-            dt = fmaf(pv.w, out[2 * i + 1].im, dt);
-          }
-          dots[0] += (double)dt;
-        }
-        if (valid) {
-          float4* yo = reinterpret_cast<float4*>(y + at);
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-            yo[i] = make_float4(out[2 * i].re, out[2 * i].im, out[2 * i + 1].re, out[2 * i + 1].im);
-        }
+        for (int i = 0; i < 3; ++i)
+          ya[i] = make_float4(out[2 * i].re, out[2 * i].im, out[2 * i + 1].re, out[2 * i + 1].im);
       }
-    }
-  }
-  if constexpr (EPI) {
-    const int nb = gfirst ? gridDim.y : gridDim.x;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const double t = pr_block_total(valid ? dots[r] : 0.0);
-      if (threadIdx.x == 0 && (r == 0 || second)) sd.part[(int64_t)(s0 + r) * nb + blk] = t;
     }
   }
 }
 
+// Partials of the epilogue: dA, dB of a pair belong to the systems s0, s0 + 1
+// (R = 4), of one right-hand side (R = 2) both to s0.
+template <int R>
+__device__ __forceinline__ void pr_partials(double* part, int s0, int nb, int blk, bool valid, float dA, float dB) {
+  const double a = valid ? (double)dA : 0.0, b = valid ? (double)dB : 0.0;
+  const double t = pr_block_total(R == 4 ? a : a + b);
+  if (threadIdx.x == 0) part[(int64_t)s0 * nb + blk] = t;
+  if constexpr (R == 4) {
+    const double u = pr_block_total(b);
+    if (threadIdx.x == 0) part[(int64_t)(s0 + 1) * nb + blk] = u;
+  }
+}
+
+// D on `groups` packed groups of one lattice; the first one holds right-hand
+// side rhs0 (and rhs0 + 1).
+template <int R, typename LS, int OUT, bool EPI>
+__global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
+    bri_pair_kernel(Geom g, float* __restrict__ y, float4* __restrict__ yp, const float4* __restrict__ x,
+                    const LS* __restrict__ W, const float* __restrict__ cl, float diag, int rhs0, int gfirst,
+                    const __grid_constant__ PairHops H, PackedDot sd) {
+  const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
+  const int n0 = blk * blockDim.x + threadIdx.x;
+  const bool valid = n0 < g.V;
+  if (!EPI && !valid) return;  // with the epilogue every thread takes part in the block's reduction
+  const int64_t rs = g.V * 24, go = (int64_t)grp * packed_words(g.V, 3 * R);
+  const int s0 = rhs0 + grp * (R / 2);
+  float dA = 0.f, dB = 0.f, sA = 0.f, sB = 0.f;
+  if constexpr (EPI) {
+    sA = (float)sd.sig[s0];
+    sB = R == 4 ? (float)sd.sig[s0 + 1] : sA;
+  }
+  pr_site<R, LS, OUT, EPI>(g, valid ? n0 : 0, valid, y + (int64_t)s0 * rs, rs, yp + go, x + go, W, cl, diag, H,
+                           EPI ? sd.p + go : nullptr, sA, sB, dA, dB);
+  if constexpr (EPI) pr_partials<R>(sd.part, s0, gfirst ? gridDim.y : gridDim.x, blk, valid, dA, dB);
+}
+
 // Spinors [nrhs][V][12] complex64 -> packed groups; group g holds the
-// right-hand sides rhs0 + 2g, rhs0 + 2g + 1 (R = 4; the second repeats the
-// first where it does not exist) or rhs0 + g (R = 2).
-template <int R> __global__ void __launch_bounds__(256) k_pack(int64_t V, const float* __restrict__ x, int rhs0, int nrhs, float4* __restrict__ X) {
+// right-hand sides rhs0 + 2g, rhs0 + 2g + 1 (R = 4) or rhs0 + g (R = 2).
+template <int R> __global__ void __launch_bounds__(256) k_pack(int64_t V, const float* __restrict__ x, int rhs0, float4* __restrict__ X) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // 16-byte word (R = 4) or spin pair (R = 2) of a site
   if (i >= V * 6) return;
   const int64_t n = i / 6;
   const int q = (int)(i - n * 6);
   float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
   if constexpr (R == 4) {
-    const int s = rhs0 + 2 * blockIdx.y;
-    const float* p = x + s * V * 24 + i * 4;
+    const float* p = x + (rhs0 + 2 * (int64_t)blockIdx.y) * V * 24 + i * 4;
     const float4 u = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 v = s + 1 < nrhs ? __ldg(reinterpret_cast<const float4*>(p + V * 24)) : u;
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p + V * 24));
     o[(2 * q) * kPackBlock] = make_float4(u.x, v.x, u.y, v.y);
     o[(2 * q + 1) * kPackBlock] = make_float4(u.z, v.z, u.w, v.w);
   } else {
@@ -482,24 +468,47 @@ template <int R> __global__ void __launch_bounds__(256) k_pack(int64_t V, const 
   }
 }
 
-template <int R>
-inline void launch_pack(int64_t V, const float* x, int rhs0, int nrhs, int groups, float4* X, cudaStream_t s) {
-  k_pack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, x, rhs0, nrhs, X);
+// The way back.
+template <int R> __global__ void __launch_bounds__(256) k_unpack(int64_t V, const float4* __restrict__ X, int rhs0, float* __restrict__ x) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  const float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
+  if constexpr (R == 4) {
+    float* p = x + (rhs0 + 2 * (int64_t)blockIdx.y) * V * 24 + i * 4;
+    const float4 u = __ldg(o + (2 * q) * kPackBlock), v = __ldg(o + (2 * q + 1) * kPackBlock);
+    *reinterpret_cast<float4*>(p) = make_float4(u.x, u.z, v.x, v.z);
+    *reinterpret_cast<float4*>(p + V * 24) = make_float4(u.y, u.w, v.y, v.w);
+  } else {
+    float2* p = reinterpret_cast<float2*>(x + (rhs0 + (int64_t)blockIdx.y) * V * 24 + n * 24) + q + 3 * (q / 3);
+    const float4 u = __ldg(o + q * kPackBlock);
+    p[0] = make_float2(u.x, u.z);
+    p[3] = make_float2(u.y, u.w);
+  }
+}
+
+template <int R> inline void launch_pack(int64_t V, const float* x, int rhs0, int groups, float4* X, cudaStream_t s) {
+  k_pack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, x, rhs0, X);
+  note_launch();
+}
+template <int R> inline void launch_unpack(int64_t V, const float4* X, int rhs0, int groups, float* x, cudaStream_t s) {
+  k_unpack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, X, rhs0, x);
   note_launch();
 }
 
 // y (or packed yp) = D x for `groups` packed groups starting at right-hand side rhs0.
 template <int R, typename LS>
 inline void launch_pair(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
-                        int dagger, int rhs0, int nrhs, int groups, cudaStream_t s, const ShiftDot<float>* sd) {
+                        int dagger, int rhs0, int groups, cudaStream_t s, const PackedDot* sd) {
   const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
-  const ShiftDot<float> none{nullptr, nullptr, nullptr};
+  const PackedDot none{nullptr, nullptr, nullptr};
   if (sd)
-    bri_pair_kernel<R, LS, 0, true><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), *sd);
+    bri_pair_kernel<R, LS, 1, true><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), *sd);
   else if (yp)
-    bri_pair_kernel<R, LS, 1, false><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), none);
+    bri_pair_kernel<R, LS, 1, false><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), none);
   else
-    bri_pair_kernel<R, LS, 0, false><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, nrhs, sg.gfirst, pair_hops(dagger), none);
+    bri_pair_kernel<R, LS, 0, false><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), none);
   note_launch();
 }
 

@@ -16,16 +16,14 @@
 
 namespace bri {
 
+// y = D x on the S sites of block blk for one right-hand side (x, y, p0 its
+// vectors); EPI: y = D x + sg p0, returns this thread's part of Re<p0, y>.
 template <typename R, typename LS, int S, int G, bool EPI>
-__global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
-    bri_split_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, const LS* __restrict__ W,
-                     const R* __restrict__ cl, R diag, R sgn, int gfirst, const __grid_constant__ HopTable<R> H,
-                     ShiftDot<R> sd) {
+__device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restrict__ yout, const R* __restrict__ xin,
+                                              const LS* __restrict__ W, const R* __restrict__ cl, R diag, R sgn,
+                                              const HopTable<R>& H, const R* __restrict__ p0, R sg) {
   __shared__ R red[G][24][S];
-  const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   const int V = (int)g.V;
-  const int64_t rs = g.V * 24;
-  const R* xin = x + s * rs;
   {
     const int site = threadIdx.x % S, grp = threadIdx.x / S;
     const int n = min(blk * S + site, V - 1);
@@ -142,16 +140,27 @@ __global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
         }
       }
     }
-    const int64_t at = s * rs + (int64_t)n * 24 + 2 * e;
+    const int64_t at = (int64_t)n * 24 + 2 * e;
     if constexpr (EPI) {
-      const C<R> p = *reinterpret_cast<const C<R>*>(sd.p + at);
-      const R sg = (R)sd.sig[s];
+      const C<R> p = *reinterpret_cast<const C<R>*>(p0 + at);
       o.re = fma(sg, p.re, o.re);
       o.im = fma(sg, p.im, o.im);
       dot += (double)fma(p.re, o.re, p.im * o.im);
     }
-    *reinterpret_cast<C<R>*>(y + at) = o;
+    *reinterpret_cast<C<R>*>(yout + at) = o;
   }
+  return dot;
+}
+
+template <typename R, typename LS, int S, int G, bool EPI>
+__global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
+    bri_split_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, const LS* __restrict__ W,
+                     const R* __restrict__ cl, R diag, R sgn, int gfirst, const __grid_constant__ HopTable<R> H,
+                     ShiftDot<R> sd) {
+  const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
+  const int64_t o = s * (g.V * 24);
+  double dot = split_block<R, LS, S, G, EPI>(g, blk, y + o, x + o, W, cl, diag, sgn, H, EPI ? sd.p + o : nullptr,
+                                             EPI ? (R)sd.sig[s] : (R)0);
   if constexpr (EPI) {
     __shared__ double sh[(S * G + 31) / 32];
 #pragma unroll

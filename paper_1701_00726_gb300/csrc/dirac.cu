@@ -46,17 +46,16 @@ int dirac_kernel(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int da
 }
 
 int dirac_bri_packed(bri_ctx* c, float* y, void* yp, const void* X, int nrhs, int na, double m0, int dagger, int prec,
-                     cudaStream_t s, const float* p, const double* sig, double* part, int* sd_blocks) {
+                     cudaStream_t s, const void* p, const double* sig, double* part, int* sd_blocks) {
   const float diag = (float)(15.0 / 8.0 + m0);
   const float* cl = c->have_clover ? c->C32 : nullptr;
-  const ShiftDot<float> sd{p, sig, part};
   cudaEvent_t ev;
   int rc = prof_begin(c, s, &ev);
   if (rc) return rc;
   if (prec == BRI_PREC_F32_BF16)
-    rc = bri_f32_on_packed<__nv_bfloat162>(c->g, y, yp, X, c->W16, cl, diag, nrhs, na, dagger, s, p ? &sd : nullptr, sd_blocks);
+    rc = bri_f32_on_packed<__nv_bfloat162>(c->g, y, yp, X, c->W16, cl, diag, nrhs, na, dagger, s, p, sig, part, sd_blocks);
   else
-    rc = bri_f32_on_packed<float2>(c->g, y, yp, X, c->W32, cl, diag, nrhs, na, dagger, s, p ? &sd : nullptr, sd_blocks);
+    rc = bri_f32_on_packed<float2>(c->g, y, yp, X, c->W32, cl, diag, nrhs, na, dagger, s, p, sig, part, sd_blocks);
   if (rc) return rc;
   return prof_end(c, s, ev, 0, prec, (double)c->g.V * na);
 }

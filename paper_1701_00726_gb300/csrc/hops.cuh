@@ -94,19 +94,4 @@ __device__ __forceinline__ void gamma_term(C<R> acc[4], const C<R> v[4], R c) {
   }
 }
 
-// One colour of the accumulator (four spins): acc += a u + sum_mu cs_mu gamma_mu v.
-template <typename R>
-__device__ __forceinline__ void add_pair_terms(C<R> acc[4], const C<R> u[4], const C<R> v[4], R a, R c1, R c2,
-                                               R c3, R c4) {
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    acc[s].re = fma(a, u[s].re, acc[s].re);
-    acc[s].im = fma(a, u[s].im, acc[s].im);
-  }
-  gamma_term<1>(acc, v, c1);
-  gamma_term<2>(acc, v, c2);
-  gamma_term<3>(acc, v, c3);
-  gamma_term<4>(acc, v, c4);
-}
-
 }  // namespace bri

@@ -29,7 +29,7 @@
 #include "internal.cuh"
 #include "cplx.cuh"
 #include "bri_pair.cuh"
-#include "bri_site.cuh"
+#include "bri_split.cuh"
 
 #include <algorithm>
 #include <chrono>
@@ -60,6 +60,7 @@ struct MsState {
   double a_s[NS], b_s[NS];
   int active[NS];
   int nshift, done, iters, maxiter, error;
+  int pend;  // this iteration's alpha holds (also in the iteration that converges)
 };
 
 // Deferred shifted updates (FP32 solves): the coefficients of up to DW
@@ -324,52 +325,6 @@ __global__ void k_update_p0(int64_t n2, const MsState* __restrict__ st, const ty
   }
 }
 
-// The same with the packed copy X of the directions (bri_pair.cuh: pairs of
-// systems, then the odd one) written in the same pass: the next application of
-// D reads X.  One thread per site and 16-byte word (R = 4) or spin pair (R = 2).
-template <int R>
-__global__ void __launch_bounds__(256) k_update_p0_packed(int64_t V, int s0, const MsState* __restrict__ st,
-                                                          const float* __restrict__ r, float* __restrict__ p,
-                                                          float4* __restrict__ X) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= V * 6) return;
-  const int64_t n = i / 6;
-  const int q = (int)(i - n * 6);
-  float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
-  if constexpr (R == 4) {
-    const int s = s0 + 2 * blockIdx.y;
-    const bool da = st[s].done, db = st[s + 1].done;
-    if (da && db) return;
-    float4 v[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int64_t at = (s + k) * V * 24 + i * 4;
-      v[k] = *reinterpret_cast<const float4*>(p + at);
-      if (k ? db : da) continue;
-      const float bt = (float)st[s + k].b_s[0];
-      const float4 rv = __ldg(reinterpret_cast<const float4*>(r + at));
-      v[k] = make_float4(fmaf(bt, v[k].x, rv.x), fmaf(bt, v[k].y, rv.y), fmaf(bt, v[k].z, rv.z), fmaf(bt, v[k].w, rv.w));
-      *reinterpret_cast<float4*>(p + at) = v[k];
-    }
-    o[(2 * q) * kPackBlock] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
-    o[(2 * q + 1) * kPackBlock] = make_float4(v[0].z, v[1].z, v[0].w, v[1].w);
-  } else {
-    const int s = s0 + blockIdx.y;
-    if (st[s].done) return;
-    const float bt = (float)st[s].b_s[0];
-    const int64_t at = s * V * 24 + n * 24 + 2 * (q + 3 * (q / 3));  // spins 2h, 2h + 1 of colour q % 3, h = q / 3
-    float2 v[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      float2* pp = reinterpret_cast<float2*>(p + at) + 3 * k;
-      const float2 rv = __ldg(reinterpret_cast<const float2*>(r + at) + 3 * k);
-      v[k] = make_float2(fmaf(bt, pp->x, rv.x), fmaf(bt, pp->y, rv.y));
-      *pp = v[k];
-    }
-    o[q * kPackBlock] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
-  }
-}
-
 // ----------------------------------------------------------------- scalar kernels (one block per system)
 __global__ void k_scalar_init(MsState* st, const double* part, int nblk) {
   const int s = blockIdx.x;
@@ -396,80 +351,106 @@ __global__ void k_scalar_init(MsState* st, const double* part, int nblk) {
   }
 }
 
-__global__ void k_scalar_alpha(MsState* st, const double* part, int nblk, ShiftHist* hist = nullptr) {
+// alpha = ||r||^2 / <p, q> and the shifts' zeta_{k+1}, alpha^i (thread k: shift
+// k).  hist: the coefficients of this iteration for the deferred updates, shift
+// 0 among them with lag0; reset starts a new window.
+__global__ void k_scalar_alpha(MsState* st, const double* part, int nblk, ShiftHist* hist = nullptr, int reset = 0,
+                               int lag0 = 0) {
   const int s = blockIdx.x;
-  if (st[s].done) return;
+  MsState& S = st[s];
+  if (hist && reset && threadIdx.x == 0) hist[s].n = 0;
+  if (S.done) {
+    if (threadIdx.x == 0) S.pend = 0;
+    return;
+  }
   double acc = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += part[s * nblk + i];
-  double pq = block_sum(acc);
-  if (threadIdx.x == 0) {
-    MsState& S = st[s];
-    if (!(pq > 0.0) || !isfinite(pq)) {
+  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += part[s * (int64_t)nblk + i];
+  __shared__ double spq;
+  const double t = block_sum(acc);
+  if (threadIdx.x == 0) spq = t;
+  __syncthreads();
+  const double pq = spq;
+  const int k = threadIdx.x;
+  if (!(pq > 0.0) || !isfinite(pq)) {
+    if (k < S.nshift) S.active[k] = 0;
+    if (k == 0) {
       S.error = 1;
       S.done = 1;
-      for (int k = 0; k < S.nshift; ++k) S.active[k] = 0;
-      return;
+      S.pend = 0;
     }
-    const double alpha = S.rr / pq;
-    S.pq = pq;
-    S.alpha = alpha;
-    // Lanczos diagonal T_kk = 1/alpha_k + beta_{k-1}/alpha_{k-1}
-    const double tkk = 1.0 / alpha + (S.iters > 0 ? S.beta_prev / S.alpha_prev : 0.0);
-    S.lam_max = fmax(S.lam_max, tkk);
-    for (int k = 0; k < S.nshift; ++k) {
-      if (!S.active[k]) continue;  // frozen shifts keep their last coefficients
+    return;
+  }
+  const double alpha = S.rr / pq;
+  const int m = hist ? hist[s].n : 0;
+  if (k < S.nshift) {
+    const int act = S.active[k];
+    if (act) {  // frozen shifts keep their last coefficients
       const double den = alpha * S.beta_prev * (S.zeta_prev[k] - S.zeta[k]) +
                          S.zeta_prev[k] * S.alpha_prev * (1.0 + S.delta[k] * alpha);
       const double zn = S.zeta[k] * S.zeta_prev[k] * S.alpha_prev / den;
       S.zeta_next[k] = zn;
       S.a_s[k] = alpha * zn / S.zeta[k];
     }
-    if (hist) {  // the coefficients this iteration's shifted update (i > 0) uses
+    if (hist) {
       ShiftHist& h = hist[s];
-      const int m = h.n++;
-      h.first[m] = S.iters == 0;
-      for (int k = 0; k < S.nshift; ++k) {
-        h.act[m][k] = (k > 0 && S.active[k]) ? 1 : 0;
-        h.z[m][k] = (float)S.zeta[k];
-        h.b[m][k] = (float)S.b_s[k];
-        h.a[m][k] = S.a_s[k];
-      }
+      h.act[m][k] = ((k > 0 || lag0) && act) ? 1 : 0;
+      h.z[m][k] = (float)S.zeta[k];
+      h.b[m][k] = (float)S.b_s[k];
+      h.a[m][k] = S.a_s[k];
+    }
+  }
+  __syncthreads();
+  if (k == 0) {
+    S.pq = pq;
+    S.alpha = alpha;
+    S.pend = 1;
+    // Lanczos diagonal T_kk = 1/alpha_k + beta_{k-1}/alpha_{k-1}
+    const double tkk = 1.0 / alpha + (S.iters > 0 ? S.beta_prev / S.alpha_prev : 0.0);
+    S.lam_max = fmax(S.lam_max, tkk);
+    if (hist) {
+      hist[s].first[m] = S.iters == 0;
+      hist[s].n = m + 1;
     }
   }
 }
 
+// beta = ||r_new||^2 / ||r||^2, the shifts' beta^i, and convergence (thread k: shift k).
 __global__ void k_scalar_beta(MsState* st, const double* part, int nblk) {
   const int s = blockIdx.x;
-  if (st[s].done) return;
+  MsState& S = st[s];
+  if (S.done) return;
   double acc = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += part[s * nblk + i];
-  double rr = block_sum(acc);
-  if (threadIdx.x == 0) {
-    MsState& S = st[s];
-    if (!isfinite(rr)) {
+  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += part[s * (int64_t)nblk + i];
+  __shared__ double srr;
+  const double t = block_sum(acc);
+  if (threadIdx.x == 0) srr = t;
+  __syncthreads();
+  const double rr = srr;
+  const int k = threadIdx.x;
+  if (!isfinite(rr)) {
+    if (k < S.nshift) S.active[k] = 0;
+    if (k == 0) {
       S.error = 1;
       S.done = 1;
-      for (int k = 0; k < S.nshift; ++k) S.active[k] = 0;
-      return;
     }
-    const double beta = rr / S.rr;
-    for (int k = 0; k < S.nshift; ++k) {
-      if (!S.active[k]) continue;
-      const double ratio = S.zeta_next[k] / S.zeta[k];
-      S.b_s[k] = beta * ratio * ratio;
-      S.zeta_prev[k] = S.zeta[k];
-      S.zeta[k] = S.zeta_next[k];
-    }
+    return;
+  }
+  const double beta = rr / S.rr;
+  if (k < S.nshift && S.active[k]) {
+    const double zn = S.zeta_next[k], ratio = zn / S.zeta[k];
+    S.b_s[k] = beta * ratio * ratio;
+    S.zeta_prev[k] = S.zeta[k];
+    S.zeta[k] = zn;
+    if (zn * zn * rr <= S.tol2 * S.bnorm2) S.active[k] = 0;
+  }
+  __syncthreads();
+  if (k == 0) {
     S.alpha_prev = S.alpha;
     S.beta_prev = beta;
     S.rr = rr;
     S.iters += 1;
-    for (int k = 0; k < S.nshift; ++k)
-      if (S.active[k] && S.zeta[k] * S.zeta[k] * rr <= S.tol2 * S.bnorm2) S.active[k] = 0;
-    if (!S.active[0] || S.iters >= S.maxiter) {
-      // p updates of the still-active (larger) shifts are skipped once the base stops
-      S.done = 1;
-    }
+    // p updates of the still-active (larger) shifts are skipped once the base stops
+    if (!S.active[0] || S.iters >= S.maxiter) S.done = 1;
   }
 }
 
@@ -597,26 +578,20 @@ struct SysDesc {
   int64_t n2, off, offn;
 };
 
-// NR = 2: the item's system s and s + 1 (same lattice, adjacent in the table)
-// share the link loads, as in the lattice-wide kernel with two right-hand
-// sides per thread; the pair is skipped only when both have converged.
-template <typename R, typename LS, int NR, int MINB>
-__global__ void __launch_bounds__(128, MINB)
+// FP64 stencil on the work list: item (system, block of S sites), the hop pairs
+// of a site split over the block's groups (bri_split.cuh).
+template <int S, int G>
+__global__ void __launch_bounds__(S* G, 2)
     kb_stencil(const __grid_constant__ BatchTab T, const SysDesc* __restrict__ sd, const int2* __restrict__ items,
-               const MsState* __restrict__ st, typename P2<R>::T* y, const typename P2<R>::T* x, int x_from_p,
-               int nshift, R sgn, const __grid_constant__ HopTable<R> H) {
+               const MsState* __restrict__ st, double2* y, const double2* x, int x_from_p, double sgn,
+               const __grid_constant__ HopTable<double> H) {
   const int2 it = items[blockIdx.x];
-  const int s = it.x;
-  const bool live = !st[s].done || (NR == 2 && !st[s + 1].done);
-  if (!live) return;
-  const SysDesc d = sd[s];
+  if (st[it.x].done) return;
+  const SysDesc d = sd[it.x];
   const BatchLat& L = T.lat[d.lat];
-  const int n = it.y * 128 + threadIdx.x;
-  if (n >= L.g.V) return;
-  const R* xin = reinterpret_cast<const R*>(x + (x_from_p ? d.offn : d.off));
-  R* yout = reinterpret_cast<R*>(y + d.off);
-  const int64_t xstride = 2 * (x_from_p ? (int64_t)nshift * d.n2 : d.n2), ystride = 2 * d.n2;
-  bri_site<R, LS, NR>(L.g, n, yout, xin, xstride, ystride, (const LS*)L.W, (const R*)L.C, (R)L.diag, sgn, H);
+  split_block<double, double2, S, G, false>(L.g, it.y, reinterpret_cast<double*>(y + d.off),
+                                            reinterpret_cast<const double*>(x + (x_from_p ? d.offn : d.off)),
+                                            (const double2*)L.W, (const double*)L.C, L.diag, sgn, H, nullptr, 0.0);
 }
 
 // r = b, p_k = b, x_k = 0, partial ||b||^2
@@ -739,8 +714,9 @@ __global__ void kb_update_p0(const SysDesc* __restrict__ sd, const MsState* __re
 // cap, so the loop ends after at most maxiter passes).
 __global__ void kb_while(cudaGraphConditionalHandle h, const MsState* __restrict__ st, int nsys) {
   int any = 0;
-  for (int s = 0; s < nsys; ++s) any |= !st[s].done;
-  cudaGraphSetConditional(h, any ? 1u : 0u);
+  for (int s = threadIdx.x; s < nsys; s += 32) any |= !st[s].done;
+  any = __any_sync(0xffffffffu, any);
+  if (threadIdx.x == 0) cudaGraphSetConditional(h, any ? 1u : 0u);
 }
 
 // X_l[k][r][i] (one lattice's layout) = x[offn(s) + k n2 + i] of system s = s0 + r
@@ -823,6 +799,54 @@ template <> int op_prec<double>(int) { return BRI_PREC_F64; }
 template <> int op_prec<float>(int prec) { return prec == BRI_PREC_F32_BF16 ? BRI_PREC_F32_BF16 : BRI_PREC_F32; }
 
 
+#include "packed_solve.cuh"
+
+// One lattice's FP32 solve on packed vectors (multishift_solve's arguments).
+int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, const double* sig, const float* b, float* x,
+                         double tol, int maxiter, int* iters_out, Counters* cnt, const double* tols, double* lam_out,
+                         double* x64) {
+  cudaStream_t st = c->stream;
+  const int64_t V = c->g.V, n2 = V * 12;
+  PackedProblem pb;
+  pb.nsys = nsys;
+  pb.nshift = nshift;
+  pb.maxiter = maxiter;
+  pb.sig.assign(sig, sig + (size_t)nsys * nshift);
+  for (int s = 0; s < nsys; ++s) pb.tol.push_back(tols ? tols[s] : tol);
+  for (int s = 0; s < nsys;) {
+    GroupDesc g;
+    memset(&g, 0, sizeof(g));
+    g.s0 = s;
+    g.two = s + 1 < nsys;
+    g.V = V;
+    g.poff = pb.words;
+    g.offn = s * n2;
+    g.kstr = nsys * n2;
+    pb.words += packed_words(V, g.two ? 12 : 6);
+    pb.grp.push_back(g);
+    s += g.two ? 2 : 1;
+  }
+  const int nb = blocks_for(V, 128);
+  DevBuf bsig, bsd, bx;
+  int rc;
+  if ((rc = bsig.alloc(sizeof(double) * nsys, st))) return rc;
+  if ((rc = bsd.alloc(sizeof(double) * nsys * nb, st))) return rc;
+  if (!x64 && (rc = bx.alloc(sizeof(float4) * pb.words, st))) return rc;
+  std::vector<double> hsig(nsys);
+  for (int s = 0; s < nsys; ++s) hsig[s] = sig[(size_t)s * nshift];
+  BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));
+  auto pack = [&](float4* dst) { return bri_f32_pack(V, b, nsys, dst, st); };
+  auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int na) {
+    return dirac_bri_packed(c, nullptr, Y, X, nsys, na, m0, dagger, prec, st, P, bsig.as<double>(), bsd.as<double>());
+  };
+  const bool graphs = graphs_enabled() && !c->prof_on && st != nullptr;
+  rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), nb, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
+                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out);
+  if (rc < 0 || x64) return rc;
+  const int q = bri_f32_unpack(V, bx.p, nsys, x, st);
+  return q ? q : rc;
+}
+
 // Solve (A + sig[s][k]) x[k][s] = b[s] for nsys systems with nshift shifts each.
 // sig: host [nsys][nshift], increasing within a system.  x64 (R = float only):
 // the solutions are accumulated in FP64 there instead of in x (x unused).
@@ -831,17 +855,20 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
                      double tol, int maxiter, int* iters_out, Counters* cnt, const double* tols,
                      double* lam_out = nullptr, const KernelOp* op = nullptr, double* x64 = nullptr) {
   using T = typename P2<R>::T;
+  const int oprec = op_prec<R>(prec);
+  // FP32 solves large enough for the packed stencil keep their vectors in its layout
+  if constexpr (sizeof(R) == 4) {
+    if (!op && c->kernel == BRI_KERNEL_BRILLOUIN && bri_f32_packed(c->g.V, nsys) && (x64 || nshift == 1))
+      return packed_lattice_solve(c, oprec, m0, nsys, nshift, sig, b, x, tol, maxiter, iters_out, cnt, tols, lam_out, x64);
+  }
   cudaStream_t st = c->stream;
   const int64_t n2 = c->g.V * 12;  // complex pairs per system
   const int nblk = grid_for(n2, nsys);
-  const int oprec = op_prec<R>(prec);
   DevBuf br, bp, bt, bq, bst, bpart;
   int rc;
   if ((rc = br.alloc(sizeof(T) * n2 * nsys, st))) return rc;
   if ((rc = bp.alloc(sizeof(T) * n2 * nsys * nshift, st))) return rc;
-  // t may hold a packed vector (whole blocks of 32 sites)
-  const size_t t_bytes = sizeof(R) == 4 ? std::max(sizeof(T) * n2 * nsys, bri_f32_packed_bytes(c->g.V, nsys)) : sizeof(T) * n2 * nsys;
-  if ((rc = bt.alloc(t_bytes, st))) return rc;
+  if ((rc = bt.alloc(sizeof(T) * n2 * nsys, st))) return rc;
   if ((rc = bq.alloc(sizeof(T) * n2 * nsys, st))) return rc;
   if ((rc = bst.alloc(sizeof(MsState) * nsys, st))) return rc;
   if ((rc = bpart.alloc(sizeof(double) * nblk * nsys, st))) return rc;
@@ -868,11 +895,6 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   // and the partials of Re<p_0, q> come out of the stencil's epilogue, so
   // k_shift_dot's pass over q and p_0 is not needed.
   const bool fused = op == nullptr && c->kernel == BRI_KERNEL_BRILLOUIN;
-  // FP32 solves large enough for the packed stencil keep p_0 and t = D p_0 in
-  // its layout: D writes t packed, the direction update writes p_0 both ways.
-  const bool packed = sizeof(R) == 4 && fused && bri_f32_packed(c->g.V, nsys);
-  DevBuf bpk;
-  if (packed && (rc = bpk.alloc(bri_f32_packed_bytes(c->g.V, nsys), st))) return rc;
   // Deferred shifted updates (FP32 solve with FP64 solutions): the shifted
   // directions and solutions are advanced every DW iterations from a ring of
   // the residuals of those iterations (same arithmetic, fewer passes).
@@ -900,7 +922,6 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   note_launch();
   k_scalar_init<<<nsys, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
   BRI_LAUNCH_CHECK("multishift init");
-  if (packed && (rc = bri_f32_pack(c->g.V, (const float*)p, nsys, bpk.p, st))) return rc;
 
   int* hdone = (int*)c->host_pinned;  // pinned scratch, >= 4 KB
   const int check_every = 8;
@@ -922,16 +943,9 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
         if ((q = op->apply((double2*)q_vec, (const double2*)t, na, 1))) return q;
       } else if (fused) {
         int nb = 0;
-        if (packed) {
-          if ((q = dirac_bri_packed(c, nullptr, t, bpk.p, nsys, na, m0, 0, oprec, st))) return q;
-          if ((q = dirac_bri_packed(c, (float*)q_vec, nullptr, t, nsys, na, m0, 1, oprec, st, (const float*)p,
-                                    bsig.as<double>(), bpart_sd.as<double>(), &nb)))
-            return q;
-        } else if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) {
+        if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) return q;
+        if ((q = dirac_bri_shiftdot(c, q_vec, t, na, m0, oprec, st, p, bsig.as<double>(), bpart_sd.as<double>(), &nb)))
           return q;
-        } else if ((q = dirac_bri_shiftdot(c, q_vec, t, na, m0, oprec, st, p, bsig.as<double>(), bpart_sd.as<double>(), &nb))) {
-          return q;
-        }
         k_scalar_alpha<<<na, RED_THREADS, 0, st>>>(S, bpart_sd.as<double>(), nb, hist); note_launch();
       } else {
         if ((q = dirac_kernel(c, t, p, na, m0, 0, oprec, st))) return q;
@@ -951,21 +965,7 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
         k_update_fused<R><<<vga, RED_THREADS, 0, st>>>(n2, nsys, S, q_vec, r, p, (T*)x, part, it0 + j == 0 ? 1 : 0);
       note_launch();
       k_scalar_beta<<<na, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
-      if (packed) {
-        const int pairs = nsys / 2, act = std::min(pairs, (na + 1) / 2);
-        const int vb = blocks_for(c->g.V * 6, 256);
-        if (act) {
-          k_update_p0_packed<4><<<dim3(vb, act), 256, 0, st>>>(c->g.V, 0, S, (const float*)r, (float*)p, bpk.as<float4>());
-          note_launch();
-        }
-        if (nsys % 2 && na == nsys) {
-          k_update_p0_packed<2><<<dim3(vb, 1), 256, 0, st>>>(c->g.V, nsys - 1, S, (const float*)r, (float*)p,
-                                                             bpk.as<float4>() + packed_words(c->g.V, 12) * pairs);
-          note_launch();
-        }
-      } else {
-        k_update_p0<R><<<vga, RED_THREADS, 0, st>>>(n2, S, r, p); note_launch();
-      }
+      k_update_p0<R><<<vga, RED_THREADS, 0, st>>>(n2, S, r, p); note_launch();
       if (defer && ((j + 1) % DW == 0 || j == count - 1)) {
         k_flush_shifts<<<vga, RED_THREADS, 0, st>>>(n2, nsys, hist, (const float2*)bring.p, (float2*)p,
                                                     (double2*)x64);
@@ -1303,32 +1303,27 @@ int refine_mixed(bri_ctx* c, const double* b, int nrhs, int n, const double* sig
   return solve_rc;
 }
 
-// Phase 1 on the system table: multi-shift CG of every system of every
+// FP64 phase on the system table: multi-shift CG of every system of every
 // lattice at once.  The first iteration is launched directly; the rest run
 // inside one CUDA graph whose WHILE node repeats the iteration body until
 // every system is done (the condition is set on the device by kb_while), so
 // the host neither polls nor relaunches.  x = [system][shift][n2].
-template <typename R, typename LS>
-int batch_multishift(cudaStream_t st, const BatchTab& tab, const std::vector<SysDesc>& sdh, int nshift,
-                     const double* sig, const typename P2<R>::T* b, double2* x, double tol, int maxiter,
-                     int* iters_out, Counters* cnt, double* lam_out) {
-  using T = typename P2<R>::T;
+int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector<SysDesc>& sdh, int nshift,
+                         const double* sig, const double2* b, double2* x, double tol, int maxiter, int* iters_out,
+                         Counters* cnt, double* lam_out) {
+  using R = double;
+  using T = double2;
   const int S = (int)sdh.size();
   int64_t tot = 0, maxn2 = 0;
-  // work items: (first system of a same-lattice pair, block) and (single system, block)
-  std::vector<int2> items2, items1;
+  std::vector<int2> items;  // (system, block of sites)
   for (int s = 0; s < S; ++s) {
     tot += sdh[s].n2;
     maxn2 = std::max(maxn2, sdh[s].n2);
   }
-  for (int s = 0; s < S;) {
-    const int64_t nb = (tab.lat[sdh[s].lat].g.V + 127) / 128;
-    const bool pair = s + 1 < S && sdh[s + 1].lat == sdh[s].lat;
-    for (int64_t k = 0; k < nb; ++k) (pair ? items2 : items1).push_back(make_int2(s, (int)k));
-    s += pair ? 2 : 1;
-  }
-  const int n2items = (int)items2.size(), n1items = (int)items1.size();
-  const int nitems = n2items + n1items;
+  const int sites = split_sites(tot / 12);
+  for (int s = 0; s < S; ++s)
+    for (int k = 0; k < blocks_for(sdh[s].n2 / 12, sites); ++k) items.push_back(make_int2(s, k));
+  const int nitems = (int)items.size();
   const int nblk = grid_for(maxn2, S);
   DevBuf bsd, bit, br, bt, bq, bp, bst, bpart;
   int rc;
@@ -1355,31 +1350,24 @@ int batch_multishift(cudaStream_t st, const BatchTab& tab, const std::vector<Sys
     h.maxiter = maxiter;
   }
   BRI_CUDA(cudaMemcpyAsync(bsd.p, sdh.data(), sizeof(SysDesc) * S, cudaMemcpyHostToDevice, st));
-  if (n2items)
-    BRI_CUDA(cudaMemcpyAsync(bit.p, items2.data(), sizeof(int2) * n2items, cudaMemcpyHostToDevice, st));
-  if (n1items)
-    BRI_CUDA(cudaMemcpyAsync(bit.as<int2>() + n2items, items1.data(), sizeof(int2) * n1items, cudaMemcpyHostToDevice,
-                             st));
+  BRI_CUDA(cudaMemcpyAsync(bit.p, items.data(), sizeof(int2) * nitems, cudaMemcpyHostToDevice, st));
   BRI_CUDA(cudaMemcpyAsync(S_, hs.data(), sizeof(MsState) * S, cudaMemcpyHostToDevice, st));
   // the host copies above read pageable vectors: complete them before they go out of scope
   BRI_CUDA(cudaStreamSynchronize(st));
   const dim3 vg(nblk, S);
-  constexpr int MINB1 = sizeof(R) == 8 ? 2 : 4, MINB2 = sizeof(R) == 8 ? 2 : 3;
-  const HopTable<R>& H = hop_table<R>();
-  const int2* it2 = bit.as<int2>();
-  const int2* it1 = bit.as<int2>() + n2items;
-  auto stencil = [&](typename P2<R>::T* out, const typename P2<R>::T* in, int from_p, R sgn) {
-    if (n2items)
-      kb_stencil<R, LS, 2, MINB2><<<n2items, 128, 0, st>>>(tab, sd, it2, S_, out, in, from_p, nshift, sgn, H);
-    if (n1items)
-      kb_stencil<R, LS, 1, MINB1><<<n1items, 128, 0, st>>>(tab, sd, it1, S_, out, in, from_p, nshift, sgn, H);
+  const HopTable<double>& H = hop_table<double>();
+  const int2* itd = bit.as<int2>();
+  auto stencil = [&](double2* out, const double2* in, int from_p, double sgn) {
+    if (sites == 32) kb_stencil<32, 5><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
+    else if (sites == 16) kb_stencil<16, 10><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
+    else kb_stencil<8, 20><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
   };
-  const int nst = (n2items ? 1 : 0) + (n1items ? 1 : 0);  // stencil launches per application
+  const int nst = 1;  // stencil launches per application
   kb_init<R><<<vg, RED_THREADS, 0, st>>>(sd, nshift, b, r, p, x, part); note_launch();
   k_scalar_init<<<S, RED_THREADS, 0, st>>>(S_, part, nblk); note_launch();
   auto iteration = [&](int first) {
-    stencil(t, p, 1, (R)1);
-    stencil(q, t, 0, (R)-1);
+    stencil(t, p, 1, 1.0);
+    stencil(q, t, 0, -1.0);
     kb_shift_dot<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, p, q, part);
     k_scalar_alpha<<<S, RED_THREADS, 0, st>>>(S_, part, nblk);
     kb_update<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, q, r, p, x, part, first);
@@ -1416,7 +1404,7 @@ int batch_multishift(cudaStream_t st, const BatchTab& tab, const std::vector<Sys
   e = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return fail(e, "batched multi-shift: capture");
   iteration(0);
-  kb_while<<<1, 1, 0, st>>>(handle, S_, S);
+  kb_while<<<1, 32, 0, st>>>(handle, S_, S);
   e = cudaStreamEndCapture(st, &body);
   if (e != cudaSuccess) return fail(e, "batched multi-shift: end capture");
   e = cudaGraphInstantiate(&gexec, graph, 0);
@@ -1439,7 +1427,7 @@ int batch_multishift(cudaStream_t st, const BatchTab& tab, const std::vector<Sys
   note_launches((long long)(6 + 2 * nst) * std::max(0, maxit - 1));
   *iters_out = maxit;
   cnt->matvecs += 2 * maxit;
-  if (sizeof(R) == 8) cnt->matvecs64 += 2 * maxit;
+  cnt->matvecs64 += 2 * maxit;
   if (lam_out) *lam_out = lm;
   if (err) {
     set_error("batched multi-shift CG: non-finite or non-positive curvature in a reduction");
@@ -1718,28 +1706,27 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
   SolveInfo info1;
   int solve_rc = BRI_OK;
   double lam_est = 0.0;
-  auto phase1 = [&](auto tag, auto ltag) -> int {
-    using R = decltype(tag);
-    using LS = decltype(ltag);
-    using T = typename P2<R>::T;
+  std::vector<double*> Xp(nctx);  // [n][nrhs][V*24] FP64 per lattice
+  DevBuf bXall;
+  auto phase1_f64 = [&]() -> int {
     DevBuf bb, bx;
     int q;
-    if ((q = bb.alloc(sizeof(T) * off, bs))) return q;
+    if ((q = bb.alloc(sizeof(double2) * off, bs))) return q;
     if ((q = bx.alloc(sizeof(double2) * off * n, bs))) return q;
     for (int i = 0; i < nctx; ++i) {
-      kb_scatter_b<R><<<dim3(grid_for(cs[i]->g.V * 12, nrhs[i]), nrhs[i]), RED_THREADS, 0, bs>>>(
-          bsd.as<SysDesc>(), first_sys[i], (const double2*)xs[i], bb.as<T>());
+      kb_scatter_b<double><<<dim3(grid_for(cs[i]->g.V * 12, nrhs[i]), nrhs[i]), RED_THREADS, 0, bs>>>(
+          bsd.as<SysDesc>(), first_sys[i], (const double2*)xs[i], bb.as<double2>());
       note_launch();
     }
-    const double tol1 = sizeof(R) == 8 ? tol : std::max(tol, prec == BRI_PREC_F32 ? 1e-7 : 1e-6);
-    q = batch_multishift<R, LS>(bs, tab, sd, n, sig, bb.as<T>(), bx.as<double2>(), tol1, maxiter, &info1.iters, &info1.cnt,
-                                &lam_est);
+    q = batch_multishift_f64(bs, tab, sd, n, sig, bb.as<double2>(), bx.as<double2>(), tol, maxiter, &info1.iters,
+                                          &info1.cnt, &lam_est);
     if (q < 0) return q;
     solve_rc = std::max(solve_rc, q);
     for (int i = 0; i < nctx; ++i) {
       const int64_t nreal = cs[i]->g.V * 24;
       int qq;
       if ((qq = Xs[i].alloc(sizeof(double) * nreal * nrhs[i] * n, bs))) return qq;
+      Xp[i] = Xs[i].as<double>();
       kb_gather_x<<<dim3(grid_for(cs[i]->g.V * 12, nrhs[i] * n), nrhs[i], n), RED_THREADS, 0, bs>>>(
           bsd.as<SysDesc>(), first_sys[i], nrhs[i], n, bx.as<double2>(), Xs[i].as<double2>());
       note_launch();
@@ -1748,9 +1735,96 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     BRI_CUDA(cudaStreamSynchronize(bs));
     return BRI_OK;
   };
-  if (prec == BRI_PREC_F64) rc = phase1(double(), double2());
-  else if (prec == BRI_PREC_F32) rc = phase1(float(), float2());
-  else rc = phase1(float(), __nv_bfloat162());
+  // FP32: the packed solver on the groups of all lattices, its stencil on a work
+  // list of (group, 128-site block) items, the solutions in each lattice's layout.
+  auto phase1_f32 = [&](auto ltag) -> int {
+    using LS = decltype(ltag);
+    const double tol1 = std::max(tol, prec == BRI_PREC_F32 ? 1e-7 : 1e-6);
+    PackedProblem pb;
+    pb.nsys = S;
+    pb.nshift = n;
+    pb.maxiter = maxiter;
+    pb.tol.assign(S, tol1);
+    for (int s = 0; s < S; ++s) pb.sig.insert(pb.sig.end(), sig, sig + n);
+    std::vector<int2> items2, items1;
+    std::vector<int64_t> lat_poff(nctx), lat_off(nctx);
+    int nb = 0;
+    int64_t maxb = 0;
+    for (int i = 0; i < nctx; ++i) {
+      const int64_t V = cs[i]->g.V, n2 = V * 12;
+      lat_poff[i] = pb.words;
+      lat_off[i] = sd[first_sys[i]].off;
+      nb = std::max(nb, blocks_for(V, 128));
+      maxb = std::max(maxb, n2 * nrhs[i]);
+      for (int r = 0; r < nrhs[i];) {
+        GroupDesc g;
+        memset(&g, 0, sizeof(g));
+        g.s0 = first_sys[i] + r;
+        g.two = r + 1 < nrhs[i];
+        g.lat = i;
+        g.V = V;
+        g.poff = pb.words;
+        g.offn = lat_off[i] * n + r * n2;
+        g.kstr = nrhs[i] * n2;
+        pb.words += packed_words(V, g.two ? 12 : 6);
+        for (int k = 0; k < blocks_for(V, 128); ++k) (g.two ? items2 : items1).push_back(make_int2((int)pb.grp.size(), k));
+        pb.grp.push_back(g);
+        r += g.two ? 2 : 1;
+      }
+    }
+    const int n2i = (int)items2.size(), n1i = (int)items1.size();
+    DevBuf bgd, bit, bsig, bpart, bb;
+    int q;
+    if ((q = bgd.alloc(sizeof(GroupDesc) * pb.grp.size(), bs))) return q;
+    if ((q = bit.alloc(sizeof(int2) * (n2i + n1i), bs))) return q;
+    if ((q = bsig.alloc(sizeof(double) * S, bs))) return q;
+    if ((q = bpart.alloc(sizeof(double) * (size_t)S * nb, bs))) return q;
+    if ((q = bb.alloc(sizeof(float2) * maxb, bs))) return q;
+    if ((q = bXall.alloc(sizeof(double2) * off * n, bs))) return q;
+    for (int i = 0; i < nctx; ++i) Xp[i] = (double*)(bXall.as<double2>() + lat_off[i] * n);
+    const std::vector<double> hsig(S, sig[0]);
+    BRI_CUDA(cudaMemcpyAsync(bgd.p, pb.grp.data(), sizeof(GroupDesc) * pb.grp.size(), cudaMemcpyHostToDevice, bs));
+    if (n2i) BRI_CUDA(cudaMemcpyAsync(bit.p, items2.data(), sizeof(int2) * n2i, cudaMemcpyHostToDevice, bs));
+    if (n1i) BRI_CUDA(cudaMemcpyAsync(bit.as<int2>() + n2i, items1.data(), sizeof(int2) * n1i, cudaMemcpyHostToDevice, bs));
+    BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * S, cudaMemcpyHostToDevice, bs));
+    // blocks beyond a smaller lattice's volume contribute nothing to its sums
+    BRI_CUDA(cudaMemsetAsync(bpart.p, 0, sizeof(double) * (size_t)S * nb, bs));
+    auto pack = [&](float4* dst) -> int {
+      for (int i = 0; i < nctx; ++i) {
+        const int64_t V = cs[i]->g.V;
+        k_convert<double, float><<<1024, 256, 0, bs>>>(V * 24 * nrhs[i], (const double*)xs[i], bb.as<float>()); note_launch();
+        if (int e = bri_f32_pack(V, bb.as<float>(), nrhs[i], dst + lat_poff[i], bs)) return e;
+      }
+      return BRI_OK;
+    };
+    const MsState* St = nullptr;
+    auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int) -> int {
+      const PackedDot pd{P, bsig.as<double>(), bpart.as<double>()};
+      const GroupDesc* gd = bgd.as<GroupDesc>();
+      const PairHops& H = pair_hops(dagger);
+      if (n2i) {
+        if (P) kb_pair<4, LS, true><<<n2i, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
+        else kb_pair<4, LS, false><<<n2i, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
+        note_launch();
+      }
+      if (n1i) {
+        const int2* it1 = bit.as<int2>() + n2i;
+        if (P) kb_pair<2, LS, true><<<n1i, 128, 0, bs>>>(tab, gd, it1, St, Y, X, H, pd, nb);
+        else kb_pair<2, LS, false><<<n1i, 128, 0, bs>>>(tab, gd, it1, St, Y, X, H, pd, nb);
+        note_launch();
+      }
+      return BRI_OK;
+    };
+    q = packed_solve(bs, pb, pack, apply, bpart.as<double>(), nb, bXall.as<double2>(), sizeof(double2) * off * n, nullptr, true,
+                     true, nullptr, &info1.iters, &info1.cnt, &lam_est, &St);
+    if (q < 0) return q;
+    solve_rc = std::max(solve_rc, q);
+    BRI_CUDA(cudaStreamSynchronize(bs));
+    return BRI_OK;
+  };
+  if (prec == BRI_PREC_F64) rc = phase1_f64();
+  else if (prec == BRI_PREC_F32) rc = phase1_f32(float2());
+  else rc = phase1_f32(__nv_bfloat162());
   if (rc < 0) return rc;
   lam_est = 1.1 * lam_est + 1e-3;
   const double t_phase1 = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -1776,11 +1850,10 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
       };
       int q = BRI_OK;
       if (prec != BRI_PREC_F64)
-        q = refine_mixed(c, (const double*)xs[i], nrhs[i], n, sig, m0, tol, maxiter, Xs[i].as<double>(), lam_est, inf,
-                         lap);
+        q = refine_mixed(c, (const double*)xs[i], nrhs[i], n, sig, m0, tol, maxiter, Xp[i], lam_est, inf, lap);
       if (q >= 0) {
         if (prec != BRI_PREC_F64) lap(2);
-        const int q2 = finish_sign(c, (double*)ys[i], (const double*)xs[i], nrhs[i], n, c0, w, Xs[i].as<double>(), m0,
+        const int q2 = finish_sign(c, (double*)ys[i], (const double*)xs[i], nrhs[i], n, c0, w, Xp[i], m0,
                                    out_scale, b_coeff, inf.cnt, nullptr);
         if (q2) q = q2;
         cudaStreamSynchronize(c->stream);

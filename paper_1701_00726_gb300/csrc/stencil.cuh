@@ -44,13 +44,6 @@ __device__ __forceinline__ void store_spinor(double* p, const Spinor<double>& s)
   for (int e = 0; e < 12; ++e) q[e] = make_double2(s.v[e / 3][e % 3].re, s.v[e / 3][e % 3].im);
 }
 
-template <typename R> __device__ __forceinline__ void zero(Spinor<R>& s) {
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) s.v[a][b] = C<R>{0, 0};
-}
-
 // One 3x3 link in structure-of-arrays storage: element e of the link at site
 // n sits at p[e*V] (p already offset by n).
 template <typename R, typename LS>
@@ -164,23 +157,6 @@ __device__ __forceinline__ void clover_block(C<R> out[6], const R (&c)[36], cons
     }
 }
 
-// acc += C(n) x, C the two chiral 6x6 clover blocks.
-template <typename R>
-__device__ __forceinline__ void add_clover(Spinor<R>& acc, const Spinor<R>& x, const R* __restrict__ cl,
-                                           int64_t V, int64_t n) {
-#pragma unroll
-  for (int blk = 0; blk < 2; ++blk) {
-    C<R> in[6], out[6];
-    R c[36];
-    load_clover(c, cl, V, n, blk);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) in[i] = x.v[2 * blk + i / 3][i % 3];
-    clover_block(out, c, in);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) acc.v[2 * blk + i / 3][i % 3] = acc.v[2 * blk + i / 3][i % 3] + out[i];
-  }
-}
-
 // Fused solver epilogue of a stencil launch: q = D x + sigma_s p_s at every
 // site, and per block the partial sums of Re<p_s, q> in FP64 (the inner
 // product of the multi-shift CG), written to part[s * blocks + site block] for
@@ -216,13 +192,16 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
 // Packed FP32 vectors (bri_pair.cuh) for callers that keep their vectors in that
 // form: whether a launch of nrhs right-hand sides takes the packed kernels, the
 // size of such a vector, packing, and the operator on it (spinors' layout y or
-// packed yp out, first na of nrhs right-hand sides).
+// packed yp out, first na of nrhs right-hand sides; with the packed vector p the
+// fused solver epilogue, see ShiftDot).
 bool bri_f32_packed(int64_t V, int nrhs);
 size_t bri_f32_packed_bytes(int64_t V, int nrhs);
 int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s);
 template <typename LS>
 int bri_f32_on_packed(const Geom& g, float* y, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs,
-                      int na, int dagger, cudaStream_t s, const ShiftDot<float>* sd = nullptr, int* sd_blocks = nullptr);
+                      int na, int dagger, cudaStream_t s, const void* p = nullptr, const double* sig = nullptr,
+                      double* part = nullptr, int* sd_blocks = nullptr);
+int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s);
 template <typename R, typename LS>
 int launch_wil_t(const Geom& g, R* y, const R* x, const LS* U, const R* cl, R diag, int nrhs, int dagger,
                  cudaStream_t s);
