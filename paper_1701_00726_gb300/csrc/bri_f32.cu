@@ -7,61 +7,53 @@
 
 namespace bri {
 
-// The packed kernels need a thread per site and pair of right-hand sides to
-// fill the chip; below that the split kernel's 5..20 threads per site win.
-// Measured on GB300 (us, split / packed with its packing pass): 4^4 x 1 rhs
-// 6.5 / 26, 8^4 x 1 12 / 29, 8^4 x 4 31 / 39, 9.7.8.16 x 3 41 / 76, 12^4 x 1
-// 35 / 41; above the line 16^4 x 1 113 / 72, 8^3.16 x 12 118 / 84.
-bool bri_f32_packed(int64_t V, int nrhs) { return V * nrhs > 24576; }
+// The packed kernels cost a packing pass, and below some thousand sites they
+// leave the chip idle where the split kernel's 5..20 threads per site do not.
+// Measured on GB300 (us, split / packed with its packing pass): 4^4 x 1 rhs 6.5 /
+// 15, 8^4 x 1 14.7 / 15.5, 8^4 x 2 20.8 / 19.9; above the line 6^4 x 12 33 / 25,
+// 8^4 x 4 31 / 24, 12^4 x 1 39 / 30, 16^4 x 1 102 / 66.
+bool bri_f32_packed(int64_t V, int nrhs) { return V * nrhs > 8192; }
 
-// A packed vector of nrhs right-hand sides: nrhs / 2 pairs, then the odd one.
-size_t bri_f32_packed_bytes(int64_t V, int nrhs) {
-  return sizeof(float4) * (size_t)(packed_words(V, 12) * (nrhs / 2) + (nrhs % 2 ? packed_words(V, 6) : 0));
-}
+// More thread groups per site give more blocks, fewer sites per block share less
+// of each other's cache lines.  Measured on GB300 (us, 1 / 2 / 4 groups, packed
+// out): 8^4 x 1 25 / 15 / 10.6, 8^4 x 4 25 / 19 / 19, 12^4 x 4 81 / 70 / 69, 16^4 x
+// 1 66 / 61 / 62, 8^3.16 x 12 84 / 74 / 72, 16^3.32 x 1 109 / 109 / 109, x 2 191 /
+// 187 / 193, x 4 349 / 354 / 368, x 12 998 / 1023 / 1064, 24^3.48 x 1 521 / 524 / 542.
+int pack_groups(int64_t site_rhs) { return site_rhs <= 98304 ? 4 : (site_rhs <= 393216 ? 2 : 1); }
+
+// Pairs of right-hand sides share a link's loads, single ones have twice the
+// threads.  Measured on GB300 (us, spinors' own layout out, pairs / the better of
+// one and two groups of singles): 16^3.32 x 4 359 / 355, x 12 993 / 1019, 24^3.48 x 4
+// 1760 / 1811.  (Packed out the pairs lose: 381 / 349, 1048 / 998, 1853 / 1768.)
+static bool take_pairs(int64_t V, int nrhs) { return nrhs > 1 && V * nrhs > 786432; }
 
 int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s) {
-  const int pairs = nrhs / 2;
-  float4* X4 = (float4*)X;
-  if (pairs) launch_pack<4>(V, x, 0, pairs, X4, s);
-  if (nrhs % 2) launch_pack<2>(V, x, nrhs - 1, 1, X4 + packed_words(V, 12) * pairs, s);
+  launch_pack<2>(V, x, 0, nrhs, (float4*)X, s);
   BRI_LAUNCH_CHECK("k_pack");
   return BRI_OK;
 }
 
 int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s) {
-  const int pairs = nrhs / 2;
-  const float4* X4 = (const float4*)X;
-  if (pairs) launch_unpack<4>(V, X4, 0, pairs, x, s);
-  if (nrhs % 2) launch_unpack<2>(V, X4 + packed_words(V, 12) * pairs, nrhs - 1, 1, x, s);
+  k_unpack<<<dim3(blocks_for(V * 6, 256), nrhs), 256, 0, s>>>(V, (const float4*)X, x);
+  note_launch();
   BRI_LAUNCH_CHECK("k_unpack");
   return BRI_OK;
 }
 
-// y (spinors' layout) or yp (packed) = D x for the first na of nrhs right-hand
-// sides of the packed vector X (a pair whose second member is not asked for is
-// still computed whole).  With p (packed; yp only) the fused epilogue of
-// ShiftDot, sd_blocks partials per system.
+// yp = D X for nrhs packed right-hand sides, ks thread groups per site; with p the
+// fused epilogue of ShiftDot, part: [nrhs][blocks_for(V, pack_sites(ks))].
 template <typename LS>
-int bri_f32_on_packed(const Geom& g, float* y, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs,
-                      int na, int dagger, cudaStream_t s, const void* p, const double* sig, double* part, int* sd_blocks) {
-  const int pairs = nrhs / 2, act = std::min(pairs, (na + 1) / 2);
-  const int64_t o = packed_words(g.V, 12) * pairs;
-  const float4 *X4 = (const float4*)X, *P4 = (const float4*)p;
-  float4* Y4 = (float4*)yp;
-  if (sd_blocks) *sd_blocks = blocks_for(g.V, 128);
-  PackedDot sd{P4, sig, part};
-  if (act) launch_pair<4, LS>(g, y, Y4, X4, W, cl, diag, dagger, 0, act, s, p ? &sd : nullptr);
-  if (nrhs % 2 && na == nrhs) {
-    sd.p = P4 + (p ? o : 0);
-    launch_pair<2, LS>(g, y, Y4 ? Y4 + o : nullptr, X4 + o, W, cl, diag, dagger, nrhs - 1, 1, s, p ? &sd : nullptr);
-  }
+int bri_f32_on_packed(const Geom& g, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs, int ks,
+                      int dagger, cudaStream_t s, const void* p, const double* sig, double* part) {
+  const PackedDot sd{(const float4*)p, sig, part};
+  launch_singles<LS>(g, nullptr, (float4*)yp, (const float4*)X, W, cl, diag, dagger, 0, nrhs, s, p ? &sd : nullptr, ks);
   BRI_LAUNCH_CHECK("bri_pair_kernel");
   return BRI_OK;
 }
-template int bri_f32_on_packed<float2>(const Geom&, float*, void*, const void*, const float2*, const float*, float, int, int,
-                                       int, cudaStream_t, const void*, const double*, double*, int*);
-template int bri_f32_on_packed<__nv_bfloat162>(const Geom&, float*, void*, const void*, const __nv_bfloat162*, const float*,
-                                               float, int, int, int, cudaStream_t, const void*, const double*, double*, int*);
+template int bri_f32_on_packed<float2>(const Geom&, void*, const void*, const float2*, const float*, float, int, int, int,
+                                       cudaStream_t, const void*, const double*, double*);
+template int bri_f32_on_packed<__nv_bfloat162>(const Geom&, void*, const void*, const __nv_bfloat162*, const float*, float, int,
+                                               int, int, cudaStream_t, const void*, const double*, double*);
 
 // Spinors in their own layout in and out.  The packed copy of x lives in a
 // stream-ordered allocation of at most kChunk right-hand sides; where there is
@@ -73,17 +65,25 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
   if (!sd && bri_f32_packed(g.V, nrhs)) {
     configure_pool_once();
     void* X = nullptr;
-    if (cudaMallocAsync(&X, bri_f32_packed_bytes(g.V, std::min(nrhs, kChunk)), s) == cudaSuccess) {
+    if (cudaMallocAsync(&X, sizeof(float4) * packed_words(g.V, 6) * std::min(nrhs, kChunk), s) == cudaSuccess) {
       note_device_alloc();
-      int rc = BRI_OK;
-      for (int r0 = 0; r0 < nrhs && rc == BRI_OK; r0 += kChunk) {
-        const int nr = std::min(kChunk, nrhs - r0);
-        const int64_t at = r0 * g.V * 24;
-        rc = bri_f32_pack(g.V, x + at, nr, X, s);
-        if (rc == BRI_OK) rc = bri_f32_on_packed<LS>(g, y + at, nullptr, X, W, cl, diag, nr, nr, dagger, s);
+      float4* X4 = (float4*)X;
+      for (int r0 = 0; r0 < nrhs; r0 += kChunk) {
+        const int nr = std::min(kChunk, nrhs - r0), pairs = take_pairs(g.V, nr) ? nr / 2 : 0, one = nr - 2 * pairs;
+        float4* X1 = X4 + packed_words(g.V, 12) * pairs;
+        if (pairs) {
+          launch_pack<4>(g.V, x, r0, pairs, X4, s);
+          launch_pairs<LS>(g, y, X4, W, cl, diag, dagger, r0, pairs, s);
+        }
+        if (one) {
+          const int r1 = r0 + 2 * pairs;
+          launch_pack<2>(g.V, x, r1, one, X1, s);
+          launch_singles<LS>(g, y, nullptr, X1, W, cl, diag, dagger, r1, one, s, nullptr, pack_groups(g.V * one));
+        }
       }
       cudaFreeAsync(X, s);
-      return rc;
+      BRI_LAUNCH_CHECK("bri_pair_kernel");
+      return BRI_OK;
     }
     cudaGetLastError();
   }

@@ -27,8 +27,8 @@
 // sides; 71 % busy at 16^3 x 32, L1 46 %, DRAM 19 %), for one right-hand side
 // at 24^3 x 48 also the link stream.  GB300, packing pass included, against the
 // kernels before it (array-of-structs spinors, links as five strided streams):
-// 16^3 x 32, 12 rhs 1208 -> 1024 us; 24^3 x 48, 1 rhs 653 -> 578 us; BF16
-// links, 18.15.14.21, 3 rhs 278 -> 237 us.  Two right-hand sides per thread run
+// 16^3 x 32, 12 rhs 1208 -> 1015 us; 24^3 x 48, 1 rhs 653 -> 560 us; BF16
+// links, 18.15.14.21, 3 rhs 278 -> 178 us (237 with one thread group per site).  Two right-hand sides per thread run
 // at 12 warps per SM (168 registers), one at 16 (128); more warps with spills
 // were slower (0.80 against 0.62 ns per site and rhs), as were blocks that
 // stage a 4D tile and its halo in shared memory (0.78: filling the halo takes
@@ -212,11 +212,11 @@ __device__ __forceinline__ void pr_gamma(CP (&acc)[2][3], const CP (&v)[2][3], f
   }
 }
 
-// Sum over the 80 hops at site n into acc; x = packed vector (R = 4: a pair of
-// right-hand sides, R = 2: one).
-template <int R, typename LS>
+// Sum over the hops at site n into acc (all 80, or those of every KS-th offset
+// pair from i0 on); x = packed vector (R = 4: a pair of right-hand sides, R = 2: one).
+template <int R, typename LS, int KS>
 __device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, const float4* __restrict__ x,
-                                        const LS* __restrict__ W, const PairHops& H) {
+                                        const LS* __restrict__ W, const PairHops& H, int i0) {
   const int V = (int)g.V;
   // index steps to the neighbours in each direction (periodic)
   int up[4], dn[4];
@@ -247,12 +247,13 @@ __device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, c
     for (int aa = 0; aa < 3; ++aa) acc[q][aa] = CP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   C<float> w[3][3], wm[3][3];
   int mp, mm;
-  sites(0, mp, mm);
-  load_stored_link<float, LS>(w, W, H.j[0], n, V);
-  load_stored_link<float, LS>(wm, W, H.j[0], mm, V);
+  if constexpr (KS == 1) i0 = 0;
+  sites(i0, mp, mm);
+  load_stored_link<float, LS>(w, W, H.j[i0], n, V);
+  load_stored_link<float, LS>(wm, W, H.j[i0], mm, V);
 #pragma unroll 1
-  for (int j = 0; j < 40; ++j) {
-    const int jn = j < 39 ? j + 1 : 39;
+  for (int j = i0; j < 40; j += KS) {
+    const int jn = KS == 1 ? (j < 39 ? j + 1 : 39) : (j < 40 - KS ? j + KS : j);
     const float a = H.a[j];
     const int op = packed_at<3 * R>(mp), om = packed_at<3 * R>(mm);
     CP P[R][3];
@@ -319,36 +320,61 @@ struct PackedDot {
   double* part;       // [nsys][blocks]
 };
 
-// D x (EPI: + sig p, dA and dB this site's Re<p, y> of the two components'
-// systems) at site n of one packed group: x, yo, p are the group's packed
-// vectors, y0 its first right-hand side in the spinors' own layout (rs reals
-// apart).  OUT = 0 writes y0, OUT = 1 writes yo.
-template <int R, typename LS, int OUT, bool EPI>
-__device__ __forceinline__ void pr_site(const Geom& g, int n, bool valid, float* __restrict__ y0, int64_t rs,
-                                        float4* __restrict__ yo, const float4* __restrict__ x, const LS* __restrict__ W,
-                                        const float* __restrict__ cl, float diag, const PairHops& H,
-                                        const float4* __restrict__ p, float sA, float sB, float& dA, float& dB) {
+// The thread group of a 128-thread block; a warp is of one group.  Told so, the
+// compiler keeps the offset's constants in uniform registers (16^3.32 x 12, two
+// groups: 1089 -> 1027 us).
+template <int KS> __device__ __forceinline__ int pr_group() {
+  if constexpr (KS == 1) return 0;
+  return __shfl_sync(0xffffffffu, threadIdx.x / (128 / KS), 0);
+}
+
+// D x at the sites of block blk of one packed group, a site's offset pairs split
+// over KS thread groups: each takes every KS-th pair, their sums meet in shared
+// memory and the groups 0 and 1 finish one chirality each.  x, yp: the group's
+// packed vectors, y0: its first right-hand side in the spinors' own layout (OUT =
+// 0 writes y0, OUT = 1 yp).  EPI (R = 2, OUT = 1): the epilogue of system s, p at
+// word po of sd.p.
+template <int R, typename LS, int OUT, bool EPI, int KS>
+__device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restrict__ y0, float4* __restrict__ yp,
+                                         const float4* __restrict__ x, const LS* __restrict__ W,
+                                         const float* __restrict__ cl, float diag, const PairHops& H, const PackedDot& sd,
+                                         int64_t po, int s, int nb) {
+  static_assert(R == 2 || (OUT == 0 && KS == 1), "pairs: spinors' own layout out, one thread per site");
+  static_assert(!EPI || OUT == 1, "the epilogue writes packed vectors");
+  constexpr int SB = 128 / KS;
+  constexpr bool STAGE = R == 2 && OUT == 0 && KS == 1;
+  const int n0 = blk * SB + (KS == 1 ? threadIdx.x : threadIdx.x % SB);
+  const bool valid = n0 < g.V;
+  if (R == 4 && !valid) return;  // else every thread takes part in the block's exchanges
+  const int n = valid ? n0 : 0, grp = pr_group<KS>();
   CP acc[R][3];
-  pr_hops<R, LS>(acc, g, n, x, W, H);
-  const float4* xo = x + packed_at<3 * R>(n);
-  const float2 sig = make_float2(sA, sB);
-  // one word: epilogue and packed store
-  auto put = [&](int row, CP v) {
-    const int64_t at = packed_at<3 * R>(n) + row * kPackBlock;
-    if constexpr (EPI) {
-      const CP pv = cp_of(__ldg(p + at));
-      v.re = pr_fma(pv.re, sig, v.re);
-      v.im = pr_fma(pv.im, sig, v.im);
-      dA = fmaf(pv.re.x, v.re.x, dA);
-      dB = fmaf(pv.re.y, v.re.y, dB);
-      dA = fmaf(pv.im.x, v.im.x, dA);
-      dB = fmaf(pv.im.y, v.im.y, dB);
-    }
-    if (valid) yo[at] = cp_word(v);
-  };
+  pr_hops<R, LS, KS>(acc, g, n, x, W, H, grp);
+  if constexpr (KS > 1) {
+    __shared__ float4 red[KS][6][SB];
+    const int l = threadIdx.x % SB;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if constexpr (R == 4) {
+    for (int i = 0; i < 6; ++i) red[grp][i][l] = cp_word(acc[i / 3][i % 3]);
+    __syncthreads();
+    if (grp < 2) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        CP t = cp_of(red[0][grp * 3 + i][l]);
+#pragma unroll
+        for (int k = 1; k < KS; ++k) {
+          const CP u = cp_of(red[k][grp * 3 + i][l]);
+          t.re = make_float2(t.re.x + u.re.x, t.re.y + u.re.y);
+          t.im = make_float2(t.im.x + u.im.x, t.im.y + u.im.y);
+        }
+        acc[0][i] = t;  // this group's chirality, whichever it is
+        acc[1][i] = t;
+      }
+    }
+  }
+  const float4* xo = x + packed_at<3 * R>(n);
+  if constexpr (R == 4) {
+    const int64_t rs = g.V * 24;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
       CP own[6], out[6];
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
@@ -365,19 +391,21 @@ __device__ __forceinline__ void pr_site(const Geom& g, int n, bool valid, float*
           out[i].im = make_float2(out[i].im.x + co[i].im.x, out[i].im.y + co[i].im.y);
         }
       }
-      if constexpr (OUT == 1) {
+      float4* ya = reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
+      float4* yb = reinterpret_cast<float4*>(y0 + rs + (int64_t)n * 24 + h * 12);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) put(h * 6 + i, out[i]);
-      } else if (valid) {
-        float4* ya = reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
-        float4* yb = reinterpret_cast<float4*>(y0 + rs + (int64_t)n * 24 + h * 12);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          ya[i] = make_float4(out[2 * i].re.x, out[2 * i].im.x, out[2 * i + 1].re.x, out[2 * i + 1].im.x);
-          yb[i] = make_float4(out[2 * i].re.y, out[2 * i].im.y, out[2 * i + 1].re.y, out[2 * i + 1].im.y);
-        }
+      for (int i = 0; i < 3; ++i) {
+        ya[i] = make_float4(out[2 * i].re.x, out[2 * i].im.x, out[2 * i + 1].re.x, out[2 * i + 1].im.x);
+        yb[i] = make_float4(out[2 * i].re.y, out[2 * i].im.y, out[2 * i + 1].re.y, out[2 * i + 1].im.y);
       }
-    } else {
+    }
+  } else {
+    __shared__ float4 stage[STAGE ? 128 * 7 : 1];
+    const float sig = EPI ? (float)sd.sig[s] : 0.f;
+    float dA = 0.f, dB = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (KS > 1 && h != grp) continue;
       C<float> in[6], out[6];
 #pragma unroll
       for (int aa = 0; aa < 3; ++aa) {
@@ -398,52 +426,59 @@ __device__ __forceinline__ void pr_site(const Geom& g, int n, bool valid, float*
       }
       if constexpr (OUT == 1) {
 #pragma unroll
-        for (int aa = 0; aa < 3; ++aa)
-          put(h * 3 + aa, CP{make_float2(out[aa].re, out[3 + aa].re), make_float2(out[aa].im, out[3 + aa].im)});
-      } else if (valid) {
-        float4* ya = reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
+        for (int aa = 0; aa < 3; ++aa) {
+          const int at = packed_at<6>(n) + (h * 3 + aa) * kPackBlock;
+          CP v{make_float2(out[aa].re, out[3 + aa].re), make_float2(out[aa].im, out[3 + aa].im)};
+          if constexpr (EPI) {
+            const CP pv = cp_of(__ldg(sd.p + po + at));
+            v.re = pr_fma(pv.re, pr_bc(sig), v.re);
+            v.im = pr_fma(pv.im, pr_bc(sig), v.im);
+            dA = fmaf(pv.re.x, v.re.x, dA);
+            dB = fmaf(pv.re.y, v.re.y, dB);
+            dA = fmaf(pv.im.x, v.im.x, dA);
+            dB = fmaf(pv.im.y, v.im.y, dB);
+          }
+          if (valid) yp[at] = cp_word(v);
+        }
+      } else {
+        float4* ya = STAGE ? stage + threadIdx.x * 7 + h * 3 : reinterpret_cast<float4*>(y0 + (int64_t)n * 24 + h * 12);
+        if (STAGE || valid) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-          ya[i] = make_float4(out[2 * i].re, out[2 * i].im, out[2 * i + 1].re, out[2 * i + 1].im);
+          for (int i = 0; i < 3; ++i)
+            ya[i] = make_float4(out[2 * i].re, out[2 * i].im, out[2 * i + 1].re, out[2 * i + 1].im);
+        }
       }
     }
-  }
-}
-
-// Partials of the epilogue: dA, dB of a pair belong to the systems s0, s0 + 1
-// (R = 4), of one right-hand side (R = 2) both to s0.
-template <int R>
-__device__ __forceinline__ void pr_partials(double* part, int s0, int nb, int blk, bool valid, float dA, float dB) {
-  const double a = valid ? (double)dA : 0.0, b = valid ? (double)dB : 0.0;
-  const double t = pr_block_total(R == 4 ? a : a + b);
-  if (threadIdx.x == 0) part[(int64_t)s0 * nb + blk] = t;
-  if constexpr (R == 4) {
-    const double u = pr_block_total(b);
-    if (threadIdx.x == 0) part[(int64_t)(s0 + 1) * nb + blk] = u;
+    if constexpr (STAGE) {
+      // a warp's 32 sites are 3 KB of y, stored in whole sectors (16^3.32 x 12: 1063 -> 1019 us)
+      __syncwarp();
+      const int lane = threadIdx.x & 31, w0 = threadIdx.x - lane, m = ((int)g.V - blk * SB - w0) * 6;
+      float4* yw = reinterpret_cast<float4*>(y0 + (int64_t)(blk * SB + w0) * 24);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        const int k = i * 32 + lane;
+        if (k < m) yw[k] = stage[(w0 + k / 6) * 7 + k % 6];
+      }
+    }
+    if constexpr (EPI) {
+      const double t = pr_block_total(valid ? (double)dA + (double)dB : 0.0);
+      if (threadIdx.x == 0) sd.part[(int64_t)s * nb + blk] = t;
+    }
   }
 }
 
 // D on `groups` packed groups of one lattice; the first one holds right-hand
 // side rhs0 (and rhs0 + 1).
-template <int R, typename LS, int OUT, bool EPI>
+template <int R, typename LS, int OUT, bool EPI, int KS>
 __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
     bri_pair_kernel(Geom g, float* __restrict__ y, float4* __restrict__ yp, const float4* __restrict__ x,
                     const LS* __restrict__ W, const float* __restrict__ cl, float diag, int rhs0, int gfirst,
                     const __grid_constant__ PairHops H, PackedDot sd) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  const int n0 = blk * blockDim.x + threadIdx.x;
-  const bool valid = n0 < g.V;
-  if (!EPI && !valid) return;  // with the epilogue every thread takes part in the block's reduction
-  const int64_t rs = g.V * 24, go = (int64_t)grp * packed_words(g.V, 3 * R);
+  const int64_t go = (int64_t)grp * packed_words(g.V, 3 * R);
   const int s0 = rhs0 + grp * (R / 2);
-  float dA = 0.f, dB = 0.f, sA = 0.f, sB = 0.f;
-  if constexpr (EPI) {
-    sA = (float)sd.sig[s0];
-    sB = R == 4 ? (float)sd.sig[s0 + 1] : sA;
-  }
-  pr_site<R, LS, OUT, EPI>(g, valid ? n0 : 0, valid, y + (int64_t)s0 * rs, rs, yp + go, x + go, W, cl, diag, H,
-                           EPI ? sd.p + go : nullptr, sA, sB, dA, dB);
-  if constexpr (EPI) pr_partials<R>(sd.part, s0, gfirst ? gridDim.y : gridDim.x, blk, valid, dA, dB);
+  pr_block<R, LS, OUT, EPI, KS>(g, blk, y + (int64_t)s0 * g.V * 24, yp + go, x + go, W, cl, diag, H, sd, go, s0,
+                                gfirst ? gridDim.y : gridDim.x);
 }
 
 // Spinors [nrhs][V][12] complex64 -> packed groups; group g holds the
@@ -468,48 +503,51 @@ template <int R> __global__ void __launch_bounds__(256) k_pack(int64_t V, const 
   }
 }
 
-// The way back.
-template <int R> __global__ void __launch_bounds__(256) k_unpack(int64_t V, const float4* __restrict__ X, int rhs0, float* __restrict__ x) {
+// The way back (single right-hand sides).
+inline __global__ void __launch_bounds__(256) k_unpack(int64_t V, const float4* __restrict__ X, float* __restrict__ x) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= V * 6) return;
   const int64_t n = i / 6;
   const int q = (int)(i - n * 6);
-  const float4* o = X + (int64_t)blockIdx.y * packed_words(V, 3 * R) + packed_at<3 * R>((int)n);
-  if constexpr (R == 4) {
-    float* p = x + (rhs0 + 2 * (int64_t)blockIdx.y) * V * 24 + i * 4;
-    const float4 u = __ldg(o + (2 * q) * kPackBlock), v = __ldg(o + (2 * q + 1) * kPackBlock);
-    *reinterpret_cast<float4*>(p) = make_float4(u.x, u.z, v.x, v.z);
-    *reinterpret_cast<float4*>(p + V * 24) = make_float4(u.y, u.w, v.y, v.w);
-  } else {
-    float2* p = reinterpret_cast<float2*>(x + (rhs0 + (int64_t)blockIdx.y) * V * 24 + n * 24) + q + 3 * (q / 3);
-    const float4 u = __ldg(o + q * kPackBlock);
-    p[0] = make_float2(u.x, u.z);
-    p[3] = make_float2(u.y, u.w);
-  }
+  const float4 u = __ldg(X + (int64_t)blockIdx.y * packed_words(V, 6) + packed_at<6>((int)n) + q * kPackBlock);
+  float2* p = reinterpret_cast<float2*>(x + (int64_t)blockIdx.y * V * 24 + n * 24) + q + 3 * (q / 3);
+  p[0] = make_float2(u.x, u.z);
+  p[3] = make_float2(u.y, u.w);
 }
 
 template <int R> inline void launch_pack(int64_t V, const float* x, int rhs0, int groups, float4* X, cudaStream_t s) {
   k_pack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, x, rhs0, X);
   note_launch();
 }
-template <int R> inline void launch_unpack(int64_t V, const float4* X, int rhs0, int groups, float* x, cudaStream_t s) {
-  k_unpack<R><<<dim3(blocks_for(V * 6, 256), groups), 256, 0, s>>>(V, X, rhs0, x);
+// y = D x for `groups` pairs of right-hand sides starting at rhs0.
+template <typename LS>
+inline void launch_pairs(const Geom& g, float* y, const float4* X, const LS* W, const float* cl, float diag, int dagger,
+                         int rhs0, int groups, cudaStream_t s) {
+  const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
+  bri_pair_kernel<4, LS, 0, false, 1><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst,
+                                                              pair_hops(dagger), PackedDot{nullptr, nullptr, nullptr});
   note_launch();
 }
 
-// y (or packed yp) = D x for `groups` packed groups starting at right-hand side rhs0.
-template <int R, typename LS>
-inline void launch_pair(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
-                        int dagger, int rhs0, int groups, cudaStream_t s, const PackedDot* sd) {
-  const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
+// y or packed yp = D x for `n` single right-hand sides starting at rhs0, with sd
+// (yp only) the solver's epilogue.
+template <typename LS, int KS>
+inline void launch_singles_ks(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
+                              int dagger, int rhs0, int n, cudaStream_t s, const PackedDot* sd) {
+  const StencilGrid sg = stencil_grid(blocks_for(g.V, 128 / KS), n);
   const PackedDot none{nullptr, nullptr, nullptr};
-  if (sd)
-    bri_pair_kernel<R, LS, 1, true><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), *sd);
-  else if (yp)
-    bri_pair_kernel<R, LS, 1, false><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), none);
-  else
-    bri_pair_kernel<R, LS, 0, false><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger), none);
+  const PairHops& H = pair_hops(dagger);
+  if (sd) bri_pair_kernel<2, LS, 1, true, KS><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, H, *sd);
+  else if (yp) bri_pair_kernel<2, LS, 1, false, KS><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, H, none);
+  else bri_pair_kernel<2, LS, 0, false, KS><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst, H, none);
   note_launch();
+}
+template <typename LS>
+inline void launch_singles(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
+                           int dagger, int rhs0, int n, cudaStream_t s, const PackedDot* sd, int ks) {
+  if (ks == 4) launch_singles_ks<LS, 4>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
+  else if (ks == 2) launch_singles_ks<LS, 2>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
+  else launch_singles_ks<LS, 1>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
 }
 
 }  // namespace bri

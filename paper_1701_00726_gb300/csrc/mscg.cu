@@ -813,20 +813,11 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
   pb.maxiter = maxiter;
   pb.sig.assign(sig, sig + (size_t)nsys * nshift);
   for (int s = 0; s < nsys; ++s) pb.tol.push_back(tols ? tols[s] : tol);
-  for (int s = 0; s < nsys;) {
-    GroupDesc g;
-    memset(&g, 0, sizeof(g));
-    g.s0 = s;
-    g.two = s + 1 < nsys;
-    g.V = V;
-    g.poff = pb.words;
-    g.offn = s * n2;
-    g.kstr = nsys * n2;
-    pb.words += packed_words(V, g.two ? 12 : 6);
-    pb.grp.push_back(g);
-    s += g.two ? 2 : 1;
+  for (int s = 0; s < nsys; ++s) {
+    pb.sys.push_back(PackedSys{0, V, pb.words, s * n2, nsys * n2});
+    pb.words += packed_words(V, 6);
   }
-  const int nb = blocks_for(V, 128);
+  const int ks = pack_groups(V * nsys), nb = blocks_for(V, pack_sites(ks));
   DevBuf bsig, bsd, bx;
   int rc;
   if ((rc = bsig.alloc(sizeof(double) * nsys, st))) return rc;
@@ -837,7 +828,7 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
   BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));
   auto pack = [&](float4* dst) { return bri_f32_pack(V, b, nsys, dst, st); };
   auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int na) {
-    return dirac_bri_packed(c, nullptr, Y, X, nsys, na, m0, dagger, prec, st, P, bsig.as<double>(), bsd.as<double>());
+    return dirac_bri_packed(c, Y, X, na, ks, m0, dagger, prec, st, P, bsig.as<double>(), bsd.as<double>());
   };
   const bool graphs = graphs_enabled() && !c->prof_on && st != nullptr;
   rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), nb, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
@@ -1736,7 +1727,7 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     return BRI_OK;
   };
   // FP32: the packed solver on the groups of all lattices, its stencil on a work
-  // list of (group, 128-site block) items, the solutions in each lattice's layout.
+  // list of (group, site block) items, the solutions in each lattice's layout.
   auto phase1_f32 = [&](auto ltag) -> int {
     using LS = decltype(ltag);
     const double tol1 = std::max(tol, prec == BRI_PREC_F32 ? 1e-7 : 1e-6);
@@ -1746,46 +1737,37 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     pb.maxiter = maxiter;
     pb.tol.assign(S, tol1);
     for (int s = 0; s < S; ++s) pb.sig.insert(pb.sig.end(), sig, sig + n);
-    std::vector<int2> items2, items1;
+    std::vector<int2> items;
     std::vector<int64_t> lat_poff(nctx), lat_off(nctx);
     int nb = 0;
-    int64_t maxb = 0;
+    int64_t maxb = 0, site_rhs = 0;
+    for (int i = 0; i < nctx; ++i) site_rhs += cs[i]->g.V * nrhs[i];
+    const int ks = pack_groups(site_rhs), sb = pack_sites(ks);
     for (int i = 0; i < nctx; ++i) {
       const int64_t V = cs[i]->g.V, n2 = V * 12;
       lat_poff[i] = pb.words;
       lat_off[i] = sd[first_sys[i]].off;
-      nb = std::max(nb, blocks_for(V, 128));
+      nb = std::max(nb, blocks_for(V, sb));
       maxb = std::max(maxb, n2 * nrhs[i]);
-      for (int r = 0; r < nrhs[i];) {
-        GroupDesc g;
-        memset(&g, 0, sizeof(g));
-        g.s0 = first_sys[i] + r;
-        g.two = r + 1 < nrhs[i];
-        g.lat = i;
-        g.V = V;
-        g.poff = pb.words;
-        g.offn = lat_off[i] * n + r * n2;
-        g.kstr = nrhs[i] * n2;
-        pb.words += packed_words(V, g.two ? 12 : 6);
-        for (int k = 0; k < blocks_for(V, 128); ++k) (g.two ? items2 : items1).push_back(make_int2((int)pb.grp.size(), k));
-        pb.grp.push_back(g);
-        r += g.two ? 2 : 1;
+      for (int r = 0; r < nrhs[i]; ++r) {
+        for (int k = 0; k < blocks_for(V, sb); ++k) items.push_back(make_int2((int)pb.sys.size(), k));
+        pb.sys.push_back(PackedSys{i, V, pb.words, lat_off[i] * n + r * n2, nrhs[i] * n2});
+        pb.words += packed_words(V, 6);
       }
     }
-    const int n2i = (int)items2.size(), n1i = (int)items1.size();
+    const int ni = (int)items.size();
     DevBuf bgd, bit, bsig, bpart, bb;
     int q;
-    if ((q = bgd.alloc(sizeof(GroupDesc) * pb.grp.size(), bs))) return q;
-    if ((q = bit.alloc(sizeof(int2) * (n2i + n1i), bs))) return q;
+    if ((q = bgd.alloc(sizeof(PackedSys) * pb.sys.size(), bs))) return q;
+    if ((q = bit.alloc(sizeof(int2) * ni, bs))) return q;
     if ((q = bsig.alloc(sizeof(double) * S, bs))) return q;
     if ((q = bpart.alloc(sizeof(double) * (size_t)S * nb, bs))) return q;
     if ((q = bb.alloc(sizeof(float2) * maxb, bs))) return q;
     if ((q = bXall.alloc(sizeof(double2) * off * n, bs))) return q;
     for (int i = 0; i < nctx; ++i) Xp[i] = (double*)(bXall.as<double2>() + lat_off[i] * n);
     const std::vector<double> hsig(S, sig[0]);
-    BRI_CUDA(cudaMemcpyAsync(bgd.p, pb.grp.data(), sizeof(GroupDesc) * pb.grp.size(), cudaMemcpyHostToDevice, bs));
-    if (n2i) BRI_CUDA(cudaMemcpyAsync(bit.p, items2.data(), sizeof(int2) * n2i, cudaMemcpyHostToDevice, bs));
-    if (n1i) BRI_CUDA(cudaMemcpyAsync(bit.as<int2>() + n2i, items1.data(), sizeof(int2) * n1i, cudaMemcpyHostToDevice, bs));
+    BRI_CUDA(cudaMemcpyAsync(bgd.p, pb.sys.data(), sizeof(PackedSys) * pb.sys.size(), cudaMemcpyHostToDevice, bs));
+    BRI_CUDA(cudaMemcpyAsync(bit.p, items.data(), sizeof(int2) * ni, cudaMemcpyHostToDevice, bs));
     BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * S, cudaMemcpyHostToDevice, bs));
     // blocks beyond a smaller lattice's volume contribute nothing to its sums
     BRI_CUDA(cudaMemsetAsync(bpart.p, 0, sizeof(double) * (size_t)S * nb, bs));
@@ -1800,19 +1782,17 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     const MsState* St = nullptr;
     auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int) -> int {
       const PackedDot pd{P, bsig.as<double>(), bpart.as<double>()};
-      const GroupDesc* gd = bgd.as<GroupDesc>();
+      const PackedSys* gd = bgd.as<PackedSys>();
       const PairHops& H = pair_hops(dagger);
-      if (n2i) {
-        if (P) kb_pair<4, LS, true><<<n2i, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
-        else kb_pair<4, LS, false><<<n2i, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
+      auto run = [&](auto ktag) {
+        constexpr int KS = decltype(ktag)::value;
+        if (P) kb_pair<LS, true, KS><<<ni, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
+        else kb_pair<LS, false, KS><<<ni, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
         note_launch();
-      }
-      if (n1i) {
-        const int2* it1 = bit.as<int2>() + n2i;
-        if (P) kb_pair<2, LS, true><<<n1i, 128, 0, bs>>>(tab, gd, it1, St, Y, X, H, pd, nb);
-        else kb_pair<2, LS, false><<<n1i, 128, 0, bs>>>(tab, gd, it1, St, Y, X, H, pd, nb);
-        note_launch();
-      }
+      };
+      if (ks == 4) run(std::integral_constant<int, 4>());
+      else if (ks == 2) run(std::integral_constant<int, 2>());
+      else run(std::integral_constant<int, 1>());
       return BRI_OK;
     };
     q = packed_solve(bs, pb, pack, apply, bpart.as<double>(), nb, bXall.as<double2>(), sizeof(double2) * off * n, nullptr, true,

@@ -1,6 +1,7 @@
 // Multi-shift CG on packed FP32 vectors (included by mscg.cu): one or several
-// lattices as groups of packed systems (bri_pair.cuh).  Base direction p_0,
-// t = D p_0, q = (A + sigma) p_0 and the residuals live in the stencil's layout;
+// lattices' systems, each a packed vector of one right-hand side (bri_pair.cuh;
+// as pairs the two stencils of an iteration took 381 + 363 us for 4 systems of
+// 16^3 x 32 where single ones take 349 + 351).  Base direction p_0, t = D p_0, q = (A + sigma) p_0 and the residuals live in the stencil's layout;
 // per iteration
 //   t = D p, q = D^dagger t + sigma p with the partials of <p, q>,   (stencil)
 //   alpha; r_{j+1} = r_j - alpha q_j with the partials of ||r||^2;   (3 vectors)
@@ -13,39 +14,25 @@
 
 constexpr int kRing = 8;  // residual slots; also the iterations of one graph block
 
-// One group of the problem: systems s0 (and s0 + 1 when two), lattice lat.
-struct GroupDesc {
-  int s0, two, lat, pad;
+// One system of the problem, on lattice lat.
+struct PackedSys {
+  int lat;
   int64_t V;
-  int64_t poff;        // offset of the group in the packed vectors, 16-byte words
-  int64_t offn, kstr;  // complex offset of system s0's shift 0 in p and x, and from shift to shift
+  int64_t poff;        // offset in the packed vectors, 16-byte words
+  int64_t offn, kstr;  // complex offset of its shift 0 in p and x, and from shift to shift
 };
 
-__device__ __forceinline__ int64_t group_words(const GroupDesc& g) { return packed_words(g.V, g.two ? 12 : 6); }
-
-// partial sums of the two components of a group's words (a pair: one system
-// each, a single right-hand side: both its own)
-__device__ __forceinline__ void group_partials(const GroupDesc& g, double* part, double a, double b) {
-  const double t = block_sum(g.two ? a : a + b);
-  if (threadIdx.x == 0) part[(int64_t)g.s0 * gridDim.x + blockIdx.x] = t;
-  if (g.two) {
-    __syncthreads();
-    const double u = block_sum(b);
-    if (threadIdx.x == 0) part[(int64_t)(g.s0 + 1) * gridDim.x + blockIdx.x] = u;
-  }
-}
-
-__global__ void __launch_bounds__(256) kp_norm(const GroupDesc* __restrict__ gd, const float4* __restrict__ r, double* part) {
-  const GroupDesc g = gd[blockIdx.y];
-  const int64_t nw = group_words(g);
+__global__ void __launch_bounds__(256) kp_norm(const PackedSys* __restrict__ gd, const float4* __restrict__ r, double* part) {
+  const PackedSys g = gd[blockIdx.y];
+  const int64_t nw = packed_words(g.V, 6);
   const float4* v = r + g.poff;
-  double a = 0.0, b = 0.0;
+  double a = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nw; i += (int64_t)gridDim.x * blockDim.x) {
     const float4 x = v[i];
-    a += (double)x.x * x.x + (double)x.z * x.z;
-    b += (double)x.y * x.y + (double)x.w * x.w;
+    a += (double)x.x * x.x + (double)x.y * x.y + (double)x.z * x.z + (double)x.w * x.w;
   }
-  group_partials(g, part, a, b);
+  const double t = block_sum(a);
+  if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
 // (h, l) += v^2 on two components: exact square and sum by TwoProduct and TwoSum
@@ -60,21 +47,19 @@ __device__ __forceinline__ void add_square(float2& h, float2& l, float2 v) {
   l = __fadd2_rn(l, __fadd2_rn(t, e));
 }
 
-// rout = rin - alpha q, partials of ||rout||^2 (rin may be rout).  A converged
-// system of a pair keeps its residual.  The squares of four words are summed in
+// rout = rin - alpha q, partials of ||rout||^2 (rin may be rout).  The squares of four words are summed in
 // double-word FP32 (48 bits), those sums in FP64: one FP64 addition per eight
 // squares instead of eight, which bound the kernel (102 -> 43 us on average in the
 // 16^3 x 32 solves; the random 2^-47 of a chunk vanish below 2^-53 in the sum).
-__global__ void __launch_bounds__(256) kp_update_r(const GroupDesc* __restrict__ gd, const MsState* __restrict__ st,
+__global__ void __launch_bounds__(256) kp_update_r(const PackedSys* __restrict__ gd, const MsState* __restrict__ st,
                                                    const float4* __restrict__ q, const float4* rin, float4* rout, double* part) {
-  const GroupDesc g = gd[blockIdx.y];
-  const int sb = g.two ? g.s0 + 1 : g.s0;
-  if (st[g.s0].done && st[sb].done) return;
-  const float2 f = make_float2(st[g.s0].done ? 0.f : -(float)st[g.s0].alpha, st[sb].done ? 0.f : -(float)st[sb].alpha);
-  const int64_t nw = group_words(g), stride = (int64_t)gridDim.x * blockDim.x;
+  const PackedSys g = gd[blockIdx.y];
+  if (st[blockIdx.y].done) return;
+  const float2 f = pr_bc(-(float)st[blockIdx.y].alpha);
+  const int64_t nw = packed_words(g.V, 6), stride = (int64_t)gridDim.x * blockDim.x;
   const float4 *qv = q + g.poff, *ri = rin + g.poff;
   float4* ro = rout + g.poff;
-  double a = 0.0, b = 0.0;
+  double a = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nw; i += 4 * stride) {
     float4 x[4], v[4];
 #pragma unroll
@@ -93,46 +78,35 @@ __global__ void __launch_bounds__(256) kp_update_r(const GroupDesc* __restrict__
         add_square(h, l, re);
         add_square(h, l, im);
       }
-    a += (double)h.x + (double)l.x;
-    b += (double)h.y + (double)l.y;
+    a += ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);
   }
-  group_partials(g, part, a, b);
+  const double t = block_sum(a);
+  if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
 // x += alpha p (XUP: single-shift solves, also in the iteration that converged),
 // p = r + beta p.
 template <bool XUP>
-__global__ void __launch_bounds__(256) kp_update_p(const GroupDesc* __restrict__ gd, const MsState* __restrict__ st,
+__global__ void __launch_bounds__(256) kp_update_p(const PackedSys* __restrict__ gd, const MsState* __restrict__ st,
                                                    const float4* __restrict__ r, float4* p, float4* x) {
-  const GroupDesc g = gd[blockIdx.y];
-  const MsState &A = st[g.s0], &B = st[g.two ? g.s0 + 1 : g.s0];
-  const bool ua = !A.done, ub = !B.done, xa = XUP && A.pend, xb = XUP && B.pend;
-  if (!(ua || ub || xa || xb)) return;
-  const float ba = (float)A.b_s[0], bb = (float)B.b_s[0];
-  const float aa = xa ? (float)A.a_s[0] : 0.f, ab = xb ? (float)B.a_s[0] : 0.f;
-  const int64_t nw = group_words(g);
+  const PackedSys g = gd[blockIdx.y];
+  const MsState& A = st[blockIdx.y];
+  const bool up = !A.done, xup = XUP && A.pend;
+  if (!(up || xup)) return;
+  const float b = (float)A.b_s[0], a = xup ? (float)A.a_s[0] : 0.f;
+  const int64_t nw = packed_words(g.V, 6);
   const float4* rv = r + g.poff;
   float4 *pv = p + g.poff, *xv = x + g.poff;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nw; i += (int64_t)gridDim.x * blockDim.x) {
-    float4 v = pv[i];
+    const float4 v = pv[i];
     if constexpr (XUP) {
-      float4 s = xv[i];
-      s.x = fmaf(aa, v.x, s.x);
-      s.y = fmaf(ab, v.y, s.y);
-      s.z = fmaf(aa, v.z, s.z);
-      s.w = fmaf(ab, v.w, s.w);
-      xv[i] = s;
+      const float4 s = xv[i];
+      xv[i] = make_float4(fmaf(a, v.x, s.x), fmaf(a, v.y, s.y), fmaf(a, v.z, s.z), fmaf(a, v.w, s.w));
     }
-    const float4 w = rv[i];
-    if (ua) {
-      v.x = fmaf(ba, v.x, w.x);
-      v.z = fmaf(ba, v.z, w.z);
+    if (up) {
+      const float4 w = rv[i];
+      pv[i] = make_float4(fmaf(b, v.x, w.x), fmaf(b, v.y, w.y), fmaf(b, v.z, w.z), fmaf(b, v.w, w.w));
     }
-    if (ub) {
-      v.y = fmaf(bb, v.y, w.y);
-      v.w = fmaf(bb, v.w, w.w);
-    }
-    pv[i] = v;
   }
 }
 
@@ -217,79 +191,51 @@ __device__ __forceinline__ void flush_system(const FlushCoef& c, const float2 (&
 // Every shift's recorded steps (ring slots base, base + 1, ...), in order:
 // p_i = zeta_i r_m + beta_i p_i (not on the first iteration), x_i += alpha_i p_i.
 // Runs while a system may already be done (its last steps still pending).  One
-// thread per site and 16-byte word of the spinors' own layout, so that p and x
-// stream; the ring is read in rows of five to six sites.
-__global__ void __launch_bounds__(256) kp_flush(const GroupDesc* __restrict__ gd, const ShiftHist* __restrict__ hist,
+// thread per site and packed word (two spins), neighbouring threads on one site,
+// so that p and x stream; the ring is read in rows of five to six sites.
+__global__ void __launch_bounds__(256) kp_flush(const PackedSys* __restrict__ gd, const ShiftHist* __restrict__ hist,
                                                 const float4* __restrict__ ring, int64_t rstride, int base, float2* p,
                                                 double2* x) {
-  const GroupDesc g = gd[blockIdx.y];
-  __shared__ FlushCoef ca, cb;
-  load_flush_coef(ca, hist[g.s0]);
-  if (g.two) load_flush_coef(cb, hist[g.s0 + 1]);
+  const PackedSys g = gd[blockIdx.y];
+  __shared__ FlushCoef c;
+  load_flush_coef(c, hist[blockIdx.y]);
   __syncthreads();
-  const int na = ca.n, nb = g.two ? cb.n : 0, nmax = max(na, nb);
-  if (nmax == 0) return;
-  const int64_t n2 = g.V * 12;
+  const int nm = c.n;
+  if (nm == 0) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < g.V * 6; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t n = i / 6;
     const int q = (int)(i - n * 6);
-    float2 a0[DW], a1[DW], b0[DW], b1[DW];
-    if (g.two) {
-      const float4* rr = ring + g.poff + packed_at<12>((int)n) + 2 * q * kPackBlock;
+    float2 a0[DW], a1[DW];
+    const float4* rr = ring + g.poff + packed_at<6>((int)n) + q * kPackBlock;
 #pragma unroll
-      for (int m = 0; m < DW; ++m)
-        if (m < nmax) {
-          const float4* rs = rr + (int64_t)((base + m) % kRing) * rstride;
-          const float4 u = __ldg(rs), v = __ldg(rs + kPackBlock);
-          a0[m] = make_float2(u.x, u.z);
-          b0[m] = make_float2(u.y, u.w);
-          a1[m] = make_float2(v.x, v.z);
-          b1[m] = make_float2(v.y, v.w);
-        }
-      const int64_t o = g.offn + 2 * i;
-      flush_system(ca, a0, a1, p, x, o, 1, g.kstr);
-      flush_system(cb, b0, b1, p, x, o + n2, 1, g.kstr);
-    } else {
-      const float4* rr = ring + g.poff + packed_at<6>((int)n) + q * kPackBlock;
-#pragma unroll
-      for (int m = 0; m < DW; ++m)
-        if (m < nmax) {
-          const float4 u = __ldg(rr + (int64_t)((base + m) % kRing) * rstride);
-          a0[m] = make_float2(u.x, u.z);
-          a1[m] = make_float2(u.y, u.w);
-        }
-      flush_system(ca, a0, a1, p, x, g.offn + n * 12 + q + 3 * (q / 3), 3, g.kstr);
-    }
+    for (int m = 0; m < DW; ++m)
+      if (m < nm) {
+        const float4 u = __ldg(rr + (int64_t)((base + m) % kRing) * rstride);
+        a0[m] = make_float2(u.x, u.z);
+        a1[m] = make_float2(u.y, u.w);
+      }
+    flush_system(c, a0, a1, p, x, g.offn + n * 12 + q + 3 * (q / 3), 3, g.kstr);
   }
 }
 
-// Stencil on the work list of several lattices: item (group, 128-site block);
-// groups whose systems have all converged are skipped.
-template <int R, typename LS, bool EPI>
-__global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
-    kb_pair(const __grid_constant__ BatchTab T, const GroupDesc* __restrict__ gd, const int2* __restrict__ items,
+// Stencil on the work list of several lattices: item (system, block of 128 / KS
+// sites); converged systems are skipped.
+template <typename LS, bool EPI, int KS>
+__global__ void __launch_bounds__(128, 4)
+    kb_pair(const __grid_constant__ BatchTab T, const PackedSys* __restrict__ gd, const int2* __restrict__ items,
             const MsState* __restrict__ st, float4* __restrict__ Y, const float4* __restrict__ X,
             const __grid_constant__ PairHops H, PackedDot sd, int nb) {
   const int2 it = items[blockIdx.x];
-  const GroupDesc gr = gd[it.x];
-  if (st[gr.s0].done && (R == 2 || st[gr.s0 + 1].done)) return;
+  const PackedSys gr = gd[it.x];
+  if (st[it.x].done) return;
   const BatchLat& L = T.lat[gr.lat];
-  const int n0 = it.y * 128 + threadIdx.x;
-  const bool valid = n0 < L.g.V;
-  float dA = 0.f, dB = 0.f, sA = 0.f, sB = 0.f;
-  if constexpr (EPI) {
-    sA = (float)sd.sig[gr.s0];
-    sB = R == 4 ? (float)sd.sig[gr.s0 + 1] : sA;
-  }
-  pr_site<R, LS, 1, EPI>(L.g, valid ? n0 : 0, valid, nullptr, 0, Y + gr.poff, X + gr.poff, (const LS*)L.W, (const float*)L.C,
-                         (float)L.diag, H, EPI ? sd.p + gr.poff : nullptr, sA, sB, dA, dB);
-  if constexpr (EPI) pr_partials<R>(sd.part, gr.s0, nb, it.y, valid, dA, dB);
+  pr_block<2, LS, 1, EPI, KS>(L.g, it.y, nullptr, Y + gr.poff, X + gr.poff, (const LS*)L.W, (const float*)L.C, (float)L.diag, H,
+                           sd, gr.poff, it.x, nb);
 }
 
-// A problem on packed vectors: groups in the order of their systems (pairs of a
-// lattice first, then its odd one), `words` 16-byte words per packed vector.
+// A problem on packed vectors: `words` 16-byte words per packed vector.
 struct PackedProblem {
-  std::vector<GroupDesc> grp;
+  std::vector<PackedSys> sys;
   int nsys = 0, nshift = 0, maxiter = 0;
   int64_t words = 0;
   std::vector<double> sig;  // [nsys][nshift], increasing within a system
@@ -298,7 +244,7 @@ struct PackedProblem {
 
 // Solves (A + sig[s][k]) x[k][s] = b[s].  pack(dst) writes the packed right-hand
 // sides; apply(dagger, X, Y, P, na) enqueues Y = D X (P null) or Y = D^dagger X +
-// sigma P with partials [nsys][nb] in sdpart, for at least the first na systems.
+// sigma P with partials [nsys][nb] in sdpart, for the first na systems.
 // Several shifts: solutions in x64 (zeroed here).  One shift: packed in xp.
 // whole: all iterations in one WHILE-node graph (no host polling), else host
 // polling every kRing iterations and a shrinking prefix of systems.
@@ -306,18 +252,18 @@ template <typename Pack, typename Apply>
 int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& apply, double* sdpart, int nb,
                  double2* x64, size_t x64_bytes, float4* xp, bool whole, bool graphs, int* hdone,
                  int* iters_out, Counters* cnt, double* lam_out, const MsState** state_out = nullptr) {
-  const int nsys = pb.nsys, nshift = pb.nshift, ngrp = (int)pb.grp.size();
+  const int nsys = pb.nsys, nshift = pb.nshift;
   const bool defer = x64 != nullptr;
   const size_t vb = sizeof(float4) * (size_t)pb.words;
   int64_t maxw = 0, n2all = 0;
-  for (const GroupDesc& g : pb.grp) {
-    maxw = std::max(maxw, packed_words(g.V, g.two ? 12 : 6));
-    n2all += g.V * 12 * (g.two ? 2 : 1);
+  for (const PackedSys& g : pb.sys) {
+    maxw = std::max(maxw, packed_words(g.V, 6));
+    n2all += g.V * 12;
   }
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((maxw + 255) / 256, std::max(1, kMaxPartials / ngrp)));
+  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((maxw + 255) / 256, std::max(1, kMaxPartials / nsys)));
   DevBuf bgd, bst, bpart, bring, bP, bT, bQ, bpk, bhist, bflags;
   int rc;
-  if ((rc = bgd.alloc(sizeof(GroupDesc) * ngrp, st))) return rc;
+  if ((rc = bgd.alloc(sizeof(PackedSys) * nsys, st))) return rc;
   if ((rc = bst.alloc(sizeof(MsState) * nsys, st))) return rc;
   if ((rc = bpart.alloc(sizeof(double) * nblk * nsys, st))) return rc;
   if ((rc = bring.alloc(vb * (defer ? kRing : 1), st))) return rc;
@@ -327,7 +273,7 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
   if (defer && (rc = bpk.alloc(sizeof(float2) * n2all * nshift, st))) return rc;
   if (defer && (rc = bhist.alloc(sizeof(ShiftHist) * nsys, st))) return rc;
   if ((rc = bflags.alloc(sizeof(int) * nsys, st))) return rc;
-  const GroupDesc* gd = bgd.as<GroupDesc>();
+  const PackedSys* gd = bgd.as<PackedSys>();
   MsState* S = bst.as<MsState>();
   ShiftHist* hist = defer ? bhist.as<ShiftHist>() : nullptr;
   double* part = bpart.as<double>();
@@ -343,7 +289,7 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
     h.tol2 = pb.tol[s] * pb.tol[s];
     h.maxiter = pb.maxiter;
   }
-  BRI_CUDA(cudaMemcpyAsync(bgd.p, pb.grp.data(), sizeof(GroupDesc) * ngrp, cudaMemcpyHostToDevice, st));
+  BRI_CUDA(cudaMemcpyAsync(bgd.p, pb.sys.data(), sizeof(PackedSys) * nsys, cudaMemcpyHostToDevice, st));
   BRI_CUDA(cudaMemcpyAsync(S, hs.data(), sizeof(MsState) * nsys, cudaMemcpyHostToDevice, st));
   // rows of the sites that pad a volume to whole blocks stay zero in every vector
   for (float4* v : {ring, P, T, Q}) BRI_CUDA(cudaMemsetAsync(v, 0, v == ring ? vb * (defer ? kRing : 1) : vb, st));
@@ -355,32 +301,25 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
   }
   if ((rc = pack(ring))) return rc;
   BRI_CUDA(cudaMemcpyAsync(P, ring, vb, cudaMemcpyDeviceToDevice, st));
-  kp_norm<<<dim3(nblk, ngrp), 256, 0, st>>>(gd, ring, part); note_launch();
+  kp_norm<<<dim3(nblk, nsys), 256, 0, st>>>(gd, ring, part); note_launch();
   k_scalar_init<<<nsys, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
   BRI_LAUNCH_CHECK("packed multi-shift init");
 
-  // systems and groups of the active prefix (a pair counts whole)
-  auto prefix = [&](int na, int* ns, int* ng) {
-    *ns = 0;
-    *ng = 0;
-    while (*ns < na && *ng < ngrp) *ns += pb.grp[(*ng)++].two ? 2 : 1;
-  };
   // `count` iterations from ring slot 0 on (every block of iterations starts there)
   auto enqueue = [&](int na, int count) -> int {
-    int ns, ng, q;
-    prefix(na, &ns, &ng);
+    int q;
     for (int j = 0; j < count; ++j) {
       if ((q = apply(0, P, T, (const float4*)nullptr, na))) return q;
       if ((q = apply(1, T, Q, (const float4*)P, na))) return q;
-      k_scalar_alpha<<<ns, RED_THREADS, 0, st>>>(S, sdpart, nb, hist, defer && j % DW == 0, 1); note_launch();
+      k_scalar_alpha<<<na, RED_THREADS, 0, st>>>(S, sdpart, nb, hist, defer && j % DW == 0, 1); note_launch();
       float4 *rin = defer ? ring + (j % kRing) * pb.words : ring, *rout = defer ? ring + ((j + 1) % kRing) * pb.words : ring;
-      kp_update_r<<<dim3(nblk, ng), 256, 0, st>>>(gd, S, Q, rin, rout, part); note_launch();
-      k_scalar_beta<<<ns, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
-      if (defer) kp_update_p<false><<<dim3(nblk, ng), 256, 0, st>>>(gd, S, rout, P, nullptr);
-      else kp_update_p<true><<<dim3(nblk, ng), 256, 0, st>>>(gd, S, rout, P, xp);
+      kp_update_r<<<dim3(nblk, na), 256, 0, st>>>(gd, S, Q, rin, rout, part); note_launch();
+      k_scalar_beta<<<na, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
+      if (defer) kp_update_p<false><<<dim3(nblk, na), 256, 0, st>>>(gd, S, rout, P, nullptr);
+      else kp_update_p<true><<<dim3(nblk, na), 256, 0, st>>>(gd, S, rout, P, xp);
       note_launch();
       if (defer && ((j + 1) % DW == 0 || j == count - 1)) {
-        kp_flush<<<dim3(nblk, ng), 256, 0, st>>>(gd, hist, ring, pb.words, j / DW * DW, bpk.as<float2>(), x64);
+        kp_flush<<<dim3(nblk, na), 256, 0, st>>>(gd, hist, ring, pb.words, j / DW * DW, bpk.as<float2>(), x64);
         note_launch();
       }
     }
