@@ -40,21 +40,6 @@ int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s)
   return BRI_OK;
 }
 
-// yp = D X for nrhs packed right-hand sides, ks thread groups per site; with p the
-// fused epilogue of ShiftDot, part: [nrhs][blocks_for(V, pack_sites(ks))].
-template <typename LS>
-int bri_f32_on_packed(const Geom& g, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs, int ks,
-                      int dagger, cudaStream_t s, const void* p, const double* sig, double* part) {
-  const PackedDot sd{(const float4*)p, sig, part};
-  launch_singles<LS>(g, nullptr, (float4*)yp, (const float4*)X, W, cl, diag, dagger, 0, nrhs, s, p ? &sd : nullptr, ks);
-  BRI_LAUNCH_CHECK("bri_pair_kernel");
-  return BRI_OK;
-}
-template int bri_f32_on_packed<float2>(const Geom&, void*, const void*, const float2*, const float*, float, int, int, int,
-                                       cudaStream_t, const void*, const double*, double*);
-template int bri_f32_on_packed<__nv_bfloat162>(const Geom&, void*, const void*, const __nv_bfloat162*, const float*, float, int,
-                                               int, int, cudaStream_t, const void*, const double*, double*);
-
 // Spinors in their own layout in and out.  The packed copy of x lives in a
 // stream-ordered allocation of at most kChunk right-hand sides; where there is
 // no memory for it the split kernel, which needs none, takes over.
@@ -78,7 +63,7 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
         if (one) {
           const int r1 = r0 + 2 * pairs;
           launch_pack<2>(g.V, x, r1, one, X1, s);
-          launch_singles<LS>(g, y, nullptr, X1, W, cl, diag, dagger, r1, one, s, nullptr, pack_groups(g.V * one));
+          launch_singles<LS>(g, y, X1, W, cl, diag, dagger, r1, one, s);
         }
       }
       cudaFreeAsync(X, s);

@@ -467,18 +467,16 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
   }
 }
 
-// D on `groups` packed groups of one lattice; the first one holds right-hand
+// y = D x on `groups` packed groups of one lattice; the first one holds right-hand
 // side rhs0 (and rhs0 + 1).
-template <int R, typename LS, int OUT, bool EPI, int KS>
+template <int R, typename LS, int KS>
 __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
-    bri_pair_kernel(Geom g, float* __restrict__ y, float4* __restrict__ yp, const float4* __restrict__ x,
-                    const LS* __restrict__ W, const float* __restrict__ cl, float diag, int rhs0, int gfirst,
-                    const __grid_constant__ PairHops H, PackedDot sd) {
+    bri_pair_kernel(Geom g, float* __restrict__ y, const float4* __restrict__ x, const LS* __restrict__ W,
+                    const float* __restrict__ cl, float diag, int rhs0, int gfirst, const __grid_constant__ PairHops H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  const int64_t go = (int64_t)grp * packed_words(g.V, 3 * R);
-  const int s0 = rhs0 + grp * (R / 2);
-  pr_block<R, LS, OUT, EPI, KS>(g, blk, y + (int64_t)s0 * g.V * 24, yp + go, x + go, W, cl, diag, H, sd, go, s0,
-                                gfirst ? gridDim.y : gridDim.x);
+  pr_block<R, LS, 0, false, KS>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
+                                x + (int64_t)grp * packed_words(g.V, 3 * R), W, cl, diag, H,
+                                PackedDot{nullptr, nullptr, nullptr}, 0, 0, 0);
 }
 
 // Spinors [nrhs][V][12] complex64 -> packed groups; group g holds the
@@ -524,30 +522,20 @@ template <typename LS>
 inline void launch_pairs(const Geom& g, float* y, const float4* X, const LS* W, const float* cl, float diag, int dagger,
                          int rhs0, int groups, cudaStream_t s) {
   const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
-  bri_pair_kernel<4, LS, 0, false, 1><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst,
-                                                              pair_hops(dagger), PackedDot{nullptr, nullptr, nullptr});
+  bri_pair_kernel<4, LS, 1><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger));
   note_launch();
 }
 
-// y or packed yp = D x for `n` single right-hand sides starting at rhs0, with sd
-// (yp only) the solver's epilogue.
-template <typename LS, int KS>
-inline void launch_singles_ks(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
-                              int dagger, int rhs0, int n, cudaStream_t s, const PackedDot* sd) {
-  const StencilGrid sg = stencil_grid(blocks_for(g.V, 128 / KS), n);
-  const PackedDot none{nullptr, nullptr, nullptr};
-  const PairHops& H = pair_hops(dagger);
-  if (sd) bri_pair_kernel<2, LS, 1, true, KS><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, H, *sd);
-  else if (yp) bri_pair_kernel<2, LS, 1, false, KS><<<sg.grid, 128, 0, s>>>(g, nullptr, yp, X, W, cl, diag, rhs0, sg.gfirst, H, none);
-  else bri_pair_kernel<2, LS, 0, false, KS><<<sg.grid, 128, 0, s>>>(g, y, nullptr, X, W, cl, diag, rhs0, sg.gfirst, H, none);
-  note_launch();
-}
+// y = D x for `n` single right-hand sides starting at rhs0.
 template <typename LS>
-inline void launch_singles(const Geom& g, float* y, float4* yp, const float4* X, const LS* W, const float* cl, float diag,
-                           int dagger, int rhs0, int n, cudaStream_t s, const PackedDot* sd, int ks) {
-  if (ks == 4) launch_singles_ks<LS, 4>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
-  else if (ks == 2) launch_singles_ks<LS, 2>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
-  else launch_singles_ks<LS, 1>(g, y, yp, X, W, cl, diag, dagger, rhs0, n, s, sd);
+inline void launch_singles(const Geom& g, float* y, const float4* X, const LS* W, const float* cl, float diag, int dagger,
+                           int rhs0, int n, cudaStream_t s) {
+  const int ks = pack_groups(g.V * n);
+  const StencilGrid sg = stencil_grid(blocks_for(g.V, pack_sites(ks)), n);
+  with_groups(ks, [&](auto k) {
+    bri_pair_kernel<2, LS, decltype(k)::value><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger));
+  });
+  note_launch();
 }
 
 }  // namespace bri

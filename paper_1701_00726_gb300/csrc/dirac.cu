@@ -45,21 +45,6 @@ int dirac_kernel(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int da
   return dirac_bri(c, y, x, nrhs, m0, dagger, prec, s);
 }
 
-int dirac_bri_packed(bri_ctx* c, void* yp, const void* X, int nrhs, int ks, double m0, int dagger, int prec,
-                     cudaStream_t s, const void* p, const double* sig, double* part) {
-  const float diag = (float)(15.0 / 8.0 + m0);
-  const float* cl = c->have_clover ? c->C32 : nullptr;
-  cudaEvent_t ev;
-  int rc = prof_begin(c, s, &ev);
-  if (rc) return rc;
-  if (prec == BRI_PREC_F32_BF16)
-    rc = bri_f32_on_packed<__nv_bfloat162>(c->g, yp, X, c->W16, cl, diag, nrhs, ks, dagger, s, p, sig, part);
-  else
-    rc = bri_f32_on_packed<float2>(c->g, yp, X, c->W32, cl, diag, nrhs, ks, dagger, s, p, sig, part);
-  if (rc) return rc;
-  return prof_end(c, s, ev, 0, prec, (double)c->g.V * nrhs);
-}
-
 int dirac_bri(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec, cudaStream_t s) {
   const double diag = 15.0 / 8.0 + m0;
   cudaEvent_t ev;

@@ -142,11 +142,6 @@ int dirac_bri_shiftdot(bri_ctx* c, void* y, const void* x, int nrhs, double m0, 
 // the Brillouin stencil (Eq. def_bril) or the Wilson stencil (Eq. def_wils).
 int dirac_kernel(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec,
                  cudaStream_t s);
-// The FP32 stencil on packed vectors (bri_f32_on_packed): yp = D X or D^dagger X
-// for nrhs right-hand sides; with the packed vector p the fused epilogue of
-// dirac_bri_shiftdot.
-int dirac_bri_packed(bri_ctx* c, void* yp, const void* X, int nrhs, int ks, double m0, int dagger, int prec,
-                     cudaStream_t s, const void* p, const double* sig, double* part);
 // Keeps freed blocks of the device's stream-ordered pool for the next
 // allocation (set once; the memory goes back when the last context is destroyed).
 void configure_pool_once();

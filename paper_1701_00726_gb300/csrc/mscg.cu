@@ -817,22 +817,41 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
     pb.sys.push_back(PackedSys{0, V, pb.words, s * n2, nsys * n2});
     pb.words += packed_words(V, 6);
   }
-  const int ks = pack_groups(V * nsys), nb = blocks_for(V, pack_sites(ks));
+  auto blocks = [&](int na) { return blocks_for(V, pack_sites(pack_groups(V * na))); };
   DevBuf bsig, bsd, bx;
   int rc;
   if ((rc = bsig.alloc(sizeof(double) * nsys, st))) return rc;
-  if ((rc = bsd.alloc(sizeof(double) * nsys * nb, st))) return rc;
+  if ((rc = bsd.alloc(sizeof(double) * nsys * blocks_for(V, pack_sites(4)), st))) return rc;
   if (!x64 && (rc = bx.alloc(sizeof(float4) * pb.words, st))) return rc;
   std::vector<double> hsig(nsys);
   for (int s = 0; s < nsys; ++s) hsig[s] = sig[(size_t)s * nshift];
   BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));
   auto pack = [&](float4* dst) { return bri_f32_pack(V, b, nsys, dst, st); };
-  auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int na) {
-    return dirac_bri_packed(c, Y, X, na, ks, m0, dagger, prec, st, P, bsig.as<double>(), bsd.as<double>());
+  const MsState* S = nullptr;
+  auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int na) -> int {
+    const PackedDot pd{P, bsig.as<double>(), bsd.as<double>()};
+    const float* cl = c->have_clover ? c->C32 : nullptr;
+    const float diag = (float)(15.0 / 8.0 + m0);
+    const StencilGrid sg = stencil_grid(blocks(na), na);
+    cudaEvent_t ev;
+    if (int e = prof_begin(c, st, &ev)) return e;
+    with_groups(pack_groups(V * na), [&](auto ktag) {
+      constexpr int KS = decltype(ktag)::value;
+      auto run = [&](const auto* W) {
+        using LS = std::decay_t<decltype(*W)>;
+        if (P) kp_stencil<LS, true, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops(dagger), pd);
+        else kp_stencil<LS, false, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops(dagger), pd);
+      };
+      if (prec == BRI_PREC_F32_BF16) run(c->W16);
+      else run(c->W32);
+    });
+    note_launch();
+    BRI_LAUNCH_CHECK("kp_stencil");
+    return prof_end(c, st, ev, 0, prec, (double)V * na);
   };
   const bool graphs = graphs_enabled() && !c->prof_on && st != nullptr;
-  rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), nb, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
-                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out);
+  rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), blocks, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
+                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out, &S);
   if (rc < 0 || x64) return rc;
   const int q = bri_f32_unpack(V, bx.p, nsys, x, st);
   return q ? q : rc;
@@ -1749,8 +1768,10 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
       lat_off[i] = sd[first_sys[i]].off;
       nb = std::max(nb, blocks_for(V, sb));
       maxb = std::max(maxb, n2 * nrhs[i]);
+      // the systems of a site block next to each other: they read the same links
+      for (int k = 0; k < blocks_for(V, sb); ++k)
+        for (int r = 0; r < nrhs[i]; ++r) items.push_back(make_int2(first_sys[i] + r, k));
       for (int r = 0; r < nrhs[i]; ++r) {
-        for (int k = 0; k < blocks_for(V, sb); ++k) items.push_back(make_int2((int)pb.sys.size(), k));
         pb.sys.push_back(PackedSys{i, V, pb.words, lat_off[i] * n + r * n2, nrhs[i] * n2});
         pb.words += packed_words(V, 6);
       }
@@ -1784,18 +1805,15 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
       const PackedDot pd{P, bsig.as<double>(), bpart.as<double>()};
       const PackedSys* gd = bgd.as<PackedSys>();
       const PairHops& H = pair_hops(dagger);
-      auto run = [&](auto ktag) {
+      with_groups(ks, [&](auto ktag) {
         constexpr int KS = decltype(ktag)::value;
         if (P) kb_pair<LS, true, KS><<<ni, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
         else kb_pair<LS, false, KS><<<ni, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);
-        note_launch();
-      };
-      if (ks == 4) run(std::integral_constant<int, 4>());
-      else if (ks == 2) run(std::integral_constant<int, 2>());
-      else run(std::integral_constant<int, 1>());
+      });
+      note_launch();
       return BRI_OK;
     };
-    q = packed_solve(bs, pb, pack, apply, bpart.as<double>(), nb, bXall.as<double2>(), sizeof(double2) * off * n, nullptr, true,
+    q = packed_solve(bs, pb, pack, apply, bpart.as<double>(), [&](int) { return nb; }, bXall.as<double2>(), sizeof(double2) * off * n, nullptr, true,
                      true, nullptr, &info1.iters, &info1.cnt, &lam_est, &St);
     if (q < 0) return q;
     solve_rc = std::max(solve_rc, q);

@@ -218,6 +218,20 @@ __global__ void __launch_bounds__(256) kp_flush(const PackedSys* __restrict__ gd
   }
 }
 
+// Stencil on the systems of one lattice, the systems of a site block next to each
+// other (stencil_grid); converged systems are skipped, not only the trailing ones
+// that the host has dropped at its last look.
+template <typename LS, bool EPI, int KS>
+__global__ void __launch_bounds__(128, 4)
+    kp_stencil(Geom g, const MsState* __restrict__ st, float4* __restrict__ Y, const float4* __restrict__ X,
+               const LS* __restrict__ W, const float* __restrict__ cl, float diag, int gfirst,
+               const __grid_constant__ PairHops H, PackedDot sd) {
+  const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
+  if (st[s].done) return;
+  const int64_t o = s * packed_words(g.V, 6);
+  pr_block<2, LS, 1, EPI, KS>(g, blk, nullptr, Y + o, X + o, W, cl, diag, H, sd, o, s, gfirst ? gridDim.y : gridDim.x);
+}
+
 // Stencil on the work list of several lattices: item (system, block of 128 / KS
 // sites); converged systems are skipped.
 template <typename LS, bool EPI, int KS>
@@ -244,12 +258,12 @@ struct PackedProblem {
 
 // Solves (A + sig[s][k]) x[k][s] = b[s].  pack(dst) writes the packed right-hand
 // sides; apply(dagger, X, Y, P, na) enqueues Y = D X (P null) or Y = D^dagger X +
-// sigma P with partials [nsys][nb] in sdpart, for the first na systems.
+// sigma P with partials [na][blocks(na)] in sdpart, for the first na systems.
 // Several shifts: solutions in x64 (zeroed here).  One shift: packed in xp.
 // whole: all iterations in one WHILE-node graph (no host polling), else host
 // polling every kRing iterations and a shrinking prefix of systems.
-template <typename Pack, typename Apply>
-int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& apply, double* sdpart, int nb,
+template <typename Pack, typename Apply, typename Blocks>
+int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& apply, double* sdpart, Blocks&& blocks,
                  double2* x64, size_t x64_bytes, float4* xp, bool whole, bool graphs, int* hdone,
                  int* iters_out, Counters* cnt, double* lam_out, const MsState** state_out = nullptr) {
   const int nsys = pb.nsys, nshift = pb.nshift;
@@ -311,7 +325,7 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
     for (int j = 0; j < count; ++j) {
       if ((q = apply(0, P, T, (const float4*)nullptr, na))) return q;
       if ((q = apply(1, T, Q, (const float4*)P, na))) return q;
-      k_scalar_alpha<<<na, RED_THREADS, 0, st>>>(S, sdpart, nb, hist, defer && j % DW == 0, 1); note_launch();
+      k_scalar_alpha<<<na, RED_THREADS, 0, st>>>(S, sdpart, blocks(na), hist, defer && j % DW == 0, 1); note_launch();
       float4 *rin = defer ? ring + (j % kRing) * pb.words : ring, *rout = defer ? ring + ((j + 1) % kRing) * pb.words : ring;
       kp_update_r<<<dim3(nblk, na), 256, 0, st>>>(gd, S, Q, rin, rout, part); note_launch();
       k_scalar_beta<<<na, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();

@@ -189,19 +189,19 @@ int launch_bri_f64(const Geom& g, double* y, const double* x, const double2* W, 
 template <typename LS>
 int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const float* cl, float diag, int nrhs,
                    int dagger, cudaStream_t s, const ShiftDot<float>* sd = nullptr, int* sd_blocks = nullptr);
-// Packed FP32 vectors of single right-hand sides (bri_pair.cuh) for callers that
-// keep their vectors in that form: whether a launch of nrhs right-hand sides takes
-// the packed kernels, packing, and the operator on such a vector (packed yp out,
-// for nrhs right-hand sides; with the packed vector p the fused solver epilogue,
-// see ShiftDot).  pack_groups(V * nrhs): the thread groups that share a site's
-// offsets, pack_sites of it: the sites of a block (one partial each).
+// Packed FP32 vectors of single right-hand sides (bri_pair.cuh) for the solver,
+// which keeps its vectors in that form: whether a launch of nrhs right-hand sides
+// takes the packed kernels, and packing.  pack_groups(V * nrhs): the thread groups
+// that share a site's offsets, pack_sites of it: the sites of a block.
 bool bri_f32_packed(int64_t V, int nrhs);
 int pack_groups(int64_t site_rhs);
 inline int pack_sites(int ks) { return 128 / ks; }
+template <typename F> inline void with_groups(int ks, F&& f) {
+  if (ks == 4) f(std::integral_constant<int, 4>());
+  else if (ks == 2) f(std::integral_constant<int, 2>());
+  else f(std::integral_constant<int, 1>());
+}
 int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s);
-template <typename LS>
-int bri_f32_on_packed(const Geom& g, void* yp, const void* X, const LS* W, const float* cl, float diag, int nrhs, int ks,
-                      int dagger, cudaStream_t s, const void* p, const double* sig, double* part);
 int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s);
 template <typename R, typename LS>
 int launch_wil_t(const Geom& g, R* y, const R* x, const LS* U, const R* cl, R diag, int nrhs, int dagger,
