@@ -148,14 +148,18 @@ const HopTableDW& hop_table_dw() {
 constexpr int kDwLinkWords = 9 * kLinkBlock;  // one offset of one block of sites
 
 // One thread per site and right-hand side (grid groups = right-hand sides, in
-// the order of stencil_grid).  The hop loop is rolled so that the body fits the
-// instruction cache.
+// the order of stencil_grid), or KS groups of threads that share a site's offsets
+// and meet in shared memory, where the first two finish one chirality each.  The
+// hop loop is rolled so that the body fits the instruction cache.
+template <int KS>
 __global__ void __launch_bounds__(128, 3)
     bri_kernel_dw(Geom g, float4* __restrict__ y, const float4* __restrict__ x, const float4* __restrict__ W,
                   const float2* __restrict__ cl, DW diag, float sgn, int gfirst, const __grid_constant__ HopTableDW H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  const int n = blk * blockDim.x + threadIdx.x;
-  if (n >= g.V) return;
+  constexpr int SB = 128 / KS;
+  const int n0 = blk * SB + threadIdx.x % SB;
+  if (KS == 1 && n0 >= g.V) return;
+  const int n = KS == 1 ? n0 : min(n0, (int)g.V - 1), ksg = KS == 1 ? 0 : threadIdx.x / SB;
   const int64_t roff = (int64_t)grp * packed_words(g.V, 12);
   const float4* xin = x + roff;
   int up[4], dn[4];
@@ -177,7 +181,7 @@ __global__ void __launch_bounds__(128, 3)
     for (int aa = 0; aa < 3; ++aa) acc[q][aa] = CDP{zero_dp(), zero_dp()};
 
 #pragma unroll 1
-  for (int j = 0; j < 40; ++j) {
+  for (int j = ksg; j < 40; j += KS) {
     int mp = n, mm = n;
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
@@ -288,6 +292,32 @@ __global__ void __launch_bounds__(128, 3)
         renorm(acc[q][aa].im);
       }
   }
+  if constexpr (KS > 1) {
+    __shared__ float4 red[KS][12][SB];
+    const int l = threadIdx.x % SB;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const CDP& v = acc[i / 3][i % 3];
+      red[ksg][2 * i][l] = make_float4(v.re.h.x, v.re.h.y, v.re.l.x, v.re.l.y);
+      red[ksg][2 * i + 1][l] = make_float4(v.im.h.x, v.im.h.y, v.im.l.x, v.im.l.y);
+    }
+    __syncthreads();
+    if (ksg >= 2 || n0 >= g.V) return;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      CDP t{zero_dp(), zero_dp()};
+#pragma unroll
+      for (int k = 0; k < KS; ++k) {
+        const float4 r = red[k][6 * ksg + 2 * i][l], m = red[k][6 * ksg + 2 * i + 1][l];
+        add(t.re, DP{make_float2(r.x, r.y), make_float2(r.z, r.w)}, pr_bc(1.f));
+        add(t.im, DP{make_float2(m.x, m.y), make_float2(m.z, m.w)}, pr_bc(1.f));
+      }
+      renorm(t.re);
+      renorm(t.im);
+      acc[0][i] = t;  // this group's chirality, whichever it is
+      acc[1][i] = t;
+    }
+  }
   // diagonal and clover terms at the site itself.  A chirality's clover block is
   // [[X, M], [M^dagger, -X]] on its two spins: X (3 reals, 3 complex above the
   // diagonal) acts with the signs (+, -), M and M^dagger on the exchanged spins.
@@ -296,6 +326,7 @@ __global__ void __launch_bounds__(128, 3)
   const float2 dh = pr_bc(diag.h), dl = pr_bc(diag.l);
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
+    if (KS > 1 && q != ksg) continue;
     CDP in[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
@@ -436,6 +467,12 @@ int ensure_dw_links(bri_ctx* c) {
   return BRI_OK;
 }
 
+// Four groups of threads per site until one thread per site fills several waves.
+// GB300, us with one group / four (conversions included): 8^4 x 1 rhs 158 / 56, 8^3.16
+// x 1 162 / 84, 12^4 x 1 296 / 195, 16^4 x 1 567 / 489, 8^3.16 x 12 739 / 662, 16^4 x 2
+// 911 / 884, 16^3.32 x 2 1749 / 1711, x 4 3289 / 3315.
+static int dw_groups(int64_t site_rhs) { return site_rhs <= 393216 ? 4 : 1; }
+
 // y = D x or D^dagger x on double-word vectors (Brillouin kernel).
 int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, cudaStream_t s) {
   int rc = ensure_dw_links(c);
@@ -444,11 +481,15 @@ int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int da
   DW diag;
   diag.h = (float)dg;
   diag.l = (float)(dg - (double)diag.h);
-  const int threads = 128;
-  const StencilGrid sg = stencil_grid(blocks_for(c->g.V, threads), nrhs);
-  bri_kernel_dw<<<sg.grid, threads, 0, s>>>(c->g, (float4*)y, (const float4*)x, (const float4*)c->Wdw,
-                                             c->have_clover ? (const float2*)c->Cdw : nullptr, diag,
-                                             dagger ? -1.f : 1.f, sg.gfirst, hop_table_dw());
+  const int ks = dw_groups(c->g.V * nrhs);
+  const StencilGrid sg = stencil_grid(blocks_for(c->g.V, 128 / ks), nrhs);
+  auto run = [&](auto kernel) {
+    kernel<<<sg.grid, 128, 0, s>>>(c->g, (float4*)y, (const float4*)x, (const float4*)c->Wdw,
+                                   c->have_clover ? (const float2*)c->Cdw : nullptr, diag, dagger ? -1.f : 1.f, sg.gfirst,
+                                   hop_table_dw());
+  };
+  if (ks == 4) run(bri_kernel_dw<4>);
+  else run(bri_kernel_dw<1>);
   note_launch();
   BRI_LAUNCH_CHECK("bri_kernel_dw");
   return BRI_OK;

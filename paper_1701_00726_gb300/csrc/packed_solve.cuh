@@ -274,7 +274,14 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
     maxw = std::max(maxw, packed_words(g.V, 6));
     n2all += g.V * 12;
   }
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((maxw + 255) / 256, std::max(1, kMaxPartials / nsys)));
+  // Reductions: four words per thread in flight (kp_update_r), but two blocks per SM
+  // as long as there is a word for every thread; partials as everywhere.  8^3 x 16,
+  // 12 systems: 24 us with 170 blocks per system, 12 with 48.
+  const int64_t one = (maxw + 255) / 256, four = (maxw + 1023) / 1024;
+  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(four, std::min<int64_t>(one, 304 / nsys)),
+                                                               std::max(1, kMaxPartials / nsys)));
+  // the other vector kernels: a word per thread, so that no block has a round more than the next
+  const int nvec = (int)std::min<int64_t>(one, 65536);
   DevBuf bgd, bst, bpart, bring, bP, bT, bQ, bpk, bhist, bflags;
   int rc;
   if ((rc = bgd.alloc(sizeof(PackedSys) * nsys, st))) return rc;
@@ -329,11 +336,11 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
       float4 *rin = defer ? ring + (j % kRing) * pb.words : ring, *rout = defer ? ring + ((j + 1) % kRing) * pb.words : ring;
       kp_update_r<<<dim3(nblk, na), 256, 0, st>>>(gd, S, Q, rin, rout, part); note_launch();
       k_scalar_beta<<<na, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
-      if (defer) kp_update_p<false><<<dim3(nblk, na), 256, 0, st>>>(gd, S, rout, P, nullptr);
-      else kp_update_p<true><<<dim3(nblk, na), 256, 0, st>>>(gd, S, rout, P, xp);
+      if (defer) kp_update_p<false><<<dim3(nvec, na), 256, 0, st>>>(gd, S, rout, P, nullptr);
+      else kp_update_p<true><<<dim3(nvec, na), 256, 0, st>>>(gd, S, rout, P, xp);
       note_launch();
       if (defer && ((j + 1) % DW == 0 || j == count - 1)) {
-        kp_flush<<<dim3(nblk, na), 256, 0, st>>>(gd, hist, ring, pb.words, j / DW * DW, bpk.as<float2>(), x64);
+        kp_flush<<<dim3(nvec, na), 256, 0, st>>>(gd, hist, ring, pb.words, j / DW * DW, bpk.as<float2>(), x64);
         note_launch();
       }
     }

@@ -58,6 +58,19 @@ def test_bri_apply_every_path(dims, nrhs, dagger):
         assert relerr(lat.bri_apply(x32, -1.0, dagger=dagger, bf16_links=bf16).cpu().numpy(), want) < bound
 
 
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((3, 2, 5, 2), 3), (LARGE, 2), (LARGE, 46)])
+@pytest.mark.parametrize("dagger", [False, True])
+def test_double_word_forms(dims, nrhs, dagger):
+    """Double-word stencil with four groups of threads per site and (394128 sites x rhs) with one: 1e-13 of
+    the largest element, as in the parity tests (48-bit operands, a few hundred roundings)."""
+    some = [0, nrhs - 1] if nrhs > 4 else list(range(nrhs))
+    x = sf.gaussian_source(dims, nrhs, 1035)
+    op = _operator(dims, True)[1]
+    want = op.apply_dagger(x[some]) if dagger else op.apply(x[some])
+    y = _lattice(dims, anti=True).bri_apply(torch.from_numpy(x).cuda(), -1.0, dagger=dagger, double_word=True)
+    assert relerr(y[some].cpu().numpy(), want) < 1e-13
+
+
 @pytest.mark.parametrize("dims,nrhs", [((8, 6, 7, 10), 19), (LARGE, 17), ((16, 15, 17, 19), 7), ((16, 15, 17, 19), 15)])
 def test_packed_forms_and_chunks(dims, nrhs):
     """Chunks of 16 right-hand sides (the packed buffer's size) and what is left, in every packed form:
