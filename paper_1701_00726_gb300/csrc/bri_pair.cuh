@@ -72,42 +72,6 @@ template <int ROWS> __device__ __forceinline__ int packed_at(int m) {
   return (m / kPackBlock) * (ROWS * kPackBlock) + m % kPackBlock;
 }
 
-// Per-offset data of the packed kernels: index of the stored offset,
-// displacement signs, a_k, and the gamma weights for V = -(P - Q), c_mu =
-// -(sign) c_k s_mu.  The offsets come with the most hops (the smallest
-// weights) first, so the accumulator stays small for most of its roundings
-// (relative error against FP64 at 16^3 x 32 and 24^3 x 48: 7.5e-8 sorted, 1.0e-7 in
-// storage order).
-struct PairHops {
-  int j[40];
-  int d[40][4];
-  float a[40];
-  float c[40][4];
-};
-inline const PairHops& pair_hops(int dagger) {
-  static const auto make = [](float sgn) {
-    PairHops t;
-    const HopTable<float>& h = hop_table<float>();
-    int i = 0;
-    for (int k = 4; k >= 1; --k)
-      for (int j = 0; j < 40; ++j) {
-        int hops = 0;
-        for (int mu = 0; mu < 4; ++mu) hops += h.site_d[j][mu] != 0;
-        if (hops != k) continue;
-        t.j[i] = j;
-        t.a[i] = h.a[j];
-        for (int mu = 0; mu < 4; ++mu) {
-          t.d[i][mu] = h.site_d[j][mu];
-          t.c[i][mu] = -sgn * h.cs[j][mu];
-        }
-        ++i;
-      }
-    return t;
-  };
-  static const PairHops t0 = make(1.f), t1 = make(-1.f);
-  return dagger ? t1 : t0;
-}
-
 // P = w x (rows of x: R spinor rows, component q at row 3 q + colour)
 template <int R> __device__ __forceinline__ void pr_fwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
 #pragma unroll
@@ -216,7 +180,7 @@ __device__ __forceinline__ void pr_gamma(CP (&acc)[2][3], const CP (&v)[2][3], f
 // pair from i0 on); x = packed vector (R = 4: a pair of right-hand sides, R = 2: one).
 template <int R, typename LS, int KS>
 __device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, const float4* __restrict__ x,
-                                        const LS* __restrict__ W, const PairHops& H, int i0) {
+                                        const LS* __restrict__ W, const PairHops<float>& H, int i0) {
   const int V = (int)g.V;
   // index steps to the neighbours in each direction (periodic)
   int up[4], dn[4];
@@ -337,7 +301,7 @@ template <int KS> __device__ __forceinline__ int pr_group() {
 template <int R, typename LS, int OUT, bool EPI, int KS>
 __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restrict__ y0, float4* __restrict__ yp,
                                          const float4* __restrict__ x, const LS* __restrict__ W,
-                                         const float* __restrict__ cl, float diag, const PairHops& H, const PackedDot& sd,
+                                         const float* __restrict__ cl, float diag, const PairHops<float>& H, const PackedDot& sd,
                                          int64_t po, int s, int nb) {
   static_assert(R == 2 || (OUT == 0 && KS == 1), "pairs: spinors' own layout out, one thread per site");
   static_assert(!EPI || OUT == 1, "the epilogue writes packed vectors");
@@ -472,7 +436,7 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
 template <int R, typename LS, int KS>
 __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
     bri_pair_kernel(Geom g, float* __restrict__ y, const float4* __restrict__ x, const LS* __restrict__ W,
-                    const float* __restrict__ cl, float diag, int rhs0, int gfirst, const __grid_constant__ PairHops H) {
+                    const float* __restrict__ cl, float diag, int rhs0, int gfirst, const __grid_constant__ PairHops<float> H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   pr_block<R, LS, 0, false, KS>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
                                 x + (int64_t)grp * packed_words(g.V, 3 * R), W, cl, diag, H,
@@ -522,7 +486,7 @@ template <typename LS>
 inline void launch_pairs(const Geom& g, float* y, const float4* X, const LS* W, const float* cl, float diag, int dagger,
                          int rhs0, int groups, cudaStream_t s) {
   const StencilGrid sg = stencil_grid(blocks_for(g.V, 128), groups);
-  bri_pair_kernel<4, LS, 1><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger));
+  bri_pair_kernel<4, LS, 1><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops<float>(dagger));
   note_launch();
 }
 
@@ -533,7 +497,7 @@ inline void launch_singles(const Geom& g, float* y, const float4* X, const LS* W
   const int ks = pack_groups(g.V * n);
   const StencilGrid sg = stencil_grid(blocks_for(g.V, pack_sites(ks)), n);
   with_groups(ks, [&](auto k) {
-    bri_pair_kernel<2, LS, decltype(k)::value><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops(dagger));
+    bri_pair_kernel<2, LS, decltype(k)::value><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops<float>(dagger));
   });
   note_launch();
 }

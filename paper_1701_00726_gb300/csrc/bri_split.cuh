@@ -20,8 +20,8 @@ namespace bri {
 // vectors); EPI: y = D x + sg p0, returns this thread's part of Re<p0, y>.
 template <typename R, typename LS, int S, int G, bool EPI>
 __device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restrict__ yout, const R* __restrict__ xin,
-                                              const LS* __restrict__ W, const R* __restrict__ cl, R diag, R sgn,
-                                              const HopTable<R>& H, const R* __restrict__ p0, R sg) {
+                                              const LS* __restrict__ W, const R* __restrict__ cl, R diag,
+                                              const PairHops<R>& H, const R* __restrict__ p0, R sg) {
   __shared__ R red[G][24][S];
   const int V = (int)g.V;
   {
@@ -45,11 +45,12 @@ __device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restr
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[aa][q] = C<R>{0, 0};
 #pragma unroll 1
-    for (int j = grp; j < 40; j += G) {
+    for (int i = grp; i < 40; i += G) {
+      const int j = H.j[i];
       int mp = n, mm = n;
 #pragma unroll
       for (int mu = 0; mu < 4; ++mu) {
-        const int d = H.site_d[j][mu];
+        const int d = H.d[i][mu];
         mp += d > 0 ? up[mu] : (d < 0 ? dn[mu] : 0);
         mm += d > 0 ? dn[mu] : (d < 0 ? up[mu] : 0);
       }
@@ -59,7 +60,7 @@ __device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restr
       load_spinor(xp, xin + (int64_t)mp * 24);
       load_stored_link<R, LS>(wm, W, j, mm, V);
       load_spinor(xm, xin + (int64_t)mm * 24);
-      const R a = H.a[j], a2 = 2 * a;
+      const R a = H.a[i], a2 = 2 * a;
       // P = w x+, V = wm^dagger x- - P, acc += 2 a P + a V - c G V
       C<R> v[3][4];
 #pragma unroll
@@ -83,8 +84,9 @@ __device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restr
           acc[aa][q].re = fma(a, v[aa][q].re, acc[aa][q].re);
           acc[aa][q].im = fma(a, v[aa][q].im, acc[aa][q].im);
         }
-      // gamma terms of vanishing weight are skipped (uniform within a group)
-      const R c1 = -sgn * H.cs[j][0], c2 = -sgn * H.cs[j][1], c3 = -sgn * H.cs[j][2], c4 = -sgn * H.cs[j][3];
+      // gamma terms of vanishing weight are skipped (uniform within a group,
+      // and nearly so within a warp, see pair_hops)
+      const R c1 = H.c[i][0], c2 = H.c[i][1], c3 = H.c[i][2], c4 = H.c[i][3];
       if (c1 != (R)0)
 #pragma unroll
         for (int aa = 0; aa < 3; ++aa) gamma_term<1>(acc[aa], v[aa], c1);
@@ -155,11 +157,11 @@ __device__ __forceinline__ double split_block(const Geom& g, int blk, R* __restr
 template <typename R, typename LS, int S, int G, bool EPI>
 __global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
     bri_split_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, const LS* __restrict__ W,
-                     const R* __restrict__ cl, R diag, R sgn, int gfirst, const __grid_constant__ HopTable<R> H,
+                     const R* __restrict__ cl, R diag, int gfirst, const __grid_constant__ PairHops<R> H,
                      ShiftDot<R> sd) {
   const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   const int64_t o = s * (g.V * 24);
-  double dot = split_block<R, LS, S, G, EPI>(g, blk, y + o, x + o, W, cl, diag, sgn, H, EPI ? sd.p + o : nullptr,
+  double dot = split_block<R, LS, S, G, EPI>(g, blk, y + o, x + o, W, cl, diag, H, EPI ? sd.p + o : nullptr,
                                              EPI ? (R)sd.sig[s] : (R)0);
   if constexpr (EPI) {
     __shared__ double sh[(S * G + 31) / 32];
@@ -176,13 +178,13 @@ __global__ void __launch_bounds__(S* G, sizeof(R) == 8 ? 2 : 3)
 }
 
 template <typename R, typename LS, int S, int G>
-inline void launch_split_sg(const Geom& g, R* y, const R* x, const LS* W, const R* cl, R diag, R sgn, int nrhs,
+inline void launch_split_sg(const Geom& g, R* y, const R* x, const LS* W, const R* cl, R diag, int dagger, int nrhs,
                             cudaStream_t st, const ShiftDot<R>* sd) {
   const StencilGrid sg = stencil_grid(blocks_for(g.V, S), nrhs);
   if (sd)
-    bri_split_kernel<R, LS, S, G, true><<<sg.grid, S * G, 0, st>>>(g, y, x, W, cl, diag, sgn, sg.gfirst, hop_table<R>(), *sd);
+    bri_split_kernel<R, LS, S, G, true><<<sg.grid, S * G, 0, st>>>(g, y, x, W, cl, diag, sg.gfirst, pair_hops<R>(dagger), *sd);
   else
-    bri_split_kernel<R, LS, S, G, false><<<sg.grid, S * G, 0, st>>>(g, y, x, W, cl, diag, sgn, sg.gfirst, hop_table<R>(),
+    bri_split_kernel<R, LS, S, G, false><<<sg.grid, S * G, 0, st>>>(g, y, x, W, cl, diag, sg.gfirst, pair_hops<R>(dagger),
                                                                    ShiftDot<R>{nullptr, nullptr, nullptr});
   note_launch();
 }
@@ -196,12 +198,11 @@ inline int split_sites(int64_t site_rhs) {
 template <typename R, typename LS>
 inline int launch_split(const Geom& g, R* y, const R* x, const LS* W, const R* cl, R diag, int nrhs, int dagger,
                         cudaStream_t st, const ShiftDot<R>* sd, int* sd_blocks) {
-  const R sgn = (R)(dagger ? -1 : 1);
   const int S = split_sites(g.V * nrhs);
   if (sd_blocks) *sd_blocks = blocks_for(g.V, S);
-  if (S == 32) launch_split_sg<R, LS, 32, 5>(g, y, x, W, cl, diag, sgn, nrhs, st, sd);
-  else if (S == 16) launch_split_sg<R, LS, 16, 10>(g, y, x, W, cl, diag, sgn, nrhs, st, sd);
-  else launch_split_sg<R, LS, 8, 20>(g, y, x, W, cl, diag, sgn, nrhs, st, sd);
+  if (S == 32) launch_split_sg<R, LS, 32, 5>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
+  else if (S == 16) launch_split_sg<R, LS, 16, 10>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
+  else launch_split_sg<R, LS, 8, 20>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
   BRI_LAUNCH_CHECK("bri_split_kernel");
   return BRI_OK;
 }

@@ -583,15 +583,15 @@ struct SysDesc {
 template <int S, int G>
 __global__ void __launch_bounds__(S* G, 2)
     kb_stencil(const __grid_constant__ BatchTab T, const SysDesc* __restrict__ sd, const int2* __restrict__ items,
-               const MsState* __restrict__ st, double2* y, const double2* x, int x_from_p, double sgn,
-               const __grid_constant__ HopTable<double> H) {
+               const MsState* __restrict__ st, double2* y, const double2* x, int x_from_p,
+               const __grid_constant__ PairHops<double> H) {
   const int2 it = items[blockIdx.x];
   if (st[it.x].done) return;
   const SysDesc d = sd[it.x];
   const BatchLat& L = T.lat[d.lat];
   split_block<double, double2, S, G, false>(L.g, it.y, reinterpret_cast<double*>(y + d.off),
                                             reinterpret_cast<const double*>(x + (x_from_p ? d.offn : d.off)),
-                                            (const double2*)L.W, (const double*)L.C, L.diag, sgn, H, nullptr, 0.0);
+                                            (const double2*)L.W, (const double*)L.C, L.diag, H, nullptr, 0.0);
 }
 
 // r = b, p_k = b, x_k = 0, partial ||b||^2
@@ -839,8 +839,8 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
       constexpr int KS = decltype(ktag)::value;
       auto run = [&](const auto* W) {
         using LS = std::decay_t<decltype(*W)>;
-        if (P) kp_stencil<LS, true, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops(dagger), pd);
-        else kp_stencil<LS, false, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops(dagger), pd);
+        if (P) kp_stencil<LS, true, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops<float>(dagger), pd);
+        else kp_stencil<LS, false, KS><<<sg.grid, 128, 0, st>>>(c->g, S, Y, X, W, cl, diag, sg.gfirst, pair_hops<float>(dagger), pd);
       };
       if (prec == BRI_PREC_F32_BF16) run(c->W16);
       else run(c->W32);
@@ -1365,19 +1365,19 @@ int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector
   // the host copies above read pageable vectors: complete them before they go out of scope
   BRI_CUDA(cudaStreamSynchronize(st));
   const dim3 vg(nblk, S);
-  const HopTable<double>& H = hop_table<double>();
   const int2* itd = bit.as<int2>();
-  auto stencil = [&](double2* out, const double2* in, int from_p, double sgn) {
-    if (sites == 32) kb_stencil<32, 5><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
-    else if (sites == 16) kb_stencil<16, 10><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
-    else kb_stencil<8, 20><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, sgn, H);
+  auto stencil = [&](double2* out, const double2* in, int from_p, int dagger) {
+    const PairHops<double>& H = pair_hops<double>(dagger);
+    if (sites == 32) kb_stencil<32, 5><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, H);
+    else if (sites == 16) kb_stencil<16, 10><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, H);
+    else kb_stencil<8, 20><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, H);
   };
   const int nst = 1;  // stencil launches per application
   kb_init<R><<<vg, RED_THREADS, 0, st>>>(sd, nshift, b, r, p, x, part); note_launch();
   k_scalar_init<<<S, RED_THREADS, 0, st>>>(S_, part, nblk); note_launch();
   auto iteration = [&](int first) {
-    stencil(t, p, 1, 1.0);
-    stencil(q, t, 0, -1.0);
+    stencil(t, p, 1, 0);
+    stencil(q, t, 0, 1);
     kb_shift_dot<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, p, q, part);
     k_scalar_alpha<<<S, RED_THREADS, 0, st>>>(S_, part, nblk);
     kb_update<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, q, r, p, x, part, first);
@@ -1804,7 +1804,7 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int) -> int {
       const PackedDot pd{P, bsig.as<double>(), bpart.as<double>()};
       const PackedSys* gd = bgd.as<PackedSys>();
-      const PairHops& H = pair_hops(dagger);
+      const PairHops<float>& H = pair_hops<float>(dagger);
       with_groups(ks, [&](auto ktag) {
         constexpr int KS = decltype(ktag)::value;
         if (P) kb_pair<LS, true, KS><<<ni, 128, 0, bs>>>(tab, gd, bit.as<int2>(), St, Y, X, H, pd, nb);

@@ -225,7 +225,7 @@ template <typename LS, bool EPI, int KS>
 __global__ void __launch_bounds__(128, 4)
     kp_stencil(Geom g, const MsState* __restrict__ st, float4* __restrict__ Y, const float4* __restrict__ X,
                const LS* __restrict__ W, const float* __restrict__ cl, float diag, int gfirst,
-               const __grid_constant__ PairHops H, PackedDot sd) {
+               const __grid_constant__ PairHops<float> H, PackedDot sd) {
   const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   if (st[s].done) return;
   const int64_t o = s * packed_words(g.V, 6);
@@ -238,7 +238,7 @@ template <typename LS, bool EPI, int KS>
 __global__ void __launch_bounds__(128, 4)
     kb_pair(const __grid_constant__ BatchTab T, const PackedSys* __restrict__ gd, const int2* __restrict__ items,
             const MsState* __restrict__ st, float4* __restrict__ Y, const float4* __restrict__ X,
-            const __grid_constant__ PairHops H, PackedDot sd, int nb) {
+            const __grid_constant__ PairHops<float> H, PackedDot sd, int nb) {
   const int2 it = items[blockIdx.x];
   const PackedSys gr = gd[it.x];
   if (st[it.x].done) return;
