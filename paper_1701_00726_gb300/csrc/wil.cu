@@ -2,13 +2,16 @@
 // flop count): for each of the 8 hops the 4-spinor is projected to 2 spin
 // components with (1 -+ gamma_mu), transported, and rebuilt.
 //
-// The FP32 kernel is bound by HBM (thin links 288, clover 288 and two spinors of
-// 96 bytes per site): links and clover come in 16-byte words of 32-site chunks
-// and serve NR right-hand sides per thread.  GB300, 24^3 x 48, 2 rhs, clover:
-// 302 us with element-wise link and clover streams read once per right-hand
-// side, 168 us now (3.8 TB/s of the bytes it cannot do without); one rhs per
-// thread 176 us at 5 blocks per SM, 206 us unbounded; two 176 us unbounded,
-// 197 us at 5 blocks.
+// FP32: links and clover come in 16-byte words of 32-site chunks; a block works on
+// 64 sites of two right-hand sides, whose links the second finds in L1.  HBM could
+// deliver its bytes (thin links 288, clover 288 and two spinors of 96 per site) in
+// 94 us at 24^3 x 48, 2 rhs, clover; what bounds it is the latency of the gathers
+// (12 to 16 warps per SM, DRAM and L2 half busy).  GB300, that case: 302 us with
+// element-wise link and clover streams read once per right-hand side, 168 us with
+// two right-hand sides per thread, 154 us now.  Against this: spinor words in order
+// (load_words; L1 83 % busy instead of 56) 168 us; one block of 128 sites per rhs
+// 176; 2, 4, 5 and 6 blocks per SM 187, 156, 174 and 186; prefetching a block's links and
+// clover into L2 188 (two rhs per thread).
 #include "stencil.cuh"
 
 namespace bri {
@@ -97,105 +100,126 @@ __device__ __forceinline__ void load_thin(C<float> u[3][3], const float2* __rest
   load_link_chunk<4>(u, U, mu, (int)m);
 }
 
-// forward: -1/2 (1 - gamma_mu) U_mu(n) x(n+mu); backward: -1/2 (1 + gamma_mu) U_mu(n-mu)^+ x(n-mu)
-// (dagger swaps the two projectors).
-template <int MU, int NR, typename R, typename LS, bool DAG>
-__device__ __forceinline__ void wil_dir(Spinor<R> (&acc)[NR], const R* __restrict__ xin, int64_t rs, const LS* __restrict__ U,
-                                        int64_t V, int64_t n, const Nb<R>& nb) {
-  const int64_t mf = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][2];
-  const int64_t mb = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][0];
-  C<R> u[3][3];
-  load_thin(u, U, MU, n, V);
+// N 16-byte words of a lane's spinor.  Neighbouring lanes are 96 bytes apart, so
+// of eight lanes that read the same word two at a time meet in a bank; the lanes
+// with bit 2 set take each pair of words the other way round, and none do.
+template <int N> __device__ __forceinline__ void load_words(float4 (&v)[N], const float4* __restrict__ q) {
+  const int odd = (threadIdx.x >> 2) & 1;
 #pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    Spinor<R> xs;
-    load_spinor(xs, xin + r * rs + mf * 24);
-    C<R> h[2][3], uh[2][3];
-    project<MU, DAG>(xs, h);
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        uh[s][a] = C<R>{0, 0};
-#pragma unroll
-        for (int b = 0; b < 3; ++b) cfma(uh[s][a], u[a][b], h[s][b]);
-      }
-    reconstruct<MU, DAG>(acc[r], uh);
+  for (int i = 0; i + 1 < N; i += 2) {
+    const float4 a = __ldg(q + i + odd), b = __ldg(q + i + 1 - odd);
+    v[i] = make_float4(odd ? b.x : a.x, odd ? b.y : a.y, odd ? b.z : a.z, odd ? b.w : a.w);
+    v[i + 1] = make_float4(odd ? a.x : b.x, odd ? a.y : b.y, odd ? a.z : b.z, odd ? a.w : b.w);
   }
-  load_thin(u, U, MU, mb, V);
+  if constexpr (N % 2 == 1) v[N - 1] = __ldg(q + N - 1);
+}
+__device__ __forceinline__ void load_site(Spinor<float>& s, const float* p) {
+  float4 v[6];
+  load_words<6>(v, reinterpret_cast<const float4*>(p));
 #pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    Spinor<R> xs;
-    load_spinor(xs, xin + r * rs + mb * 24);
-    C<R> h[2][3], uh[2][3];
-    project<MU, !DAG>(xs, h);
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        uh[s][a] = C<R>{0, 0};
-#pragma unroll
-        for (int b = 0; b < 3; ++b) cfma_cj(uh[s][a], u[b][a], h[s][b]);
-      }
-    reconstruct<MU, !DAG>(acc[r], uh);
+  for (int i = 0; i < 6; ++i) {
+    s.v[2 * i / 3][2 * i % 3] = C<float>{v[i].x, v[i].y};
+    s.v[(2 * i + 1) / 3][(2 * i + 1) % 3] = C<float>{v[i].z, v[i].w};
   }
 }
+__device__ __forceinline__ void load_site(Spinor<double>& s, const double* p) { load_spinor(s, p); }
+// the six components of chirality h
+__device__ __forceinline__ void load_chirality(C<float> (&o)[6], const float* p, int h) {
+  float4 v[3];
+  load_words<3>(v, reinterpret_cast<const float4*>(p) + 3 * h);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    o[2 * i] = C<float>{v[i].x, v[i].y};
+    o[2 * i + 1] = C<float>{v[i].z, v[i].w};
+  }
+}
+__device__ __forceinline__ void load_chirality(C<double> (&o)[6], const double* p, int h) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) o[i] = ld2(reinterpret_cast<const double2*>(p) + 6 * h + i);
+}
 
-template <typename R, typename LS, int NR, bool DAG, bool CLOV>
-__global__ void __launch_bounds__(128, sizeof(R) == 8 ? 1 : (NR == 2 ? 4 : 5)) wil_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, int rhs0,
+// forward: -1/2 (1 - gamma_mu) U_mu(n) x(n+mu); backward: -1/2 (1 + gamma_mu) U_mu(n-mu)^+ x(n-mu)
+// (dagger swaps the two projectors).
+template <int MU, typename R, typename LS, bool DAG>
+__device__ __forceinline__ void wil_dir(Spinor<R>& acc, const R* __restrict__ xin, const LS* __restrict__ U, int64_t V, int64_t n,
+                                        const Nb<R>& nb) {
+  const int64_t mf = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][2];
+  const int64_t mb = nb.o[0][1] + nb.o[1][1] + nb.o[2][1] + nb.o[3][1] - nb.o[MU][1] + nb.o[MU][0];
+  C<R> u[3][3], h[2][3], uh[2][3];
+  Spinor<R> xs;
+  load_thin(u, U, MU, n, V);
+  load_site(xs, xin + mf * 24);
+  project<MU, DAG>(xs, h);
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      uh[s][a] = C<R>{0, 0};
+#pragma unroll
+      for (int b = 0; b < 3; ++b) cfma(uh[s][a], u[a][b], h[s][b]);
+    }
+  reconstruct<MU, DAG>(acc, uh);
+  load_thin(u, U, MU, mb, V);
+  load_site(xs, xin + mb * 24);
+  project<MU, !DAG>(xs, h);
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      uh[s][a] = C<R>{0, 0};
+#pragma unroll
+      for (int b = 0; b < 3; ++b) cfma_cj(uh[s][a], u[b][a], h[s][b]);
+    }
+  reconstruct<MU, !DAG>(acc, uh);
+}
+
+// RB right-hand sides per block of 128 threads, one per thread
+template <typename R, typename LS, int RB, bool DAG, bool CLOV>
+__global__ void __launch_bounds__(128, sizeof(R) == 8 ? 1 : 3) wil_kernel(Geom g, R* __restrict__ y, const R* __restrict__ x, int rhs0,
                                                   const LS* __restrict__ U, const R* __restrict__ cl, R diag) {
-  const int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  constexpr int SB = 128 / RB;
+  const int64_t n = blockIdx.x * (int64_t)SB + threadIdx.x % SB;
   if (n >= g.V) return;
-  const int64_t rs = g.V * 24, rhs_off = (rhs0 + (int64_t)blockIdx.y * NR) * rs;
+  const int64_t rhs_off = (rhs0 + (int64_t)blockIdx.y * RB + threadIdx.x / SB) * g.V * 24;
   const R* xin = x + rhs_off;
   Nb<R> nb;
   neighbours(g, n, nb);
-  Spinor<R> acc[NR];
+  Spinor<R> acc;
+  load_site(acc, xin + n * 24);
 #pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    Spinor<R> xc;
-    load_spinor(xc, xin + r * rs + n * 24);
+  for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) acc[r].v[s][a] = diag * xc.v[s][a];
-  }
-  wil_dir<0, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
-  wil_dir<1, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
-  wil_dir<2, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
-  wil_dir<3, NR, R, LS, DAG>(acc, xin, rs, U, g.V, n, nb);
+    for (int a = 0; a < 3; ++a) acc.v[s][a] = diag * acc.v[s][a];
+  wil_dir<0, R, LS, DAG>(acc, xin, U, g.V, n, nb);
+  wil_dir<1, R, LS, DAG>(acc, xin, U, g.V, n, nb);
+  wil_dir<2, R, LS, DAG>(acc, xin, U, g.V, n, nb);
+  wil_dir<3, R, LS, DAG>(acc, xin, U, g.V, n, nb);
   if constexpr (CLOV) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       R c[36];
       load_clover(c, cl, g.V, n, h);
+      C<R> in[6], out[6];
+      load_chirality(in, xin + n * 24, h);
+      clover_block(out, c, in);
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const C<R>* xn = reinterpret_cast<const C<R>*>(xin + r * rs + n * 24) + 6 * h;
-        C<R> in[6], out[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) in[i] = xn[i];
-        clover_block(out, c, in);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) acc[r].v[2 * h + i / 3][i % 3] = acc[r].v[2 * h + i / 3][i % 3] + out[i];
-      }
+      for (int i = 0; i < 6; ++i) acc.v[2 * h + i / 3][i % 3] = acc.v[2 * h + i / 3][i % 3] + out[i];
     }
   }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) store_spinor(y + rhs_off + r * rs + n * 24, acc[r]);
+  store_spinor(y + rhs_off + n * 24, acc);
 }
 
-template <typename R, typename LS, int NR>
-void launch_wil_nr(const Geom& g, R* y, const R* x, int rhs0, int groups, const LS* U, const R* cl, R diag, int dagger,
+template <typename R, typename LS, int RB>
+void launch_wil_rb(const Geom& g, R* y, const R* x, int rhs0, int groups, const LS* U, const R* cl, R diag, int dagger,
                    cudaStream_t s) {
   const int th = 128;
-  const dim3 grid(blocks_for(g.V, th), groups);
+  const dim3 grid(blocks_for(g.V, th / RB), groups);
   if (dagger) {
-    if (cl) wil_kernel<R, LS, NR, true, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
-    else wil_kernel<R, LS, NR, true, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    if (cl) wil_kernel<R, LS, RB, true, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    else wil_kernel<R, LS, RB, true, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
   } else {
-    if (cl) wil_kernel<R, LS, NR, false, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
-    else wil_kernel<R, LS, NR, false, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    if (cl) wil_kernel<R, LS, RB, false, true><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
+    else wil_kernel<R, LS, RB, false, false><<<grid, th, 0, s>>>(g, y, x, rhs0, U, cl, diag);
   }
   note_launch();
 }
@@ -205,10 +229,10 @@ void launch_wil_nr(const Geom& g, R* y, const R* x, int rhs0, int groups, const 
 template <typename R, typename LS>
 int launch_wil_t(const Geom& g, R* y, const R* x, const LS* U, const R* cl, R diag, int nrhs, int dagger,
                  cudaStream_t s) {
-  constexpr int NR = sizeof(R) == 4 ? 2 : 1;
-  const int groups = nrhs / NR;
-  if (groups) launch_wil_nr<R, LS, NR>(g, y, x, 0, groups, U, cl, diag, dagger, s);
-  if (nrhs > groups * NR) launch_wil_nr<R, LS, 1>(g, y, x, groups * NR, nrhs - groups * NR, U, cl, diag, dagger, s);
+  constexpr int RB = sizeof(R) == 4 ? 2 : 1;
+  const int groups = nrhs / RB;
+  if (groups) launch_wil_rb<R, LS, RB>(g, y, x, 0, groups, U, cl, diag, dagger, s);
+  if (nrhs > groups * RB) launch_wil_rb<R, LS, 1>(g, y, x, groups * RB, nrhs - groups * RB, U, cl, diag, dagger, s);
   BRI_LAUNCH_CHECK("wil_kernel");
   return BRI_OK;
 }

@@ -58,6 +58,17 @@ def test_bri_apply_every_path(dims, nrhs, dagger):
         assert relerr(lat.bri_apply(x32, -1.0, dagger=dagger, bf16_links=bf16).cpu().numpy(), want) < bound
 
 
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((5, 4, 6, 3), 3), ((7, 5, 6, 5), 2), ((4, 4, 4, 5), 5)])
+@pytest.mark.parametrize("dagger", [False, True])
+def test_wils_apply_blocks(dims, nrhs, dagger):
+    """The FP32 Wilson kernel's blocks of 64 sites x 2 right-hand sides and 128 x 1 (the odd one), full
+    (320 sites) and with a partial last block: 1e-5 of the largest element."""
+    x = sf.gaussian_source(dims, nrhs, 1036)
+    op = dirac.DiracOperator(sf.gauge_field(dims, 31), "wil", m0=-1.0, c_sw=1.0, antiperiodic_t=True)
+    y = _lattice(dims, anti=True).wils_apply(torch.from_numpy(x).to(torch.complex64).cuda(), -1.0, dagger=dagger)
+    assert relerr(y.cpu().numpy(), op.apply_dagger(x) if dagger else op.apply(x)) < 1e-5
+
+
 @pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((3, 2, 5, 2), 3), (LARGE, 2), (LARGE, 46)])
 @pytest.mark.parametrize("dagger", [False, True])
 def test_double_word_forms(dims, nrhs, dagger):
