@@ -828,6 +828,7 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
   BRI_CUDA(cudaMemcpyAsync(bsig.p, hsig.data(), sizeof(double) * nsys, cudaMemcpyHostToDevice, st));
   auto pack = [&](float4* dst) { return bri_f32_pack(V, b, nsys, dst, st); };
   const MsState* S = nullptr;
+  double counted = 0.0;
   auto apply = [&](int dagger, const float4* X, float4* Y, const float4* P, int na) -> int {
     const PackedDot pd{P, bsig.as<double>(), bsd.as<double>()};
     const float* cl = c->have_clover ? c->C32 : nullptr;
@@ -847,11 +848,15 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
     });
     note_launch();
     BRI_LAUNCH_CHECK("kp_stencil");
+    counted += (double)V * na;
     return prof_end(c, st, ev, 0, prec, (double)V * na);
   };
   const bool graphs = graphs_enabled() && !c->prof_on && st != nullptr;
+  int64_t all_iters = 0;
   rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), blocks, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
-                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out, &S);
+                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out, &S, &all_iters);
+  // the tracing counts the systems that ran, not those a launch was sized for
+  if (c->prof_on && !c->prof_pending.empty()) c->prof_pending.back().units += 2.0 * V * all_iters - counted;
   if (rc < 0 || x64) return rc;
   const int q = bri_f32_unpack(V, bx.p, nsys, x, st);
   return q ? q : rc;

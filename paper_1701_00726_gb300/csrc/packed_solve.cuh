@@ -1,8 +1,8 @@
 // Multi-shift CG on packed FP32 vectors (included by mscg.cu): one or several
 // lattices' systems, each a packed vector of one right-hand side (bri_pair.cuh;
 // as pairs the two stencils of an iteration took 381 + 363 us for 4 systems of
-// 16^3 x 32 where single ones take 349 + 351).  Base direction p_0, t = D p_0, q = (A + sigma) p_0 and the residuals live in the stencil's layout;
-// per iteration
+// 16^3 x 32 where single ones take 349 + 351).  Base direction p_0, t = D p_0,
+// q = (A + sigma) p_0 and the residuals live in the stencil's layout; per iteration
 //   t = D p, q = D^dagger t + sigma p with the partials of <p, q>,   (stencil)
 //   alpha; r_{j+1} = r_j - alpha q_j with the partials of ||r||^2;   (3 vectors)
 //   beta; p = r + beta p, and for a single shift x += alpha p first. (3 or 5)
@@ -261,11 +261,13 @@ struct PackedProblem {
 // sigma P with partials [na][blocks(na)] in sdpart, for the first na systems.
 // Several shifts: solutions in x64 (zeroed here).  One shift: packed in xp.
 // whole: all iterations in one WHILE-node graph (no host polling), else host
-// polling every kRing iterations and a shrinking prefix of systems.
+// polling every kRing iterations and a shrinking prefix of systems.  all_iters: the
+// systems' iterations in all.
 template <typename Pack, typename Apply, typename Blocks>
 int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& apply, double* sdpart, Blocks&& blocks,
                  double2* x64, size_t x64_bytes, float4* xp, bool whole, bool graphs, int* hdone,
-                 int* iters_out, Counters* cnt, double* lam_out, const MsState** state_out = nullptr) {
+                 int* iters_out, Counters* cnt, double* lam_out, const MsState** state_out = nullptr,
+                 int64_t* all_iters = nullptr) {
   const int nsys = pb.nsys, nshift = pb.nshift;
   const bool defer = x64 != nullptr;
   const size_t vb = sizeof(float4) * (size_t)pb.words;
@@ -453,6 +455,10 @@ int packed_solve(cudaStream_t st, const PackedProblem& pb, Pack&& pack, Apply&& 
     lm = std::max(lm, h.lam_max - h.sig_base);
   }
   *iters_out = maxit;
+  if (all_iters) {
+    *all_iters = 0;
+    for (const MsState& h : hs) *all_iters += h.iters;
+  }
   if (lam_out) *lam_out = lm;
   if (err) {
     set_error("multi-shift CG: non-finite or non-positive curvature in a reduction");
