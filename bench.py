@@ -549,7 +549,7 @@ def main():
     t_alu = alg_flops / (fp32_peak * 1e12)
     traffic = stencil_traffic()
     lt = "bf16x2" if prec == PREC_F32_BF16 else "float2"
-    common = {"kernel": f"bri_pair_kernel<4|2,{lt}> (two or one rhs per thread)",
+    common = {"kernel": f"kp_stencil, bri_pair_kernel ({lt} links, packed spinors)",
               "launches": nlaunch, "avg_launch_ms": round(kms / max(nlaunch, 1), 4),
               "avg_rhs_per_launch": round(units / max(nlaunch, 1) / vol, 3),
               "alg_bytes_per_launch": int(alg_bytes / max(nlaunch, 1)),
