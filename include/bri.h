@@ -113,6 +113,9 @@ int bri_set_kernel(bri_ctx* ctx, int kernel);
  * used by wils_apply and, when c_sw != 0, the clover term
  * -(c_sw/2) sum_{mu<nu} sigma_{mu nu} F_{mu nu} with F the traceless
  * anti-Hermitian part of the four-leaf clover divided by 8i.
+ * Without memory for a rebuild (BRI_ERR_OOM) the context keeps its links and
+ * clover; after any other failure operators answer BRI_ERR_NOLINKS until a
+ * build succeeds.
  * U: device, [V][4][3][3] complex128, read once; may be freed afterwards. */
 int bri_build_links(bri_ctx* ctx, const double* U, double c_sw);
 

@@ -441,18 +441,14 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
     note_device_alloc();
     return BRI_OK;
   };
+  // Everything is allocated before the first write: without memory for a rebuild the
+  // links and clover of the last one stay as they were.
   int rc;
   if ((rc = alloc((void**)&c->W64, sizeof(double2) * 360 * V))) return rc;
   if ((rc = alloc((void**)&c->W32, kLinkBytes32 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->W16, kLinkBytes16 * kLinkBlock * 40 * link_blocks(V)))) return rc;
   if ((rc = alloc((void**)&c->U64, sizeof(double2) * 36 * V))) return rc;
   if ((rc = alloc((void**)&c->U32, kLinkBytes32 * kLinkBlock * 4 * link_blocks(V)))) return rc;
-  const int th = 128;
-  thin_links_kernel<<<blocks_for(V, th), th, 0, st>>>(g, (const double2*)U, c->U64, c->U32,
-                                                       (c->flags & BRI_ANTIPERIODIC_T) ? 1 : 0); note_launch();
-  c->have_clover = false;
-  c->dw_valid = false;
-  c->c_sw = c_sw;
   // the two paths of every stored two-hop offset, kept for the clover leaves
   LevelList two = stored_level(2);
   double2* AB = nullptr;
@@ -464,6 +460,14 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
     if (e != cudaSuccess) return cuda_fail(e, "bri_build_links: cudaMallocAsync");
     note_device_alloc();
   }
+  // no operator runs on what a failure from here on leaves behind
+  c->have_links = false;
+  c->have_clover = false;
+  c->dw_valid = false;
+  c->c_sw = c_sw;
+  const int th = 128;
+  thin_links_kernel<<<blocks_for(V, th), th, 0, st>>>(g, (const double2*)U, c->U64, c->U32,
+                                                       (c->flags & BRI_ANTIPERIODIC_T) ? 1 : 0); note_launch();
   stored1_kernel<<<dim3(blocks_for(V, th), 4), th, 0, st>>>(g, c->U64, c->W64, c->W32, c->W16); note_launch();
   for (int k = 2; k <= 4; ++k) {
     const LevelList lst = stored_level(k);
