@@ -131,8 +131,11 @@ int bri_get_links(bri_ctx* ctx, double* W);
  * arithmetic (relative error ~1e-15, the FP64 operator's accuracy class) and
  * the call allocates two double-word work vectors of nrhs right-hand sides
  * (stream-ordered) plus, on first use after bri_build_links, the double-word
- * link and clover copies (5760 + 576 bytes per site).  x and y must not
- * alias. */
+ * link and clover copies (5760 + 576 bytes per site).  FP32 and BF16 calls on
+ * more than 8192 sites x right-hand sides take a stream-ordered copy of at
+ * most 16 right-hand sides of x (96 bytes per site each); where there is no
+ * memory for it, and while the stream is being captured into a graph, they run
+ * without one (same result, up to a fifth slower).  x and y must not alias. */
 int bri_apply(bri_ctx* ctx, void* y, const void* x, int nrhs, double m0, int dagger, int prec);
 
 /* y = D_wil x or D_wil^dagger x (Eq. def_wils): 9-point stencil over the thin

@@ -40,14 +40,23 @@ int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s)
   return BRI_OK;
 }
 
+// Under capture an allocation would become a node of the caller's graph, which then
+// could be no child graph, no body of a conditional node and be instantiated only once.
+static bool may_allocate(cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) return cap == cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
 // Spinors in their own layout in and out.  The packed copy of x lives in a
 // stream-ordered allocation of at most kChunk right-hand sides; where there is
-// no memory for it the split kernel, which needs none, takes over.
+// no memory for it, or under capture, the kernels read x as it is.
 template <typename LS>
 int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const float* cl, float diag, int nrhs, int dagger,
                    cudaStream_t s, const ShiftDot<float>* sd, int* sd_blocks) {
   constexpr int kChunk = 16;
-  if (!sd && bri_f32_packed(g.V, nrhs)) {
+  if (!sd && bri_f32_packed(g.V, nrhs) && may_allocate(s)) {
     configure_pool_once();
     void* X = nullptr;
     if (cudaMallocAsync(&X, sizeof(float4) * packed_words(g.V, 6) * std::min(nrhs, kChunk), s) == cudaSuccess) {
@@ -71,6 +80,11 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
       return BRI_OK;
     }
     cudaGetLastError();
+  }
+  if (!sd && bri_f32_packed(g.V, nrhs)) {
+    launch_singles<LS, true>(g, y, (const float4*)x, W, cl, diag, dagger, 0, nrhs, s);
+    BRI_LAUNCH_CHECK("bri_pair_kernel");
+    return BRI_OK;
   }
   return launch_split<float, LS>(g, y, x, W, cl, diag, nrhs, dagger, s, sd, sd_blocks);
 }

@@ -72,13 +72,60 @@ template <int ROWS> __device__ __forceinline__ int packed_at(int m) {
   return (m / kPackBlock) * (ROWS * kPackBlock) + m % kPackBlock;
 }
 
+// The words of a spinor in one of two layouts: rows of a block of sites as above, or
+// (OWN, single right-hand sides) the caller's 96 bytes of a site, whose spins meet in
+// registers.  OWN needs no packed copy of x: 16^3 x 32, 4 and 12 rhs 422 and 1205 us
+// against 382 and 1023 with one (packing included), 24^3 x 48, 1 rhs 621 against 565,
+// 16^4, 1 rhs 68 against 70; its 16-byte words in order 510 and 1472 us, 3 blocks per SM 446
+// and 1291; the split kernel (bri_split.cuh), which needs no copy either, 713 and 2056.
+template <int R, bool OWN> struct SpinorWords {
+  CP v[R][3];
+  // Neighbouring lanes are 96 bytes apart: the lanes with bit 2 set read each pair of
+  // words the other way round, so that no two of eight meet in a bank.
+  __device__ __forceinline__ void load(const float4* __restrict__ x) {
+    if constexpr (OWN) {
+      static_assert(R == 2, "single right-hand sides");
+      const int odd = (threadIdx.x >> 2) & 1;
+      float4 u[6];
+#pragma unroll
+      for (int i = 0; i < 6; i += 2) {
+        const float4 a = __ldg(x + i + odd), b = __ldg(x + i + 1 - odd);
+        u[i] = make_float4(odd ? b.x : a.x, odd ? b.y : a.y, odd ? b.z : a.z, odd ? b.w : a.w);
+        u[i + 1] = make_float4(odd ? a.x : b.x, odd ? a.y : b.y, odd ? a.z : b.z, odd ? a.w : b.w);
+      }
+#pragma unroll
+      for (int q = 0; q < R; ++q) join(u[3 * q], u[3 * q + 1], u[3 * q + 2], v[q]);
+    }
+  }
+  __device__ __forceinline__ static void join(const float4& a, const float4& b, const float4& c, CP (&o)[3]) {
+    o[0] = CP{make_float2(a.x, b.z), make_float2(a.y, b.w)};
+    o[1] = CP{make_float2(a.z, c.x), make_float2(a.w, c.y)};
+    o[2] = CP{make_float2(b.x, c.z), make_float2(b.y, c.w)};
+  }
+  __device__ __forceinline__ static void load_half(const float4* __restrict__ x, int q, CP (&o)[3]) {
+    if constexpr (OWN) {
+      join(__ldg(x + 3 * q), __ldg(x + 3 * q + 1), __ldg(x + 3 * q + 2), o);
+    } else {
+#pragma unroll
+      for (int aa = 0; aa < 3; ++aa) o[aa] = cp_of(__ldg(x + (q * 3 + aa) * kPackBlock));
+    }
+  }
+  __device__ __forceinline__ CP word(const float4* __restrict__ x, int q, int b) const {
+    if constexpr (OWN) return v[q][b];
+    else return cp_of(__ldg(x + (q * 3 + b) * kPackBlock));
+  }
+  __device__ __forceinline__ static int at(int m) { return OWN ? m * 6 : packed_at<3 * R>(m); }
+};
+
 // P = w x (rows of x: R spinor rows, component q at row 3 q + colour)
-template <int R> __device__ __forceinline__ void pr_fwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+template <int R, bool OWN> __device__ __forceinline__ void pr_fwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+  SpinorWords<R, OWN> xs;
+  xs.load(x);
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
     CP v[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = cp_of(__ldg(x + (q * 3 + b) * kPackBlock));
+    for (int q = 0; q < R; ++q) v[q] = xs.word(x, q, b);
 #pragma unroll
     for (int q = 0; q < R; ++q) {
 #pragma unroll
@@ -97,12 +144,14 @@ template <int R> __device__ __forceinline__ void pr_fwd(CP (&P)[R][3], const flo
   }
 }
 // P = w^dagger x - P
-template <int R> __device__ __forceinline__ void pr_bwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+template <int R, bool OWN> __device__ __forceinline__ void pr_bwd(CP (&P)[R][3], const float4* __restrict__ x, const C<float> (&w)[3][3]) {
+  SpinorWords<R, OWN> xs;
+  xs.load(x);
 #pragma unroll
   for (int b = 0; b < 3; ++b) {
     CP v[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) v[q] = cp_of(__ldg(x + (q * 3 + b) * kPackBlock));
+    for (int q = 0; q < R; ++q) v[q] = xs.word(x, q, b);
 #pragma unroll
     for (int q = 0; q < R; ++q) {
 #pragma unroll
@@ -178,7 +227,7 @@ __device__ __forceinline__ void pr_gamma(CP (&acc)[2][3], const CP (&v)[2][3], f
 
 // Sum over the hops at site n into acc (all 80, or those of every KS-th offset
 // pair from i0 on); x = packed vector (R = 4: a pair of right-hand sides, R = 2: one).
-template <int R, typename LS, int KS>
+template <int R, typename LS, int KS, bool OWN>
 __device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, const float4* __restrict__ x,
                                         const LS* __restrict__ W, const PairHops<float>& H, int i0) {
   const int V = (int)g.V;
@@ -219,13 +268,13 @@ __device__ __forceinline__ void pr_hops(CP (&acc)[R][3], const Geom& g, int n, c
   for (int j = i0; j < 40; j += KS) {
     const int jn = KS == 1 ? (j < 39 ? j + 1 : 39) : (j < 40 - KS ? j + KS : j);
     const float a = H.a[j];
-    const int op = packed_at<3 * R>(mp), om = packed_at<3 * R>(mm);
+    const int op = SpinorWords<R, OWN>::at(mp), om = SpinorWords<R, OWN>::at(mm);
     CP P[R][3];
-    pr_fwd<R>(P, x + op, w);
+    pr_fwd<R, OWN>(P, x + op, w);
     sites(jn, mp, mm);
     load_stored_link<float, LS>(w, W, H.j[jn], n, V);
     pr_axpy<R>(acc, P, 2.f * a);
-    pr_bwd<R>(P, x + om, wm);
+    pr_bwd<R, OWN>(P, x + om, wm);
     load_stored_link<float, LS>(wm, W, H.j[jn], mm, V);
     pr_axpy<R>(acc, P, a);
     pr_gamma(acc, P, H.c[j][0], H.c[j][1], H.c[j][2], H.c[j][3]);
@@ -298,7 +347,7 @@ template <int KS> __device__ __forceinline__ int pr_group() {
 // packed vectors, y0: its first right-hand side in the spinors' own layout (OUT =
 // 0 writes y0, OUT = 1 yp).  EPI (R = 2, OUT = 1): the epilogue of system s, p at
 // word po of sd.p.
-template <int R, typename LS, int OUT, bool EPI, int KS>
+template <int R, typename LS, int OUT, bool EPI, int KS, bool OWN = false>
 __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restrict__ y0, float4* __restrict__ yp,
                                          const float4* __restrict__ x, const LS* __restrict__ W,
                                          const float* __restrict__ cl, float diag, const PairHops<float>& H, const PackedDot& sd,
@@ -312,7 +361,7 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
   if (R == 4 && !valid) return;  // else every thread takes part in the block's exchanges
   const int n = valid ? n0 : 0, grp = pr_group<KS>();
   CP acc[R][3];
-  pr_hops<R, LS, KS>(acc, g, n, x, W, H, grp);
+  pr_hops<R, LS, KS, OWN>(acc, g, n, x, W, H, grp);
   if constexpr (KS > 1) {
     __shared__ float4 red[KS][6][SB];
     const int l = threadIdx.x % SB;
@@ -334,7 +383,7 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
       }
     }
   }
-  const float4* xo = x + packed_at<3 * R>(n);
+  const float4* xo = x + SpinorWords<R, OWN>::at(n);
   if constexpr (R == 4) {
     const int64_t rs = g.V * 24;
 #pragma unroll
@@ -371,9 +420,11 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
     for (int h = 0; h < 2; ++h) {
       if (KS > 1 && h != grp) continue;
       C<float> in[6], out[6];
+      CP xh[3];
+      SpinorWords<R, OWN>::load_half(xo, h, xh);
 #pragma unroll
       for (int aa = 0; aa < 3; ++aa) {
-        const CP own = cp_of(__ldg(xo + (h * 3 + aa) * kPackBlock));
+        const CP own = xh[aa];
         cp_add(acc[h][aa], own, diag);
         in[aa] = C<float>{own.re.x, own.im.x};
         in[3 + aa] = C<float>{own.re.y, own.im.y};
@@ -432,14 +483,14 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
 }
 
 // y = D x on `groups` packed groups of one lattice; the first one holds right-hand
-// side rhs0 (and rhs0 + 1).
-template <int R, typename LS, int KS>
+// side rhs0 (and rhs0 + 1).  OWN: x in its own layout, a group one right-hand side.
+template <int R, typename LS, int KS, bool OWN = false>
 __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
     bri_pair_kernel(Geom g, float* __restrict__ y, const float4* __restrict__ x, const LS* __restrict__ W,
                     const float* __restrict__ cl, float diag, int rhs0, int gfirst, const __grid_constant__ PairHops<float> H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  pr_block<R, LS, 0, false, KS>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
-                                x + (int64_t)grp * packed_words(g.V, 3 * R), W, cl, diag, H,
+  pr_block<R, LS, 0, false, KS, OWN>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
+                                x + (int64_t)grp * (OWN ? g.V * 6 : packed_words(g.V, 3 * R)), W, cl, diag, H,
                                 PackedDot{nullptr, nullptr, nullptr}, 0, 0, 0);
 }
 
@@ -490,14 +541,14 @@ inline void launch_pairs(const Geom& g, float* y, const float4* X, const LS* W, 
   note_launch();
 }
 
-// y = D x for `n` single right-hand sides starting at rhs0.
-template <typename LS>
+// y = D x for `n` single right-hand sides starting at rhs0; OWN: X is x itself.
+template <typename LS, bool OWN = false>
 inline void launch_singles(const Geom& g, float* y, const float4* X, const LS* W, const float* cl, float diag, int dagger,
                            int rhs0, int n, cudaStream_t s) {
   const int ks = pack_groups(g.V * n);
   const StencilGrid sg = stencil_grid(blocks_for(g.V, pack_sites(ks)), n);
   with_groups(ks, [&](auto k) {
-    bri_pair_kernel<2, LS, decltype(k)::value><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops<float>(dagger));
+    bri_pair_kernel<2, LS, decltype(k)::value, OWN><<<sg.grid, 128, 0, s>>>(g, y, X, W, cl, diag, rhs0, sg.gfirst, pair_hops<float>(dagger));
   });
   note_launch();
 }

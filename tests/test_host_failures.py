@@ -88,3 +88,24 @@ def test_failed_rebuild_of_the_links(run, first, second):
     assert lib.bri_apply(h, y, x, 1, -1.0, 0, 1) == {NOLINKS} and lib.wils_apply(h, y, x, 1, -1.0, 0, 1) == {NOLINKS}
     assert lib.bri_build_links(h, u, {second}) == 0 and lib.bri_apply(h, y, x, 1, -1.0, 0, 1) == 0
     """)
+
+
+@pytest.mark.parametrize("nrhs,prec", [(1, 1), (3, 2), (40, 1)])
+def test_large_fp32_application_without_scratch(run, nrhs, prec):
+    """Under capture an application leaves kernels only in the caller's graph (an allocation node would bar it from child
+    graphs, conditional bodies and a second instantiation), and without memory for packed spinors it runs all the same:
+    one launch, nothing allocated."""
+    run(f"""
+    h, V = lattice(10, 9, 10, 11), 9900
+    u, x, y = device(V * 576), device(V * 96 * {nrhs}), device(V * 96 * {nrhs})
+    assert lib.bri_build_links(h, u, 0.0) == 0
+    for setting in ("capture", "memory"):
+        fake.fake_forget()
+        fake.fake_largest()
+        (fake.fake_capturing if setting == "capture" else fake.fake_memory_left)(1 if setting == "capture" else 0)
+        assert lib.bri_apply(h, y, x, {nrhs}, -1.0, 0, {prec}) == 0
+        assert fake.fake_largest() == 0
+        kernels = launched()
+        assert len(kernels) == 1 and "bri_pair_kernel" in kernels[0], kernels
+        fake.fake_capturing(0)
+    """)
