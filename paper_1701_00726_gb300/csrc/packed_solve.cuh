@@ -35,27 +35,17 @@ __global__ void __launch_bounds__(256) kp_norm(const PackedSys* __restrict__ gd,
   if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
 }
 
-// (h, l) += v^2 on two components: exact square and sum by TwoProduct and TwoSum
-// (bri_dw.cu), their errors collected in l.
-__device__ __forceinline__ void add_square(float2& h, float2& l, float2 v) {
-  const float2 p = __fmul2_rn(v, v);
-  const float2 e = __ffma2_rn(v, v, pr_neg(p));
-  const float2 s = __fadd2_rn(h, p);
-  const float2 bb = __fadd2_rn(s, pr_neg(h));
-  const float2 t = __fadd2_rn(__fadd2_rn(h, pr_neg(__fadd2_rn(s, pr_neg(bb)))), __fadd2_rn(p, pr_neg(bb)));
-  h = s;
-  l = __fadd2_rn(l, __fadd2_rn(t, e));
-}
-
 // rout = rin - alpha q, partials of ||rout||^2 (rin may be rout).  The squares of four words are summed in
-// double-word FP32 (48 bits), those sums in FP64: one FP64 addition per eight
-// squares instead of eight, which bound the kernel (102 -> 43 us on average in the
-// 16^3 x 32 solves; the random 2^-47 of a chunk vanish below 2^-53 in the sum).
+// three FP32 words (sum3.cuh, scaled by the residual's norm so far) and those sums in FP64.  FP64 squares bound
+// the kernel (102 us on average in the 16^3 x 32 solves against 43 with two FP32 words, which kept only 2^-47 and
+// FP32's range); the third word costs the whole solve 0.4 %.
 __global__ void __launch_bounds__(256) kp_update_r(const PackedSys* __restrict__ gd, const MsState* __restrict__ st,
                                                    const float4* __restrict__ q, const float4* rin, float4* rout, double* part) {
   const PackedSys g = gd[blockIdx.y];
   if (st[blockIdx.y].done) return;
   const float2 f = pr_bc(-(float)st[blockIdx.y].alpha);
+  const int k2 = unit_exponent(st[blockIdx.y].rr);
+  const float2 sc = pr_bc(exp2_float(k2));
   const int64_t nw = packed_words(g.V, 6), stride = (int64_t)gridDim.x * blockDim.x;
   const float4 *qv = q + g.poff, *ri = rin + g.poff;
   float4* ro = rout + g.poff;
@@ -68,20 +58,21 @@ __global__ void __launch_bounds__(256) kp_update_r(const PackedSys* __restrict__
         x[k] = __ldg(qv + i + k * stride);
         v[k] = ri[i + k * stride];
       }
-    float2 h = make_float2(0.f, 0.f), l = h;
+    Sum3 sum = sum3_zero();
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       if (i + k * stride < nw) {
         const float2 re = __ffma2_rn(f, make_float2(x[k].x, x[k].y), make_float2(v[k].x, v[k].y));
         const float2 im = __ffma2_rn(f, make_float2(x[k].z, x[k].w), make_float2(v[k].z, v[k].w));
         ro[i + k * stride] = make_float4(re.x, re.y, im.x, im.y);
-        add_square(h, l, re);
-        add_square(h, l, im);
+        const float2 u = __fmul2_rn(re, sc), v = __fmul2_rn(im, sc);
+        sum3_add(sum, u, u);
+        sum3_add(sum, v, v);
       }
-    a += ((double)h.x + (double)l.x) + ((double)h.y + (double)l.y);
+    a += sum3_total(sum);
   }
   const double t = block_sum(a);
-  if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+  if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t * exp2_square(k2);
 }
 
 // x += alpha p (XUP: single-shift solves, also in the iteration that converged),

@@ -2,7 +2,10 @@
 or against the common form, with the tolerances of the parity tests (FP32 1e-5 and BF16 links 1e-2 of the largest
 element, FP64 1e-12, mixed solves 1e-10).
 """
+import ctypes
 import functools
+import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -10,7 +13,7 @@ import torch
 
 import synthetic_fields as sf
 from oracle import dirac
-from paper_1701_00726_gb300 import Lattice
+from paper_1701_00726_gb300 import Lattice, build
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +62,51 @@ def test_captured_application(dims, nrhs, bf16, dagger):
         want = op.apply_dagger(xs) if dagger else op.apply(xs)
         assert relerr(y[some].cpu().numpy(), want) < (1e-2 if bf16 else 1e-5)
         assert relerr(y.cpu().numpy(), eager.cpu().numpy()) < 1e-6  # the same operands, a few roundings apart
+
+
+SUM3 = r"""
+#include "sum3.cuh"
+using namespace bri;
+__global__ void k(int n, const float2* x, const float2* y, double n2, double* out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, e = unit_exponent(n2);
+  const float2 f = make_float2(exp2_float(e), exp2_float(e));
+  Sum3 s = sum3_zero();
+  for (int i = 0; i < n; ++i) sum3_add(s, __fmul2_rn(x[t * n + i], f), __fmul2_rn(y[t * n + i], f));
+  out[t] = sum3_total(s) * exp2_square(e);
+}
+extern "C" int run(int threads, int n, const float2* x, const float2* y, double n2, double* out) {
+  k<<<threads / 64, 64>>>(n, x, y, n2, out);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def sum3(tmp_path_factory):
+    d = tmp_path_factory.mktemp("sum3")
+    (d / "t.cu").write_text(SUM3)
+    subprocess.run([build.nvcc(), *build.ARCH, "-O3", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", build.CSRC, "-o",
+                    str(d / "t.so"), str(d / "t.cu")], check=True)
+    return ctypes.CDLL(str(d / "t.so"))
+
+
+@pytest.mark.parametrize("n", [1, 8, 24])
+@pytest.mark.parametrize("scale", [-120, -65, 0, 62, 110])
+@pytest.mark.parametrize("square", [True, False])
+def test_fp32_sums_of_products_to_fp64_accuracy(sum3, n, scale, square):
+    """The reductions of the packed solver, at element scales whose FP32 squares under- and overflow: two FP64 roundings
+    of the absolute sum (2^-52; the rounding of the third word adds 2^-54 for 24 products), where FP64 multiply-adds
+    may err by one rounding per product and a double-word sum by 2^-48 for each."""
+    rng = np.random.default_rng(31 + n)
+    threads = 128
+    x = (rng.standard_normal((threads, n, 2)) * 10.0 ** rng.uniform(-5, 0, (threads, n, 2))).astype(np.float32)
+    y = x if square else rng.standard_normal(x.shape).astype(np.float32)
+    f = 2.0 ** scale
+    xt, yt = (torch.from_numpy((v.astype(np.float64) * f).astype(np.float32)).cuda() for v in (x, y))
+    out = torch.zeros(threads, dtype=torch.float64, device="cuda")
+    assert sum3.run(threads, n, *(ctypes.c_void_p(v.data_ptr()) for v in (xt, yt)), ctypes.c_double(f * f),
+                    ctypes.c_void_p(out.data_ptr())) == 0
+    xs, ys = xt.cpu().tolist(), yt.cpu().tolist()  # (at 2^-120 the small ones were rounded to FP32 subnormals)
+    for t, got in enumerate(out.cpu().tolist()):
+        prods = [Fraction(a) * Fraction(b) for i in range(n) for a, b in zip(xs[t][i], ys[t][i])]
+        assert abs(Fraction(got) - sum(prods)) <= Fraction(5, 4) * Fraction(2) ** -52 * sum(map(abs, prods))
