@@ -38,6 +38,7 @@
 #pragma once
 
 #include "hops.cuh"
+#include "sum3.cuh"
 
 namespace bri {
 
@@ -326,7 +327,9 @@ __device__ __forceinline__ void pr_clover(CP (&o)[6], const float* __restrict__ 
 }
 
 // The solver's epilogue on packed vectors: y = D x + sig_s p_s and the site
-// block's partial of Re<p_s, y> in part[s * blocks + block].
+// block's partial of Re<p_s, y> in part[s * blocks + block].  A thread's products are
+// summed in FP32 (EPI = 1, one lattice) or to FP64 accuracy and range (EPI = 2,
+// batched lattices: sum3.cuh, p and y scaled by 2^k2).
 struct PackedDot {
   const float4* p;    // packed base directions
   const double* sig;  // per system
@@ -345,13 +348,13 @@ template <int KS> __device__ __forceinline__ int pr_group() {
 // over KS thread groups: each takes every KS-th pair, their sums meet in shared
 // memory and the groups 0 and 1 finish one chirality each.  x, yp: the group's
 // packed vectors, y0: its first right-hand side in the spinors' own layout (OUT =
-// 0 writes y0, OUT = 1 yp).  EPI (R = 2, OUT = 1): the epilogue of system s, p at
+// 0 writes y0, OUT = 1 yp).  EPI > 0 (R = 2, OUT = 1): the epilogue of system s, p at
 // word po of sd.p.
-template <int R, typename LS, int OUT, bool EPI, int KS, bool OWN = false>
+template <int R, typename LS, int OUT, int EPI, int KS, bool OWN = false>
 __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restrict__ y0, float4* __restrict__ yp,
                                          const float4* __restrict__ x, const LS* __restrict__ W,
                                          const float* __restrict__ cl, float diag, const PairHops<float>& H, const PackedDot& sd,
-                                         int64_t po, int s, int nb) {
+                                         int64_t po, int s, int nb, int k2 = 0) {
   static_assert(R == 2 || (OUT == 0 && KS == 1), "pairs: spinors' own layout out, one thread per site");
   static_assert(!EPI || OUT == 1, "the epilogue writes packed vectors");
   constexpr int SB = 128 / KS;
@@ -416,6 +419,8 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
     __shared__ float4 stage[STAGE ? 128 * 7 : 1];
     const float sig = EPI ? (float)sd.sig[s] : 0.f;
     float dA = 0.f, dB = 0.f;
+    Sum3 sum = sum3_zero();
+    const float2 sc = pr_bc(exp2_float(k2));
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (KS > 1 && h != grp) continue;
@@ -448,10 +453,15 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
             const CP pv = cp_of(__ldg(sd.p + po + at));
             v.re = pr_fma(pv.re, pr_bc(sig), v.re);
             v.im = pr_fma(pv.im, pr_bc(sig), v.im);
-            dA = fmaf(pv.re.x, v.re.x, dA);
-            dB = fmaf(pv.re.y, v.re.y, dB);
-            dA = fmaf(pv.im.x, v.im.x, dA);
-            dB = fmaf(pv.im.y, v.im.y, dB);
+            if constexpr (EPI == 1) {
+              dA = fmaf(pv.re.x, v.re.x, dA);
+              dB = fmaf(pv.re.y, v.re.y, dB);
+              dA = fmaf(pv.im.x, v.im.x, dA);
+              dB = fmaf(pv.im.y, v.im.y, dB);
+            } else {
+              sum3_add(sum, pr_mul(pv.re, sc), pr_mul(v.re, sc));
+              sum3_add(sum, pr_mul(pv.im, sc), pr_mul(v.im, sc));
+            }
           }
           if (valid) yp[at] = cp_word(v);
         }
@@ -476,8 +486,9 @@ __device__ __forceinline__ void pr_block(const Geom& g, int blk, float* __restri
       }
     }
     if constexpr (EPI) {
-      const double t = pr_block_total(valid ? (double)dA + (double)dB : 0.0);
-      if (threadIdx.x == 0) sd.part[(int64_t)s * nb + blk] = t;
+      const double d = EPI == 1 ? (double)dA + (double)dB : sum3_total(sum);
+      const double t = pr_block_total(valid ? d : 0.0);
+      if (threadIdx.x == 0) sd.part[(int64_t)s * nb + blk] = EPI == 1 ? t : t * exp2_square(k2);
     }
   }
 }
@@ -489,7 +500,7 @@ __global__ void __launch_bounds__(128, R == 4 ? 3 : 4)
     bri_pair_kernel(Geom g, float* __restrict__ y, const float4* __restrict__ x, const LS* __restrict__ W,
                     const float* __restrict__ cl, float diag, int rhs0, int gfirst, const __grid_constant__ PairHops<float> H) {
   const int grp = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
-  pr_block<R, LS, 0, false, KS, OWN>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
+  pr_block<R, LS, 0, 0, KS, OWN>(g, blk, y + (int64_t)(rhs0 + grp * (R / 2)) * g.V * 24, nullptr,
                                 x + (int64_t)grp * (OWN ? g.V * 6 : packed_words(g.V, 3 * R)), W, cl, diag, H,
                                 PackedDot{nullptr, nullptr, nullptr}, 0, 0, 0);
 }

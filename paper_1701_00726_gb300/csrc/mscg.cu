@@ -30,7 +30,6 @@
 #include "cplx.cuh"
 #include "bri_pair.cuh"
 #include "bri_split.cuh"
-#include "sum3.cuh"
 
 #include <algorithm>
 #include <chrono>

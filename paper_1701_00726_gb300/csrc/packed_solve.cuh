@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(128, 4)
   const int s = gfirst ? blockIdx.x : blockIdx.y, blk = gfirst ? blockIdx.y : blockIdx.x;
   if (st[s].done) return;
   const int64_t o = s * packed_words(g.V, 6);
-  pr_block<2, LS, 1, EPI, KS>(g, blk, nullptr, Y + o, X + o, W, cl, diag, H, sd, o, s, gfirst ? gridDim.y : gridDim.x);
+  pr_block<2, LS, 1, EPI ? 1 : 0, KS>(g, blk, nullptr, Y + o, X + o, W, cl, diag, H, sd, o, s, gfirst ? gridDim.y : gridDim.x);
 }
 
 // Stencil on the work list of several lattices: item (system, block of 128 / KS
@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(128, 4)
   const PackedSys gr = gd[it.x];
   if (st[it.x].done) return;
   const BatchLat& L = T.lat[gr.lat];
-  pr_block<2, LS, 1, EPI, KS>(L.g, it.y, nullptr, Y + gr.poff, X + gr.poff, (const LS*)L.W, (const float*)L.C, (float)L.diag, H,
-                           sd, gr.poff, it.x, nb);
+  pr_block<2, LS, 1, EPI ? 2 : 0, KS>(L.g, it.y, nullptr, Y + gr.poff, X + gr.poff, (const LS*)L.W, (const float*)L.C, (float)L.diag,
+                                     H, sd, gr.poff, it.x, nb, EPI ? unit_exponent(st[it.x].rr) : 0);
 }
 
 // A problem on packed vectors: `words` 16-byte words per packed vector.

@@ -7,6 +7,9 @@
 // eight, and converting the words to FP64 adds two roundings of 2^-53, where FP64
 // multiply-adds take one per product.  Two sums run side by side (f32x2).
 //
+// Measured: a batch of 8^3 x 16 and three more lattices 172.6 -> 173.1 ms with this in
+// the residual norms and in <p, q>.
+//
 // The products must neither overflow nor, where they count, lose bits below 2^-126:
 // the operands are first scaled by a power of two (unit_exponent), exactly.
 #pragma once

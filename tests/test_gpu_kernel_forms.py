@@ -13,7 +13,7 @@ import torch
 
 import synthetic_fields as sf
 from oracle import dirac
-from paper_1701_00726_gb300 import Lattice, build
+from paper_1701_00726_gb300 import PREC_F32, Lattice, build, overlap_apply_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -110,3 +110,18 @@ def test_fp32_sums_of_products_to_fp64_accuracy(sum3, n, scale, square):
     for t, got in enumerate(out.cpu().tolist()):
         prods = [Fraction(a) * Fraction(b) for i in range(n) for a, b in zip(xs[t][i], ys[t][i])]
         assert abs(Fraction(got) - sum(prods)) <= Fraction(5, 4) * Fraction(2) ** -52 * sum(map(abs, prods))
+
+
+@pytest.mark.parametrize("scale", [-65, 66])
+def test_batch_of_small_and_large_sources(scale):
+    """Sources whose elements' squares leave FP32's range: the batched solve takes its inner products to FP64 range, so
+    that a source scaled by a power of two gives the scaled result bit by bit (at 1e-3 the first phase is all there is;
+    the FP32 corrections' own inner products are in FP32)."""
+    dims = [LARGE, (6, 5, 4, 3)]
+    lats = [_lattice(d) for d in dims]
+    xs = [torch.from_numpy(sf.gaussian_source(d, r, 1042)).cuda() for d, r in zip(dims, (2, 3))]
+    want, _ = overlap_apply_batch(lats, xs, n=4, tol=1e-3, prec=PREC_F32)
+    got, st = overlap_apply_batch(lats, [x * 2.0 ** scale for x in xs], n=4, tol=1e-3, prec=PREC_F32)
+    assert all(s["refinements"] == 0 for s in st)
+    for g, w in zip(got, want):
+        assert torch.equal(g, w * 2.0 ** scale)
