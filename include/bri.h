@@ -34,6 +34,13 @@
  * stream; calls return once the work is enqueued unless documented otherwise
  * (solvers synchronise the stream to test convergence).
  *
+ * Device memory between calls: besides what the contexts own, the library
+ * keeps per device up to 1 GiB of stream-ordered scratch of its operator calls
+ * and link constructions, and solver workspaces in the device's default
+ * stream-ordered pool, whose release threshold the first solver call on the
+ * device raises.  Both go back, and the threshold is set back, when the
+ * process's last context is destroyed.
+ *
  * Errors: functions return BRI_OK (0), BRI_NOT_CONVERGED (1, output written)
  * or a negative code; bri_last_error() gives a thread-local message.
  */
@@ -116,7 +123,9 @@ int bri_set_kernel(bri_ctx* ctx, int kernel);
  * Without memory for a rebuild (BRI_ERR_OOM) the context keeps its links and
  * clover; after any other failure operators answer BRI_ERR_NOLINKS until a
  * build succeeds.
- * U: device, [V][4][3][3] complex128, read once; may be freed afterwards. */
+ * U: device, [V][4][3][3] complex128, read once; may be freed afterwards.
+ * Allocates the context's arrays on first use (about 12 KB per site with
+ * clover) and, when c_sw != 0, 3456 bytes per site of scratch on each call. */
 int bri_build_links(bri_ctx* ctx, const double* U, double c_sw);
 
 /* Export the stored links in the App. C layout [V][40][3][3] complex128

@@ -31,28 +31,80 @@ int graphs_enabled() {
   return v && current_arena() == nullptr;
 }
 
-// Contexts alive; when the last one goes, the pool's kept blocks go back too.
+// Device memory kept between calls, per device, until the last context goes:
+//  * scratch of the operator calls and the link construction, in a pool of the
+//    library's own that keeps at most kScratchKept (the packed copy of 16 right-hand
+//    sides at 24^3 x 48) once its stream has synchronised;
+//  * solver workspaces, in the device's default pool, whose release threshold is
+//    raised by the first solver call there and set back with the last context.
+constexpr int kMaxDevices = 64;
+constexpr uint64_t kScratchKept = uint64_t(1) << 30;
+struct DevicePools {
+  cudaMemPool_t scratch = nullptr;
+  bool solver = false;
+  uint64_t threshold = 0;  // the default pool's own
+};
+static std::mutex g_pool_mu;
+static DevicePools g_pools[kMaxDevices];
 static std::atomic<int> g_contexts{0};
 
-void configure_pool_once() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-      uint64_t thr = UINT64_MAX;
-      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-    }
-    cudaGetLastError();
-  });
+static int pool_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices ? dev : -1;
 }
 
-static void trim_pool() {
-  int dev = 0;
+void configure_solver_pool() {
+  const int dev = pool_device();
+  if (dev < 0) return;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevicePools& d = g_pools[dev];
   cudaMemPool_t pool;
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
-    cudaMemPoolTrimTo(pool, 0);
+  uint64_t all = UINT64_MAX;
+  if (!d.solver && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &d.threshold) == cudaSuccess)
+    d.solver = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &all) == cudaSuccess;
+  cudaGetLastError();
+}
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = nullptr;
+  const int dev = pool_device();
+  if (dev >= 0) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    DevicePools& d = g_pools[dev];
+    if (!d.scratch) {
+      cudaMemPoolProps props;
+      memset(&props, 0, sizeof(props));
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      uint64_t keep = kScratchKept;
+      if (cudaMemPoolCreate(&d.scratch, &props) == cudaSuccess)
+        cudaMemPoolSetAttribute(d.scratch, cudaMemPoolAttrReleaseThreshold, &keep);
+      else
+        d.scratch = nullptr;
+    }
+    pool = d.scratch;
+  }
+  const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+  cudaGetLastError();
+  if (e == cudaSuccess) note_device_alloc();
+  return e;
+}
+
+static void give_back_pools() {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_contexts.load() != 0) return;
+  for (int dev = 0; dev < kMaxDevices; ++dev) {
+    DevicePools& d = g_pools[dev];
+    cudaMemPool_t pool;
+    if (d.scratch) cudaMemPoolTrimTo(d.scratch, 0);
+    if (d.solver && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &d.threshold);
+      cudaMemPoolTrimTo(pool, 0);
+      d.solver = false;
+    }
+  }
   cudaGetLastError();
 }
 
@@ -222,7 +274,7 @@ void bri_destroy(bri_ctx* c) {
   cudaFreeHost(c->host_pinned);
   cudaGetLastError();
   delete c;
-  if (g_contexts.fetch_sub(1) == 1) trim_pool();
+  if (g_contexts.fetch_sub(1) == 1) give_back_pools();
 }
 
 int bri_set_stream(bri_ctx* c, void* stream) {
@@ -306,14 +358,11 @@ int bri_apply(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagge
   if (prec != BRI_PREC_DW) return dirac_bri(c, y, x, nrhs, m0, dagger ? 1 : 0, prec, c->stream);
   void* tmp = nullptr;
   const size_t bytes = 2 * dw_vector_bytes(c->g.V) * nrhs;
-  configure_pool_once();
-  cudaError_t e = cudaMallocAsync(&tmp, bytes, c->stream);
+  const cudaError_t e = scratch_alloc(&tmp, bytes, c->stream);
   if (e != cudaSuccess) {
-    cudaGetLastError();
     set_error(std::string("bri_apply: cudaMallocAsync failed: ") + cudaGetErrorString(e));
     return BRI_ERR_OOM;
   }
-  note_device_alloc();
   rc = dirac_bri_dw64(c, (double*)y, (const double*)x, nrhs, m0, dagger ? 1 : 0, tmp, c->stream);
   cudaFreeAsync(tmp, c->stream);
   return rc;

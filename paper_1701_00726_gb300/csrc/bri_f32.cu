@@ -57,10 +57,8 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
                    cudaStream_t s, const ShiftDot<float>* sd, int* sd_blocks) {
   constexpr int kChunk = 16;
   if (!sd && bri_f32_packed(g.V, nrhs) && may_allocate(s)) {
-    configure_pool_once();
     void* X = nullptr;
-    if (cudaMallocAsync(&X, sizeof(float4) * packed_words(g.V, 6) * std::min(nrhs, kChunk), s) == cudaSuccess) {
-      note_device_alloc();
+    if (scratch_alloc(&X, sizeof(float4) * packed_words(g.V, 6) * std::min(nrhs, kChunk), s) == cudaSuccess) {
       float4* X4 = (float4*)X;
       for (int r0 = 0; r0 < nrhs; r0 += kChunk) {
         const int nr = std::min(kChunk, nrhs - r0), pairs = take_pairs(g.V, nr) ? nr / 2 : 0, one = nr - 2 * pairs;
@@ -79,7 +77,6 @@ int launch_bri_f32(const Geom& g, float* y, const float* x, const LS* W, const f
       BRI_LAUNCH_CHECK("bri_pair_kernel");
       return BRI_OK;
     }
-    cudaGetLastError();
   }
   if (!sd && bri_f32_packed(g.V, nrhs)) {
     launch_singles<LS, true>(g, y, (const float4*)x, W, cl, diag, dagger, 0, nrhs, s);

@@ -142,9 +142,12 @@ int dirac_bri_shiftdot(bri_ctx* c, void* y, const void* x, int nrhs, double m0, 
 // the Brillouin stencil (Eq. def_bril) or the Wilson stencil (Eq. def_wils).
 int dirac_kernel(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, int prec,
                  cudaStream_t s);
-// Keeps freed blocks of the device's stream-ordered pool for the next
-// allocation (set once; the memory goes back when the last context is destroyed).
-void configure_pool_once();
+// The current device's default pool keeps what solver workspaces free, until the last
+// context is destroyed.
+void configure_solver_pool();
+// Stream-ordered scratch of one call (cudaFreeAsync gives it back) from the library's
+// pool on the current device; an error is returned, not left pending.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 
 // Device scratch from a caller-provided block (used by the entry point that
 // allocates nothing); when no arena is set the solvers allocate from the

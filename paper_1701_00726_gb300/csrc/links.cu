@@ -455,10 +455,8 @@ int launch_build_links(bri_ctx* c, const double* U, double c_sw) {
   if (c_sw != 0.0) {
     if ((rc = alloc((void**)&c->C64, sizeof(double) * 72 * V))) return rc;
     if ((rc = alloc((void**)&c->C32, sizeof(float4) * clover_words32(V)))) return rc;
-    configure_pool_once();
-    const cudaError_t e = cudaMallocAsync(&AB, sizeof(double2) * 9 * 2 * two.count * V, st);
+    const cudaError_t e = scratch_alloc((void**)&AB, sizeof(double2) * 9 * 2 * two.count * V, st);
     if (e != cudaSuccess) return cuda_fail(e, "bri_build_links: cudaMallocAsync");
-    note_device_alloc();
   }
   // no operator runs on what a failure from here on leaves behind
   c->have_links = false;

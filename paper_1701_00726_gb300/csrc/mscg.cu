@@ -1586,7 +1586,7 @@ int sign_apply(bri_ctx* c, double2* y, const double2* x, int nrhs, int n, int ki
                double tol, int prec, double out_scale, double b_coeff, bri_stats* stats, const KernelOp* op) {
   StreamScope scope(c);
   auto t0 = std::chrono::steady_clock::now();
-  configure_pool_once();
+  configure_solver_pool();
   cudaStream_t st = c->stream;
   const int64_t nreal = c->g.V * 24;
   const double m0 = -rho;
@@ -1667,7 +1667,7 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
       return BRI_ERR_INVALID;
     }
   auto t0 = std::chrono::steady_clock::now();
-  configure_pool_once();
+  configure_solver_pool();
   double c0, w[NS], sig[NS];
   int rc = kl_host(n, kind, scale, &c0, w, sig);
   if (rc) return rc;

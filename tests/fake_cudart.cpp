@@ -3,6 +3,7 @@
 // touch.  It gives the host code of the library the failures a GPU test must not provoke: an allocation that fails, a
 // launch that fails, a stream under capture, a second device.
 #include <cuda_runtime_api.h>
+#include <sys/mman.h>
 
 #include <algorithm>
 #include <cstdlib>
@@ -58,7 +59,8 @@ cudaError_t give(void** p, size_t n, Pool* pool, bool dev) {
     if (pool) more = n;
     if (held() + more > memory) return fail(cudaErrorMemoryAllocation);
   }
-  *p = calloc(n ? n : 1, 1);
+  *p = mmap(nullptr, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
+  if (*p == MAP_FAILED) abort();
   blocks[(char*)*p] = Block{n, pool, dev};
   if (dev && n > largest) largest = n;
   if (pool) {
@@ -76,8 +78,8 @@ cudaError_t take(void* p) {
   if (it == blocks.end()) return fail(cudaErrorInvalidValue);
   if (it->second.pool) it->second.pool->used -= it->second.bytes;
   else if (it->second.device) plain -= it->second.bytes;
+  munmap(p, it->second.bytes ? it->second.bytes : 1);
   blocks.erase(it);
-  free(p);
   return cudaSuccess;
 }
 void sync() {

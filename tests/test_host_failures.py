@@ -109,3 +109,36 @@ def test_large_fp32_application_without_scratch(run, nrhs, prec):
         assert len(kernels) == 1 and "bri_pair_kernel" in kernels[0], kernels
         fake.fake_capturing(0)
     """)
+
+
+def test_memory_kept_between_calls(run):
+    """Operator calls and link constructions leave at most 1 GiB of scratch in a pool (the two-hop paths of 24^3 x 28 are
+    1.3 GB); solver workspaces stay in the default pool of the device they ran on, on every device; the last context to
+    go gives all of it back and the default pools have their thresholds again."""
+    run("""
+    h, V = lattice(24, 24, 24, 28), 387072
+    u, x, y = device(V * 576), device(V * 192 * 2), device(V * 192 * 2)
+    assert lib.bri_build_links(h, u, 1.0) == 0
+    assert fake.fake_pool_kept() <= 1 << 30
+    for prec in (1, 2, 3):
+        assert lib.bri_apply(h, y, x, 2, -1.0, 0, prec) == 0
+    fake.cudaDeviceSynchronize()
+    assert fake.fake_pool_kept() <= 1 << 30 and fake.fake_default_threshold(0) == 0
+    small = []
+    for dev in (0, 1):
+        fake.fake_device(dev)
+        k = lattice(10, 9, 10, 11)
+        small.append(k)
+        assert lib.bri_build_links(k, u, 1.0) == 0
+        st = _lib.BriStats()
+        st.maxiter = 8
+        assert lib.sign_apply_multishift(k, y, x, 1, 4, 0, 1.0, 1.0, 1e-3, 0, ctypes.byref(st)) >= 0
+        assert fake.fake_default_threshold(dev) > 1 << 40 and fake.fake_pool_kept_on(dev) > 0
+    for k in small:
+        lib.bri_destroy(k)
+    assert fake.fake_pool_kept_on(1) > 0
+    fake.fake_device(0)
+    lib.bri_destroy(h)
+    for dev in (0, 1):
+        assert fake.fake_pool_kept_on(dev) == 0 and fake.fake_default_threshold(dev) == 0
+    """)
