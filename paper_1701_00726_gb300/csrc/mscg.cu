@@ -871,10 +871,15 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
                      double* lam_out = nullptr, const KernelOp* op = nullptr, double* x64 = nullptr) {
   using T = typename P2<R>::T;
   const int oprec = op_prec<R>(prec);
-  // FP32 solves large enough for the packed stencil keep their vectors in its layout
+  // FP32 solves large enough for the packed stencil keep their vectors in its layout.
+  // That takes up to four vectors more than the spinors' own layout does (96 bytes per
+  // site and system each): where the memory ends between the two, the latter serves.
   if constexpr (sizeof(R) == 4) {
-    if (!op && c->kernel == BRI_KERNEL_BRILLOUIN && bri_f32_packed(c->g.V, nsys) && (x64 || nshift == 1))
-      return packed_lattice_solve(c, oprec, m0, nsys, nshift, sig, b, x, tol, maxiter, iters_out, cnt, tols, lam_out, x64);
+    if (!op && c->kernel == BRI_KERNEL_BRILLOUIN && bri_f32_packed(c->g.V, nsys) && (x64 || nshift == 1)) {
+      const int prc =
+          packed_lattice_solve(c, oprec, m0, nsys, nshift, sig, b, x, tol, maxiter, iters_out, cnt, tols, lam_out, x64);
+      if (prc != BRI_ERR_OOM) return prc;
+    }
   }
   cudaStream_t st = c->stream;
   const int64_t n2 = c->g.V * 12;  // complex pairs per system

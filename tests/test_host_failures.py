@@ -142,3 +142,22 @@ def test_memory_kept_between_calls(run):
     for dev in (0, 1):
         assert fake.fake_pool_kept_on(dev) == 0 and fake.fake_default_threshold(dev) == 0
     """)
+
+
+@pytest.mark.parametrize("n,nrhs", [(1, 2), (4, 3)])
+def test_mixed_solve_at_the_memory_limit(run, n, nrhs):
+    """A mixed solve runs in the memory that the spinors' own layout needs: solutions 192 n, source 96, and 96 bytes for
+    each of the n directions, r, t, q and the ring of four residuals, per site and right-hand side (the packed form's
+    ring has eight); with a sixteenth less it is refused."""
+    run(f"""
+    h, V = lattice(10, 9, 10, 11), 9900
+    u, x, y = device(V * 576), device(V * 192 * {nrhs}), device(V * 192 * {nrhs})
+    assert lib.bri_build_links(h, u, 0.0) == 0
+    assert lib.bri_apply(h, y, x, 1, -1.0, 0, 3) == 0  # the double-word links of the residuals, kept by the context
+    need = V * {nrhs} * (192 * {n} + 96 + 96 * ({n} + 7))
+    st = _lib.BriStats()
+    st.maxiter = 8
+    for left, rcs in ((need * 2, (0, 1)), (need + V * {nrhs} * 8 + 65536, (0, 1)), (need - need // 16, ({OOM},))):
+        fake.fake_memory_left(left)
+        assert lib.sign_apply_multishift(h, y, x, {nrhs}, {n}, 0, 1.0, 1.0, 1e-3, 1, ctypes.byref(st)) in rcs
+    """)
