@@ -238,7 +238,7 @@ int bri_create(bri_ctx** out, const int dims[4], int flags, void* stream) {
   c->g.str[3] = (int64_t)dims[0] * dims[1] * dims[2];
   c->flags = flags;
   c->stream = (cudaStream_t)stream;
-  cudaError_t e = cudaMallocHost(&c->host_pinned, 1 << 16);
+  cudaError_t e = cudaMallocHost(&c->host_pinned, kPinnedBytes);
   if (e != cudaSuccess) {
     delete c;
     return cuda_fail(e, "bri_create: cudaMallocHost");

@@ -41,6 +41,8 @@ struct Workspace {
   size_t bytes = 0;
 };
 
+constexpr size_t kPinnedBytes = 1 << 16;  // bri_ctx::host_pinned
+
 // Event-bracketed stencil launches (profiling), per operator x precision.
 struct ProfRec {
   cudaEvent_t a, b;

@@ -799,6 +799,16 @@ template <> int op_prec<double>(int) { return BRI_PREC_F64; }
 template <> int op_prec<float>(int prec) { return prec == BRI_PREC_F32_BF16 ? BRI_PREC_F32_BF16 : BRI_PREC_F32; }
 
 
+// Where the host reads the systems' done flags: the context's pinned block, or
+// pageable memory for more systems than fit there.
+struct DoneFlags {
+  std::vector<int> many;
+  int* p;
+  DoneFlags(bri_ctx* c, int nsys) : many(sizeof(int) * nsys > kPinnedBytes ? nsys : 0) {
+    p = many.empty() ? (int*)c->host_pinned : many.data();
+  }
+};
+
 #include "packed_solve.cuh"
 
 // One lattice's FP32 solve on packed vectors (multishift_solve's arguments).
@@ -852,9 +862,10 @@ int packed_lattice_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, 
     return prof_end(c, st, ev, 0, prec, (double)V * na);
   };
   const bool graphs = graphs_enabled() && !c->prof_on && st != nullptr;
+  const DoneFlags done(c, nsys);
   int64_t all_iters = 0;
   rc = packed_solve(st, pb, pack, apply, bsd.as<double>(), blocks, (double2*)x64, sizeof(double2) * n2 * nsys * nshift,
-                    bx.as<float4>(), false, graphs, (int*)c->host_pinned, iters_out, cnt, lam_out, &S, &all_iters);
+                    bx.as<float4>(), false, graphs, done.p, iters_out, cnt, lam_out, &S, &all_iters);
   // the tracing counts the systems that ran, not those a launch was sized for
   if (c->prof_on && !c->prof_pending.empty()) c->prof_pending.back().units += 2.0 * V * all_iters - counted;
   if (rc < 0 || x64) return rc;
@@ -943,7 +954,8 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
   k_scalar_init<<<nsys, RED_THREADS, 0, st>>>(S, part, nblk); note_launch();
   BRI_LAUNCH_CHECK("multishift init");
 
-  int* hdone = (int*)c->host_pinned;  // pinned scratch, >= 4 KB
+  const DoneFlags done(c, nsys);
+  int* hdone = done.p;
   const int check_every = 8;
   int it = 0;
   // Systems [nact, nsys) have all converged: the stencil and the vector

@@ -161,3 +161,17 @@ def test_mixed_solve_at_the_memory_limit(run, n, nrhs):
         fake.fake_memory_left(left)
         assert lib.sign_apply_multishift(h, y, x, {nrhs}, {n}, 0, 1.0, 1.0, 1e-3, 1, ctypes.byref(st)) in rcs
     """)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_flags_of_many_systems(run, prec):
+    """The done flags of more systems than the context's pinned block holds (16384) go elsewhere: no copy leaves its block."""
+    run(f"""
+    h, V, nrhs = lattice(2, 2, 2, 2), 16, 16400
+    u, x, y = device(V * 576), device(V * 192 * nrhs), device(V * 192 * nrhs)
+    assert lib.bri_build_links(h, u, 0.0) == 0
+    st = _lib.BriStats()
+    st.maxiter = 8
+    rc = lib.sign_apply_multishift(h, y, x, nrhs, 1, 0, 1.0, 1.0, 1e-3, {prec}, ctypes.byref(st))
+    assert fake.fake_out_of_range() == 0 and rc >= 0, lib.bri_last_error()
+    """)
