@@ -33,6 +33,18 @@ int bri_f32_pack(int64_t V, const float* x, int nrhs, void* X, cudaStream_t s) {
   return BRI_OK;
 }
 
+// Packed single right-hand sides -> spinors [nrhs][V][12] complex64.
+static __global__ void __launch_bounds__(256) k_unpack(int64_t V, const float4* __restrict__ X, float* __restrict__ x) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= V * 6) return;
+  const int64_t n = i / 6;
+  const int q = (int)(i - n * 6);
+  const float4 u = __ldg(X + (int64_t)blockIdx.y * packed_words(V, 6) + packed_at<6>((int)n) + q * kPackBlock);
+  float2* p = reinterpret_cast<float2*>(x + (int64_t)blockIdx.y * V * 24 + n * 24) + q + 3 * (q / 3);
+  p[0] = make_float2(u.x, u.z);
+  p[3] = make_float2(u.y, u.w);
+}
+
 int bri_f32_unpack(int64_t V, const void* X, int nrhs, float* x, cudaStream_t s) {
   k_unpack<<<dim3(blocks_for(V * 6, 256), nrhs), 256, 0, s>>>(V, (const float4*)X, x);
   note_launch();

@@ -7,9 +7,9 @@
 // FP64 runs it at every size: the FP64 pipe (1/64 of the FP32 rate) is busy
 // with a few warps, so what counts is that every SM gets the same number of
 // sites, which blocks of 8..32 sites give where blocks of 128 leave a partly
-// filled last wave.  FP32 runs it on lattices too small to fill the chip with a
-// thread per site, where the serial chain of 40 gathers per thread was the
-// whole time.
+// filled last wave.  FP32 runs it, in blocks of 8 sites, on lattices too small to
+// fill the chip with a thread per site, where the serial chain of 40 gathers per
+// thread was the whole time.
 #pragma once
 
 #include "hops.cuh"
@@ -198,11 +198,14 @@ inline int split_sites(int64_t site_rhs) {
 template <typename R, typename LS>
 inline int launch_split(const Geom& g, R* y, const R* x, const LS* W, const R* cl, R diag, int nrhs, int dagger,
                         cudaStream_t st, const ShiftDot<R>* sd, int* sd_blocks) {
-  const int S = split_sites(g.V * nrhs);
+  // (FP32 is here for small calls, and for a solve that has no memory for packed vectors)
+  const int S = sizeof(R) == 4 ? 8 : split_sites(g.V * nrhs);
   if (sd_blocks) *sd_blocks = blocks_for(g.V, S);
-  if (S == 32) launch_split_sg<R, LS, 32, 5>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
-  else if (S == 16) launch_split_sg<R, LS, 16, 10>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
-  else launch_split_sg<R, LS, 8, 20>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
+  if constexpr (sizeof(R) == 8) {
+    if (S == 32) launch_split_sg<R, LS, 32, 5>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
+    if (S == 16) launch_split_sg<R, LS, 16, 10>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
+  }
+  if (S == 8) launch_split_sg<R, LS, 8, 20>(g, y, x, W, cl, diag, dagger, nrhs, st, sd);
   BRI_LAUNCH_CHECK("bri_split_kernel");
   return BRI_OK;
 }

@@ -150,16 +150,14 @@ __global__ void k_shift_dot(int64_t n2, const MsState* __restrict__ st, const ty
 // The per-shift coefficients are staged in shared memory once per block (the
 // active shifts compacted to a list), so the element loop reads no scalars
 // from global memory.
-template <typename R, typename XT = typename P2<R>::T>
+template <typename R>
 __global__ void k_update_fused(int64_t n2, int nsys, const MsState* __restrict__ st,
                                const typename P2<R>::T* __restrict__ q, typename P2<R>::T* r, typename P2<R>::T* p,
-                               XT* x, double* part, int first) {
+                               typename P2<R>::T* x, double* part, int first) {
   using T = typename P2<R>::T;
-  using XR = decltype(XT::x);
   const int s = blockIdx.y;
   if (st[s].done) return;
-  __shared__ R sz[NS], sb[NS];
-  __shared__ XR sa[NS];
+  __shared__ R sz[NS], sb[NS], sa[NS];
   __shared__ int sk[NS], snact;
   if (threadIdx.x == 0) {
     int m = 0;
@@ -168,7 +166,7 @@ __global__ void k_update_fused(int64_t n2, int nsys, const MsState* __restrict__
         sk[m] = k;
         sz[m] = (R)st[s].zeta[k];
         sb[m] = (R)st[s].b_s[k];
-        sa[m] = (XR)st[s].a_s[k];
+        sa[m] = (R)st[s].a_s[k];
         ++m;
       }
     snact = m;
@@ -189,10 +187,10 @@ __global__ void k_update_fused(int64_t n2, int nsys, const MsState* __restrict__
         pv.y = fma(bt, pv.y, z * rv.y);
         p[o] = pv;
       }
-      const XR a = sa[m];
-      XT xv = x[o];
-      xv.x = fma(a, (XR)pv.x, xv.x);
-      xv.y = fma(a, (XR)pv.y, xv.y);
+      const R a = sa[m];
+      T xv = x[o];
+      xv.x = fma(a, pv.x, xv.x);
+      xv.y = fma(a, pv.y, xv.y);
       x[o] = xv;
     }
     const T qv = q[s * n2 + i];
@@ -595,66 +593,59 @@ __global__ void __launch_bounds__(S* G, 2)
 }
 
 // r = b, p_k = b, x_k = 0, partial ||b||^2
-template <typename R>
-__global__ void kb_init(const SysDesc* __restrict__ sd, int nshift, const typename P2<R>::T* __restrict__ b,
-                        typename P2<R>::T* r, typename P2<R>::T* p, double2* x, double* part) {
-  using T = typename P2<R>::T;
+__global__ void kb_init(const SysDesc* __restrict__ sd, int nshift, const double2* __restrict__ b,
+                        double2* r, double2* p, double2* x, double* part) {
   const int s = blockIdx.y;
   const SysDesc d = sd[s];
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n2; i += (int64_t)gridDim.x * blockDim.x) {
-    const T v = b[d.off + i];
+    const double2 v = b[d.off + i];
     r[d.off + i] = v;
     for (int k = 0; k < nshift; ++k) {
       p[d.offn + k * d.n2 + i] = v;
       x[d.offn + k * d.n2 + i] = make_double2(0.0, 0.0);
     }
-    acc += (double)v.x * v.x + (double)v.y * v.y;
+    acc += v.x * v.x + v.y * v.y;
   }
   double t = block_sum(acc);
   if (threadIdx.x == 0) part[s * gridDim.x + blockIdx.x] = t;
 }
 
 // q += sigma_base p_0 ; partial Re <p_0, q>
-template <typename R>
 __global__ void kb_shift_dot(const SysDesc* __restrict__ sd, const MsState* __restrict__ st,
-                             const typename P2<R>::T* __restrict__ p, typename P2<R>::T* q, double* part) {
-  using T = typename P2<R>::T;
+                             const double2* __restrict__ p, double2* q, double* part) {
   const int s = blockIdx.y;
   if (st[s].done) return;
   const SysDesc d = sd[s];
-  const R sb = (R)st[s].sig_base;
+  const double sb = st[s].sig_base;
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n2; i += (int64_t)gridDim.x * blockDim.x) {
-    const T pv = p[d.offn + i];
-    T qv = q[d.off + i];
+    const double2 pv = p[d.offn + i];
+    double2 qv = q[d.off + i];
     qv.x = fma(sb, pv.x, qv.x);
     qv.y = fma(sb, pv.y, qv.y);
     q[d.off + i] = qv;
-    acc += (double)pv.x * qv.x + (double)pv.y * qv.y;
+    acc += pv.x * qv.x + pv.y * qv.y;
   }
   double t = block_sum(acc);
   if (threadIdx.x == 0) part[s * gridDim.x + blockIdx.x] = t;
 }
 
-// the fused shift pass of k_update_fused on the system table (solutions in FP64)
-template <typename R>
+// the fused shift pass of k_update_fused on the system table
 __global__ void kb_update(const SysDesc* __restrict__ sd, const MsState* __restrict__ st,
-                          const typename P2<R>::T* __restrict__ q, typename P2<R>::T* r, typename P2<R>::T* p,
+                          const double2* __restrict__ q, double2* r, double2* p,
                           double2* x, double* part, int first) {
-  using T = typename P2<R>::T;
   const int s = blockIdx.y;
   if (st[s].done) return;
-  __shared__ R sz[NS], sb[NS];
-  __shared__ double sa[NS];
+  __shared__ double sz[NS], sb[NS], sa[NS];
   __shared__ int sk[NS], snact;
   if (threadIdx.x == 0) {
     int m = 0;
     for (int k = 0; k < st[s].nshift; ++k)
       if (st[s].active[k]) {
         sk[m] = k;
-        sz[m] = (R)st[s].zeta[k];
-        sb[m] = (R)st[s].b_s[k];
+        sz[m] = st[s].zeta[k];
+        sb[m] = st[s].b_s[k];
         sa[m] = st[s].a_s[k];
         ++m;
       }
@@ -663,46 +654,44 @@ __global__ void kb_update(const SysDesc* __restrict__ sd, const MsState* __restr
   __syncthreads();
   const SysDesc d = sd[s];
   const int nact = snact;
-  const R alpha = (R)st[s].alpha;
+  const double alpha = st[s].alpha;
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n2; i += (int64_t)gridDim.x * blockDim.x) {
-    T rv = r[d.off + i];
+    double2 rv = r[d.off + i];
     for (int m = 0; m < nact; ++m) {
       const int k = sk[m];
       const int64_t o = d.offn + k * d.n2 + i;
-      T pv = p[o];
+      double2 pv = p[o];
       if (k > 0 && !first) {
         pv.x = fma(sb[m], pv.x, sz[m] * rv.x);
         pv.y = fma(sb[m], pv.y, sz[m] * rv.y);
         p[o] = pv;
       }
       double2 xv = x[o];
-      xv.x = fma(sa[m], (double)pv.x, xv.x);
-      xv.y = fma(sa[m], (double)pv.y, xv.y);
+      xv.x = fma(sa[m], pv.x, xv.x);
+      xv.y = fma(sa[m], pv.y, xv.y);
       x[o] = xv;
     }
-    const T qv = q[d.off + i];
+    const double2 qv = q[d.off + i];
     rv.x = fma(-alpha, qv.x, rv.x);
     rv.y = fma(-alpha, qv.y, rv.y);
     r[d.off + i] = rv;
-    acc += (double)rv.x * rv.x + (double)rv.y * rv.y;
+    acc += rv.x * rv.x + rv.y * rv.y;
   }
   double t = block_sum(acc);
   if (threadIdx.x == 0) part[s * gridDim.x + blockIdx.x] = t;
 }
 
 // p_0 = r + beta p_0
-template <typename R>
 __global__ void kb_update_p0(const SysDesc* __restrict__ sd, const MsState* __restrict__ st,
-                             const typename P2<R>::T* __restrict__ r, typename P2<R>::T* p) {
-  using T = typename P2<R>::T;
+                             const double2* __restrict__ r, double2* p) {
   const int s = blockIdx.y;
   if (st[s].done) return;
   const SysDesc d = sd[s];
-  const R bt = (R)st[s].b_s[0];
+  const double bt = st[s].b_s[0];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n2; i += (int64_t)gridDim.x * blockDim.x) {
-    const T rv = r[d.off + i];
-    T pv = p[d.offn + i];
+    const double2 rv = r[d.off + i];
+    double2 pv = p[d.offn + i];
     pv.x = fma(bt, pv.x, rv.x);
     pv.y = fma(bt, pv.y, rv.y);
     p[d.offn + i] = pv;
@@ -729,14 +718,12 @@ __global__ void kb_gather_x(const SysDesc* __restrict__ sd, int s0, int nrhs, in
 }
 
 // b of one lattice (FP64, [nrhs][n2]) into the system table's vector
-template <typename R>
 __global__ void kb_scatter_b(const SysDesc* __restrict__ sd, int s0, const double2* __restrict__ b,
-                             typename P2<R>::T* out) {
+                             double2* out) {
   const int r = blockIdx.y;
   const SysDesc d = sd[s0 + r];
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d.n2; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = b[(int64_t)r * d.n2 + i];
-    out[d.off + i] = typename P2<R>::T{(R)v.x, (R)v.y};
+    out[d.off + i] = b[(int64_t)r * d.n2 + i];
   }
 }
 
@@ -990,9 +977,6 @@ int multishift_solve(bri_ctx* c, int prec, double m0, int nsys, int nshift, cons
       if (defer)
         k_update_base<<<vga, RED_THREADS, 0, st>>>(n2, nsys, S, hist, (const float2*)q_vec, (float2*)r,
                                                    (const float2*)p, (double2*)x64, (float2*)bring.p, part);
-      else if (x64)
-        k_update_fused<R, double2><<<vga, RED_THREADS, 0, st>>>(n2, nsys, S, q_vec, r, p, (double2*)x64, part,
-                                                                it0 + j == 0 ? 1 : 0);
       else
         k_update_fused<R><<<vga, RED_THREADS, 0, st>>>(n2, nsys, S, q_vec, r, p, (T*)x, part, it0 + j == 0 ? 1 : 0);
       note_launch();
@@ -1343,8 +1327,6 @@ int refine_mixed(bri_ctx* c, const double* b, int nrhs, int n, const double* sig
 int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector<SysDesc>& sdh, int nshift,
                          const double* sig, const double2* b, double2* x, double tol, int maxiter, int* iters_out,
                          Counters* cnt, double* lam_out) {
-  using R = double;
-  using T = double2;
   const int S = (int)sdh.size();
   int64_t tot = 0, maxn2 = 0;
   std::vector<int2> items;  // (system, block of sites)
@@ -1361,16 +1343,16 @@ int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector
   int rc;
   if ((rc = bsd.alloc(sizeof(SysDesc) * S, st))) return rc;
   if ((rc = bit.alloc(sizeof(int2) * nitems, st))) return rc;
-  if ((rc = br.alloc(sizeof(T) * tot, st))) return rc;
-  if ((rc = bt.alloc(sizeof(T) * tot, st))) return rc;
-  if ((rc = bq.alloc(sizeof(T) * tot, st))) return rc;
-  if ((rc = bp.alloc(sizeof(T) * tot * nshift, st))) return rc;
+  if ((rc = br.alloc(sizeof(double2) * tot, st))) return rc;
+  if ((rc = bt.alloc(sizeof(double2) * tot, st))) return rc;
+  if ((rc = bq.alloc(sizeof(double2) * tot, st))) return rc;
+  if ((rc = bp.alloc(sizeof(double2) * tot * nshift, st))) return rc;
   if ((rc = bst.alloc(sizeof(MsState) * S, st))) return rc;
   if ((rc = bpart.alloc(sizeof(double) * std::max<int64_t>((int64_t)nblk * S, kMaxPartials), st))) return rc;
   const SysDesc* sd = bsd.as<SysDesc>();
   MsState* S_ = bst.as<MsState>();
   double* part = bpart.as<double>();
-  T *r = br.as<T>(), *t = bt.as<T>(), *q = bq.as<T>(), *p = bp.as<T>();
+  double2 *r = br.as<double2>(), *t = bt.as<double2>(), *q = bq.as<double2>(), *p = bp.as<double2>();
   std::vector<MsState> hs(S);
   for (int s = 0; s < S; ++s) {
     MsState& h = hs[s];
@@ -1394,20 +1376,19 @@ int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector
     else if (sites == 16) kb_stencil<16, 10><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, H);
     else kb_stencil<8, 20><<<nitems, 160, 0, st>>>(tab, sd, itd, S_, out, in, from_p, H);
   };
-  const int nst = 1;  // stencil launches per application
-  kb_init<R><<<vg, RED_THREADS, 0, st>>>(sd, nshift, b, r, p, x, part); note_launch();
+  kb_init<<<vg, RED_THREADS, 0, st>>>(sd, nshift, b, r, p, x, part); note_launch();
   k_scalar_init<<<S, RED_THREADS, 0, st>>>(S_, part, nblk); note_launch();
   auto iteration = [&](int first) {
     stencil(t, p, 1, 0);
     stencil(q, t, 0, 1);
-    kb_shift_dot<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, p, q, part);
+    kb_shift_dot<<<vg, RED_THREADS, 0, st>>>(sd, S_, p, q, part);
     k_scalar_alpha<<<S, RED_THREADS, 0, st>>>(S_, part, nblk);
-    kb_update<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, q, r, p, x, part, first);
+    kb_update<<<vg, RED_THREADS, 0, st>>>(sd, S_, q, r, p, x, part, first);
     k_scalar_beta<<<S, RED_THREADS, 0, st>>>(S_, part, nblk);
-    kb_update_p0<R><<<vg, RED_THREADS, 0, st>>>(sd, S_, r, p);
+    kb_update_p0<<<vg, RED_THREADS, 0, st>>>(sd, S_, r, p);
   };
   iteration(1);
-  note_launches(5 + 2 * nst);
+  note_launches(7);
   BRI_LAUNCH_CHECK("batched multi-shift: first iteration");
   // graph: WHILE (any system running) { iteration }
   cudaGraph_t graph = nullptr;
@@ -1456,7 +1437,7 @@ int batch_multishift_f64(cudaStream_t st, const BatchTab& tab, const std::vector
     if (hs[s].active[0] && !hs[s].error) notconv = 1;
     lm = std::max(lm, hs[s].lam_max - hs[s].sig_base);
   }
-  note_launches((long long)(6 + 2 * nst) * std::max(0, maxit - 1));
+  note_launches(8LL * std::max(0, maxit - 1));
   *iters_out = maxit;
   cnt->matvecs += 2 * maxit;
   cnt->matvecs64 += 2 * maxit;
@@ -1480,7 +1461,6 @@ int solve_shifts(bri_ctx* c, const double* b, int nrhs, int n, const double* sig
   int rc = BRI_OK;
   Counters& cnt = info.cnt;
   int& iters = info.iters;
-  int& refinements = info.refinements;
   std::vector<double> sig_all((size_t)nrhs * n);
   for (int s = 0; s < nrhs; ++s)
     for (int k = 0; k < n; ++k) sig_all[(size_t)s * n + k] = sig[k];
@@ -1746,7 +1726,7 @@ int batch_sign_apply(bri_ctx* const* cs, int nctx, void* const* ys, const void* 
     if ((q = bb.alloc(sizeof(double2) * off, bs))) return q;
     if ((q = bx.alloc(sizeof(double2) * off * n, bs))) return q;
     for (int i = 0; i < nctx; ++i) {
-      kb_scatter_b<double><<<dim3(grid_for(cs[i]->g.V * 12, nrhs[i]), nrhs[i]), RED_THREADS, 0, bs>>>(
+      kb_scatter_b<<<dim3(grid_for(cs[i]->g.V * 12, nrhs[i]), nrhs[i]), RED_THREADS, 0, bs>>>(
           bsd.as<SysDesc>(), first_sys[i], (const double2*)xs[i], bb.as<double2>());
       note_launch();
     }

@@ -44,19 +44,11 @@ __device__ __forceinline__ void store_spinor(double* p, const Spinor<double>& s)
   for (int e = 0; e < 12; ++e) q[e] = make_double2(s.v[e / 3][e % 3].re, s.v[e / 3][e % 3].im);
 }
 
-// One 3x3 link in structure-of-arrays storage: element e of the link at site
+// One 3x3 FP64 link in structure-of-arrays storage: element e of the link at site
 // n sits at p[e*V] (p already offset by n).
-template <typename R, typename LS>
-__device__ __forceinline__ void load_link(C<R> w[3][3], const LS* __restrict__ p, int V) {
+__device__ __forceinline__ void load_link(C<double> w[3][3], const double2* __restrict__ p, int V) {
 #pragma unroll
-  for (int e = 0; e < 9; ++e) {
-    if constexpr (sizeof(R) == 8) {
-      w[e / 3][e % 3] = ld2(reinterpret_cast<const double2*>(p) + e * V);
-    } else {
-      C<float> f = ld2(p + e * V);
-      w[e / 3][e % 3] = C<R>{(R)f.re, (R)f.im};
-    }
-  }
+  for (int e = 0; e < 9; ++e) w[e / 3][e % 3] = ld2(p + e * V);
 }
 
 // Stored link of offset j at site m.  FP64 links are [40][9][V] (element e at
@@ -104,7 +96,7 @@ __device__ __forceinline__ void load_stored_link(C<R> w[3][3], const LS* __restr
     }
     w[2][2] = C<R>{(R)__uint_as_float(last << 16), (R)__uint_as_float(last & 0xffff0000u)};
   } else {
-    load_link<R, LS>(w, W + (int64_t)j * 9 * V + m, V);
+    load_link(w, W + (int64_t)j * 9 * V + m, V);
   }
 }
 
