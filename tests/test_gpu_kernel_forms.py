@@ -13,7 +13,7 @@ import torch
 
 import synthetic_fields as sf
 from oracle import dirac
-from paper_1701_00726_gb300 import PREC_F32, Lattice, build, overlap_apply_batch
+from paper_1701_00726_gb300 import PREC_F32, PREC_F64, Lattice, build, overlap_apply_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -125,3 +125,36 @@ def test_batch_of_small_and_large_sources(scale):
     assert all(s["refinements"] == 0 for s in st)
     for g, w in zip(got, want):
         assert torch.equal(g, w * 2.0 ** scale)
+
+
+@pytest.mark.parametrize("dagger", [False, True])
+def test_fp64_sixteen_sites_per_block(dagger):
+    """FP64 split kernel between 9728 and 19455 sites x right-hand sides (17136), against the oracle."""
+    x = sf.gaussian_source(LARGE, 2, 1043)
+    op = _operator(LARGE)[1]
+    y = _lattice(LARGE).bri_apply(torch.from_numpy(x).cuda(), -1.0, dagger=dagger).cpu().numpy()
+    assert relerr(y, op.apply_dagger(x) if dagger else op.apply(x)) < 1e-12
+
+
+@pytest.mark.parametrize("dims,nrhs", [(LARGE, 17), ((16, 15, 17, 19), 7), ((16, 15, 17, 19), 15)])
+def test_bf16_links_in_the_packed_forms(dims, nrhs):
+    """BF16 links with two thread groups per site and a rest of one right-hand side, with one group, and in pairs: the
+    oracle's result to the links' 8 bits."""
+    x = torch.from_numpy(sf.gaussian_source(dims, nrhs, 1044)).to(torch.complex64).cuda()
+    y = _lattice(dims).bri_apply(x, -1.0, bf16_links=True)
+    some = [0, nrhs - 1] if nrhs == 17 else [nrhs - 1]
+    want = _operator(dims)[1].apply(x[some].cpu().numpy().astype(np.complex128))
+    assert relerr(y[some].cpu().numpy(), want) < 1e-2
+
+
+@pytest.mark.parametrize("nrhs,prec", [((1, 4), PREC_F64), ((2, 8), PREC_F64), ((9, 24), PREC_F32), ((40, 60), PREC_F32)])
+def test_batch_of_uneven_volumes(nrhs, prec):
+    """Batches of two volumes: FP64 with 16 (12768 sites x systems) and 32 (25536) sites per block, mixed with two (102312)
+    and one (405720) thread groups per site: each lattice's own FP64 result."""
+    dims = [LARGE, (7, 5, 6, 5)]
+    lats = [_lattice(d) for d in dims]
+    xs = [torch.from_numpy(sf.gaussian_source(d, r, 1045)).cuda() for d, r in zip(dims, nrhs)]
+    ys, _ = overlap_apply_batch(lats, xs, n=4, tol=1e-13 if prec == PREC_F64 else 1e-11, prec=prec)
+    for lat, x, y in zip(lats, xs, ys):
+        want, _ = lat.overlap_apply(x, n=4, tol=1e-13, prec=PREC_F64)
+        assert relerr(y.cpu().numpy(), want.cpu().numpy()) < 1e-10
