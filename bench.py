@@ -96,8 +96,9 @@ def parse():
                     help="time the mixed-precision backward (overlap_grad, KL order 12) on 32^3x64 instead")
     ap.add_argument("--probe-nrhs", type=int, default=1)
     ap.add_argument("--probe-launches", type=int, default=4)
-    ap.add_argument("--probe-prec", choices=("f32", "dw", "f64"), default="f32",
-                    help="stencil probe precision: FP32, double-word FP32 (complex128 in/out) or FP64")
+    ap.add_argument("--probe-prec", choices=("f32", "dw", "f64", "solver"), default="f32",
+                    help="stencil probe precision: FP32, double-word FP32 (complex128 in/out) or FP64; solver: "
+                         "eight iterations of the mixed solver, whose stencil is a kernel of its own")
     return ap.parse_args()
 
 
@@ -105,7 +106,7 @@ def stencil_probe(args):
     import torch
 
     import synthetic_fields as sf
-    from paper_1701_00726_gb300 import Lattice
+    from paper_1701_00726_gb300 import PREC_F32, Lattice
     dims = tuple(int(v) for v in args.stencil_probe.split(","))
     vol = dims[0] * dims[1] * dims[2] * dims[3]
     lat = Lattice(dims)
@@ -114,6 +115,11 @@ def stencil_probe(args):
     dw = args.probe_prec == "dw"
     x = torch.randn((args.probe_nrhs, vol * 12), dtype=dt, device="cuda")
     y = torch.empty_like(x)
+    if args.probe_prec == "solver":
+        _, st = lat.sign_apply(x, 1, tol=1e-12, prec=PREC_F32, maxiter=8, out=y)
+        print(json.dumps({"stencil_probe": list(dims), "prec": "solver", "nrhs": args.probe_nrhs,
+                          "matvecs": st["matvecs"]}), flush=True)
+        return
     lat.bri_apply(x, -RHO, out=y, double_word=dw)
     torch.cuda.synchronize()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -182,10 +188,14 @@ def stencil_traffic_per_launch(traffic, vol, nlaunch, units, prec):
     return int(vol * per_site + units / nlaunch * per_site_rhs)
 
 
+# the kernel behind the step's FP32 stencil launches, and its sources
+STENCIL_KERNEL = "kp_stencil"
+STENCIL_SOURCES = ("packed_solve.cuh", "bri_pair.cuh", "sum3.cuh", "hops.cuh", "stencil.cuh", "cplx.cuh")
+
+
 def stencil_source_hash():
-    """Hash of the FP32 stencil's sources (kernel header and shared helpers)."""
     h = hashlib.sha256()
-    for f in ("bri_pair.cuh", "bri_split.cuh", "bri_f32.cu", "hops.cuh", "stencil.cuh", "cplx.cuh"):
+    for f in STENCIL_SOURCES:
         h.update(open(os.path.join(ROOT, "paper_1701_00726_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -433,7 +443,7 @@ def c5_grad(args):
     lat = Lattice(dims)
     lat.build_links(torch.from_numpy(u).cuda(), 0.0)
     del u
-    lat.overlap_apply(psi, 12, rho=RHO, tol=TOL, prec=PREC_F32)  # warm-up (autotuner, pool)
+    lat.overlap_apply(psi, 12, rho=RHO, tol=TOL, prec=PREC_F32)  # warm-up (memory pool)
     torch.cuda.synchronize()
     t0 = time.perf_counter()
     _, stf = lat.overlap_apply(psi, 12, rho=RHO, tol=TOL, prec=PREC_F32)
@@ -549,7 +559,7 @@ def main():
     t_alu = alg_flops / (fp32_peak * 1e12)
     traffic = stencil_traffic()
     lt = "bf16x2" if prec == PREC_F32_BF16 else "float2"
-    common = {"kernel": f"kp_stencil, bri_pair_kernel ({lt} links, packed spinors)",
+    common = {"kernel": f"{STENCIL_KERNEL} ({lt} links, packed spinors)",
               "launches": nlaunch, "avg_launch_ms": round(kms / max(nlaunch, 1), 4),
               "avg_rhs_per_launch": round(units / max(nlaunch, 1) / vol, 3),
               "alg_bytes_per_launch": int(alg_bytes / max(nlaunch, 1)),

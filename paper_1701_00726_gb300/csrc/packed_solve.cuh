@@ -36,9 +36,10 @@ __global__ void __launch_bounds__(256) kp_norm(const PackedSys* __restrict__ gd,
 }
 
 // rout = rin - alpha q, partials of ||rout||^2 (rin may be rout).  The squares of four words are summed in
-// three FP32 words (sum3.cuh, scaled by the residual's norm so far) and those sums in FP64.  FP64 squares bound
-// the kernel (102 us on average in the 16^3 x 32 solves against 43 with two FP32 words, which kept only 2^-47 and
-// FP32's range); the third word costs the whole solve 0.4 %.
+// three FP32 words (sum3.cuh, scaled by the residual's norm so far) and those sums in FP64.  Bound by HBM: 174 us
+// on average in the 24^3 x 48 solves of 4 rhs, 91 % of the copy rate.  FP64 squares bound it instead (102 us on
+// average in the 16^3 x 32 solves against 43 with two FP32 words, which kept only 2^-47 and FP32's range); the third
+// word costs the whole solve 0.4 %.
 __global__ void __launch_bounds__(256) kp_update_r(const PackedSys* __restrict__ gd, const MsState* __restrict__ st,
                                                    const float4* __restrict__ q, const float4* rin, float4* rout, double* part) {
   const PackedSys g = gd[blockIdx.y];
