@@ -180,11 +180,11 @@ int overlap_apply(bri_ctx* ctx, void* y, const void* x, int nrhs, int n, int kin
  * lattices): the same result as overlap_apply on
  * each context.  The multi-shift phase of every lattice and right-hand side
  * runs as one system table: each stencil launch walks a device-side work list
- * of (lattice, right-hand side, 128-site block) items, the CG scalars and
+ * of (lattice, right-hand side, site block) items, the CG scalars and
  * convergence flags of every system stay in device memory, and the iterations
- * run inside one CUDA graph whose conditional WHILE node repeats the
- * iteration until every system has converged (or reached the iteration cap),
- * with no host polling.  For the mixed precisions the FP64-class residuals, FP32
+ * run inside one CUDA graph whose conditional WHILE node repeats them until
+ * every system has converged (or reached the iteration cap), with no host
+ * polling.  For the mixed precisions the FP64-class residuals, FP32
  * corrections and the final application then run per lattice, concurrently
  * on the contexts' own streams.  At most 32 contexts, all on the current
  * device, each with the Brillouin kernel; ys[i], xs[i]: device complex128

@@ -127,8 +127,9 @@ int dirac_wil(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagge
 // Double-word FP32 Brillouin stencil (bri_dw.cu): y = D x or D^dagger x on
 // packed double-word vectors (dw_vector_bytes each), FP64 in and out through the
 // split/join kernels (tmp: two double-word vectors of nrhs right-hand sides),
-// and the normal operator D^dagger D on FP64 vectors (t1, t2 double-word
-// scratch; t2 may be out).
+// and the normal operator D^dagger D on FP64 vectors (t1, t2: nrhs * dw_vector_bytes
+// of scratch each, more than the FP64 vectors take unless 32 divides V; out may be t2
+// in a buffer of that size).
 size_t dw_vector_bytes(int64_t V);
 int ensure_dw_links(bri_ctx* c);
 int dirac_bri_dw(bri_ctx* c, void* y, const void* x, int nrhs, double m0, int dagger, cudaStream_t s);
