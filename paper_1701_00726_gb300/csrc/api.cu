@@ -58,12 +58,13 @@ void configure_solver_pool() {
   if (dev < 0) return;
   std::lock_guard<std::mutex> lk(g_pool_mu);
   DevicePools& d = g_pools[dev];
+  if (d.solver) return;
   cudaMemPool_t pool;
   uint64_t all = UINT64_MAX;
-  if (!d.solver && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &d.threshold) == cudaSuccess)
-    d.solver = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &all) == cudaSuccess;
-  cudaGetLastError();
+  d.solver = cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess &&
+             cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &d.threshold) == cudaSuccess &&
+             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &all) == cudaSuccess;
+  if (!d.solver) cudaGetLastError();
 }
 
 cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
@@ -79,16 +80,18 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
       uint64_t keep = kScratchKept;
-      if (cudaMemPoolCreate(&d.scratch, &props) == cudaSuccess)
+      if (cudaMemPoolCreate(&d.scratch, &props) == cudaSuccess) {
         cudaMemPoolSetAttribute(d.scratch, cudaMemPoolAttrReleaseThreshold, &keep);
-      else
-        d.scratch = nullptr;
+      } else {
+        cudaGetLastError();
+        d.scratch = nullptr;  // the default pool serves
+      }
     }
     pool = d.scratch;
   }
   const cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
-  cudaGetLastError();
   if (e == cudaSuccess) note_device_alloc();
+  else cudaGetLastError();
   return e;
 }
 
@@ -98,7 +101,8 @@ static void give_back_pools() {
   for (int dev = 0; dev < kMaxDevices; ++dev) {
     DevicePools& d = g_pools[dev];
     cudaMemPool_t pool;
-    if (d.scratch) cudaMemPoolTrimTo(d.scratch, 0);
+    if (d.scratch) cudaMemPoolDestroy(d.scratch);  // (takes effect once its last block is free)
+    d.scratch = nullptr;
     if (d.solver && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &d.threshold);
       cudaMemPoolTrimTo(pool, 0);

@@ -137,6 +137,11 @@ cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps* props) {
   *p = (cudaMemPool_t)pools.back();
   return cudaSuccess;
 }
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t p) {
+  ((Pool*)p)->reserved = ((Pool*)p)->used;
+  ((Pool*)p)->keep = 0;
+  return cudaSuccess;
+}
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t p, cudaMemPoolAttr a, void* v) {
   if (a == cudaMemPoolAttrReleaseThreshold) ((Pool*)p)->keep = *(uint64_t*)v;
   return cudaSuccess;
