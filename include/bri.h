@@ -318,7 +318,7 @@ int bri_fma_probe(int kind, void* stream, double* tflops, double* ms);
 long long bri_kernel_launches(void);
 
 /* Process-wide number of device allocations this library has made so far
- * (link and clover storage, solver workspaces).  Diagnostic: the
+ * (link and clover storage, solver workspaces, operator scratch).  Diagnostic: the
  * allocation-free entry point leaves it unchanged. */
 long long bri_device_allocations(void);
 

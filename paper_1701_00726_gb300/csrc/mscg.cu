@@ -1119,7 +1119,7 @@ int norms64(bri_ctx* c, int nsys, const double* X, double* part, double* dsum, d
 // to ~2^-49 of each component, the products and sums are error-free up to the
 // second word (~2^-48 of the terms, which cancel in D x), and the intermediate
 // D x is stored as a double-word pair.  Measured against the FP64 operator on
-// the 24^3 x 48 stout-smeared field: 2.5e-14 ||x|| for Gaussian x, 3.7e-14
+// the 24^3 x 48 stout-smeared field: 1.8e-14 ||x|| for Gaussian x, 2.0e-14
 // ||x|| for a smooth x (the low-mode shape of the small shifts' solutions);
 // the bound takes 1e-13.
 constexpr double kDwRelErr = 1e-13;
